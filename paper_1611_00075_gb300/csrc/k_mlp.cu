@@ -20,8 +20,10 @@ constexpr int kH = 32;
 constexpr int kNP = kH * 3 + kH + kH * kH + kH + kH + 1;  // 1217
 constexpr int kOffB1 = kH * 3, kOffW2 = kOffB1 + kH, kOffB2 = kOffW2 + kH * kH,
               kOffW3 = kOffB2 + kH, kOffB3 = kOffW3 + kH;
-constexpr int kMS = 64;        // samples per block in the gradient kernel
-constexpr int kGradThreads = 128;
+// Gradient kernel: warps of 32 samples; blocks of four warps, three per SM.
+constexpr int kGradWarps = 4;
+constexpr int kGradBlocks = 152 * 3;
+constexpr int kRow = kH + 4;  // padded row of a sample's 32 activations (conflict-free float4s)
 
 namespace {
 
@@ -54,107 +56,217 @@ __global__ void mlp_forward_kernel(const float *__restrict__ X, long long ns,
     }
 }
 
-// Stage 1: each block back-propagates kMS samples and writes its partial
-// gradient (sum over its samples) and partial squared-error sum.
-__global__ void __launch_bounds__(kGradThreads)
+// Shared memory of the gradient kernel: the weights, the products
+// V[u][k] = W2[u][k] W3[u], and per warp three arrays of 32 sample rows.
+struct GradSmem {
+    float P[(kNP + 3) & ~3];
+    float V[kH * kH];
+    float4 x[kGradWarps][32];  // a sample's inputs and dL/dyhat
+    float a1[kGradWarps][32][kRow];
+    float d2[kGradWarps][32][kRow];  // dL/dyhat where unit u of layer 2 is active, else 0
+    float s1[kGradWarps][32][kRow];  // layer 2's activations, later dL/dz of layer 1
+};
+
+// Stage 1: partial gradient (a sum over the block's samples) and partial
+// squared-error sum of every block.
+//
+// One warp takes 32 samples at a time.  First a lane is a sample: forward and
+// backward pass in registers against weights broadcast from shared memory
+// (one 16-byte read feeds four multiply-adds).  Then a lane is a tile of the
+// gradient: the layer-2 gradient sum_s d2[s][u] a1[s][k] is a 32 x 32 x 32
+// product, eight u by four k per lane, three 16-byte reads per 32
+// multiply-adds, accumulated in registers over all of the warp's groups.  With
+// d2[s][u] = dy_s W3[u] [z2_u > 0], W3[u] is a common factor of row u and is
+// multiplied in once per block, not per sample.  About 3,400 multiply-adds per
+// sample: FP32-bound.  One block holds 66 KB of shared memory, three run per SM, and
+// the grid is at most one wave, so the second stage adds 456 partials at most
+// (one block per 64 samples before: 8,457 partials of 41 MB, added by one
+// serial thread per parameter in 0.92 ms at 541,199 samples).
+__global__ void __launch_bounds__(32 * kGradWarps, 3)
 mlp_grad_partial_kernel(const float *__restrict__ X, const float *__restrict__ Y, long long ns,
                         const float *__restrict__ P, float *__restrict__ partial,
                         float *__restrict__ lossp) {
-    __shared__ float sP[kNP];
-    __shared__ float sx[kMS][3];
-    __shared__ float sa1[kMS][kH + 1], sd1[kMS][kH + 1], sa2[kMS][kH + 1], sd2[kMS][kH + 1];
-    __shared__ float sdy[kMS], sl[kMS];
-    for (int k = threadIdx.x; k < kNP; k += blockDim.x) sP[k] = P[k];
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    GradSmem &sm = *reinterpret_cast<GradSmem *>(smem_raw);
+    for (int k = threadIdx.x; k < kNP; k += blockDim.x) sm.P[k] = P[k];
     __syncthreads();
-    const float *W1 = sP, *b1 = sP + kOffB1, *W2 = sP + kOffW2, *b2 = sP + kOffB2,
-                *W3 = sP + kOffW3;
-    const int t = threadIdx.x;
-    if (t < kMS) {
-        const long long s = (long long)blockIdx.x * kMS + t;
+    for (int k = threadIdx.x; k < kH * kH; k += blockDim.x)
+        sm.V[k] = sm.P[kOffW2 + k] * sm.P[kOffW3 + k / kH];
+    __syncthreads();
+    const float *W1 = sm.P, *b1 = sm.P + kOffB1, *W2 = sm.P + kOffW2, *b2 = sm.P + kOffB2,
+                *W3 = sm.P + kOffW3;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const int ti = (lane >> 3) * 8, tj = (lane & 7) * 4;  // the lane's tile of the layer-2 gradient
+    float g2[8][4];
+#pragma unroll
+    for (int u = 0; u < 8; ++u)
+#pragma unroll
+        for (int k = 0; k < 4; ++k) g2[u][k] = 0.f;
+    float g1x = 0.f, g1y = 0.f, g1z = 0.f, gb1 = 0.f, gb2 = 0.f, g3 = 0.f, gb3 = 0.f, lsum = 0.f;
+    const float inv2 = 2.f / (float)ns;
+    const long long groups = (ns + 31) >> 5;
+    const long long stride = (long long)gridDim.x * kGradWarps;
+    for (long long gr = (long long)blockIdx.x * kGradWarps + wid; gr < groups; gr += stride) {
+        const long long s = gr * 32 + lane;
         const bool ok = s < ns;
         const float x0 = ok ? X[3 * s] : 0.f, x1 = ok ? X[3 * s + 1] : 0.f,
                     x2 = ok ? X[3 * s + 2] : 0.f;
-        sx[t][0] = x0; sx[t][1] = x1; sx[t][2] = x2;
-        float z1[kH], a1[kH];
+        float a1[kH];
+        unsigned m1 = 0;  // active units of layer 1
 #pragma unroll
         for (int u = 0; u < kH; ++u) {
-            float z = b1[u] + W1[3 * u] * x0 + W1[3 * u + 1] * x1 + W1[3 * u + 2] * x2;
-            z1[u] = z;
+            const float z = b1[u] + W1[3 * u] * x0 + W1[3 * u + 1] * x1 + W1[3 * u + 2] * x2;
             a1[u] = z > 0.f ? z : 0.f;
-            sa1[t][u] = ok ? a1[u] : 0.f;
+            m1 |= z > 0.f ? 1u << u : 0u;
         }
-        float yh = sP[kOffB3];
-        for (int u = 0; u < kH; ++u) {
-            float z = b2[u];
 #pragma unroll
-            for (int k = 0; k < kH; ++k) z += W2[kH * u + k] * a1[k];
-            const float a2 = z > 0.f ? z : 0.f;
-            sa2[t][u] = ok ? a2 : 0.f;
-            sd2[t][u] = z > 0.f ? 1.f : 0.f;  // ReLU mask for now
-            yh += W3[u] * a2;
+        for (int u = 0; u < kH; u += 4)
+            *reinterpret_cast<float4 *>(&sm.a1[wid][lane][u]) =
+                make_float4(a1[u], a1[u + 1], a1[u + 2], a1[u + 3]);
+        float yh = sm.P[kOffB3];
+        unsigned m2 = 0;  // active units of layer 2
+#pragma unroll 1
+        for (int u = 0; u < kH; u += 4) {
+            float z[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) z[q] = b2[u + q];
+#pragma unroll
+            for (int k = 0; k < kH; k += 4)
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    const float4 w = *reinterpret_cast<const float4 *>(W2 + kH * (u + q) + k);
+                    z[q] += w.x * a1[k];
+                    z[q] += w.y * a1[k + 1];
+                    z[q] += w.z * a1[k + 2];
+                    z[q] += w.w * a1[k + 3];
+                }
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                m2 |= z[q] > 0.f ? 1u << (u + q) : 0u;
+                z[q] = z[q] > 0.f ? z[q] : 0.f;
+                yh += W3[u + q] * z[q];
+            }
+            *reinterpret_cast<float4 *>(&sm.s1[wid][lane][u]) = make_float4(z[0], z[1], z[2], z[3]);
         }
         const float e = ok ? yh - Y[s] : 0.f;
-        const float dy = ok ? 2.f * e / (float)ns : 0.f;
-        sdy[t] = dy;
-        sl[t] = e * e;
-        float d2[kH];
+        const float dy = e * inv2;
+        lsum += e * e;
+        sm.x[wid][lane] = make_float4(x0, x1, x2, dy);
 #pragma unroll
+        for (int u = 0; u < kH; u += 4)
+            *reinterpret_cast<float4 *>(&sm.d2[wid][lane][u]) =
+                make_float4((m2 >> u) & 1u ? dy : 0.f, (m2 >> (u + 1)) & 1u ? dy : 0.f,
+                            (m2 >> (u + 2)) & 1u ? dy : 0.f, (m2 >> (u + 3)) & 1u ? dy : 0.f);
+        __syncwarp();
+        // output layer: lane k adds dy_s a2[s][k]
+        for (int t = 0; t < 32; ++t) g3 += sm.x[wid][t].w * sm.s1[wid][t][lane];
+        gb3 += dy;
+        __syncwarp();
+        // dL/da1[k] = dy sum_u [z2_u > 0] V[u][k]
+        float acc[kH];
+#pragma unroll
+        for (int k = 0; k < kH; ++k) acc[k] = 0.f;
+#pragma unroll 2
         for (int u = 0; u < kH; ++u) {
-            d2[u] = sd2[t][u] * dy * W3[u];
-            sd2[t][u] = d2[u];
+            const float on = (m2 >> u) & 1u ? 1.f : 0.f;
+#pragma unroll
+            for (int k = 0; k < kH; k += 4) {
+                const float4 v = *reinterpret_cast<const float4 *>(sm.V + kH * u + k);
+                acc[k] += on * v.x;
+                acc[k + 1] += on * v.y;
+                acc[k + 2] += on * v.z;
+                acc[k + 3] += on * v.w;
+            }
         }
 #pragma unroll
-        for (int k = 0; k < kH; ++k) {
-            float acc = 0.f;
-            for (int u = 0; u < kH; ++u) acc += W2[kH * u + k] * d2[u];
-            sd1[t][k] = z1[k] > 0.f ? acc : 0.f;
+        for (int k = 0; k < kH; k += 4)
+            *reinterpret_cast<float4 *>(&sm.s1[wid][lane][k]) =
+                make_float4((m1 >> k) & 1u ? dy * acc[k] : 0.f,
+                            (m1 >> (k + 1)) & 1u ? dy * acc[k + 1] : 0.f,
+                            (m1 >> (k + 2)) & 1u ? dy * acc[k + 2] : 0.f,
+                            (m1 >> (k + 3)) & 1u ? dy * acc[k + 3] : 0.f);
+        __syncwarp();
+#pragma unroll 4
+        for (int t = 0; t < 32; ++t) {
+            const float4 da = *reinterpret_cast<const float4 *>(&sm.d2[wid][t][ti]);
+            const float4 db = *reinterpret_cast<const float4 *>(&sm.d2[wid][t][ti + 4]);
+            const float4 av = *reinterpret_cast<const float4 *>(&sm.a1[wid][t][tj]);
+            const float d[8] = {da.x, da.y, da.z, da.w, db.x, db.y, db.z, db.w};
+#pragma unroll
+            for (int u = 0; u < 8; ++u) {
+                g2[u][0] += d[u] * av.x;
+                g2[u][1] += d[u] * av.y;
+                g2[u][2] += d[u] * av.z;
+                g2[u][3] += d[u] * av.w;
+            }
+            const float4 xs = sm.x[wid][t];
+            const float e1 = sm.s1[wid][t][lane];
+            g1x += e1 * xs.x;
+            g1y += e1 * xs.y;
+            g1z += e1 * xs.z;
+            gb1 += e1;
+            gb2 += sm.d2[wid][t][lane];
         }
+        __syncwarp();  // the rows are rewritten by the next group
+    }
+    // the warp's sums to shared memory, in the parameter layout, then a
+    // fixed-order sum over the warps
+    __syncthreads();
+    float *red = &sm.a1[0][0][0];  // kGradWarps x kNP: fits in the a1 and d2 rows
+    static_assert(kGradWarps * kNP <= 2 * kGradWarps * 32 * kRow, "block sums fit");
+    float *w = red + wid * kNP;
+#pragma unroll
+    for (int u = 0; u < 8; ++u)
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+            w[kOffW2 + kH * (ti + u) + tj + k] = g2[u][k] * W3[ti + u];
+    w[3 * lane] = g1x;
+    w[3 * lane + 1] = g1y;
+    w[3 * lane + 2] = g1z;
+    w[kOffB1 + lane] = gb1;
+    w[kOffB2 + lane] = gb2 * W3[lane];
+    w[kOffW3 + lane] = g3;
+    for (int o = 16; o > 0; o >>= 1) {
+        gb3 += __shfl_down_sync(0xffffffffu, gb3, o);
+        lsum += __shfl_down_sync(0xffffffffu, lsum, o);
+    }
+    float *wl = &sm.s1[0][0][0];
+    if (lane == 0) {
+        w[kOffB3] = gb3;
+        wl[wid] = lsum;
     }
     __syncthreads();
     float *out = partial + (size_t)blockIdx.x * kNP;
-    for (int p = t; p < kNP; p += blockDim.x) {
-        float acc = 0.f;
-        if (p < kOffB1) {
-            const int u = p / 3, c = p % 3;
-            for (int s = 0; s < kMS; ++s) acc += sd1[s][u] * sx[s][c];
-        } else if (p < kOffW2) {
-            const int u = p - kOffB1;
-            for (int s = 0; s < kMS; ++s) acc += sd1[s][u];
-        } else if (p < kOffB2) {
-            const int u = (p - kOffW2) / kH, k = (p - kOffW2) % kH;
-            for (int s = 0; s < kMS; ++s) acc += sd2[s][u] * sa1[s][k];
-        } else if (p < kOffW3) {
-            const int u = p - kOffB2;
-            for (int s = 0; s < kMS; ++s) acc += sd2[s][u];
-        } else if (p < kOffB3) {
-            const int k = p - kOffW3;
-            for (int s = 0; s < kMS; ++s) acc += sdy[s] * sa2[s][k];
-        } else {
-            for (int s = 0; s < kMS; ++s) acc += sdy[s];
-        }
-        out[p] = acc;
+    for (int p = threadIdx.x; p < kNP; p += blockDim.x) {
+        float t = red[p];
+#pragma unroll
+        for (int q = 1; q < kGradWarps; ++q) t += red[q * kNP + p];
+        out[p] = t;
     }
-    if (t == 0) {
-        float l = 0.f;
-        for (int s = 0; s < kMS; ++s) l += sl[s];
-        lossp[blockIdx.x] = l;
-    }
+    if (threadIdx.x == 0) lossp[blockIdx.x] = (wl[0] + wl[1]) + (wl[2] + wl[3]);
+    static_assert(kGradWarps == 4, "the sum above");
 }
 
-// Stage 2: fixed-order sums over blocks.
-__global__ void mlp_grad_reduce_kernel(const float *__restrict__ partial,
-                                       const float *__restrict__ lossp, int nblk, long long ns,
-                                       float *__restrict__ G, float *__restrict__ loss) {
-    const int p = blockIdx.x * blockDim.x + threadIdx.x;
-    if (p < kNP) {
-        float acc = 0.f;
-        for (int b = 0; b < nblk; ++b) acc += partial[(size_t)b * kNP + p];
-        G[p] = acc;
-    } else if (p == kNP && loss) {
-        double l = 0.0;
-        for (int b = 0; b < nblk; ++b) l += lossp[b];
-        *loss = (float)(l / (double)ns);
-    }
+// Stage 2: fixed-order sums over the blocks' partials, in float64.  A block
+// takes 32 parameters; its eight warps take every eighth partial.
+__global__ void __launch_bounds__(256)
+mlp_grad_reduce_kernel(const float *__restrict__ partial, const float *__restrict__ lossp,
+                       int nblk, long long ns, float *__restrict__ G, float *__restrict__ loss) {
+    __shared__ double part[8][32];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const int p = blockIdx.x * 32 + lane;
+    const bool is_loss = p == kNP;
+    double acc = 0.0;
+    if (p < kNP)
+        for (int b = wid; b < nblk; b += 8) acc += (double)partial[(size_t)b * kNP + p];
+    else if (is_loss)
+        for (int b = wid; b < nblk; b += 8) acc += (double)lossp[b];
+    part[wid][lane] = acc;
+    __syncthreads();
+    if (wid != 0) return;
+    for (int q = 1; q < 8; ++q) acc += part[q][lane];
+    if (p < kNP) G[p] = (float)acc;
+    else if (is_loss && loss) *loss = (float)(acc / (double)ns);
 }
 
 __global__ void adam_kernel(float *__restrict__ P, const float *__restrict__ G,
@@ -229,19 +341,28 @@ cudaError_t launch_mlp_forward(const float *X, long long ns, const float *P, flo
 }
 
 // scratch: at least mlp_grad_scratch_floats(ns) floats
+static int mlp_grad_blocks(long long ns) {
+    const long long nb = (ns + 32 * kGradWarps - 1) / (32 * kGradWarps);
+    return (int)(nb < kGradBlocks ? nb : kGradBlocks);
+}
 size_t mlp_grad_scratch_floats(long long ns) {
-    const long long nblk = (ns + kMS - 1) / kMS;
-    return (size_t)nblk * (kNP + 1) + 1;
+    return (size_t)mlp_grad_blocks(ns) * (kNP + 1) + 1;
 }
 
 cudaError_t launch_mlp_loss_grad(const float *X, const float *Y, long long ns, const float *P,
                                  float *G, float *loss, float *scratch, cudaStream_t s) {
-    const int nblk = (int)((ns + kMS - 1) / kMS);
+    const int nblk = mlp_grad_blocks(ns);
     float *partial = scratch;
     float *lossp = scratch + (size_t)nblk * kNP;
-    mlp_grad_partial_kernel<<<nblk, kGradThreads, 0, s>>>(X, Y, ns, P, partial, lossp);
-    mlp_grad_reduce_kernel<<<(kNP + 1 + kBlock - 1) / kBlock, kBlock, 0, s>>>(partial, lossp, nblk,
-                                                                            ns, G, loss);
+    // over 48 KB of shared memory: set on every call (a host-side attribute of
+    // the function on the current device)
+    cudaError_t e = cudaFuncSetAttribute(mlp_grad_partial_kernel,
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)sizeof(GradSmem));
+    if (e != cudaSuccess) return e;
+    mlp_grad_partial_kernel<<<nblk, 32 * kGradWarps, sizeof(GradSmem), s>>>(X, Y, ns, P, partial,
+                                                                           lossp);
+    mlp_grad_reduce_kernel<<<(kNP + 1 + 31) / 32, 256, 0, s>>>(partial, lossp, nblk, ns, G, loss);
     return cudaGetLastError();
 }
 
