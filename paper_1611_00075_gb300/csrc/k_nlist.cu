@@ -10,6 +10,10 @@
 // float64 arithmetic only runs for candidates whose float32 distance lies in
 // a thin band around r_list^2; outside the band the float32 result cannot
 // decide differently (its error bound is far below the band's half width).
+// Both precisions build this way: the float32 positions are kept on the float64
+// path too, and the accepted set is the float64 definition's either way (4,000
+// atoms in float64: 50 steps with six builds 11.9 -> 9.1 ms against float64
+// distances for every candidate, on a pipe of 1/64 of the float32 rate).
 //
 // List layout: see list_idx() -- per warp group of 32 atoms, quads of four
 // entries per atom, written here with one 16-byte store per quad.  An entry is
@@ -58,7 +62,6 @@ __device__ __forceinline__ void stencil_shift64(const Grid &g, int cx, int cy, i
 
 // How the acceptance r^2 < r_list^2 is decided for one atom's candidates.
 enum ListMode {
-    LM_EXACT = 0,  // float64 definition for every candidate (float64 path)
     LM_BAND = 1,   // float32 prefilter; band candidates tested in float64 at once
     LM_DEFER = 2,  // float32 prefilter; band candidates accepted, verified after
 };
@@ -87,7 +90,6 @@ __device__ __forceinline__ int list_atom(int i, const Grid &g, float lo, float h
     const int cx = c % g.nx, cy = (c / g.nx) % g.ny, cz = c / (g.nx * g.ny);
     const float4 qi = xq[i];
     const int myo = __float_as_int(qi.w);
-    const double4 ai = (LM == LM_EXACT) ? xabs[i] : make_double4(0.0, 0.0, 0.0, 0.0);
     for (int dz = -1; dz <= 1; ++dz) {
         int zz = cz + dz;
         double shz = 0.0;
@@ -138,20 +140,12 @@ __device__ __forceinline__ int list_atom(int i, const Grid &g, float lo, float h
 #pragma unroll 4
                     for (int j = b; j < e; ++j) {
                         const float4 qj = xq[j];
-                        float r2f = 0.f;
-                        bool cand = true;
-                        if (LM == LM_BAND) {
-                            const float ex = qj.x - hx, ey = qj.y - hy, ez = qj.z - hz;
-                            r2f = ex * ex + ey * ey + ez * ez;
-                            cand = r2f < hi;
-                        }
-                        cand = cand && (j != skip);
+                        const float ex = qj.x - hx, ey = qj.y - hy, ez = qj.z - hz;
+                        const float r2f = ex * ex + ey * ey + ez * ez;
+                        bool cand = (r2f < hi) && (j != skip);
                         if (HALF) cand = cand && (__float_as_int(qj.w) > myo);
                         if (!cand) continue;
-                        bool acc = true;
-                        if (LM == LM_EXACT) acc = exact_within(ai, xabs[j], shx, shy, shz, rl2);
-                        else if (r2f >= lo) acc = exact_within_band(xabs, i, j, shx, shy, shz, rl2);
-                        if (!acc) continue;
+                        if (r2f >= lo && !exact_within_band(xabs, i, j, shx, shy, shz, rl2)) continue;
                         if (WRITE && cnt < cap)
                             row[(size_t)(((cnt >> 2) << 7) | (cnt & 3))] = sbits | (uint32_t)j;
                         ++cnt;
@@ -179,7 +173,7 @@ __device__ __noinline__ int list_atom_band(int i, const Grid &g, float lo, float
 // 128-thread blocks measured 1 % faster than 256 for this kernel.
 constexpr int kListBlock = 128;
 
-template <bool PREFILTER, bool WRITE, bool HALF>
+template <bool WRITE, bool HALF>
 __global__ void __launch_bounds__(kListBlock)
 build_list_kernel(int n, const Grid *__restrict__ grids, const uint16_t *__restrict__ rep,
                   float lo, float hi, double rl2, const float4 *__restrict__ xq,
@@ -195,36 +189,30 @@ build_list_kernel(int n, const Grid *__restrict__ grids, const uint16_t *__restr
         // entry k of atom i: row[(k / 4) * 128 + k % 4]
         uint32_t *row = nlist + list_group(i, cap) + ((i & 31) << 2);
         BandNote band{0, 0, 0, 0};
-        int cnt;
-        if (!PREFILTER) {
-            cnt = list_atom<LM_EXACT, WRITE, HALF>(i, g, lo, hi, rl2, xq, xabs, c, start, row, cap,
-                                                   band);
-        } else {
-            cnt = list_atom<LM_DEFER, WRITE, HALF>(i, g, lo, hi, rl2, xq, xabs, c, start, row, cap,
-                                                   band);
-            if (band.count == 1 && WRITE && band.k >= cap) {
-                overflow = 1;  // the entry was not stored: the row is regrown anyway
-            } else if (band.count == 1) {
-                // verify the one provisional entry; drop it if the float64
-                // definition rejects it
-                if (WRITE) {
-                    const uint32_t ent = row[row_off(band.k)];
-                    band.j = (int)(ent & kIndexMask);
-                    band.s = (int)(ent >> kIndexBits);
-                }
-                const int cx = c % g.nx, cy = (c / g.nx) % g.ny, cz = c / (g.nx * g.ny);
-                double shx, shy, shz;
-                stencil_shift64(g, cx, cy, cz, band.s, shx, shy, shz);
-                if (!exact_within_band(xabs, i, band.j, shx, shy, shz, rl2)) {
-                    overflow |= (cnt > cap);  // a full row lost its tail: regrow
-                    if (WRITE)
-                        for (int k = band.k; k + 1 < min(cnt, cap); ++k)
-                            row[row_off(k)] = row[row_off(k + 1)];
-                    --cnt;
-                }
-            } else if (band.count > 1) {
-                cnt = list_atom_band<WRITE, HALF>(i, g, lo, hi, rl2, xq, xabs, c, start, row, cap);
+        int cnt = list_atom<LM_DEFER, WRITE, HALF>(i, g, lo, hi, rl2, xq, xabs, c, start, row,
+                                                   cap, band);
+        if (band.count == 1 && WRITE && band.k >= cap) {
+            overflow = 1;  // the entry was not stored: the row is regrown anyway
+        } else if (band.count == 1) {
+            // verify the one provisional entry; drop it if the float64
+            // definition rejects it
+            if (WRITE) {
+                const uint32_t ent = row[row_off(band.k)];
+                band.j = (int)(ent & kIndexMask);
+                band.s = (int)(ent >> kIndexBits);
             }
+            const int cx = c % g.nx, cy = (c / g.nx) % g.ny, cz = c / (g.nx * g.ny);
+            double shx, shy, shz;
+            stencil_shift64(g, cx, cy, cz, band.s, shx, shy, shz);
+            if (!exact_within_band(xabs, i, band.j, shx, shy, shz, rl2)) {
+                overflow |= (cnt > cap);  // a full row lost its tail: regrow
+                if (WRITE)
+                    for (int k = band.k; k + 1 < min(cnt, cap); ++k)
+                        row[row_off(k)] = row[row_off(k + 1)];
+                --cnt;
+            }
+        } else if (band.count > 1) {
+            cnt = list_atom_band<WRITE, HALF>(i, g, lo, hi, rl2, xq, xabs, c, start, row, cap);
         }
         if (WRITE && cnt <= cap) {
             // pad the last quad with self-entries that no cutoff accepts
@@ -316,21 +304,15 @@ cudaError_t launch_build_list(md_system *h, bool write, bool gated, const float4
     int n = (int)h->n;
     cudaStream_t s = h->stream;
     const float4 *xq = positions ? positions : h->xq[h->cur];
-    const bool prefilter = (h->p.precision == MD_MIXED);
     const bool half = half_variant(h->p.force_variant);
     reset_max_count_kernel<<<1, 1, 0, s>>>(h->ds, gated);
-#define MDG_LIST(PF, WR, HF)                                                                    \
-    build_list_kernel<PF, WR, HF><<<gs_blocks(n) * (kBlock / kListBlock), kListBlock, 0, s>>>(                                \
+#define MDG_LIST(WR, HF)                                                                    \
+    build_list_kernel<WR, HF><<<gs_blocks(n) * (kBlock / kListBlock), kListBlock, 0, s>>>(                                \
         n, h->grids, h->rep, h->list_lo, h->list_hi, h->rl2, xq, h->xabs, h->cell,           \
         h->cell_start,                                                                         \
         h->nlist, h->ncount, h->cap, h->ds, gated)
-    if (prefilter) {
-        if (write) { if (half) MDG_LIST(true, true, true); else MDG_LIST(true, true, false); }
-        else { if (half) MDG_LIST(true, false, true); else MDG_LIST(true, false, false); }
-    } else {
-        if (write) { if (half) MDG_LIST(false, true, true); else MDG_LIST(false, true, false); }
-        else { if (half) MDG_LIST(false, false, true); else MDG_LIST(false, false, false); }
-    }
+    if (write) { if (half) MDG_LIST(true, true); else MDG_LIST(true, false); }
+    else { if (half) MDG_LIST(false, true); else MDG_LIST(false, false); }
 #undef MDG_LIST
     return cudaGetLastError();
 }
