@@ -91,7 +91,7 @@ __global__ void __launch_bounds__(kBlock, 4) eam_density_mixed(ForceArgs a, EamT
             const float ey = (qj.y - qi.y) + sh.y[st];
             const float ez = (qj.z - qi.z) + sh.z[st];
             const float r2 = ex * ex + ey * ey + ez * ez;
-            if (r2 < rc2) r += pieces_f32<NPSI>(t.qr, t.qa, t.npsi, r2 * rsqrtf(r2), nullptr);
+            if (r2 < rc2) r += pieces_f32<NPSI>(t.qr, t.qa, t.npsi, r2 * rsqrt_fast(r2), nullptr);
         };
         for (int q = q0; q < q1; ++q) {
             const uint4 e4 = nxt;
@@ -169,7 +169,7 @@ __global__ void __launch_bounds__(kBlock, 4) eam_force_mixed(ForceArgs a, EamTab
             const float ez = (qj.z - qi.z) + sh.z[st];
             const float r2 = ex * ex + ey * ey + ez * ez;
             if (r2 < rc2) {
-                const float rinv = rsqrtf(r2);
+                const float rinv = rsqrt_fast(r2);
                 const float r = r2 * rinv;
                 float dPhi, dpsi;
                 const float Phi = pieces_f32<NPHI>(t.pr, t.pa, t.nphi, r, &dPhi);
@@ -324,7 +324,7 @@ __global__ void __launch_bounds__(kEamPairBlock, 8) eam_density_pair(ForceArgs a
         // the slot's own pair adds to both densities
         const float ex = q1.x - q0.x, ey = q1.y - q0.y, ez = q1.z - q0.z;
         const float r2 = ex * ex + ey * ey + ez * ez;
-        if (r2 < rc2) r = dup2(pieces_f32<NPSI>(t.qr, t.qa, t.npsi, r2 * rsqrtf(r2), nullptr));
+        if (r2 < rc2) r = dup2(pieces_f32<NPSI>(t.qr, t.qa, t.npsi, r2 * rsqrt_fast(r2), nullptr));
     }
     const float2 nqx = make_float2(-q0.x, -q1.x), nqy = make_float2(-q0.y, -q1.y),
                  nqz = make_float2(-q0.z, -q1.z);
@@ -336,7 +336,7 @@ __global__ void __launch_bounds__(kEamPairBlock, 8) eam_density_pair(ForceArgs a
         const float tx = qj.x + sh.x[st], ty = qj.y + sh.y[st], tz = qj.z + sh.z[st];
         const float2 dx = add2(dup2(tx), nqx), dy = add2(dup2(ty), nqy), dz = add2(dup2(tz), nqz);
         const float2 r2 = fma2(dz, dz, fma2(dy, dy, mul2(dx, dx)));
-        const float2 rr = mul2(r2, make_float2(rsqrtf(r2.x), rsqrtf(r2.y)));
+        const float2 rr = mul2(r2, make_float2(rsqrt_fast(r2.x), rsqrt_fast(r2.y)));
         r = add2(r, pieces_pair<NPSI, false>(t.qr, t.qa, t.npsi, rr, nullptr));
     };
     double R0 = 0.0, R1 = 0.0;
@@ -413,7 +413,7 @@ __global__ void __launch_bounds__(kEamPairBlock, 8) eam_force_pair(ForceArgs a, 
         const float ex = q1.x - q0.x, ey = q1.y - q0.y, ez = q1.z - q0.z;
         const float r2 = ex * ex + ey * ey + ez * ez;
         if (r2 < rc2) {
-            const float rinv = rsqrtf(r2);
+            const float rinv = rsqrt_fast(r2);
             const float rr = r2 * rinv;
             float dPhi, dpsi;
             const float Phi = pieces_f32<NPHI>(t.pr, t.pa, t.nphi, rr, &dPhi);
@@ -439,7 +439,7 @@ __global__ void __launch_bounds__(kEamPairBlock, 8) eam_force_pair(ForceArgs a, 
         const float tx = qj.x + sh.x[st], ty = qj.y + sh.y[st], tz = qj.z + sh.z[st];
         const float2 dx = add2(dup2(tx), nqx), dy = add2(dup2(ty), nqy), dz = add2(dup2(tz), nqz);
         const float2 r2 = fma2(dz, dz, fma2(dy, dy, mul2(dx, dx)));
-        const float2 rinv = make_float2(rsqrtf(r2.x), rsqrtf(r2.y));
+        const float2 rinv = make_float2(rsqrt_fast(r2.x), rsqrt_fast(r2.y));
         const float2 rr = mul2(r2, rinv);
         float2 dPhi, dpsi;
         const float2 Phi = pieces_pair<NPHI, true>(t.pr, t.pa, t.nphi, rr, &dPhi);

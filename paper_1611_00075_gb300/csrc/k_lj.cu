@@ -54,7 +54,7 @@ __device__ __forceinline__ void lj_mixed_atom(const ForceArgs &a, const ShiftTab
         const float ez = (qj.z - qi.z) + sf.z;
         const float r2 = ex * ex + ey * ey + ez * ez;
         if (r2 < rc2) {
-            const float r2i = __fdividef(1.0f, r2);
+            const float r2i = rcp_fast(r2);
             float s6 = sig2 * r2i;
             s6 = s6 * s6 * s6;
             const float fs = e48 * r2i * s6 * (s6 - 0.5f);
@@ -470,7 +470,7 @@ __device__ __forceinline__ void lj_typed_mixed_atom(const ForceArgs &a, const Ty
         const float r2 = ex * ex + ey * ey + ez * ez;
         if (r2 < rc2) {
             const int tj = species_of(__float_as_uint(qj.w));
-            const float r2i = __fdividef(1.0f, r2);
+            const float r2i = rcp_fast(r2);
             float s6 = pick_row<NT>(s2, tj) * r2i;
             s6 = s6 * s6 * s6;
             const float fs = pick_row<NT>(e48, tj) * r2i * s6 * (s6 - 0.5f);

@@ -111,7 +111,7 @@ __device__ __forceinline__ void split_pair_loop(const ForceArgs &a, const Overla
         const float ez = (qj.z - qi.z) + sh->z[st];
         const float r2 = ex * ex + ey * ey + ez * ez;
         if (mine && r2 < rc2) {
-            const float r2i = __fdividef(1.0f, r2);
+            const float r2i = rcp_fast(r2);
             float s6 = sig2 * r2i;
             s6 = s6 * s6 * s6;
             const float fs = e48 * r2i * s6 * (s6 - 0.5f);

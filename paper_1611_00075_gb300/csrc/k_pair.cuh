@@ -41,7 +41,7 @@ template <bool ENERGY>
 __device__ __forceinline__ void lj_term(const ForceConsts &fc, float ex, float ey, float ez,
                                         float r2, float &fx, float &fy, float &fz, float &en,
                                         unsigned &np) {
-    const float r2i = __fdividef(1.0f, r2);
+    const float r2i = rcp_fast(r2);
     float s6 = fc.sig2f * r2i;
     s6 = s6 * s6 * s6;
     const float fs = fc.eps48f * r2i * s6 * (s6 - 0.5f);
@@ -145,7 +145,7 @@ __device__ __forceinline__ void lj_pair_slot(const ForceArgs &a, const PairArgs 
         const float tx = qj.x + sf.x, ty = qj.y + sf.y, tz = qj.z + sf.z;
         const float2 dx = add2(dup2(tx), nqx), dy = add2(dup2(ty), nqy), dz = add2(dup2(tz), nqz);
         const float2 r2 = fma2(dz, dz, fma2(dy, dy, mul2(dx, dx)));
-        const float2 r2i = make_float2(__fdividef(1.0f, r2.x), __fdividef(1.0f, r2.y));
+        const float2 r2i = make_float2(rcp_fast(r2.x), rcp_fast(r2.y));
         const float2 s2 = mul2(dup2(a.fc.sig2f), r2i);
         const float2 s6 = mul2(mul2(s2, s2), s2);
         float2 nfs = mul2(mul2(fma2(s6, dup2(-a.fc.eps48f), dup2(0.5f * a.fc.eps48f)), s6), r2i);

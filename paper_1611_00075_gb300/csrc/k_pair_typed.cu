@@ -95,7 +95,7 @@ lj_typed_pair_kernel(ForceArgs a, PairArgs p, TypeTab tt, int store_f) {
         const float ex = q1.x - q0.x, ey = q1.y - q0.y, ez = q1.z - q0.z;
         const float r2 = ex * ex + ey * ey + ez * ez;
         if (r2 < rc2) {
-            const float r2i = __fdividef(1.0f, r2);
+            const float r2i = rcp_fast(r2);
             float s6 = row_at<NT>(s2a, t1) * r2i;
             s6 = s6 * s6 * s6;
             const float fs = row_at<NT>(e48a, t1) * r2i * s6 * (s6 - 0.5f);
@@ -121,7 +121,7 @@ lj_typed_pair_kernel(ForceArgs a, PairArgs p, TypeTab tt, int store_f) {
         const float tx = qj.x + sh.x[st], ty = qj.y + sh.y[st], tz = qj.z + sh.z[st];
         const float2 dx = add2(dup2(tx), nqx), dy = add2(dup2(ty), nqy), dz = add2(dup2(tz), nqz);
         const float2 r2 = fma2(dz, dz, fma2(dy, dy, mul2(dx, dx)));
-        const float2 r2i = make_float2(__fdividef(1.0f, r2.x), __fdividef(1.0f, r2.y));
+        const float2 r2i = make_float2(rcp_fast(r2.x), rcp_fast(r2.y));
         const float2 s2 = mul2(make_float2(row_at<NT>(s2a, tj), row_at<NT>(s2b, tj)), r2i);
         const float2 s6 = mul2(mul2(s2, s2), s2);
         const float2 e48 = make_float2(row_at<NT>(e48a, tj), row_at<NT>(e48b, tj));

@@ -101,10 +101,10 @@ __global__ void __launch_bounds__(kBlock, 4) sc_density_mixed(ForceArgs a) {
             const float ez = (qj.z - qi.z) + sh.z[st];
             const float r2 = ex * ex + ey * ey + ez * ez;
             if (r2 < rc2) {
-                const float s = a2 * __fdividef(1.0f, r2);
+                const float s = a2 * rcp_fast(r2);
                 float psi;
-                if (ME > 0) psi = ar_pow<ME>(s, (ME & 1) ? af * rsqrtf(r2) : 0.f);
-                else psi = (m & 1) ? rpow(s, m / 2) * af * rsqrtf(r2) : rpow(s, m / 2);
+                if (ME > 0) psi = ar_pow<ME>(s, (ME & 1) ? af * rsqrt_fast(r2) : 0.f);
+                else psi = (m & 1) ? rpow(s, m / 2) * af * rsqrt_fast(r2) : rpow(s, m / 2);
                 r += psi;
             }
         };
@@ -191,8 +191,8 @@ __global__ void __launch_bounds__(kBlock, 4) sc_force_mixed(ForceArgs a, int sto
                 // with an odd exponent a/r comes from one reciprocal square
                 // root, and (a/r)^2 and 1/r^2 from it without a reciprocal
                 const bool odd = (NE > 0) ? ((NE | ME) & 1) : ((nexp | mexp) & 1);
-                const float ar = odd ? af * rsqrtf(r2) : 0.f;
-                const float r2i = odd ? ar * ar * inv_a2 : __fdividef(1.0f, r2);
+                const float ar = odd ? af * rsqrt_fast(r2) : 0.f;
+                const float r2i = odd ? ar * ar * inv_a2 : rcp_fast(r2);
                 const float s = odd ? ar * ar : a2 * r2i;
                 float Phi, psi;
                 if (NE > 0) {
@@ -338,9 +338,9 @@ __global__ void __launch_bounds__(kScPairBlock, 8) sc_density_pair(ForceArgs a, 
         const float ex = q1.x - q0.x, ey = q1.y - q0.y, ez = q1.z - q0.z;
         const float r2 = ex * ex + ey * ey + ez * ez;
         if (r2 < rc2) {
-            const float sp = a2 * __fdividef(1.0f, r2);
-            const float psi = ME > 0 ? ar_pow<ME>(sp, (ME & 1) ? af * rsqrtf(r2) : 0.f)
-                                     : ((m & 1) ? rpow(sp, m / 2) * af * rsqrtf(r2)
+            const float sp = a2 * rcp_fast(r2);
+            const float psi = ME > 0 ? ar_pow<ME>(sp, (ME & 1) ? af * rsqrt_fast(r2) : 0.f)
+                                     : ((m & 1) ? rpow(sp, m / 2) * af * rsqrt_fast(r2)
                                                 : rpow(sp, m / 2));
             r = dup2(psi);
         }
@@ -355,12 +355,12 @@ __global__ void __launch_bounds__(kScPairBlock, 8) sc_density_pair(ForceArgs a, 
         const float tx = qj.x + sh.x[st], ty = qj.y + sh.y[st], tz = qj.z + sh.z[st];
         const float2 dx = add2(dup2(tx), nqx), dy = add2(dup2(ty), nqy), dz = add2(dup2(tz), nqz);
         const float2 r2 = fma2(dz, dz, fma2(dy, dy, mul2(dx, dx)));
-        const float2 sp = mul2(dup2(a2), make_float2(__fdividef(1.0f, r2.x), __fdividef(1.0f, r2.y)));
+        const float2 sp = mul2(dup2(a2), make_float2(rcp_fast(r2.x), rcp_fast(r2.y)));
         float2 psi;
         if (ME == 6) {
             psi = mul2(mul2(sp, sp), sp);
         } else {
-            const float2 ar = (m & 1) ? make_float2(af * rsqrtf(r2.x), af * rsqrtf(r2.y)) : dup2(0.f);
+            const float2 ar = (m & 1) ? make_float2(af * rsqrt_fast(r2.x), af * rsqrt_fast(r2.y)) : dup2(0.f);
             psi = ar_pow_rt(sp, ar, m);
         }
         psi.x = r2.x < rc2 ? psi.x : 0.f;
@@ -444,9 +444,9 @@ __global__ void __launch_bounds__(kScPairBlock, 7) sc_force_pair(ForceArgs a, Pa
         const float ex = q1.x - q0.x, ey = q1.y - q0.y, ez = q1.z - q0.z;
         const float r2 = ex * ex + ey * ey + ez * ez;
         if (r2 < rc2) {
-            const float r2i = __fdividef(1.0f, r2);
+            const float r2i = rcp_fast(r2);
             const float sp = a2 * r2i;
-            const float ar = odd ? af * rsqrtf(r2) : 0.f;
+            const float ar = odd ? af * rsqrt_fast(r2) : 0.f;
             float Phi, psi;
             if (NE > 0) {
                 Phi = epsf * ar_pow<NE>(sp, ar);
@@ -480,12 +480,12 @@ __global__ void __launch_bounds__(kScPairBlock, 7) sc_force_pair(ForceArgs a, Pa
         // and (a/r)^2 and 1/r^2 from it without a reciprocal
         float2 ar, sp, r2i;
         if (odd) {
-            ar = mul2(dup2(af), make_float2(rsqrtf(r2.x), rsqrtf(r2.y)));
+            ar = mul2(dup2(af), make_float2(rsqrt_fast(r2.x), rsqrt_fast(r2.y)));
             sp = mul2(ar, ar);
             r2i = mul2(sp, dup2(inv_a2));
         } else {
             ar = dup2(0.f);
-            r2i = make_float2(__fdividef(1.0f, r2.x), __fdividef(1.0f, r2.y));
+            r2i = make_float2(rcp_fast(r2.x), rcp_fast(r2.y));
             sp = mul2(dup2(a2), r2i);
         }
         float2 Phi, psi;
