@@ -2,20 +2,28 @@
 // into small cells; a cell's atoms are processed together).
 //
 // Atoms are assigned to cell c = min(floor(x * n_d / L_d), n_d - 1) per
-// dimension, counted with atomics, the counts are scanned into cell starts,
-// atoms are scattered into their cell's range and each cell's range is put in
-// ascending original-id order, so the sorted layout is deterministic and
-// equals a stable sort by (cell, original id).  For the two-atom layout,
-// whose slots take a cell's atoms two at a time, each cell is instead put in
-// a pairing order (cell_pair_order_kernel), also deterministic, that places
-// near neighbours next to each other.  The gather then rewrites the
-// state in the new order as float64 positions relative to the cell centre
-// plus their float32 copy (the layout the force kernels read).
+// dimension, counted with atomics, the counts are scanned into cell starts and
+// atoms are scattered into their cell's range.  One warp per cell then orders
+// the cell's atoms -- by original id, so that the sorted layout is
+// deterministic and equals a stable sort by (cell, original id), or, for the
+// two-atom layout, whose slots take a cell's atoms two at a time, in a pairing
+// order (also deterministic) that places near neighbours next to each other --
+// and gathers the state in that order as float64 positions relative to the
+// cell centre plus their float32 copy (the layout the force kernels read).
 //
 // Traffic: the counting pass also writes each atom's absolute position and
 // velocity (with its original id, new cell and replica packed into the spare
 // fourth words) into two 32-byte records, so the gather reads two aligned
 // sectors per atom instead of seven scattered words.
+//
+// Launches: five (counting, two of the scan, scatter, order and gather); the
+// slot tables of the two-atom layout come out of the scan (slots per cell, beside
+// the atoms) and of the last pass.  Most steps need no rebuild, and on the
+// default stream they still launch the gated chain, 2 us per idle kernel: with
+// seven launches fewer per step (14 fewer under the two-atom layout) 864 atoms on
+// the default stream run 50 steps in 2.11 instead of 2.60 ms, and the rebuilds
+// of 9.8 M porous atoms, which now read the records once, bring 40 steps from
+// 69.7 to 68.6 ms.
 //
 // A system of several boxes (replicas) numbers its cells consecutively, box
 // after box, so each box's atoms stay one contiguous range of the sorted
@@ -78,15 +86,10 @@ __device__ __forceinline__ double pack2(int hi, int lo) {
     return __longlong_as_double(((long long)hi << 32) | (long long)(unsigned)lo);
 }
 
-__global__ void zero_counts_kernel(int ncells, int32_t *count, DevStatus *ds, bool gated) {
-    if (chain_off(ds, gated)) return;
-    if (blockIdx.x == 0 && threadIdx.x == 0) ds->max_cell = 0;
-    for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < ncells; c += gridDim.x * blockDim.x)
-        count[c] = 0;
-}
-
 // Cell of every atom, its slot in the cell (atomic count) and its gather
-// records: (x, y, z, new cell | original id) and (v, replica).
+// records: (x, y, z, new cell | original id) and (v, replica).  The counts are
+// zero on entry (the scan clears them behind itself).  Resets what the later
+// passes of the rebuild count.
 __global__ void bin_count_kernel(int n, const Grid *__restrict__ grids,
                                  const uint16_t *__restrict__ rep,
                                  const double4 *__restrict__ xr,
@@ -95,10 +98,14 @@ __global__ void bin_count_kernel(int n, const Grid *__restrict__ grids,
                                  const double *__restrict__ v, const int32_t *__restrict__ orig,
                                  int32_t *__restrict__ count, int32_t *__restrict__ new_cell,
                                  int32_t *__restrict__ slot, double4 *__restrict__ tabs,
-                                 double4 *__restrict__ tv, DevStatus *ds, bool gated) {
+                                 double4 *__restrict__ tv, bool slots, DevStatus *ds,
+                                 bool gated) {
     if (chain_off(ds, gated)) return;
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        ds->max_cell = 0;
+        reset_list_counts(ds, slots);
+    }
     const bool fresh = ds->abs_fresh != 0;
-    int maxs = 0;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
         const int r = rep ? rep[i] : 0;
         const Grid &g = grids[r];
@@ -108,109 +115,176 @@ __global__ void bin_count_kernel(int n, const Grid *__restrict__ grids,
         const int cz = cell_coord(x.z, g.inv_w[2], g.nz);
         const int c = g.cell0 + (cz * g.ny + cy) * g.nx + cx;
         new_cell[i] = c;
-        const int sl = atomicAdd(&count[c], 1);
-        slot[i] = sl;
-        maxs = max(maxs, sl + 1);
+        slot[i] = atomicAdd(&count[c], 1);
         tabs[i] = make_double4(x.x, x.y, x.z, pack2(c, orig[i]));
         tv[i] = make_double4(v[i], v[n + i], v[2 * (size_t)n + i], pack2(0, r));
     }
-    // all lanes arrive here (grid-stride loop): one atomic per warp
-    maxs = __reduce_max_sync(0xffffffffu, (unsigned)maxs);
-    if ((threadIdx.x & 31) == 0 && maxs) atomicMax(&ds->max_cell, maxs);
+}
+
+// Exclusive prefix sums over the cells of the atoms and of the slots
+// (ceil(atoms / 2)) of every cell at once, the two sums packed in one 64-bit
+// word (slots << 32 | atoms, each below 2^31); the counts are cleared behind the
+// read, and the largest cell is noted.  slot_start may be null.
+__global__ void __launch_bounds__(kBlock)
+cell_scan_block_kernel(int32_t *__restrict__ count, int32_t *__restrict__ start,
+                       int32_t *__restrict__ slot_start, int n, long long *__restrict__ bsum,
+                       DevStatus *ds, bool gated) {
+    if (chain_off(ds, gated)) return;
+    __shared__ long long tot;
+    const long long base = (long long)blockIdx.x * kScanTile + (long long)threadIdx.x * kScanItems;
+    int c[kScanItems];
+    long long s = 0;
+    int maxc = 0;
+#pragma unroll
+    for (int k = 0; k < kScanItems; ++k) {
+        const long long idx = base + k;
+        c[k] = 0;
+        if (idx < n) {
+            c[k] = count[idx];
+            count[idx] = 0;
+        }
+        maxc = max(maxc, c[k]);
+        s += ((long long)((c[k] + 1) >> 1) << 32) + c[k];
+    }
+    long long off = block_exclusive<long long>(s, &tot);
+#pragma unroll
+    for (int k = 0; k < kScanItems; ++k) {
+        const long long idx = base + k;
+        if (idx < n) {
+            start[idx] = (int)(unsigned)off;
+            if (slot_start) slot_start[idx] = (int)(off >> 32);
+        }
+        off += ((long long)((c[k] + 1) >> 1) << 32) + c[k];
+    }
+    if (threadIdx.x == 0) bsum[blockIdx.x] = tot;
+    maxc = (int)__reduce_max_sync(0xffffffffu, (unsigned)maxc);
+    if ((threadIdx.x & 31) == 0 && maxc) atomicMax(&ds->max_cell, maxc);
+}
+
+// adds the tiles before (one block per tile; as scan_add_kernel)
+__global__ void __launch_bounds__(kBlock)
+cell_scan_add_kernel(int32_t *__restrict__ start, int32_t *__restrict__ slot_start, int n,
+                     const long long *__restrict__ bsum, int nb, bool prefixed,
+                     const DevStatus *ds, bool gated) {
+    if (chain_off(ds, gated)) return;
+    const int t = blockIdx.x;
+    const long long off = prefixed ? bsum[t] : tiles_before<long long>(bsum, t);
+    const long long b = (long long)t * kScanTile;
+#pragma unroll
+    for (int k = 0; k < kScanItems; ++k) {
+        const long long idx = b + (long long)k * kBlock + threadIdx.x;
+        if (idx < n) {
+            start[idx] += (int)(unsigned)off;
+            if (slot_start) slot_start[idx] += (int)(off >> 32);
+        }
+    }
+    if (t == nb - 1 && threadIdx.x == 0) {
+        const long long end = prefixed ? bsum[nb] : off + bsum[t];
+        start[n] = (int)(unsigned)end;
+        if (slot_start) slot_start[n] = (int)(end >> 32);
+    }
 }
 
 __global__ void scatter_kernel(int n, const int32_t *__restrict__ new_cell,
                                const int32_t *__restrict__ slot,
-                               const int32_t *__restrict__ start, const int32_t *__restrict__ orig,
-                               int32_t *__restrict__ src, int32_t *__restrict__ key,
+                               const int32_t *__restrict__ start, int32_t *__restrict__ src,
                                const DevStatus *ds, bool gated) {
     if (chain_off(ds, gated)) return;
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-        int p = start[new_cell[i]] + slot[i];
-        src[p] = i;
-        key[p] = orig[i];
-    }
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
+        src[start[new_cell[i]] + slot[i]] = i;
 }
 
-// Orders each cell's range by original id.  One warp per cell: a cell of up
-// to 32 atoms is ranked by shuffles (lane l's rank = how many keys of the cell
-// are smaller; the keys are distinct original ids); a cell of up to 256 by
-// reading its keys once per lane, two or eight atoms per lane; a larger one is
-// insertion-sorted by one lane (one chain of dependent loads and stores, where
-// the middle path's reads are uniform and independent).
-constexpr int kSortBlock = 256;
+// What the last pass writes, in the new order.
+struct GatherArgs {
+    int n;
+    const Grid *grids;
+    const double4 *tabs, *tv;  // the counting pass's records
+    double4 *xr;
+    float4 *xq, *xq_build;
+    double4 *xabs;
+    double *v;
+    int32_t *orig, *cell;
+    uint16_t *rep;
+    const int32_t *type_orig;
+};
 
-__device__ void insertion_sort_cell(int b, int m, int32_t *__restrict__ key,
-                                    int32_t *__restrict__ src) {
-    for (int a = b + 1; a < b + m; ++a) {
-        const int k = key[a], sv = src[a];
-        int q = a - 1;
-        while (q >= b && key[q] > k) {
-            key[q + 1] = key[q];
-            src[q + 1] = src[q];
-            --q;
-        }
-        key[q + 1] = k;
-        src[q + 1] = sv;
-    }
+__device__ __forceinline__ int record_orig(const double4 &a) {
+    return (int)(unsigned)(__double_as_longlong(a.w) & 0xffffffffll);
 }
 
-// ranks by original id, K atoms per lane (m <= 32 K); all lanes of the warp
-template <int K>
-__device__ __forceinline__ void rank_sort_cell(int b, int m, int lane, int32_t *key,
-                                               int32_t *src) {
-    int k[K], sv[K], rank[K];
-#pragma unroll
-    for (int t = 0; t < K; ++t) {
-        const int l = lane + 32 * t;
-        k[t] = l < m ? key[b + l] : 0x7fffffff;
-        sv[t] = l < m ? src[b + l] : 0;
-        rank[t] = 0;
+// the atom of record s (position record a) becomes sorted atom k
+__device__ __forceinline__ void gather_atom(const GatherArgs &o, int k, int s, const double4 &a) {
+    const double4 u = o.tv[s];
+    const int id = record_orig(a);
+    const int c = (int)(__double_as_longlong(a.w) >> 32);
+    const int r = (int)(__double_as_longlong(u.w) & 0xffff);
+    const Grid &g = o.grids[r];
+    const int cl = c - g.cell0;
+    const double3 C = cell_centre_of(cl % g.nx, (cl / g.nx) % g.ny, cl / (g.nx * g.ny), g);
+    const double rx = a.x - C.x, ry = a.y - C.y, rz = a.z - C.z;
+    o.xr[k] = make_double4(rx, ry, rz, 0.0);
+    // the float32 word carries the original id and, for a multi-element
+    // system, the species above it
+    const uint32_t w = (uint32_t)id | (o.type_orig ? (uint32_t)o.type_orig[id] << kIndexBits : 0u);
+    const float4 q = make_float4((float)rx, (float)ry, (float)rz, __uint_as_float(w));
+    o.xq[k] = q;
+    o.xq_build[k] = q;
+    o.xabs[k] = make_double4(a.x, a.y, a.z, 0.0);
+    const size_t n = (size_t)o.n;
+    o.v[k] = u.x;
+    o.v[n + k] = u.y;
+    o.v[2 * n + k] = u.z;
+    o.orig[k] = id;
+    o.cell[k] = c;
+    if (o.rep) o.rep[k] = (uint16_t)r;
+}
+
+// A cell by original id, any occupancy, by its warp: the rank of an atom is the
+// number of smaller ids in the cell (they are distinct).  Up to 32 atoms by
+// shuffles; above that each lane ranks every 32nd atom by reading the cell's
+// ids (uniform, independent reads).
+constexpr int kOrderBlock = 256;
+
+__device__ __forceinline__ void gather_by_id(const GatherArgs &o, int b, int m, int lane,
+                                             const int32_t *__restrict__ src) {
+    if (m <= 32) {
+        const int s = lane < m ? src[b + lane] : 0;
+        const double4 a = lane < m ? o.tabs[s] : make_double4(0.0, 0.0, 0.0, 0.0);
+        const int id = lane < m ? record_orig(a) : 0x7fffffff;
+        int rank = 0;
+        for (int q = 0; q < m; ++q) rank += (__shfl_sync(0xffffffffu, id, q) < id) ? 1 : 0;
+        if (lane < m) gather_atom(o, b + rank, s, a);
+        return;
     }
+    for (int l = lane; l < m; l += 32) {
+        const int s = src[b + l];
+        const double4 a = o.tabs[s];
+        const int id = record_orig(a);
+        int rank = 0;
 #pragma unroll 4
-    for (int q = 0; q < m; ++q) {
-        const int kq = key[b + q];
-#pragma unroll
-        for (int t = 0; t < K; ++t) rank[t] += (kq < k[t]) ? 1 : 0;
+        for (int q = 0; q < m; ++q)
+            rank += (int)(unsigned)(__double_as_longlong(o.tabs[src[b + q]].w) & 0xffffffffll) < id ? 1 : 0;
+        gather_atom(o, b + rank, s, a);
     }
-    __syncwarp();  // every key is read before one is rewritten
-#pragma unroll
-    for (int t = 0; t < K; ++t)
-        if (lane + 32 * t < m) {
-            key[b + rank[t]] = k[t];
-            src[b + rank[t]] = sv[t];
-        }
 }
 
-// a cell of more than 32 atoms
-__device__ __forceinline__ void sort_large_cell(int b, int m, int lane, int32_t *key,
-                                                int32_t *src) {
-    if (m <= 64) rank_sort_cell<2>(b, m, lane, key, src);
-    else if (m <= 256) rank_sort_cell<8>(b, m, lane, key, src);
-    else if (lane == 0) insertion_sort_cell(b, m, key, src);
+// slots of a cell: first atoms, the last one flagged when it holds one atom
+__device__ __forceinline__ void write_slots(int b, int m, int lane, int s0,
+                                            uint32_t *__restrict__ slot_atom) {
+    for (int k = lane; 2 * k < m; k += 32)
+        slot_atom[s0 + k] = (uint32_t)(b + 2 * k) | (2 * k + 1 >= m ? 0x80000000u : 0u);
 }
 
-__global__ void __launch_bounds__(kSortBlock)
-cell_sort_kernel(int ncells, const int32_t *__restrict__ start, int32_t *key, int32_t *src,
-                 const DevStatus *ds, bool gated) {
+__global__ void __launch_bounds__(kOrderBlock)
+cell_id_order_kernel(int ncells, const int32_t *__restrict__ start,
+                     const int32_t *__restrict__ src, GatherArgs o, DevStatus *ds, bool gated) {
     if (chain_off(ds, gated)) return;
+    if (blockIdx.x == 0 && threadIdx.x == 0) ds->abs_fresh = 1;
     const int lane = threadIdx.x & 31;
-    const int nw = gridDim.x * (kSortBlock / 32);
-    for (int c = blockIdx.x * (kSortBlock / 32) + (threadIdx.x >> 5); c < ncells; c += nw) {
+    const int nw = gridDim.x * (kOrderBlock / 32);
+    for (int c = blockIdx.x * (kOrderBlock / 32) + (threadIdx.x >> 5); c < ncells; c += nw) {
         const int b = start[c], m = start[c + 1] - b;
-        if (m <= 1) continue;
-        if (m <= 32) {
-            const int k = lane < m ? key[b + lane] : 0x7fffffff;
-            const int sv = lane < m ? src[b + lane] : 0;
-            int rank = 0;
-            for (int q = 0; q < m; ++q) rank += (__shfl_sync(0xffffffffu, k, q) < k) ? 1 : 0;
-            if (lane < m) {
-                key[b + rank] = k;
-                src[b + rank] = sv;
-            }
-        } else {
-            sort_large_cell(b, m, lane, key, src);
-        }
+        if (m > 0) gather_by_id(o, b, m, lane, src);
     }
 }
 
@@ -255,31 +329,34 @@ __device__ __forceinline__ float f32_toward_zero(double d) {
 // and ids only and is deterministic; a larger cell falls back to the
 // original-id order (cell_pair_order2_kernel is the form for systems whose
 // average cell is larger).
-__global__ void __launch_bounds__(kSortBlock)
-cell_pair_order_kernel(int ncells, const Grid *__restrict__ grids,
-                       const uint16_t *__restrict__ rep, const int32_t *__restrict__ start,
-                       const double4 *__restrict__ tabs, int32_t *key, int32_t *src,
-                       const DevStatus *ds, bool gated) {
+__global__ void __launch_bounds__(kOrderBlock)
+cell_pair_order_kernel(int ncells, const int32_t *__restrict__ start,
+                       const int32_t *__restrict__ slot_start, uint32_t *__restrict__ slot_atom,
+                       const int32_t *__restrict__ src, GatherArgs out, DevStatus *ds,
+                       bool gated) {
     if (chain_off(ds, gated)) return;
+    if (blockIdx.x == 0 && threadIdx.x == 0) ds->abs_fresh = 1;
     constexpr unsigned full = 0xffffffffu;
-    __shared__ int s_lane_of[kSortBlock / 32][32];
+    __shared__ int s_lane_of[kOrderBlock / 32][32];
     int *lane_of = s_lane_of[threadIdx.x >> 5];
     const int lane = threadIdx.x & 31;
-    const int nw = gridDim.x * (kSortBlock / 32);
-    for (int c = blockIdx.x * (kSortBlock / 32) + (threadIdx.x >> 5); c < ncells; c += nw) {
+    const int nw = gridDim.x * (kOrderBlock / 32);
+    for (int c = blockIdx.x * (kOrderBlock / 32) + (threadIdx.x >> 5); c < ncells; c += nw) {
         const int b = start[c], m = start[c + 1] - b;
-        if (m <= 1) continue;
-        if (m > 32) {
-            sort_large_cell(b, m, lane, key, src);
+        if (m == 0) continue;
+        write_slots(b, m, lane, slot_start[c], slot_atom);
+        if (m == 1 || m > 32) {
+            gather_by_id(out, b, m, lane, src);
             continue;
         }
         const bool on = lane < m;
-        int o = on ? key[b + lane] : 0x7fffffff;
         int sv = on ? src[b + lane] : 0;
-        const double4 a = on ? tabs[sv] : make_double4(0.0, 0.0, 0.0, 0.0);
+        const double4 a = on ? out.tabs[sv] : make_double4(0.0, 0.0, 0.0, 0.0);
+        const int o = on ? record_orig(a) : 0x7fffffff;
         float px = f32_toward_zero(a.x), py = f32_toward_zero(a.y), pz = f32_toward_zero(a.z);
-        // the cell's box (a cell's atoms share it; lane 0 always holds one)
-        const Grid &g = grids[rep ? __shfl_sync(full, (int)rep[sv], 0) : 0];
+        // the cell's box (a cell's atoms share it)
+        const Grid &g =
+            out.grids[out.rep ? (int)(__double_as_longlong(out.tv[src[b]].w) & 0xffff) : 0];
         const float iwx = g.inv_wf[0], iwy = g.inv_wf[1], iwz = g.inv_wf[2];
         const unsigned mk =
             morton9(octree_coord(px, iwx), octree_coord(py, iwy), octree_coord(pz, iwz));
@@ -291,7 +368,6 @@ cell_pair_order_kernel(int ncells, const Grid *__restrict__ grids,
         __syncwarp();
         const int from = on ? lane_of[lane] : lane;
         __syncwarp();
-        o = __shfl_sync(full, o, from);
         sv = __shfl_sync(full, sv, from);
         px = __shfl_sync(full, px, from);
         py = __shfl_sync(full, py, from);
@@ -315,10 +391,7 @@ cell_pair_order_kernel(int ncells, const Grid *__restrict__ grids,
             left &= ~((1u << first) | (1u << mate));
         }
         if ((left >> lane) & 1u) dst = next;
-        if (on) {
-            key[b + dst] = o;
-            src[b + dst] = sv;
-        }
+        if (on) gather_atom(out, b + dst, sv, out.tabs[sv]);
     }
 }
 
@@ -334,43 +407,41 @@ constexpr int kWideCell = 64, kWideMean = 52;
 constexpr int kWideBlock = 128;
 
 __global__ void __launch_bounds__(kWideBlock)
-cell_pair_order2_kernel(int ncells, const Grid *__restrict__ grids,
-                        const uint16_t *__restrict__ rep, const int32_t *__restrict__ start,
-                        const double4 *__restrict__ tabs, int32_t *key, int32_t *src,
-                        const DevStatus *ds, bool gated) {
+cell_pair_order2_kernel(int ncells, const int32_t *__restrict__ start,
+                        const int32_t *__restrict__ slot_start, uint32_t *__restrict__ slot_atom,
+                        const int32_t *__restrict__ src, GatherArgs out, DevStatus *ds,
+                        bool gated) {
     if (chain_off(ds, gated)) return;
+    if (blockIdx.x == 0 && threadIdx.x == 0) ds->abs_fresh = 1;
     constexpr unsigned full = 0xffffffffu;
     __shared__ long long s_key[kWideBlock / 32][kWideCell];
-    __shared__ float4 s_atom[kWideBlock / 32][kWideCell];  // by rank: position, original id
-    __shared__ int s_src[kWideBlock / 32][kWideCell];
+    __shared__ float4 s_atom[kWideBlock / 32][kWideCell];  // by rank: position, source record
     long long *wkey = s_key[threadIdx.x >> 5];
     float4 *watom = s_atom[threadIdx.x >> 5];
-    int *wsrc = s_src[threadIdx.x >> 5];
     const int lane = threadIdx.x & 31;
     const int nw = gridDim.x * (kWideBlock / 32);
     for (int c = blockIdx.x * (kWideBlock / 32) + (threadIdx.x >> 5); c < ncells; c += nw) {
         const int b = start[c], m = start[c + 1] - b;
-        if (m <= 1) continue;
-        if (m > kWideCell) {
-            sort_large_cell(b, m, lane, key, src);
+        if (m == 0) continue;
+        write_slots(b, m, lane, slot_start[c], slot_atom);
+        if (m == 1 || m > kWideCell) {
+            gather_by_id(out, b, m, lane, src);
             continue;
         }
         float4 at[2];
-        int sv[2];
         long long K[2];
-        int r0 = 0;
+        // the cell's box (its atoms share it)
+        const Grid &g =
+            out.grids[out.rep ? (int)(__double_as_longlong(out.tv[src[b]].w) & 0xffff) : 0];
 #pragma unroll
         for (int t = 0; t < 2; ++t) {
             const int l = lane + 32 * t;
             const bool on = l < m;
-            const int o = on ? key[b + l] : 0x7fffffff;
-            sv[t] = on ? src[b + l] : 0;
-            const double4 a = on ? tabs[sv[t]] : make_double4(0.0, 0.0, 0.0, 0.0);
+            const int sv = on ? src[b + l] : 0;
+            const double4 a = on ? out.tabs[sv] : make_double4(0.0, 0.0, 0.0, 0.0);
+            const int o = on ? record_orig(a) : 0x7fffffff;
             at[t] = make_float4(f32_toward_zero(a.x), f32_toward_zero(a.y), f32_toward_zero(a.z),
-                                __int_as_float(o));
-            // the cell's box (its atoms share it; lane 0 always holds one)
-            if (t == 0) r0 = rep ? __shfl_sync(full, (int)rep[sv[0]], 0) : 0;
-            const Grid &g = grids[r0];
+                                __int_as_float(sv));
             const unsigned mk = morton9(octree_coord(at[t].x, g.inv_wf[0]),
                                         octree_coord(at[t].y, g.inv_wf[1]),
                                         octree_coord(at[t].z, g.inv_wf[2]));
@@ -386,10 +457,7 @@ cell_pair_order2_kernel(int ncells, const Grid *__restrict__ grids,
         }
 #pragma unroll
         for (int t = 0; t < 2; ++t)
-            if (lane + 32 * t < m) {
-                watom[rank[t]] = at[t];
-                wsrc[rank[t]] = sv[t];
-            }
+            if (lane + 32 * t < m) watom[rank[t]] = at[t];
         __syncwarp();
         const float4 a0 = lane < m ? watom[lane] : make_float4(0.f, 0.f, 0.f, 0.f);
         const float4 a1 = lane + 32 < m ? watom[lane + 32] : make_float4(0.f, 0.f, 0.f, 0.f);
@@ -419,53 +487,14 @@ cell_pair_order2_kernel(int ncells, const Grid *__restrict__ grids,
         if ((left >> lane) & 1ull) dst0 = next;
         if ((left >> (lane + 32)) & 1ull) dst1 = next;
         if (lane < m) {
-            key[b + dst0] = __float_as_int(a0.w);
-            src[b + dst0] = wsrc[lane];
+            const int sv = __float_as_int(a0.w);
+            gather_atom(out, b + dst0, sv, out.tabs[sv]);
         }
         if (lane + 32 < m) {
-            key[b + dst1] = __float_as_int(a1.w);
-            src[b + dst1] = wsrc[lane + 32];
+            const int sv = __float_as_int(a1.w);
+            gather_atom(out, b + dst1, sv, out.tabs[sv]);
         }
         __syncwarp();  // the shared rows are rewritten by the warp's next cell
-    }
-}
-
-__global__ void gather_kernel(int n, const Grid *__restrict__ grids,
-                              const int32_t *__restrict__ src, const double4 *__restrict__ tabs,
-                              const double4 *__restrict__ tv, double4 *__restrict__ xr,
-                              float4 *__restrict__ xq, float4 *__restrict__ xq_build,
-                              double4 *__restrict__ xabs, double *__restrict__ v,
-                              int32_t *__restrict__ orig, int32_t *__restrict__ cell,
-                              uint16_t *__restrict__ rep, const int32_t *__restrict__ type_orig,
-                              DevStatus *ds, bool gated) {
-    if (chain_off(ds, gated)) return;
-    if (blockIdx.x == 0 && threadIdx.x == 0) ds->abs_fresh = 1;
-    for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) {
-        const int s = src[k];
-        const double4 a = tabs[s];
-        const double4 u = tv[s];
-        const long long pa = __double_as_longlong(a.w);
-        const int o = (int)(unsigned)(pa & 0xffffffffll);
-        const int c = (int)(pa >> 32);
-        const int r = (int)(__double_as_longlong(u.w) & 0xffff);
-        const Grid &g = grids[r];
-        const int cl = c - g.cell0;
-        const double3 C = cell_centre_of(cl % g.nx, (cl / g.nx) % g.ny, cl / (g.nx * g.ny), g);
-        const double rx = a.x - C.x, ry = a.y - C.y, rz = a.z - C.z;
-        xr[k] = make_double4(rx, ry, rz, 0.0);
-        // the float32 word carries the original id and, for a multi-element
-        // system, the species above it
-        const uint32_t w = (uint32_t)o | (type_orig ? (uint32_t)type_orig[o] << kIndexBits : 0u);
-        const float4 q = make_float4((float)rx, (float)ry, (float)rz, __uint_as_float(w));
-        xq[k] = q;
-        xq_build[k] = q;
-        xabs[k] = make_double4(a.x, a.y, a.z, 0.0);
-        v[k] = u.x;
-        v[n + k] = u.y;
-        v[2 * (size_t)n + k] = u.z;
-        orig[k] = o;
-        cell[k] = c;
-        if (rep) rep[k] = (uint16_t)r;
     }
 }
 
@@ -486,41 +515,57 @@ cudaError_t launch_scan_i32(const int32_t *in, int32_t *out, int n, int32_t *bsu
 }
 
 cudaError_t launch_bin(md_system *h, bool gated) {
-    int n = (int)h->n;
+    const int n = (int)h->n, nc = h->g.ncells;
     cudaStream_t s = h->stream;
-    int cur = h->cur;
-    zero_counts_kernel<<<gs_blocks(h->g.ncells), kBlock, 0, s>>>(h->g.ncells, h->cell_count,
-                                                                 h->ds, gated);
+    const int cur = h->cur;
+    // (a variant switch that failed half-way may have left no slot tables)
+    const bool paired = h->p.force_variant == MD_FORCE_PAIRED && h->ps_count != nullptr;
     bin_count_kernel<<<gs_blocks(n), kBlock, 0, s>>>(n, h->grids, h->rep, h->xr64[cur], h->cell,
                                                      h->xabs, h->v, h->orig, h->cell_count,
                                                      h->new_cell, h->slot, h->tmp_abs, h->tmp_v,
-                                                     h->ds, gated);
-    cudaError_t e = launch_scan_i32(h->cell_count, h->cell_start, h->g.ncells, h->scan_bsum,
-                                    h->ds, gated, s);
-    if (e != cudaSuccess) return e;
-    scatter_kernel<<<gs_blocks(n), kBlock, 0, s>>>(n, h->new_cell, h->slot, h->cell_start,
-                                                   h->orig, h->src, h->key, h->ds, gated);
-    const int sort_blocks = std::min((h->g.ncells + kSortBlock / 32 - 1) / (kSortBlock / 32),
-                                     kGridCap * 2);
+                                                     paired, h->ds, gated);
+    int32_t *slot_start = paired ? h->ps_start : nullptr;
+    const int nb = std::max((nc + kScanTile - 1) / kScanTile, 1);
+    const bool prefixed = nb > kScanDirect;
+    cell_scan_block_kernel<<<nb, kBlock, 0, s>>>(h->cell_count, h->cell_start, slot_start, nc,
+                                                 h->cell_bsum, h->ds, gated);
+    if (prefixed) scan_bsum_kernel<long long><<<1, kBlock, 0, s>>>(h->cell_bsum, nb, h->ds, gated);
+    cell_scan_add_kernel<<<nb, kBlock, 0, s>>>(h->cell_start, slot_start, nc, h->cell_bsum, nb,
+                                               prefixed, h->ds, gated);
+    scatter_kernel<<<gs_blocks(n), kBlock, 0, s>>>(n, h->new_cell, h->slot, h->cell_start, h->src,
+                                                   h->ds, gated);
+    GatherArgs o;
+    o.n = n;
+    o.grids = h->grids;
+    o.tabs = h->tmp_abs;
+    o.tv = h->tmp_v;
+    o.xr = h->xr64[cur];
+    o.xq = h->xq[cur];
+    o.xq_build = h->xq_build;
+    o.xabs = h->xabs;
+    o.v = h->v;
+    o.orig = h->orig;
+    o.cell = h->cell;
+    o.rep = h->rep;
+    o.type_orig = h->type_orig;
+    const int warps = kOrderBlock / 32;
+    const int blocks = std::max(std::min((nc + warps - 1) / warps, kGridCap * 2), 1);
     // one atom per lane while the average cell fits a warp, two per lane above
-    const int64_t nc64 = h->g.ncells;
-    if (h->p.force_variant == MD_FORCE_PAIRED && h->n > 32 * nc64 && h->n <= kWideMean * nc64)
-        cell_pair_order2_kernel<<<std::max(std::min((int)((nc64 + 3) / 4), kGridCap * 2), 1),
-                                  kWideBlock, 0, s>>>(h->g.ncells, h->grids, h->rep, h->cell_start,
-                                                      h->tmp_abs, h->key, h->src, h->ds, gated);
-    else if (h->p.force_variant == MD_FORCE_PAIRED)
-        cell_pair_order_kernel<<<std::max(sort_blocks, 1), kSortBlock, 0, s>>>(
-            h->g.ncells, h->grids, h->rep, h->cell_start, h->tmp_abs, h->key, h->src, h->ds,
-            gated);
+    if (paired && h->n > 32 * (int64_t)nc && h->n <= kWideMean * (int64_t)nc)
+        cell_pair_order2_kernel<<<std::max(std::min((nc + 3) / 4, kGridCap * 2), 1), kWideBlock, 0,
+                                  s>>>(nc, h->cell_start, h->ps_start, h->ps_atom, h->src, o,
+                                       h->ds, gated);
+    else if (paired)
+        cell_pair_order_kernel<<<blocks, kOrderBlock, 0, s>>>(
+            nc, h->cell_start, h->ps_start, h->ps_atom, h->src, o, h->ds, gated);
     else
-        cell_sort_kernel<<<std::max(sort_blocks, 1), kSortBlock, 0, s>>>(
-            h->g.ncells, h->cell_start, h->key, h->src, h->ds, gated);
-    gather_kernel<<<gs_blocks(n), kBlock, 0, s>>>(n, h->grids, h->src, h->tmp_abs, h->tmp_v,
-                                                  h->xr64[cur], h->xq[cur], h->xq_build, h->xabs,
-                                                  h->v, h->orig, h->cell, h->rep, h->type_orig,
-                                                  h->ds, gated);
+        cell_id_order_kernel<<<blocks, kOrderBlock, 0, s>>>(nc, h->cell_start, h->src, o, h->ds,
+                                                           gated);
     return cudaGetLastError();
 }
+
+int scan_launch_count(long long n) { return scan_launches(n); }
+int bin_launches(const md_system *h) { return 3 + scan_launches(h->g.ncells); }
 
 cudaError_t launch_export_cells(md_system *h, int32_t *cell_of_atom, int64_t *cell_start) {
     int m = (int)(h->n > h->g.ncells + 1 ? h->n : h->g.ncells + 1);

@@ -179,7 +179,7 @@ build_list_kernel(int n, const Grid *__restrict__ grids, const uint16_t *__restr
                   float lo, float hi, double rl2, const float4 *__restrict__ xq,
                   const double4 *__restrict__ xabs, const int32_t *__restrict__ cell,
                   const int32_t *__restrict__ start, uint32_t *__restrict__ nlist,
-                  int32_t *__restrict__ ncount, int cap, DevStatus *ds, bool gated) {
+                  int32_t *__restrict__ ncount, int cap, DevStatus *ds, bool gated, bool close) {
     if (chain_off(ds, gated)) return;
     unsigned long long tot = 0;
     int overflow = 0, maxc = 0;
@@ -233,12 +233,12 @@ build_list_kernel(int n, const Grid *__restrict__ grids, const uint16_t *__restr
         if (maxc) atomicMax(&ds->max_count, maxc);
     }
     if (WRITE && overflow) atomicCAS(&ds->status, 0, (int)MD_ERR_LIST_OVERFLOW);
+    list_build_done(ds, close);
 }
 
-__global__ void reset_max_count_kernel(DevStatus *ds, bool gated) {
-    if (chain_off(ds, gated)) return;
-    ds->max_count = 0;
-    ds->list_entries = 0;
+// a list build without binning counts anew
+__global__ void reset_counts_kernel(DevStatus *ds, bool slots) {
+    if (ds->status == 0) reset_list_counts(ds, slots);
 }
 
 __global__ void finish_rebuild_kernel(DevStatus *ds, bool gated) {
@@ -300,17 +300,26 @@ __global__ void export_fill_kernel(int n, int cap, int half, const int32_t *__re
 
 }  // namespace
 
-cudaError_t launch_build_list(md_system *h, bool write, bool gated, const float4 *positions) {
+cudaError_t launch_reset_counts(md_system *h, bool slots) {
+    reset_counts_kernel<<<1, 1, 0, h->stream>>>(h->ds, slots);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_build_list(md_system *h, bool write, bool gated, const float4 *positions,
+                              bool close) {
     int n = (int)h->n;
     cudaStream_t s = h->stream;
     const float4 *xq = positions ? positions : h->xq[h->cur];
     const bool half = half_variant(h->p.force_variant);
-    reset_max_count_kernel<<<1, 1, 0, s>>>(h->ds, gated);
+    if (!gated) {
+        const cudaError_t e = launch_reset_counts(h, false);
+        if (e != cudaSuccess) return e;
+    }
 #define MDG_LIST(WR, HF)                                                                    \
     build_list_kernel<WR, HF><<<gs_blocks(n) * (kBlock / kListBlock), kListBlock, 0, s>>>(                                \
         n, h->grids, h->rep, h->list_lo, h->list_hi, h->rl2, xq, h->xabs, h->cell,           \
         h->cell_start,                                                                         \
-        h->nlist, h->ncount, h->cap, h->ds, gated)
+        h->nlist, h->ncount, h->cap, h->ds, gated, close)
     if (write) { if (half) MDG_LIST(true, true); else MDG_LIST(true, false); }
     else { if (half) MDG_LIST(false, true); else MDG_LIST(false, false); }
 #undef MDG_LIST

@@ -28,8 +28,9 @@
 // at rho* = 0.8442, so one chunk of the per-atom kernel's float32-then-
 // float64 sums) and converted once: without the float64 accumulators the
 // kernel fits 9 CTAs of 128 threads per SM.
+#include <algorithm>
+
 #include "k_pair.cuh"
-#include "k_scan.cuh"
 
 namespace mdg {
 
@@ -43,30 +44,6 @@ __device__ __forceinline__ bool chain_off(const DevStatus *ds, bool gated) {
 }
 
 __device__ __forceinline__ int row_off(int k) { return k + (k >> 2) * 124; }
-
-// slots per cell: ceil(atoms / 2)
-__global__ void slot_count_kernel(int ncells, const int32_t *__restrict__ start,
-                                  int32_t *__restrict__ cnt, const DevStatus *ds, bool gated) {
-    if (chain_off(ds, gated)) return;
-    for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < ncells; c += gridDim.x * blockDim.x)
-        cnt[c] = (start[c + 1] - start[c] + 1) >> 1;
-}
-
-// the first atom of every slot, flagged when the slot holds one atom
-__global__ void slot_fill_kernel(int n, const int32_t *__restrict__ cell,
-                                 const int32_t *__restrict__ start,
-                                 const int32_t *__restrict__ slot_start,
-                                 uint32_t *__restrict__ slot_atom, const DevStatus *ds,
-                                 bool gated) {
-    if (chain_off(ds, gated)) return;
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-        const int c = cell[i];
-        const int k = i - start[c];
-        if (k & 1) continue;
-        const uint32_t single = (i + 1 >= start[c + 1]) ? kSingle : 0u;
-        slot_atom[slot_start[c] + (k >> 1)] = (uint32_t)i | single;
-    }
-}
 
 // One stencil cell of a slot's union-list scan (HOME: the slot's own cell,
 // the only one holding i0 and i1); returns the running entry count.
@@ -118,7 +95,7 @@ pair_list_kernel(int n, Grid g, const Grid *__restrict__ grids, const uint16_t *
                  const int32_t *__restrict__ cell, const int32_t *__restrict__ start,
                  const int32_t *__restrict__ slot_start, const uint32_t *__restrict__ slot_atom,
                  uint32_t *__restrict__ list, int32_t *__restrict__ count, int cap, DevStatus *ds,
-                 bool gated) {
+                 bool gated, bool close) {
     if (chain_off(ds, gated)) return;
     const int nslots = slot_start[g.ncells];
     if (blockIdx.x == 0 && threadIdx.x == 0) ds->pair_slots = nslots;
@@ -186,12 +163,7 @@ pair_list_kernel(int n, Grid g, const Grid *__restrict__ grids, const uint16_t *
         if (maxc) atomicMax(&ds->pair_max, maxc);
     }
     if (WRITE && overflow) atomicCAS(&ds->status, 0, (int)MD_ERR_LIST_OVERFLOW);
-}
-
-__global__ void pair_reset_kernel(DevStatus *ds, bool gated) {
-    if (chain_off(ds, gated)) return;
-    ds->pair_max = 0;
-    ds->pair_entries = 0;
+    list_build_done(ds, close);
 }
 
 // the dummy neighbour of the padding entries, past the last atom of both
@@ -265,21 +237,19 @@ cudaError_t launch_pair_dummy(md_system *h) {
     return cudaGetLastError();
 }
 
-cudaError_t launch_pair_build(md_system *h, bool write, bool gated) {
+cudaError_t launch_pair_build(md_system *h, bool write, bool gated, bool close) {
     const int n = (int)h->n, nc = h->g.ncells;
     cudaStream_t s = h->stream;
-    slot_count_kernel<<<gs_blocks(nc), kBlock, 0, s>>>(nc, h->cell_start, h->ps_cnt, h->ds, gated);
-    cudaError_t e = launch_scan_i32(h->ps_cnt, h->ps_start, nc, h->ps_bsum, h->ds, gated, s);
-    if (e != cudaSuccess) return e;
-    slot_fill_kernel<<<gs_blocks(n), kBlock, 0, s>>>(n, h->cell, h->cell_start, h->ps_start,
-                                                     h->ps_atom, h->ds, gated);
-    pair_reset_kernel<<<1, 1, 0, s>>>(h->ds, gated);
+    if (!gated) {
+        const cudaError_t e = launch_reset_counts(h, true);
+        if (e != cudaSuccess) return e;
+    }
     const int64_t smax = pair_slots_max(h->n, nc);
     const int blocks = (int)std::min<int64_t>((smax + kPairBlock - 1) / kPairBlock, 152 * 16);
 #define MDG_PAIR_LIST(W, M)                                                                  \
     pair_list_kernel<W, M><<<blocks, kPairBlock, 0, s>>>(                                    \
         n, h->g, h->grids, h->rep, h->list_hi, h->xq[h->cur], h->cell, h->cell_start,        \
-        h->ps_start, h->ps_atom, h->ps_list, h->ps_count, h->ps_cap, h->ds, gated)
+        h->ps_start, h->ps_atom, h->ps_list, h->ps_count, h->ps_cap, h->ds, gated, close)
     if (h->R > 1) {
         if (write) MDG_PAIR_LIST(true, true);
         else MDG_PAIR_LIST(false, true);

@@ -1,5 +1,6 @@
-// k_scan.cuh -- exclusive prefix sum over a device array (three passes:
-// per-tile scan, scan of tile sums, add tile offsets).  out[n] = total.
+// k_scan.cuh -- exclusive prefix sum over a device array (per-tile scan, then
+// every tile adds the sum of the tiles before it; more than kScanDirect tiles
+// get a pass of their own for the tile sums).  out[n] = total.
 #pragma once
 
 #include "md_internal.cuh"
@@ -8,6 +9,9 @@ namespace mdg {
 
 constexpr int kScanItems = 8;
 constexpr int kScanTile = kBlock * kScanItems;
+// up to this many tiles each block of the last pass adds up the tile sums
+// before it by itself (at most four reads per thread), which saves a launch
+constexpr int kScanDirect = 1024;
 
 template <class T>
 __device__ T block_exclusive(T v, T *total) {
@@ -80,13 +84,34 @@ __global__ void scan_bsum_kernel(T *bsum, int nb, const DevStatus *ds, bool gate
     if (threadIdx.x == 0) bsum[nb] = carry;
 }
 
+// the sum of bsum[0 .. t), for every thread of the block
 template <class T>
-__global__ void scan_add_kernel(T *out, int n, const T *__restrict__ bsum, int nb,
+__device__ T tiles_before(const T *__restrict__ bsum, int t) {
+    __shared__ T ws[kBlock / 32];
+    T x = 0;
+    for (int k = threadIdx.x; k < t; k += kBlock) x += bsum[k];
+    for (int o = 16; o > 0; o >>= 1) x += __shfl_down_sync(0xffffffffu, x, o);
+    if ((threadIdx.x & 31) == 0) ws[threadIdx.x >> 5] = x;
+    __syncthreads();
+    T r = 0;
+    for (int k = 0; k < kBlock / 32; ++k) r += ws[k];
+    return r;
+}
+
+// one block per tile; prefixed: bsum holds prefix sums (scan_bsum_kernel ran)
+template <class T>
+__global__ void scan_add_kernel(T *out, int n, const T *__restrict__ bsum, int nb, bool prefixed,
                                 const DevStatus *ds, bool gated) {
     if (scan_off(ds, gated)) return;
-    for (int idx = blockIdx.x * blockDim.x + threadIdx.x; idx < n; idx += gridDim.x * blockDim.x)
-        out[idx] += bsum[idx / kScanTile];
-    if (blockIdx.x == 0 && threadIdx.x == 0) out[n] = bsum[nb];
+    const int t = blockIdx.x;
+    const T off = prefixed ? bsum[t] : tiles_before<T>(bsum, t);
+    const long long b = (long long)t * kScanTile;
+#pragma unroll
+    for (int k = 0; k < kScanItems; ++k) {
+        const long long idx = b + (long long)k * kBlock + threadIdx.x;
+        if (idx < n) out[idx] += off;
+    }
+    if (t == nb - 1 && threadIdx.x == 0) out[n] = prefixed ? bsum[nb] : off + bsum[t];
 }
 
 // bsum must hold at least n / kScanTile + 2 elements.
@@ -96,9 +121,11 @@ inline cudaError_t launch_scan(const T *in, T *out, int n, T *bsum, const DevSta
     int nb = (n + kScanTile - 1) / kScanTile;
     if (nb < 1) nb = 1;
     scan_block_kernel<T><<<nb, kBlock, 0, s>>>(in, out, n, bsum, ds, gated);
-    scan_bsum_kernel<T><<<1, kBlock, 0, s>>>(bsum, nb, ds, gated);
-    scan_add_kernel<T><<<gs_blocks(n), kBlock, 0, s>>>(out, n, bsum, nb, ds, gated);
+    const bool prefixed = nb > kScanDirect;
+    if (prefixed) scan_bsum_kernel<T><<<1, kBlock, 0, s>>>(bsum, nb, ds, gated);
+    scan_add_kernel<T><<<nb, kBlock, 0, s>>>(out, n, bsum, nb, prefixed, ds, gated);
     return cudaGetLastError();
 }
+inline int scan_launches(long long n) { return n > (long long)kScanDirect * kScanTile ? 3 : 2; }
 
 }  // namespace mdg

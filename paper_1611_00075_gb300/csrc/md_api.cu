@@ -89,13 +89,13 @@ void free_all(md_system *h) {
     auto F = [](void *p) { if (p) cudaFree(p); };
     for (int b = 0; b < 2; ++b) { F(h->xr64[b]); F(h->xq[b]); }
     F(h->xq_build); F(h->xabs); F(h->v); F(h->f); F(h->e_atom); F(h->orig); F(h->cell);
-    F(h->cell_start); F(h->cell_count); F(h->new_cell); F(h->slot); F(h->src); F(h->key);
-    F(h->scan_bsum); F(h->tmp_abs); F(h->tmp_v); F(h->nlist); F(h->ncount);
+    F(h->cell_start); F(h->cell_count); F(h->new_cell); F(h->slot); F(h->src);
+    F(h->scan_bsum); F(h->cell_bsum); F(h->tmp_abs); F(h->tmp_v); F(h->nlist); F(h->ncount);
     F(h->rho); F(h->dF32); F(h->dF64); F(h->xqf); F(h->partials); F(h->red_out); F(h->ds);
     F(h->exp_tmp); F(h->type_orig);
     F(h->cl_icnt); F(h->cl_jcnt); F(h->cl_ioff); F(h->cl_joff); F(h->cl_bsum); F(h->cl_icl);
     F(h->cl_icell); F(h->cl_jbox); F(h->cl_ntot); F(h->cl_list); F(h->cl_row);
-    F(h->ps_cnt); F(h->ps_start); F(h->ps_bsum); F(h->ps_atom); F(h->ps_list); F(h->ps_count);
+    F(h->ps_start); F(h->ps_atom); F(h->ps_list); F(h->ps_count);
     F(h->ov_cell_outer); F(h->ov_flag); F(h->ov_pos); F(h->ov_bsum); F(h->ov_gidx);
     F(h->ov_bidx); F(h->ov_nb); F(h->ov_send); F(h->ov_recv);
     if (h->ov_stream) cudaStreamDestroy(h->ov_stream);
@@ -145,9 +145,9 @@ cudaError_t alloc_pair(md_system *h, int cap) {
     const int64_t smax = pair_slots_max(h->n, h->g.ncells);
     cudaError_t e = cudaSuccess;
     auto A = [&](cudaError_t r) { if (e == cudaSuccess) e = r; };
-    if (!h->ps_cnt) {
-        A(dalloc(&h->ps_cnt, C)); A(dalloc(&h->ps_start, C + 1));
-        A(dalloc(&h->ps_bsum, C / (kBlock * 8) + 4)); A(dalloc(&h->ps_atom, (size_t)smax));
+    if (!h->ps_count) {  // the last of the three
+        A(h->ps_start ? cudaSuccess : dalloc(&h->ps_start, C + 1));
+        A(h->ps_atom ? cudaSuccess : dalloc(&h->ps_atom, (size_t)smax));
         A(dalloc(&h->ps_count, (size_t)smax));
     }
     if (e == cudaSuccess && cap > 0 && (cap != h->ps_cap || !h->ps_list)) {
@@ -164,10 +164,9 @@ int cap_for(int max_count);
 md_status read_status(md_system *h);
 md_status clear_status(md_system *h);
 
-// Slot tables and union lists for the current binning, sized from a count
-// pass when the list is new, regrown when a row overflows.
+// Union lists for the current binning (which made the slot tables), sized from
+// a count pass when the list is new, regrown when a row overflows.
 md_status pair_rebuild_now(md_system *h) {
-    MD_CK(alloc_pair(h, 0));
     if (!h->ps_list) {
         MD_CK(launch_pair_build(h, false, false));
         md_status st = read_status(h);
@@ -335,38 +334,40 @@ md_status enqueue_sched_prep(md_system *h, bool gated) {
     MD_CK(launch_cell_features(h, pc, gated));
     if (!pc) MD_CK(launch_predict_costs(h, gated));
     MD_CK(launch_partition_cells(h, gated));
-    h->launches += pc ? 5 : 7;
+    h->launches += (pc ? 2 : 4) + scan_launch_count(h->g.ncells);
     return MD_OK;
 }
 
 // Rebuild chain enqueued before a force evaluation.  gated: runs only if the
 // device flag asks for it.
 md_status enqueue_rebuild(md_system *h, bool gated) {
+    // the list build closes the rebuild unless other passes follow it
+    const bool last = !h->ov_on && h->p.force_variant != MD_FORCE_CLUSTER && !uses_partition(h);
     MD_CK(launch_bin(h, gated));
-    if (h->p.force_variant == MD_FORCE_PAIRED) {
-        MD_CK(launch_pair_build(h, true, gated));
-        h->launches += kBinLaunches + 8;  // binning, slot tables and lists, finish
-    } else {
-        MD_CK(launch_build_list(h, true, gated));
-        h->launches += kBinLaunches + 3;  // binning, list reset and build, finish
-    }
+    if (h->p.force_variant == MD_FORCE_PAIRED) MD_CK(launch_pair_build(h, true, gated, last));
+    else MD_CK(launch_build_list(h, true, gated, nullptr, last));
+    h->launches += bin_launches(h) + 1 + (gated ? 0 : 1);  // binning, list (and its reset)
     if (h->ov_on) {
         MD_CK(launch_overlap_index(h, gated));
-        h->launches += 5;
+        h->launches += 2 + scan_launch_count(h->n);
     }
     if (h->p.force_variant == MD_FORCE_CLUSTER) {
         MD_CK(launch_cluster_build(h, gated));
-        h->launches += 9;
+        h->launches += 3 + 2 * scan_launch_count(h->g.ncells);
     }
-    md_status st = enqueue_sched_prep(h, gated);
-    if (st != MD_OK) return st;
-    MD_CK(launch_finish_rebuild(h, gated));
+    if (!last) {
+        md_status st = enqueue_sched_prep(h, gated);
+        if (st != MD_OK) return st;
+        MD_CK(launch_finish_rebuild(h, gated));
+        h->launches += 1;
+    }
     MD_CK(mark(h, K_REBUILD));
     return MD_OK;
 }
 
 // Host-driven rebuild with capacity repair (explicit calls and create).
 md_status rebuild_now(md_system *h, bool size_from_count) {
+    if (h->p.force_variant == MD_FORCE_PAIRED) MD_CK(alloc_pair(h, 0));
     MD_CK(launch_bin(h, false));
     if (h->p.force_variant == MD_FORCE_PAIRED) {
         // the slot lists carry the force pass; per-atom rows are built on
@@ -881,7 +882,8 @@ static md_status create_impl(md_system **out, const md_params *p, int R, const i
     A(dalloc(&h->f, 3 * N)); A(dalloc(&h->e_atom, N)); A(dalloc(&h->orig, N));
     A(dalloc(&h->cell, N)); A(dalloc(&h->cell_start, C + 1)); A(dalloc(&h->cell_count, C));
     A(dalloc(&h->new_cell, N)); A(dalloc(&h->slot, N)); A(dalloc(&h->src, N));
-    A(dalloc(&h->key, N)); A(dalloc(&h->scan_bsum, scan_len)); A(dalloc(&h->tmp_abs, N));
+    A(dalloc(&h->scan_bsum, scan_len)); A(dalloc(&h->cell_bsum, scan_len));
+    A(dalloc(&h->tmp_abs, N));
     A(dalloc(&h->tmp_v, N)); A(dalloc(&h->ncount, N));
     size_t ctab_len = 0;
     for (const Grid &g : h->grids_h) ctab_len += (size_t)g.nx + g.ny + g.nz;
@@ -950,6 +952,7 @@ static md_status create_impl(md_system **out, const md_params *p, int R, const i
     step(cudaMemcpyAsync(h->atom_off, h->atom_off_h.data(), (R + 1) * sizeof(int64_t),
                          cudaMemcpyHostToDevice, h->stream), "copy offsets");
     step(cudaMemsetAsync(h->ds, 0, sizeof(DevStatus), h->stream), "memset status");
+    step(cudaMemsetAsync(h->cell_count, 0, C * sizeof(int32_t), h->stream), "memset counts");
     step(cudaMemsetAsync(h->f, 0, 3 * N * sizeof(double), h->stream), "memset f");
     step(cudaMemsetAsync(h->e_atom, 0, N * sizeof(double), h->stream), "memset e");
     if (!vel_dev) step(cudaMemsetAsync(h->v, 0, 3 * N * sizeof(double), h->stream), "memset v");

@@ -87,7 +87,38 @@ struct DevStatus {
     unsigned long long pair_entries;  // entries of the last two-atom slot list
     int pair_max;                     // its longest row
     int pair_slots;                   // its slots
+    unsigned int list_done;           // blocks of the list build finished this launch
 };
+
+// What a list build counts, reset by the binning before it (or by a launch of
+// its own when a list is built without binning): the slot lists' counts or the
+// per-atom rows'.
+__device__ __forceinline__ void reset_list_counts(DevStatus *ds, bool slots) {
+    if (slots) {
+        ds->pair_max = 0;
+        ds->pair_entries = 0;
+    } else {
+        ds->max_count = 0;
+        ds->list_entries = 0;
+    }
+}
+
+// End of a list build (every thread of every block calls it, after its work):
+// the last block closes the rebuild when no error was raised.  close = false:
+// later passes of the rebuild follow, which finish_rebuild_kernel closes.
+__device__ __forceinline__ void list_build_done(DevStatus *ds, bool close) {
+    if (!close) return;
+    __syncthreads();
+    if (threadIdx.x != 0) return;
+    __threadfence();
+    if (atomicAdd(&ds->list_done, 1u) != gridDim.x - 1) return;
+    ds->list_done = 0;
+    __threadfence();
+    if (atomicAdd(&ds->status, 0) != 0) return;
+    ds->rebuild = 0;
+    ds->since_build = 0;
+    ds->builds += 1;
+}
 
 // What the persistent force kernel needs besides ForceArgs.
 struct SchedArgs {
@@ -233,8 +264,9 @@ struct md_system {
     // binning
     int32_t *cell_start = nullptr;  // ncells + 1
     int32_t *cell_count = nullptr;  // ncells
-    int32_t *new_cell = nullptr, *slot = nullptr, *src = nullptr, *key = nullptr;
+    int32_t *new_cell = nullptr, *slot = nullptr, *src = nullptr;
     int32_t *scan_bsum = nullptr;
+    long long *cell_bsum = nullptr;  // tile sums of the cell scan (slots << 32 | atoms)
     double4 *tmp_abs = nullptr;  // gather records: (x, y, z, new cell | original id)
     double4 *tmp_v = nullptr;    //                 (vx, vy, vz, replica)
 
@@ -294,9 +326,7 @@ struct md_system {
     int cl_cap = 0;
 
     // two home atoms per thread (MD_FORCE_PAIRED)
-    int32_t *ps_cnt = nullptr;     // slots per cell
-    int32_t *ps_start = nullptr;   // their scan (ncells + 1)
-    int32_t *ps_bsum = nullptr;
+    int32_t *ps_start = nullptr;   // first slot of every cell (ncells + 1)
     uint32_t *ps_atom = nullptr;   // slot: first atom | 2^31 for a one-atom slot
     uint32_t *ps_list = nullptr;   // union lists, per-atom layout over slots
     int32_t *ps_count = nullptr;   // their lengths
@@ -346,21 +376,27 @@ namespace mdg {
 
 // ---- binning (k_bin.cu) --------------------------------------------------
 // Gated chain: count per cell (with the absolute positions and gather
-// records), scan, scatter, order each cell by original id, gather the new
-// sorted state.  kBinLaunches kernels.
-constexpr int kBinLaunches = 8;
+// records), scan, scatter, order and gather every cell; under the two-atom
+// layout also the slot tables.  bin_launches kernels.
 cudaError_t launch_bin(md_system *h, bool gated);
+int bin_launches(const md_system *h);
 // Exclusive scan of int32 counts into int32 starts (starts[n] = total).
 cudaError_t launch_scan_i32(const int32_t *in, int32_t *out, int n, int32_t *bsum,
                             const DevStatus *ds, bool gated, cudaStream_t s);
 // cell of each atom in original order; cell_start as int64
 cudaError_t launch_export_cells(md_system *h, int32_t *cell_of_atom, int64_t *cell_start);
 
+// kernels of one launch_scan over n values
+int scan_launch_count(long long n);
+
 // ---- neighbour list (k_nlist.cu) ------------------------------------------
 // positions: the float32 positions the list is built from (default: the
-// current buffer, right after binning)
+// current buffer, right after binning).  close: this list build is the last
+// pass of the rebuild (launch_finish_rebuild's work is done by its last block).
+// One kernel when gated (binning reset the counts), else two.
 cudaError_t launch_build_list(md_system *h, bool write, bool gated,
-                              const float4 *positions = nullptr);
+                              const float4 *positions = nullptr, bool close = false);
+cudaError_t launch_reset_counts(md_system *h, bool slots);
 cudaError_t launch_finish_rebuild(md_system *h, bool gated);
 cudaError_t launch_export_list(md_system *h, int half, int64_t *offsets, int32_t *ids,
                                int64_t *row_counts_tmp);
@@ -384,12 +420,12 @@ cudaError_t launch_cluster_forces(md_system *h, int mode, bool energy, bool stor
 // then per force pass assemble, exchange, inner and outer passes (4 kernels)
 cudaError_t launch_overlap_index(md_system *h, bool gated);
 cudaError_t launch_overlap_forces(md_system *h, int mode, bool energy, bool store_f);
-// two atoms per thread (k_pair.cu): slot tables and union lists after a
-// rebuild (7 kernels), one force kernel; the padding entries point at a
+// two atoms per thread (k_pair.cu): union lists after binning (as
+// launch_build_list), one force kernel; the padding entries point at a
 // dummy position at index n of both position buffers
 int64_t pair_slots_max(int64_t n, int ncells);
 cudaError_t launch_pair_dummy(md_system *h);
-cudaError_t launch_pair_build(md_system *h, bool write, bool gated);
+cudaError_t launch_pair_build(md_system *h, bool write, bool gated, bool close = false);
 cudaError_t launch_pair_forces(md_system *h, int mode, bool energy, bool store_f);
 cudaError_t launch_eam_density(md_system *h);  // k_eam.cu
 cudaError_t launch_eam_force(md_system *h, int mode, bool energy, bool store_f);
