@@ -26,6 +26,9 @@
 // buffer of a double-buffered pair; FM_FUSED_HALF applies the closing half
 // kick (v += dt f / 2m).  The drift also measures the displacement since the
 // last list build and raises the rebuild flag past half the skin (Sec. 3.3).
+#include <type_traits>
+
+#include "k_fp64.cuh"
 #include "k_pair.cuh"
 
 namespace mdg {
@@ -102,37 +105,41 @@ __device__ __forceinline__ void lj_mixed_atom(const ForceArgs &a, const ShiftTab
     if (MODE != FM_STORE) vv_epilogue<MODE>(a, i, Fx, Fy, Fz, qi.w);
 }
 
-// Float64 cell shifts (dx, dy, dz) * w of the 27 stencil cells.
-__device__ __forceinline__ void load_shifts_f64(const Grid &g, double3 *sh) {
-    if (threadIdx.x < kStencil) {
-        const int s = threadIdx.x;
-        const int dx = s % 3 - 1, dy = (s / 3) % 3 - 1, dz = s / 9 - 1;
-        sh[s] = make_double3(dx * g.w[0], dy * g.w[1], dz * g.w[2]);
+// Stores and the velocity-Verlet epilogue of one atom of the float64 path.
+template <int MODE, bool ENERGY, bool SPECIES>
+__device__ __forceinline__ void f64_atom_out(const ForceArgs &a, int i, double fx, double fy,
+                                             double fz, double e, float qw, int store_f) {
+    const size_t n = (size_t)a.n;
+    if (MODE == FM_STORE || store_f) {
+        a.f[i] = fx;
+        a.f[n + i] = fy;
+        a.f[2 * n + i] = fz;
     }
+    if (ENERGY) a.e_atom[i] = e;
+    if (MODE != FM_STORE) vv_epilogue<MODE, SPECIES>(a, i, fx, fy, fz, qw);
 }
 
-// The whole per-atom job of the plain float64 path for sorted atom i.
-template <int MODE, bool ENERGY>
-__device__ __forceinline__ void lj_fp64_atom(const ForceArgs &a, const double3 *sh, int i,
-                                             int store_f) {
-    const double4 ri = a.xr[i];
-    const int cnt = min(a.ncount[i], a.cap);
-    const double rc2 = a.fc.rc2, sig2 = a.fc.sig2, e48 = a.fc.eps48;
+// The whole per-atom job of the plain float64 path for sorted atom i, shared by
+// P lanes (lane `part`); on: the atom exists (all lanes of a warp call this).
+// The force scalar 48 eps r^-2 s6 (s6 - 1/2) with u = (sigma/r)^2 is
+// (48 eps / r^2) u^3 (u^3 - 1/2).
+template <int MODE, bool ENERGY, int P>
+__device__ __forceinline__ void lj_fp64_atom(const ForceArgs &a, const ShiftTab *sh, Home64 *h,
+                                             int i, int part, bool on, int store_f) {
     double fx = 0.0, fy = 0.0, fz = 0.0, e = 0.0;
     unsigned npair = 0;
-    for (int k = 0; k < cnt; ++k) {
-        const uint32_t ent = __ldg(a.nlist + list_idx(i, k, a.cap));
-        const double4 rj = a.xr[ent & kIndexMask];
-        const double3 sd = sh[ent >> kIndexBits];
-        const double ex = (rj.x - ri.x) + sd.x;
-        const double ey = (rj.y - ri.y) + sd.y;
-        const double ez = (rj.z - ri.z) + sd.z;
-        const double r2 = ex * ex + ey * ey + ez * ez;
-        if (r2 < rc2) {
-            const double r2i = 1.0 / r2;
+    float qw = 0.f;
+    if (on) {
+        const float4 qi = a.xq[i];
+        qw = qi.w;
+        load_home64(a, i, h);
+        const double sig2 = a.fc.sig2, e48 = a.fc.eps48;
+        const bool seeded = a.fc.f64_seeded;
+        f64_pairs<P>(a, sh, h, i, part, qi, [&](int, double ex, double ey, double ez, double r2) {
+            const double r2i = rcp_f64(r2, seeded);
             double s6 = sig2 * r2i;
             s6 = s6 * s6 * s6;
-            const double fs = e48 * r2i * s6 * (s6 - 0.5);
+            const double fs = (e48 * r2i) * fma(s6, s6, -0.5 * s6);
             fx -= fs * ex;
             fy -= fs * ey;
             fz -= fs * ez;
@@ -140,22 +147,16 @@ __device__ __forceinline__ void lj_fp64_atom(const ForceArgs &a, const double3 *
                 e += a.fc.eps4 * s6 * (s6 - 1.0) - a.fc.shift;
                 ++npair;
             }
-        }
+        });
     }
-    const size_t n = (size_t)a.n;
-    if (MODE == FM_STORE || store_f) {
-        a.f[i] = fx;
-        a.f[n + i] = fy;
-        a.f[2 * n + i] = fz;
+    if (P > 1) {
+        fx = lanes_sum<P>(fx);
+        fy = lanes_sum<P>(fy);
+        fz = lanes_sum<P>(fz);
+        if (ENERGY) e = lanes_sum<P>(e);
     }
-    if (ENERGY) {
-        a.e_atom[i] = 0.5 * e;
-        count_pairs(a.ds, npair);
-    }
-    if (MODE != FM_STORE) {
-        const float4 qi = a.xq[i];
-        vv_epilogue<MODE>(a, i, fx, fy, fz, qi.w);
-    }
+    if (ENERGY && on) count_pairs(a.ds, npair);
+    if (on && part == 0) f64_atom_out<MODE, ENERGY, false>(a, i, fx, fy, fz, 0.5 * e, qw, store_f);
 }
 
 // One thread per sorted atom; the hardware block scheduler spreads the work.
@@ -240,6 +241,7 @@ __device__ __forceinline__ void prefetch_l2(const void *p) {
 // 1.359 ms against 1.395 ms for 256 threads at 48 registers on the 9.8 M-atom
 // porous system.
 constexpr int kPersistBlock = 128;
+static_assert(kPersistBlock == kF64Block, "the float64 job's shared columns");
 // The slot job holds twice the accumulators: its persistent kernel gets up to
 // 64 registers (8 CTAs per SM) instead of spilling at 56.
 constexpr int kPersistPairedCtas = 9;
@@ -252,11 +254,10 @@ lj_mixed_persist(ForceArgs a, int store_f, SchedArgs sa, PairArgs pa) {
     static_assert(!(F64 && MULTI), "batches run the mixed path");
     static_assert(!(PAIRED && (F64 || MULTI || ENERGY)), "slots: one box, mixed path, forces");
     __shared__ ShiftTab sh;
-    __shared__ double3 sh64[F64 ? kStencil : 1];
+    __shared__ typename std::conditional<F64, Home64, int>::type home;
     __shared__ int s_first[kSchedRounds], s_pre[kSchedRounds + 1], s_next;  // this CTA's ranges
     __shared__ int s_stop;
-    if (F64) load_shifts_f64(a.g, sh64);
-    else if (!MULTI) load_shifts_f32(a.g, &sh);
+    if (!MULTI) load_shifts_f32(a.g, &sh);
     // one read of the status word for the whole CTA: every thread must take the
     // same branch, since the CTA meets barriers below
     if (threadIdx.x == 0) s_stop = a.ds->status;
@@ -370,9 +371,10 @@ lj_mixed_persist(ForceArgs a, int store_f, SchedArgs sa, PairArgs pa) {
             __syncwarp();
             t0 = clock64();
         }
-        if (active) {
+        if constexpr (F64) {
+            lj_fp64_atom<MODE, ENERGY, 1>(a, &sh, &home, active ? i : 0, 0, active, store_f);
+        } else if (active) {
             if (PAIRED) lj_pair_slot<MODE, false>(a, pa, &sh, i, store_f);
-            else if (F64) lj_fp64_atom<MODE, ENERGY>(a, sh64, i, store_f);
             else lj_mixed_atom<MODE, ENERGY, MULTI>(a, &sh, i, store_f);
         }
         if (TIMING) {
@@ -401,15 +403,31 @@ lj_mixed_persist(ForceArgs a, int store_f, SchedArgs sa, PairArgs pa) {
     }
 }
 
-template <int MODE, bool ENERGY>
-__global__ void __launch_bounds__(kBlock) lj_fp64_kernel(ForceArgs a, int store_f) {
-    __shared__ double3 sh[kStencil];
-    load_shifts_f64(a.g, sh);
+template <int MODE, bool ENERGY, int P>
+__global__ void __launch_bounds__(kF64Block) lj_fp64_kernel(ForceArgs a, int store_f) {
+    __shared__ ShiftTab sh;
+    __shared__ Home64 home;
+    load_shifts_f32(a.g, &sh);
     __syncthreads();
     if (a.ds->status != 0) return;
     step_bookkeeping<MODE>(a);
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < a.n) lj_fp64_atom<MODE, ENERGY>(a, sh, i, store_f);
+    const long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+    const bool on = t < (long long)a.n * P;
+    lj_fp64_atom<MODE, ENERGY, P>(a, &sh, &home, on ? (int)(t / P) : 0, (int)(t % P), on, store_f);
+}
+
+template <int P>
+cudaError_t launch_lj_fp64(const ForceArgs &a, int mode, bool energy, int sf, cudaStream_t s) {
+    const int nb = nblocks((int64_t)a.n * P, kF64Block);
+    switch (mode) {
+        case FM_STORE:
+            if (energy) lj_fp64_kernel<FM_STORE, true, P><<<nb, kF64Block, 0, s>>>(a, sf);
+            else lj_fp64_kernel<FM_STORE, false, P><<<nb, kF64Block, 0, s>>>(a, sf);
+            break;
+        case FM_FUSED_FULL: lj_fp64_kernel<FM_FUSED_FULL, false, P><<<nb, kF64Block, 0, s>>>(a, sf); break;
+        default: lj_fp64_kernel<FM_FUSED_HALF, false, P><<<nb, kF64Block, 0, s>>>(a, sf); break;
+    }
+    return cudaGetLastError();
 }
 
 // ---- multi-element Lennard-Jones (Sec. 2.2 pair loop, Sec. 3.1 Cu-Au) ------
@@ -516,36 +534,30 @@ __device__ __forceinline__ void lj_typed_mixed_atom(const ForceArgs &a, const Ty
     if (MODE != FM_STORE) vv_epilogue<MODE, true>(a, i, Fx, Fy, Fz, qi.w);
 }
 
-template <int MODE, bool ENERGY, int NT>
+template <int MODE, bool ENERGY, int NT, int P>
 __device__ __forceinline__ void lj_typed_fp64_atom(const ForceArgs &a, const TypeTab &tt,
-                                                   const double3 *sh, int i, int store_f) {
-    const double4 ri = a.xr[i];
-    const float4 qi = a.xq[i];
-    const int ti = species_of(__float_as_uint(qi.w));
-    double e48[NT], e4[NT], s2[NT], shd[NT];
-    load_row<NT>(tt.e48d, ti, e48);
-    load_row<NT>(tt.e4d, ti, e4);
-    load_row<NT>(tt.s2d, ti, s2);
-    load_row<NT>(tt.shd, ti, shd);
-    const int cnt = min(a.ncount[i], a.cap);
-    const double rc2 = a.fc.rc2;
+                                                   const ShiftTab *sh, Home64 *h, int i, int part,
+                                                   bool on, int store_f) {
     double fx = 0.0, fy = 0.0, fz = 0.0, e = 0.0;
     unsigned npair = 0;
-    for (int k = 0; k < cnt; ++k) {
-        const uint32_t ent = __ldg(a.nlist + list_idx(i, k, a.cap));
-        const int j = (int)(ent & kIndexMask);
-        const double4 rj = a.xr[j];
-        const double3 sd = sh[ent >> kIndexBits];
-        const double ex = (rj.x - ri.x) + sd.x;
-        const double ey = (rj.y - ri.y) + sd.y;
-        const double ez = (rj.z - ri.z) + sd.z;
-        const double r2 = ex * ex + ey * ey + ez * ez;
-        if (r2 < rc2) {
+    float qw = 0.f;
+    if (on) {
+        const float4 qi = a.xq[i];
+        qw = qi.w;
+        load_home64(a, i, h);
+        const int ti = species_of(__float_as_uint(qi.w));
+        double e48[NT], e4[NT], s2[NT], shd[NT];
+        load_row<NT>(tt.e48d, ti, e48);
+        load_row<NT>(tt.e4d, ti, e4);
+        load_row<NT>(tt.s2d, ti, s2);
+        load_row<NT>(tt.shd, ti, shd);
+        const bool seeded = a.fc.f64_seeded;
+        f64_pairs<P>(a, sh, h, i, part, qi, [&](int j, double ex, double ey, double ez, double r2) {
             const int tj = species_of(__float_as_uint(__ldg(&a.xq[j].w)));
-            const double r2i = 1.0 / r2;
+            const double r2i = rcp_f64(r2, seeded);
             double s6 = pick_row<NT>(s2, tj) * r2i;
             s6 = s6 * s6 * s6;
-            const double fs = pick_row<NT>(e48, tj) * r2i * s6 * (s6 - 0.5);
+            const double fs = (pick_row<NT>(e48, tj) * r2i) * fma(s6, s6, -0.5 * s6);
             fx -= fs * ex;
             fy -= fs * ey;
             fz -= fs * ez;
@@ -553,65 +565,99 @@ __device__ __forceinline__ void lj_typed_fp64_atom(const ForceArgs &a, const Typ
                 e += pick_row<NT>(e4, tj) * s6 * (s6 - 1.0) - pick_row<NT>(shd, tj);
                 ++npair;
             }
-        }
+        });
     }
-    const size_t n = (size_t)a.n;
-    if (MODE == FM_STORE || store_f) {
-        a.f[i] = fx;
-        a.f[n + i] = fy;
-        a.f[2 * n + i] = fz;
+    if (P > 1) {
+        fx = lanes_sum<P>(fx);
+        fy = lanes_sum<P>(fy);
+        fz = lanes_sum<P>(fz);
+        if (ENERGY) e = lanes_sum<P>(e);
     }
-    if (ENERGY) {
-        a.e_atom[i] = 0.5 * e;
-        count_pairs(a.ds, npair);
-    }
-    if (MODE != FM_STORE) vv_epilogue<MODE, true>(a, i, fx, fy, fz, qi.w);
+    if (ENERGY && on) count_pairs(a.ds, npair);
+    if (on && part == 0) f64_atom_out<MODE, ENERGY, true>(a, i, fx, fy, fz, 0.5 * e, qw, store_f);
 }
 
-template <int MODE, bool ENERGY, int NT, bool F64>
+template <int MODE, bool ENERGY, int NT, int P>
+__global__ void __launch_bounds__(kF64Block) lj_typed_fp64_kernel(ForceArgs a, TypeTab tt,
+                                                                  int store_f) {
+    __shared__ ShiftTab sh;
+    __shared__ Home64 home;
+    load_shifts_f32(a.g, &sh);
+    __syncthreads();
+    if (a.ds->status != 0) return;
+    step_bookkeeping<MODE>(a);
+    const long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+    const bool on = t < (long long)a.n * P;
+    lj_typed_fp64_atom<MODE, ENERGY, NT, P>(a, tt, &sh, &home, on ? (int)(t / P) : 0, (int)(t % P),
+                                            on, store_f);
+}
+
+template <int MODE, bool ENERGY, int NT>
 __global__ void __launch_bounds__(128) lj_typed_kernel(ForceArgs a, TypeTab tt, int store_f) {
     __shared__ ShiftTab sh;
-    __shared__ double3 sh64[F64 ? kStencil : 1];
-    if (F64) load_shifts_f64(a.g, sh64);
-    else load_shifts_f32(a.g, &sh);
+    load_shifts_f32(a.g, &sh);
     __syncthreads();
     if (a.ds->status != 0) return;
     step_bookkeeping<MODE>(a);
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= a.n) return;
-    if (F64) lj_typed_fp64_atom<MODE, ENERGY, NT>(a, tt, sh64, i, store_f);
-    else lj_typed_mixed_atom<MODE, ENERGY, NT>(a, tt, &sh, i, store_f);
+    lj_typed_mixed_atom<MODE, ENERGY, NT>(a, tt, &sh, i, store_f);
 }
 
-template <int NT, bool F64>
-cudaError_t launch_lj_typed_nt(md_system *h, const ForceArgs &a, int mode, bool energy, int sf) {
+template <int NT>
+cudaError_t launch_lj_typed_mixed(md_system *h, const ForceArgs &a, int mode, bool energy, int sf) {
     const int nb = nblocks(a.n, 128);
     cudaStream_t s = h->stream;
     const TypeTab &tt = h->types;
     switch (mode) {
         case FM_STORE:
-            if (energy) lj_typed_kernel<FM_STORE, true, NT, F64><<<nb, 128, 0, s>>>(a, tt, sf);
-            else lj_typed_kernel<FM_STORE, false, NT, F64><<<nb, 128, 0, s>>>(a, tt, sf);
+            if (energy) lj_typed_kernel<FM_STORE, true, NT><<<nb, 128, 0, s>>>(a, tt, sf);
+            else lj_typed_kernel<FM_STORE, false, NT><<<nb, 128, 0, s>>>(a, tt, sf);
             break;
         case FM_FUSED_FULL:
-            if (energy) lj_typed_kernel<FM_FUSED_FULL, true, NT, F64><<<nb, 128, 0, s>>>(a, tt, sf);
-            else lj_typed_kernel<FM_FUSED_FULL, false, NT, F64><<<nb, 128, 0, s>>>(a, tt, sf);
+            lj_typed_kernel<FM_FUSED_FULL, false, NT><<<nb, 128, 0, s>>>(a, tt, sf);
+            break;
+        default: lj_typed_kernel<FM_FUSED_HALF, false, NT><<<nb, 128, 0, s>>>(a, tt, sf); break;
+    }
+    return cudaGetLastError();
+}
+
+template <int NT, int P>
+cudaError_t launch_lj_typed_fp64(md_system *h, const ForceArgs &a, int mode, bool energy, int sf) {
+    const int nb = nblocks((int64_t)a.n * P, kF64Block);
+    cudaStream_t s = h->stream;
+    const TypeTab &tt = h->types;
+    switch (mode) {
+        case FM_STORE:
+            if (energy) lj_typed_fp64_kernel<FM_STORE, true, NT, P><<<nb, kF64Block, 0, s>>>(a, tt, sf);
+            else lj_typed_fp64_kernel<FM_STORE, false, NT, P><<<nb, kF64Block, 0, s>>>(a, tt, sf);
+            break;
+        case FM_FUSED_FULL:
+            lj_typed_fp64_kernel<FM_FUSED_FULL, false, NT, P><<<nb, kF64Block, 0, s>>>(a, tt, sf);
             break;
         default:
-            if (energy) lj_typed_kernel<FM_FUSED_HALF, true, NT, F64><<<nb, 128, 0, s>>>(a, tt, sf);
-            else lj_typed_kernel<FM_FUSED_HALF, false, NT, F64><<<nb, 128, 0, s>>>(a, tt, sf);
+            lj_typed_fp64_kernel<FM_FUSED_HALF, false, NT, P><<<nb, kF64Block, 0, s>>>(a, tt, sf);
             break;
     }
     return cudaGetLastError();
 }
 
-template <bool F64>
-cudaError_t launch_lj_typed_p(md_system *h, const ForceArgs &a, int mode, bool energy, int sf) {
+template <int NT>
+cudaError_t launch_lj_typed_nt(md_system *h, const ForceArgs &a, int mode, bool energy, int sf) {
+    if (h->p.precision == MD_MIXED) return launch_lj_typed_mixed<NT>(h, a, mode, energy, sf);
+    switch (f64_split(h->n)) {
+        case 1: return launch_lj_typed_fp64<NT, 1>(h, a, mode, energy, sf);
+        case 4: return launch_lj_typed_fp64<NT, 4>(h, a, mode, energy, sf);
+        default: return launch_lj_typed_fp64<NT, 16>(h, a, mode, energy, sf);
+    }
+}
+
+cudaError_t launch_lj_typed(md_system *h, const ForceArgs &a, int mode, bool energy, int sf) {
     switch (h->fc.ntypes) {
-        case 1: return launch_lj_typed_nt<1, F64>(h, a, mode, energy, sf);
-        case 2: return launch_lj_typed_nt<2, F64>(h, a, mode, energy, sf);
-        case 3: return launch_lj_typed_nt<3, F64>(h, a, mode, energy, sf);
-        default: return launch_lj_typed_nt<4, F64>(h, a, mode, energy, sf);
+        case 1: return launch_lj_typed_nt<1>(h, a, mode, energy, sf);
+        case 2: return launch_lj_typed_nt<2>(h, a, mode, energy, sf);
+        case 3: return launch_lj_typed_nt<3>(h, a, mode, energy, sf);
+        default: return launch_lj_typed_nt<4>(h, a, mode, energy, sf);
     }
 }
 
@@ -646,14 +692,9 @@ ForceArgs make_force_args(md_system *h) {
 
 cudaError_t launch_lj(md_system *h, int mode, bool energy, bool store_f) {
     ForceArgs a = make_force_args(h);
-    const int nb = nblocks(a.n);
     const int sf = store_f ? 1 : 0;
     cudaStream_t s = h->stream;
-    if (h->fc.ntypes > 0) {
-        return h->p.precision == MD_MIXED ? launch_lj_typed_p<false>(h, a, mode, energy, sf)
-                                          : launch_lj_typed_p<true>(h, a, mode, energy, sf);
-    }
-#define MDG_LJ(K, M, E) K<M, E><<<nb, kBlock, 0, s>>>(a, sf)
+    if (h->fc.ntypes > 0) return launch_lj_typed(h, a, mode, energy, sf);
     if (h->R > 1) {
         // several boxes: mixed precision only (checked at creation)
         constexpr int tb = grid_block<true>();
@@ -681,13 +722,12 @@ cudaError_t launch_lj(md_system *h, int mode, bool energy, bool store_f) {
         }
 #undef MDG_LJM
     } else {
-        switch (mode) {
-            case FM_STORE: if (energy) MDG_LJ(lj_fp64_kernel, FM_STORE, true); else MDG_LJ(lj_fp64_kernel, FM_STORE, false); break;
-            case FM_FUSED_FULL: if (energy) MDG_LJ(lj_fp64_kernel, FM_FUSED_FULL, true); else MDG_LJ(lj_fp64_kernel, FM_FUSED_FULL, false); break;
-            default: if (energy) MDG_LJ(lj_fp64_kernel, FM_FUSED_HALF, true); else MDG_LJ(lj_fp64_kernel, FM_FUSED_HALF, false); break;
+        switch (f64_split(h->n)) {
+            case 1: return launch_lj_fp64<1>(a, mode, energy, sf, s);
+            case 4: return launch_lj_fp64<4>(a, mode, energy, sf, s);
+            default: return launch_lj_fp64<16>(a, mode, energy, sf, s);
         }
     }
-#undef MDG_LJ
     return cudaGetLastError();
 }
 

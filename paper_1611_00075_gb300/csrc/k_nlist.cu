@@ -13,7 +13,9 @@
 // Both precisions build this way: the float32 positions are kept on the float64
 // path too, and the accepted set is the float64 definition's either way (4,000
 // atoms in float64: 50 steps with six builds 11.9 -> 9.1 ms against float64
-// distances for every candidate, on a pipe of 1/64 of the float32 rate).
+// distances for every candidate, on a pipe of 1/64 of the float32 rate).  The
+// comparisons are written so that NaN bounds (lengths that float32 cannot hold)
+// send every candidate to the float64 test.
 //
 // List layout: see list_idx() -- per warp group of 32 atoms, quads of four
 // entries per atom, written here with one 16-byte store per quad.  An entry is
@@ -122,16 +124,16 @@ __device__ __forceinline__ int list_atom(int i, const Grid &g, float lo, float h
                         const float4 qj = xq[j];
                         const float ex = qj.x - hx, ey = qj.y - hy, ez = qj.z - hz;
                         const float r2f = ex * ex + ey * ey + ez * ez;
-                        bool acc = (r2f < hi) & (j != skip);
+                        bool acc = !(r2f >= hi) & (j != skip);
                         if (HALF) acc = acc & (__float_as_int(qj.w) > myo);
                         if (WRITE) {
                             if (acc & (cnt < cap)) row[row_off(cnt)] = sbits | (uint32_t)j;
                         } else {
-                            const bool bq = acc & (r2f >= lo);
+                            const bool bq = acc & !(r2f < lo);
                             band.j = bq ? j : band.j;
                             band.s = bq ? s : band.s;
                         }
-                        const bool bnd = acc & (r2f >= lo);
+                        const bool bnd = acc & !(r2f < lo);
                         band.k = bnd ? cnt : band.k;
                         band.count += bnd ? 1 : 0;
                         cnt += acc ? 1 : 0;
@@ -142,10 +144,10 @@ __device__ __forceinline__ int list_atom(int i, const Grid &g, float lo, float h
                         const float4 qj = xq[j];
                         const float ex = qj.x - hx, ey = qj.y - hy, ez = qj.z - hz;
                         const float r2f = ex * ex + ey * ey + ez * ez;
-                        bool cand = (r2f < hi) && (j != skip);
+                        bool cand = !(r2f >= hi) && (j != skip);
                         if (HALF) cand = cand && (__float_as_int(qj.w) > myo);
                         if (!cand) continue;
-                        if (r2f >= lo && !exact_within_band(xabs, i, j, shx, shy, shz, rl2)) continue;
+                        if (!(r2f < lo) && !exact_within_band(xabs, i, j, shx, shy, shz, rl2)) continue;
                         if (WRITE && cnt < cap)
                             row[(size_t)(((cnt >> 2) << 7) | (cnt & 3))] = sbits | (uint32_t)j;
                         ++cnt;

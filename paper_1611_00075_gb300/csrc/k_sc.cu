@@ -20,6 +20,7 @@
 // sums rho and the forces in float64 over float32 chunks; F'(rho) feeds the
 // float32 pair terms as float32.  The embedding energy is float64.
 #include "k_common.cuh"
+#include "k_fp64.cuh"
 #include "k_pair.cuh"
 
 namespace mdg {
@@ -125,32 +126,46 @@ __global__ void __launch_bounds__(kBlock, 4) sc_density_mixed(ForceArgs a) {
     a.xqf[i] = make_float4(qi.x, qi.y, qi.z, dF);
 }
 
-__global__ void __launch_bounds__(kBlock) sc_density_fp64(ForceArgs a) {
-    __shared__ double3 sh[kStencil];
-    if (threadIdx.x < kStencil) {
-        int s = threadIdx.x;
-        int dx = s % 3 - 1, dy = (s / 3) % 3 - 1, dz = s / 9 - 1;
-        sh[s] = make_double3(dx * a.g.w[0], dy * a.g.w[1], dz * a.g.w[2]);
-    }
+// (a/r)^K in float64 from s = (a/r)^2, K = 0: the run-time exponent k; an odd
+// exponent also takes ar = a/r.
+template <int K>
+__device__ __forceinline__ double ar_pow_f64(double s, double ar, int k) {
+    if (K == 6) return s * s * s;
+    if (K == 9) return (s * s) * (s * s) * ar;
+    const double p = rpowd(s, k / 2);
+    return (k & 1) ? p * ar : p;
+}
+
+// The float64 passes run the pair loop of k_fp64.cuh, P lanes per atom; NE, ME:
+// the exponents 9 and 6 at compile time, or 0.
+template <int NE, int ME, int P>
+__global__ void __launch_bounds__(kF64Block) sc_density_fp64(ForceArgs a) {
+    __shared__ ShiftTab sh;
+    __shared__ Home64 home;
+    load_shifts_f32(a.g, &sh);
     __syncthreads();
     if (a.ds->status != 0) return;
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= a.n) return;
-    const double4 ri = a.xr[i];
-    const int cnt = min(a.ncount[i], a.cap);
-    const double rc2 = a.fc.rc2, A = a.fc.sc_a;
-    const int m = a.fc.sc_m;
+    const long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+    const bool on = t < (long long)a.n * P;
+    const int i = on ? (int)(t / P) : 0, part = (int)(t % P);
     double R = 0.0;
-    for (int k = 0; k < cnt; ++k) {
-        const uint32_t ent = __ldg(a.nlist + list_idx(i, k, a.cap));
-        const double4 rj = a.xr[ent & kIndexMask];
-        const double3 sd = sh[ent >> kIndexBits];
-        const double ex = (rj.x - ri.x) + sd.x;
-        const double ey = (rj.y - ri.y) + sd.y;
-        const double ez = (rj.z - ri.z) + sd.z;
-        const double r2 = ex * ex + ey * ey + ez * ez;
-        if (r2 < rc2) R += rpowd(A / sqrt(r2), m);
+    if (on) {
+        load_home64(a, i, &home);
+        const double A = a.fc.sc_a, A2 = A * A;
+        const int m = a.fc.sc_m;
+        const bool seeded = a.fc.f64_seeded;
+        f64_pairs<P>(a, &sh, &home, i, part, a.xq[i],
+                     [&](int, double, double, double, double r2) {
+                         if (ME > 0 ? (ME & 1) : (m & 1)) {
+                             const double ar = A * rsqrt_f64(r2, seeded);
+                             R += ar_pow_f64<ME>(ar * ar, ar, m);
+                         } else {
+                             R += ar_pow_f64<ME>(A2 * rcp_f64(r2, seeded), 0.0, m);
+                         }
+                     });
     }
+    if (P > 1) R = lanes_sum<P>(R);
+    if (!on || part != 0) return;
     a.rho[i] = R;
     const double d = sc_embed_deriv_f64(R, a.fc.sc_ec);
     a.dF64[i] = d;
@@ -240,63 +255,105 @@ __global__ void __launch_bounds__(kBlock, 4) sc_force_mixed(ForceArgs a, int sto
         vv_epilogue<MODE>(a, i, Fx, Fy, Fz, reinterpret_cast<const float *>(a.xq)[4 * (size_t)i + 3]);
 }
 
-template <int MODE, bool ENERGY>
-__global__ void __launch_bounds__(kBlock) sc_force_fp64(ForceArgs a, int store_f) {
-    __shared__ double3 sh[kStencil];
-    if (threadIdx.x < kStencil) {
-        int s = threadIdx.x;
-        int dx = s % 3 - 1, dy = (s / 3) % 3 - 1, dz = s / 9 - 1;
-        sh[s] = make_double3(dx * a.g.w[0], dy * a.g.w[1], dz * a.g.w[2]);
-    }
+template <int MODE, bool ENERGY, int NE, int ME, int P>
+__global__ void __launch_bounds__(kF64Block) sc_force_fp64(ForceArgs a, int store_f) {
+    __shared__ ShiftTab sh;
+    __shared__ Home64 home;
+    load_shifts_f32(a.g, &sh);
     __syncthreads();
     if (a.ds->status != 0) return;
     step_bookkeeping<MODE>(a);
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= a.n) return;
-    const double4 ri = a.xr[i];
-    const double dFi = a.dF64[i];
-    const int cnt = min(a.ncount[i], a.cap);
-    const double rc2 = a.fc.rc2, A = a.fc.sc_a, eps = a.fc.sc_eps;
-    const int nexp = a.fc.sc_n, mexp = a.fc.sc_m;
+    const long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+    const bool on = t < (long long)a.n * P;
+    const int i = on ? (int)(t / P) : 0, part = (int)(t % P);
     double fx = 0.0, fy = 0.0, fz = 0.0, e = 0.0;
     unsigned npair = 0;
-    for (int k = 0; k < cnt; ++k) {
-        const uint32_t ent = __ldg(a.nlist + list_idx(i, k, a.cap));
-        const int j = (int)(ent & kIndexMask);
-        const double4 rj = a.xr[j];
-        const double3 sd = sh[ent >> kIndexBits];
-        const double ex = (rj.x - ri.x) + sd.x;
-        const double ey = (rj.y - ri.y) + sd.y;
-        const double ez = (rj.z - ri.z) + sd.z;
-        const double r2 = ex * ex + ey * ey + ez * ez;
-        if (r2 < rc2) {
-            const double ar = A / sqrt(r2);
-            const double Phi = eps * rpowd(ar, nexp);
-            const double psi = rpowd(ar, mexp);
-            const double fs = (nexp * Phi + mexp * (dFi + a.dF64[j]) * psi) / r2;
-            fx -= fs * ex;
-            fy -= fs * ey;
-            fz -= fs * ez;
-            if (ENERGY) {
-                e += Phi;
-                ++npair;
-            }
-        }
+    float qw = 0.f;
+    if (on) {
+        const float4 qi = a.xq[i];
+        qw = qi.w;
+        load_home64(a, i, &home);
+        const double dFi = a.dF64[i];
+        const double A = a.fc.sc_a, A2 = A * A, eps = a.fc.sc_eps;
+        const int nexp = a.fc.sc_n, mexp = a.fc.sc_m;
+        const double nd = (double)(NE > 0 ? NE : nexp), mD = (double)(ME > 0 ? ME : mexp);
+        const bool odd = NE > 0 ? ((NE | ME) & 1) : ((nexp | mexp) & 1);
+        const bool seeded = a.fc.f64_seeded;
+        f64_pairs<P>(a, &sh, &home, i, part, qi,
+                     [&](int j, double ex, double ey, double ez, double r2) {
+                         double ar = 0.0, r2i;
+                         if (odd) {
+                             const double y = rsqrt_f64(r2, seeded);
+                             ar = A * y;
+                             r2i = y * y;
+                         } else {
+                             r2i = rcp_f64(r2, seeded);
+                         }
+                         const double s = A2 * r2i;
+                         const double Phi = eps * ar_pow_f64<NE>(s, ar, nexp);
+                         const double psi = ar_pow_f64<ME>(s, ar, mexp);
+                         const double fs = (nd * Phi + mD * (dFi + a.dF64[j]) * psi) * r2i;
+                         fx -= fs * ex;
+                         fy -= fs * ey;
+                         fz -= fs * ez;
+                         if (ENERGY) {
+                             e += Phi;
+                             ++npair;
+                         }
+                     });
     }
+    if (P > 1) {
+        fx = lanes_sum<P>(fx);
+        fy = lanes_sum<P>(fy);
+        fz = lanes_sum<P>(fz);
+        if (ENERGY) e = lanes_sum<P>(e);
+    }
+    if (ENERGY && on) count_pairs(a.ds, npair);
+    if (!on || part != 0) return;
     const size_t n = (size_t)a.n;
     if (MODE == FM_STORE || store_f) {
         a.f[i] = fx;
         a.f[n + i] = fy;
         a.f[2 * n + i] = fz;
     }
-    if (ENERGY) {
-        a.e_atom[i] = 0.5 * e - a.fc.sc_ec * sqrt(a.rho[i]);
-        count_pairs(a.ds, npair);
+    if (ENERGY) a.e_atom[i] = 0.5 * e - a.fc.sc_ec * sqrt(a.rho[i]);
+    if (MODE != FM_STORE) vv_epilogue<MODE>(a, i, fx, fy, fz, qw);
+}
+
+template <int NE, int ME, int P>
+cudaError_t launch_sc_fp64(const ForceArgs &a, bool density, int mode, bool energy, int sf,
+                           cudaStream_t s) {
+    const int nb = nblocks((int64_t)a.n * P, kF64Block);
+    if (density) {
+        sc_density_fp64<NE, ME, P><<<nb, kF64Block, 0, s>>>(a);
+        return cudaGetLastError();
     }
-    if (MODE != FM_STORE) {
-        const float4 qi = a.xq[i];
-        vv_epilogue<MODE>(a, i, fx, fy, fz, qi.w);
+    switch (mode) {
+        case FM_STORE:
+            if (energy) sc_force_fp64<FM_STORE, true, NE, ME, P><<<nb, kF64Block, 0, s>>>(a, sf);
+            else sc_force_fp64<FM_STORE, false, NE, ME, P><<<nb, kF64Block, 0, s>>>(a, sf);
+            break;
+        case FM_FUSED_FULL:
+            sc_force_fp64<FM_FUSED_FULL, false, NE, ME, P><<<nb, kF64Block, 0, s>>>(a, sf);
+            break;
+        default: sc_force_fp64<FM_FUSED_HALF, false, NE, ME, P><<<nb, kF64Block, 0, s>>>(a, sf); break;
     }
+    return cudaGetLastError();
+}
+
+// the pass (density or force) in float64, its lanes per atom by size
+cudaError_t launch_sc_fp64_any(const ForceArgs &a, bool density, int mode, bool energy, int sf,
+                               cudaStream_t s) {
+    const bool cu = a.fc.sc_n == 9 && a.fc.sc_m == 6;
+#define MDG_SC64(P)                                                                   \
+    (cu ? launch_sc_fp64<9, 6, P>(a, density, mode, energy, sf, s)                    \
+        : launch_sc_fp64<0, 0, P>(a, density, mode, energy, sf, s))
+    switch (f64_split(a.n)) {
+        case 1: return MDG_SC64(1);
+        case 4: return MDG_SC64(4);
+        default: return MDG_SC64(16);
+    }
+#undef MDG_SC64
 }
 
 // ---- two atoms per thread (MD_FORCE_PAIRED) ---------------------------------
@@ -556,7 +613,7 @@ cudaError_t launch_sc_density(md_system *h) {
         if (a.fc.sc_m == 6) sc_density_mixed<6><<<nb, kBlock, 0, h->stream>>>(a);
         else sc_density_mixed<0><<<nb, kBlock, 0, h->stream>>>(a);
     } else {
-        sc_density_fp64<<<nb, kBlock, 0, h->stream>>>(a);
+        return launch_sc_fp64_any(a, true, FM_STORE, false, 0, h->stream);
     }
     return cudaGetLastError();
 }
@@ -597,11 +654,7 @@ cudaError_t launch_sc_force(md_system *h, int mode, bool energy, bool store_f) {
         }
 #undef MDG_SC
     } else {
-        switch (mode) {
-            case FM_STORE: if (energy) sc_force_fp64<FM_STORE, true><<<nb, kBlock, 0, s>>>(a, sf); else sc_force_fp64<FM_STORE, false><<<nb, kBlock, 0, s>>>(a, sf); break;
-            case FM_FUSED_FULL: if (energy) sc_force_fp64<FM_FUSED_FULL, true><<<nb, kBlock, 0, s>>>(a, sf); else sc_force_fp64<FM_FUSED_FULL, false><<<nb, kBlock, 0, s>>>(a, sf); break;
-            default: if (energy) sc_force_fp64<FM_FUSED_HALF, true><<<nb, kBlock, 0, s>>>(a, sf); else sc_force_fp64<FM_FUSED_HALF, false><<<nb, kBlock, 0, s>>>(a, sf); break;
-        }
+        return launch_sc_fp64_any(a, false, mode, energy, sf, s);
     }
     return cudaGetLastError();
 }

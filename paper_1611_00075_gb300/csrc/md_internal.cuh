@@ -181,6 +181,10 @@ struct ForceConsts {
     // integrator
     double dt, inv_m;
     float half_skin2f;
+    // float64 passes: the float32 screen around r_c^2 (NaN: undecided, every
+    // entry goes to the float64 test) and whether float32 seeds serve
+    float scr_lo, scr_hi;
+    bool f64_seeded;
     // multi-element Lennard-Jones: species count (0 = one species) and the
     // inverse mass of each species; an atom's species sits in bits 27-28 of
     // its float32 position's w word, above the original id
