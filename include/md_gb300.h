@@ -80,7 +80,9 @@ enum { MD_FORCE_FULL = 0, MD_FORCE_HALF_COLOR = 1, MD_FORCE_HALF_ATOMIC = 2,
  * cells into equal-cost ranges per persistent CTA and leave the last fifth
  * of the cost as a tail that CTAs claim tile by tile when their ranges are
  * done.  The learned model is trained on the mixed kernel's timings, so the
- * float64 path partitions by list length under MD_SCHED_MLP too. */
+ * float64 path partitions by list length under MD_SCHED_MLP too.  A system whose
+ * atoms (or two-atom slots) all fit the resident CTAs at once has nothing to
+ * schedule and runs the grid launch under every scheduler, with the same bits. */
 enum {
     MD_SCHED_GRID = 0,      /* one thread per atom, hardware block scheduler */
     MD_SCHED_PAIRCOUNT = 1, /* persistent CTAs, static partition by list length */

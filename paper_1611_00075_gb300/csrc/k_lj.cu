@@ -240,7 +240,7 @@ __device__ __forceinline__ void prefetch_l2(const void *p) {
 // CTAs of 128 threads at up to 56 registers (9 per SM) were measured fastest:
 // 1.359 ms against 1.395 ms for 256 threads at 48 registers on the 9.8 M-atom
 // porous system.
-constexpr int kPersistBlock = 128;
+constexpr int kPersistBlock = kPersistThreads;
 static_assert(kPersistBlock == kF64Block, "the float64 job's shared columns");
 // The slot job holds twice the accumulators: its persistent kernel gets up to
 // 64 registers (8 CTAs per SM) instead of spilling at 56.

@@ -253,11 +253,21 @@ void harvest(md_system *h, size_t upto = SIZE_MAX) {
 
 // ---- persistent scheduler ----------------------------------------------------
 
-// The persistent kernel serves the mixed-precision Lennard-Jones full-list
-// force pass; every other combination uses the one-thread-per-atom grid.
-bool persistent_path(const md_system *h) {
+// The persistent kernel serves the Lennard-Jones full-list and two-atom force
+// passes; every other combination uses the one-thread-per-item grid.
+bool scheduled(const md_system *h) {
     return h->p.scheduler != MD_SCHED_GRID && h->p.potential == MD_POT_LJ &&
            (h->p.force_variant == MD_FORCE_FULL || h->p.force_variant == MD_FORCE_PAIRED);
+}
+
+// A system with at most one tile of 32 items per resident warp has nothing to
+// schedule: every tile runs at once, and the grid launch (the same job per item,
+// bit for bit) does that without claims or partition -- a persistent warp claims
+// its next tile while it runs one, so half of the warps took two tiles and half
+// none: 70 against 32 us per force launch at 153,600 porous atoms in slots of two.
+bool persistent_path(const md_system *h) {
+    const int64_t items = h->p.force_variant == MD_FORCE_PAIRED ? (h->n + 1) / 2 : h->n;
+    return scheduled(h) && items > (int64_t)h->sched_ctas * kPersistThreads;
 }
 
 bool uses_partition(const md_system *h) {
@@ -326,8 +336,8 @@ md_status ensure_sched(md_system *h) {
 
 // Cost estimate and equal-cost partition of the cells over the persistent
 // CTAs; part of the rebuild chain (gated) or run right away.
-md_status enqueue_sched_prep(md_system *h, bool gated) {
-    if (!uses_partition(h)) return MD_OK;
+md_status enqueue_sched_prep(md_system *h, bool gated, bool always = false) {
+    if (!always && !uses_partition(h)) return MD_OK;
     // the cost model learns the mixed kernel's timings; the float64 path
     // partitions by pair count under either static scheduler
     const bool pc = (h->p.scheduler == MD_SCHED_PAIRCOUNT) || h->p.precision == MD_FP64;
@@ -1506,6 +1516,11 @@ md_status md_cost_model(md_system *h, int32_t op, float *loss_out) {
             // one timed force pass with the current scheduler: max / mean CTA cycles
             st = enqueue_rebuild(h, true);
             if (st != MD_OK) return st;
+            if (scheduled(h) && !uses_partition(h) && h->p.scheduler != MD_SCHED_DYNAMIC) {
+                // a system too small for the schedulers keeps no partition
+                st = enqueue_sched_prep(h, false, true);
+                if (st != MD_OK) return st;
+            }
             MD_CK(cudaMemsetAsync(h->cell_cycles, 0, (size_t)h->g.ncells * sizeof(float),
                                   h->stream));
             MD_CK(cudaMemsetAsync(h->cta_cycles, 0, (size_t)h->sched_ctas * sizeof(float),
