@@ -28,6 +28,30 @@ __device__ __forceinline__ float rsqrt_fast(float x) {
     return r;
 }
 
+// Sum over the P neighbouring lanes that share an item (P a power of two; every
+// lane of the warp calls it).
+template <int P, class T>
+__device__ __forceinline__ T split_sum(T x) {
+#pragma unroll
+    for (int o = P / 2; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+    return x;
+}
+
+// pair(entry) for every entry of the quads part, part + P, ... of an item's list
+// (lq: its first quad; quads lie 32 apart), one quad loaded ahead.
+template <int P, class Pair>
+__device__ __forceinline__ void split_quads(const uint4 *lq, int nq, int part, const Pair &pair) {
+    uint4 nxt = part < nq ? __ldcs(lq + (size_t)part * 32) : make_uint4(0u, 0u, 0u, 0u);
+    for (int q = part; q < nq; q += P) {
+        const uint4 e4 = nxt;
+        if (q + P < nq) nxt = __ldcs(lq + (size_t)(q + P) * 32);
+        pair(e4.x);
+        pair(e4.y);
+        pair(e4.z);
+        pair(e4.w);
+    }
+}
+
 struct ForceArgs {
     int n, cap, step, rebuild_every;
     const float4 *__restrict__ xq;
@@ -102,6 +126,75 @@ __device__ __forceinline__ void vv_epilogue(const ForceArgs &a, int i, double Fx
         if (!(d2 <= 3.0e38f)) atomicCAS(&a.ds->status, 0, (int)MD_ERR_NONFINITE);
         if (a.rebuild_every <= 0 && d2 > a.fc.half_skin2f) a.ds->rebuild = 1;
     }
+}
+
+// What the epilogue of one component of an atom reads, loaded before its list is
+// walked.
+struct SplitState {
+    double v, r;  // velocity and position component
+    float b;      // position component at the last build
+};
+template <int MODE>
+__device__ __forceinline__ SplitState load_split_state(const ForceArgs &a, int i, int c, bool on) {
+    SplitState t{0.0, 0.0, 0.f};
+    if (MODE != FM_STORE && on && c < 3) {
+        t.v = a.v[(size_t)c * a.n + i];
+        if (MODE == FM_FUSED_FULL) {
+            t.r = reinterpret_cast<const double *>(a.xr + i)[c];
+            t.b = reinterpret_cast<const float *>(a.xq_build + i)[c];
+        }
+    }
+    return t;
+}
+
+// Stores and the velocity-Verlet epilogue of atom i by four neighbouring lanes
+// (aligned to four; every lane of the warp calls it): lane c of the four owns
+// component c (x, y, z), lane 3 the position word qw.  on: the atom exists.  The
+// arithmetic of each component is vv_epilogue's; a float64 instruction then
+// serves three components of eight atoms where one lane per atom would spend
+// three on eight.
+template <int MODE, bool SPECIES = false>
+__device__ __forceinline__ void split_epilogue(const ForceArgs &a, int i, int c, bool on, double F,
+                                               float qw, const SplitState &t, int store_f) {
+    const size_t n = (size_t)a.n;
+    const bool comp = on && c < 3;
+    if ((MODE == FM_STORE || store_f) && comp) a.f[(size_t)c * n + i] = F;
+    if (MODE == FM_STORE) return;
+    double im = a.fc.inv_m;
+    if (SPECIES) im = pick4(a.fc.t_inv_m, species_of(__float_as_uint(qw)));
+    const double hk = (MODE == FM_FUSED_FULL) ? a.fc.dt * im : 0.5 * a.fc.dt * im;
+    const double v = t.v + hk * F;
+    if (comp) a.v[(size_t)c * n + i] = v;
+    if (MODE != FM_FUSED_FULL) return;
+    const double r = t.r + a.fc.dt * v;
+    const float q = c < 3 ? (float)r : qw;
+    if (comp) reinterpret_cast<double *>(a.xr_out + i)[c] = r;
+    if (on) reinterpret_cast<float *>(a.xq_out + i)[c] = q;
+    // the displacement since the last build, summed as in vv_epilogue
+    const float dd = q - t.b;
+    const int lane = (int)(threadIdx.x & 31) & ~3;
+    const float dx = __shfl_sync(0xffffffffu, dd, lane), dy = __shfl_sync(0xffffffffu, dd, lane + 1),
+                dz = __shfl_sync(0xffffffffu, dd, lane + 2);
+    const float d2 = dx * dx + dy * dy + dz * dz;
+    if (on && c == 0) {
+        if (!(d2 <= 3.0e38f)) atomicCAS(&a.ds->status, 0, (int)MD_ERR_NONFINITE);
+        if (a.rebuild_every <= 0 && d2 > a.fc.half_skin2f) a.ds->rebuild = 1;
+    }
+}
+
+// Lanes per work item (atom or two-atom slot) of the mixed passes: one item's
+// list is a serial chain of gathers, so a system that leaves most of the GPU
+// idle is split.  The lanes' float32 sums cover at most cap / P entries, kept
+// within the 64 of the one-lane kernels' chunks.  Force launch (LJ, timed by
+// events, which add about 4 us), one lane / four / eight: per-atom lists 14.0 /
+// 9.8 / 7.9 us at 864 atoms, 14.2 / 9.8 / 8.1 at 4,000, 16.0 / 13.8 / 24 at
+// 32,000, 22.5 / 33 / 51 at 87,808 (float64 instructions of the epilogue); slots
+// of two atoms 22.0 / - / 8.7 at 864, 24.1 / - / 8.6 at 4,000, 23.8 / 16.7 at
+// 32,000, 26.1 / 25.7 at 87,808 atoms.
+inline int mixed_split(int64_t items, int cap) {
+    if (items <= 16384 && cap <= 8 * 4 * kChunkQ) return 8;
+    if (items <= 65536 && cap <= 4 * 4 * kChunkQ) return 4;
+    return 1;
 }
 
 // Adds v over the converged lanes of the warp to the in-cutoff pair counter

@@ -36,10 +36,12 @@ namespace mdg {
 // The whole per-atom job of the mixed path for sorted atom i: pair loop over
 // its list, stores, and the velocity-Verlet epilogue.  MULTI (systems of
 // several boxes) reads the cell shifts of the atom's own box from a global
-// R x 27 table instead of the block's shared table.
-template <int MODE, bool ENERGY, bool MULTI = false>
+// R x 27 table instead of the block's shared table.  P > 1: the P lanes of the
+// atom (this one is `part`; on: the atom exists) each walk every P-th quad and
+// add their sums.
+template <int MODE, bool ENERGY, bool MULTI = false, int P = 1>
 __device__ __forceinline__ void lj_mixed_atom(const ForceArgs &a, const ShiftTab *sh, int i,
-                                              int store_f) {
+                                              int store_f, int part = 0, bool on = true) {
     const float4 *shr = MULTI ? a.shifts32 + 27 * (int)a.rep[i] : nullptr;
     const float4 qi = a.xq[i];
     const int nq = (min(a.ncount[i], a.cap) + 3) >> 2;
@@ -70,26 +72,44 @@ __device__ __forceinline__ void lj_mixed_atom(const ForceArgs &a, const ShiftTab
             }
         }
     };
-    // list quads stream through once (evict-first), one quad loaded ahead;
-    // the float64 sums run once per chunk, outside the inner loop
-    uint4 nxt = nq > 0 ? __ldcs(lq) : make_uint4(0u, 0u, 0u, 0u);
-    for (int q0 = 0; q0 < nq; q0 += kChunkQ) {
-        const int q1 = min(q0 + kChunkQ, nq);
-        for (int q = q0; q < q1; ++q) {
-            const uint4 e4 = nxt;
-            if (q + 1 < nq) nxt = __ldcs(lq + (size_t)(q + 1) * 32);
-            pair(e4.x);
-            pair(e4.y);
-            pair(e4.z);
-            pair(e4.w);
-        }
-        Fx += (double)fx;
-        Fy += (double)fy;
-        Fz += (double)fz;
-        fx = fy = fz = 0.f;
+    if constexpr (P > 1) {
+        // the float32 sums cover a P-th of the list
+        const int c = part & 3;
+        const SplitState t = load_split_state<MODE>(a, i, c, on && part < 4);
+        split_quads<P>(lq, on ? nq : 0, part, pair);
+        fx = split_sum<P>(fx);
+        fy = split_sum<P>(fy);
+        fz = split_sum<P>(fz);
         if (ENERGY) {
-            E += (double)e;
-            e = 0.f;
+            e = split_sum<P>(e);
+            if (on) count_pairs(a.ds, npair);
+            if (on && part == 0) a.e_atom[i] = 0.5 * (double)e;
+        }
+        split_epilogue<MODE>(a, i, c, on && part < 4, (double)(c == 0 ? fx : (c == 1 ? fy : fz)),
+                             qi.w, t, store_f);
+        return;
+    } else {
+        // list quads stream through once (evict-first), one quad loaded ahead;
+        // the float64 sums run once per chunk, outside the inner loop
+        uint4 nxt = nq > 0 ? __ldcs(lq) : make_uint4(0u, 0u, 0u, 0u);
+        for (int q0 = 0; q0 < nq; q0 += kChunkQ) {
+            const int q1 = min(q0 + kChunkQ, nq);
+            for (int q = q0; q < q1; ++q) {
+                const uint4 e4 = nxt;
+                if (q + 1 < nq) nxt = __ldcs(lq + (size_t)(q + 1) * 32);
+                pair(e4.x);
+                pair(e4.y);
+                pair(e4.z);
+                pair(e4.w);
+            }
+            Fx += (double)fx;
+            Fy += (double)fy;
+            Fz += (double)fz;
+            fx = fy = fz = 0.f;
+            if (ENERGY) {
+                E += (double)e;
+                e = 0.f;
+            }
         }
     }
     const size_t n = (size_t)a.n;
@@ -170,16 +190,18 @@ __device__ __forceinline__ void lj_fp64_atom(const ForceArgs &a, const ShiftTab 
 template <bool MULTI>
 constexpr int grid_block() { return MULTI ? 256 : 128; }
 
-template <int MODE, bool ENERGY, bool MULTI = false>
-__global__ void __launch_bounds__(grid_block<MULTI>(), MULTI ? 4 : 5)
+//
+// P > 1: thread t serves atom t / P (blocks of 128).
+template <int MODE, bool ENERGY, bool MULTI = false, int P = 1>
+__global__ void __launch_bounds__(P > 1 ? 128 : grid_block<MULTI>(), P > 1 ? 1 : (MULTI ? 4 : 5))
 lj_mixed_kernel(ForceArgs a, int store_f) {
     __shared__ ShiftTab sh[MULTI ? 2 : 1];
     __shared__ int s_r0, s_span;
     if (!MULTI) {
         load_shifts_f32(a.g, &sh[0]);
     } else {
-        const int i0 = blockIdx.x * blockDim.x;
-        const int r0 = a.rep[i0], r1 = a.rep[min(a.n, i0 + (int)blockDim.x) - 1];
+        const int i0 = blockIdx.x * (blockDim.x / P);
+        const int r0 = a.rep[i0], r1 = a.rep[min(a.n, i0 + (int)blockDim.x / P) - 1];
         if (threadIdx.x < 2 * kStencil) {
             const int t = threadIdx.x / kStencil, st = threadIdx.x % kStencil;
             if (t <= r1 - r0) {
@@ -197,6 +219,16 @@ lj_mixed_kernel(ForceArgs a, int store_f) {
     __syncthreads();
     if (a.ds->status != 0) return;
     step_bookkeeping<MODE>(a);
+    if constexpr (P > 1) {
+        const int t = blockIdx.x * blockDim.x + threadIdx.x;
+        const bool on = t / P < a.n;
+        const int i = on ? t / P : a.n - 1;
+        if (MULTI && s_span <= 1)
+            lj_mixed_atom<MODE, ENERGY, false, P>(a, &sh[(int)a.rep[i] - s_r0], i, store_f, t % P, on);
+        else
+            lj_mixed_atom<MODE, ENERGY, MULTI, P>(a, &sh[0], i, store_f, t % P, on);
+        return;
+    }
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= a.n) return;
     if (MULTI && s_span <= 1)
@@ -463,9 +495,10 @@ __device__ __forceinline__ void load_row(const T *tab, int ti, T *row) {
     }
 }
 
-template <int MODE, bool ENERGY, int NT>
+template <int MODE, bool ENERGY, int NT, int P>
 __device__ __forceinline__ void lj_typed_mixed_atom(const ForceArgs &a, const TypeTab &tt,
-                                                    const ShiftTab *sh, int i, int store_f) {
+                                                    const ShiftTab *sh, int i, int store_f,
+                                                    int part, bool on) {
     const float4 qi = a.xq[i];
     const int ti = species_of(__float_as_uint(qi.w));
     float e48[NT], e4[NT], s2[NT], shf[NT];
@@ -501,6 +534,22 @@ __device__ __forceinline__ void lj_typed_mixed_atom(const ForceArgs &a, const Ty
             }
         }
     };
+    if constexpr (P > 1) {
+        const int c = part & 3;
+        const SplitState t = load_split_state<MODE>(a, i, c, on && part < 4);
+        split_quads<P>(lq, on ? nq : 0, part, pair);
+        fx = split_sum<P>(fx);
+        fy = split_sum<P>(fy);
+        fz = split_sum<P>(fz);
+        if (ENERGY) {
+            e = split_sum<P>(e);
+            if (on) count_pairs(a.ds, npair);
+            if (on && part == 0) a.e_atom[i] = 0.5 * (double)e;
+        }
+        split_epilogue<MODE, true>(a, i, c, on && part < 4,
+                                   (double)(c == 0 ? fx : (c == 1 ? fy : fz)), qi.w, t, store_f);
+        return;
+    }
     uint4 nxt = nq > 0 ? __ldcs(lq) : make_uint4(0u, 0u, 0u, 0u);
     for (int q0 = 0; q0 < nq; q0 += kChunkQ) {
         const int q1 = min(q0 + kChunkQ, nq);
@@ -592,32 +641,33 @@ __global__ void __launch_bounds__(kF64Block) lj_typed_fp64_kernel(ForceArgs a, T
                                             on, store_f);
 }
 
-template <int MODE, bool ENERGY, int NT>
+template <int MODE, bool ENERGY, int NT, int P>
 __global__ void __launch_bounds__(128) lj_typed_kernel(ForceArgs a, TypeTab tt, int store_f) {
     __shared__ ShiftTab sh;
     load_shifts_f32(a.g, &sh);
     __syncthreads();
     if (a.ds->status != 0) return;
     step_bookkeeping<MODE>(a);
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= a.n) return;
-    lj_typed_mixed_atom<MODE, ENERGY, NT>(a, tt, &sh, i, store_f);
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    const bool on = t / P < a.n;
+    if (P == 1 && !on) return;
+    lj_typed_mixed_atom<MODE, ENERGY, NT, P>(a, tt, &sh, on ? t / P : a.n - 1, store_f, t % P, on);
 }
 
-template <int NT>
+template <int NT, int P>
 cudaError_t launch_lj_typed_mixed(md_system *h, const ForceArgs &a, int mode, bool energy, int sf) {
-    const int nb = nblocks(a.n, 128);
+    const int nb = nblocks((int64_t)a.n * P, 128);
     cudaStream_t s = h->stream;
     const TypeTab &tt = h->types;
     switch (mode) {
         case FM_STORE:
-            if (energy) lj_typed_kernel<FM_STORE, true, NT><<<nb, 128, 0, s>>>(a, tt, sf);
-            else lj_typed_kernel<FM_STORE, false, NT><<<nb, 128, 0, s>>>(a, tt, sf);
+            if (energy) lj_typed_kernel<FM_STORE, true, NT, P><<<nb, 128, 0, s>>>(a, tt, sf);
+            else lj_typed_kernel<FM_STORE, false, NT, P><<<nb, 128, 0, s>>>(a, tt, sf);
             break;
         case FM_FUSED_FULL:
-            lj_typed_kernel<FM_FUSED_FULL, false, NT><<<nb, 128, 0, s>>>(a, tt, sf);
+            lj_typed_kernel<FM_FUSED_FULL, false, NT, P><<<nb, 128, 0, s>>>(a, tt, sf);
             break;
-        default: lj_typed_kernel<FM_FUSED_HALF, false, NT><<<nb, 128, 0, s>>>(a, tt, sf); break;
+        default: lj_typed_kernel<FM_FUSED_HALF, false, NT, P><<<nb, 128, 0, s>>>(a, tt, sf); break;
     }
     return cudaGetLastError();
 }
@@ -644,7 +694,9 @@ cudaError_t launch_lj_typed_fp64(md_system *h, const ForceArgs &a, int mode, boo
 
 template <int NT>
 cudaError_t launch_lj_typed_nt(md_system *h, const ForceArgs &a, int mode, bool energy, int sf) {
-    if (h->p.precision == MD_MIXED) return launch_lj_typed_mixed<NT>(h, a, mode, energy, sf);
+    if (h->p.precision == MD_MIXED)
+        return mixed_split(h->n, h->cap) > 1 ? launch_lj_typed_mixed<NT, 8>(h, a, mode, energy, sf)
+                                             : launch_lj_typed_mixed<NT, 1>(h, a, mode, energy, sf);
     switch (f64_split(h->n)) {
         case 1: return launch_lj_typed_fp64<NT, 1>(h, a, mode, energy, sf);
         case 4: return launch_lj_typed_fp64<NT, 4>(h, a, mode, energy, sf);
@@ -690,37 +742,35 @@ ForceArgs make_force_args(md_system *h) {
     return a;
 }
 
+template <bool MULTI, int P>
+cudaError_t launch_lj_mixed(const ForceArgs &a, int mode, bool energy, int sf, cudaStream_t s) {
+    const int tb = P > 1 ? 128 : grid_block<MULTI>();
+    const int nb = nblocks((int64_t)a.n * P, tb);
+    switch (mode) {
+        case FM_STORE:
+            if (energy) lj_mixed_kernel<FM_STORE, true, MULTI, P><<<nb, tb, 0, s>>>(a, sf);
+            else lj_mixed_kernel<FM_STORE, false, MULTI, P><<<nb, tb, 0, s>>>(a, sf);
+            break;
+        case FM_FUSED_FULL: lj_mixed_kernel<FM_FUSED_FULL, false, MULTI, P><<<nb, tb, 0, s>>>(a, sf); break;
+        default: lj_mixed_kernel<FM_FUSED_HALF, false, MULTI, P><<<nb, tb, 0, s>>>(a, sf); break;
+    }
+    return cudaGetLastError();
+}
+
 cudaError_t launch_lj(md_system *h, int mode, bool energy, bool store_f) {
     ForceArgs a = make_force_args(h);
     const int sf = store_f ? 1 : 0;
     cudaStream_t s = h->stream;
     if (h->fc.ntypes > 0) return launch_lj_typed(h, a, mode, energy, sf);
-    if (h->R > 1) {
-        // several boxes: mixed precision only (checked at creation)
-        constexpr int tb = grid_block<true>();
-        const int nbm = nblocks(a.n, tb);
-        switch (mode) {
-            case FM_STORE:
-                if (energy) lj_mixed_kernel<FM_STORE, true, true><<<nbm, tb, 0, s>>>(a, sf);
-                else lj_mixed_kernel<FM_STORE, false, true><<<nbm, tb, 0, s>>>(a, sf);
-                break;
-            case FM_FUSED_FULL:
-                lj_mixed_kernel<FM_FUSED_FULL, false, true><<<nbm, tb, 0, s>>>(a, sf);
-                break;
-            default:
-                lj_mixed_kernel<FM_FUSED_HALF, false, true><<<nbm, tb, 0, s>>>(a, sf);
-                break;
-        }
-    } else if (h->p.precision == MD_MIXED) {
-        constexpr int tb = grid_block<false>();
-        const int nbs = nblocks(a.n, tb);
-#define MDG_LJM(M, E) lj_mixed_kernel<M, E><<<nbs, tb, 0, s>>>(a, sf)
-        switch (mode) {
-            case FM_STORE: if (energy) MDG_LJM(FM_STORE, true); else MDG_LJM(FM_STORE, false); break;
-            case FM_FUSED_FULL: if (energy) MDG_LJM(FM_FUSED_FULL, true); else MDG_LJM(FM_FUSED_FULL, false); break;
-            default: if (energy) MDG_LJM(FM_FUSED_HALF, true); else MDG_LJM(FM_FUSED_HALF, false); break;
-        }
-#undef MDG_LJM
+    if (h->p.precision == MD_MIXED) {
+        const int P = mixed_split(h->n, h->cap);
+        if (h->R > 1)
+            return P == 8 ? launch_lj_mixed<true, 8>(a, mode, energy, sf, s)
+                 : P == 4 ? launch_lj_mixed<true, 4>(a, mode, energy, sf, s)
+                          : launch_lj_mixed<true, 1>(a, mode, energy, sf, s);
+        return P == 8 ? launch_lj_mixed<false, 8>(a, mode, energy, sf, s)
+             : P == 4 ? launch_lj_mixed<false, 4>(a, mode, energy, sf, s)
+                      : launch_lj_mixed<false, 1>(a, mode, energy, sf, s);
     } else {
         switch (f64_split(h->n)) {
             case 1: return launch_lj_fp64<1>(a, mode, energy, sf, s);

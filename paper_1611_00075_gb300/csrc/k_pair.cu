@@ -188,17 +188,19 @@ __global__ void pair_dummy_kernel(float4 *xq0, float4 *xq1, float4 *xqf, int n) 
 // belong to one or two boxes (more only when a box holds fewer slots than a
 // block); the shift tables of those boxes go to shared memory like a single
 // box's, and a block that spans more boxes reads the global R x 27 table.
-template <int MODE, bool ENERGY, bool MULTI = false>
-__global__ void __launch_bounds__(kPairBlock, 9) lj_pair_kernel(ForceArgs a, PairArgs p,
-                                                                int store_f) {
+//
+// P > 1: thread t serves slot t / P.
+template <int MODE, bool ENERGY, bool MULTI = false, int P = 1>
+__global__ void __launch_bounds__(kPairBlock, P > 1 ? 1 : 9)
+lj_pair_kernel(ForceArgs a, PairArgs p, int store_f) {
     __shared__ ShiftTab sh[MULTI ? 2 : 1];
     __shared__ int s_r0, s_span;
     const int nslots = p.slot_start[p.ncells];
     if (!MULTI) {
         load_shifts_f32(a.g, &sh[0]);
     } else {
-        const int sb = blockIdx.x * blockDim.x;
-        const int se = min(nslots, sb + (int)blockDim.x) - 1;
+        const int sb = blockIdx.x * (blockDim.x / P);
+        const int se = min(nslots, sb + (int)blockDim.x / P) - 1;
         const int r0 = sb <= se ? (int)a.rep[p.slot_atom[sb] & ~kSingle] : 0;
         const int r1 = sb <= se ? (int)a.rep[p.slot_atom[se] & ~kSingle] : 0;
         if (threadIdx.x < 2 * kStencil) {
@@ -218,6 +220,19 @@ __global__ void __launch_bounds__(kPairBlock, 9) lj_pair_kernel(ForceArgs a, Pai
     __syncthreads();
     if (a.ds->status != 0) return;
     step_bookkeeping<MODE>(a);
+    if constexpr (P > 1) {
+        const int t = blockIdx.x * blockDim.x + threadIdx.x;
+        if ((t & ~31) / P >= nslots) return;  // whole warps: the lanes add their sums
+        const bool on = t / P < nslots;
+        const int s = on ? t / P : nslots - 1;
+        if (MULTI && s_span <= 1) {
+            const int r = (int)a.rep[p.slot_atom[s] & ~kSingle];
+            lj_pair_slot<MODE, ENERGY, false, P>(a, p, &sh[r - s_r0], s, store_f, t % P, on);
+        } else {
+            lj_pair_slot<MODE, ENERGY, MULTI, P>(a, p, &sh[0], s, store_f, t % P, on);
+        }
+        return;
+    }
     const int s = blockIdx.x * blockDim.x + threadIdx.x;
     if (s >= nslots) return;
     if (MULTI && s_span <= 1) {
@@ -264,31 +279,36 @@ cudaError_t launch_pair_build(md_system *h, bool write, bool gated, bool close) 
 // the multi-element variant (k_pair_typed.cu)
 cudaError_t launch_pair_typed_forces(md_system *h, int mode, bool energy, bool store_f);
 
+template <bool MULTI, int P>
+static cudaError_t launch_pair_lj(md_system *h, int mode, bool energy, int sf) {
+    const ForceArgs a = make_force_args(h);
+    const PairArgs p = make_pair_args(h);
+    const int nb = pair_grid_blocks(h, kPairBlock, P);
+    cudaStream_t s = h->stream;
+    switch (mode) {
+        case FM_STORE:
+            if (energy) lj_pair_kernel<FM_STORE, true, MULTI, P><<<nb, kPairBlock, 0, s>>>(a, p, sf);
+            else lj_pair_kernel<FM_STORE, false, MULTI, P><<<nb, kPairBlock, 0, s>>>(a, p, sf);
+            break;
+        case FM_FUSED_FULL:
+            lj_pair_kernel<FM_FUSED_FULL, false, MULTI, P><<<nb, kPairBlock, 0, s>>>(a, p, sf);
+            break;
+        default: lj_pair_kernel<FM_FUSED_HALF, false, MULTI, P><<<nb, kPairBlock, 0, s>>>(a, p, sf); break;
+    }
+    return cudaGetLastError();
+}
+
 cudaError_t launch_pair_forces(md_system *h, int mode, bool energy, bool store_f) {
     if (h->fc.ntypes > 0) return launch_pair_typed_forces(h, mode, energy, store_f);
-    ForceArgs a = make_force_args(h);
-    const PairArgs p = make_pair_args(h);
     const int sf = store_f ? 1 : 0;
-    const int blocks = pair_grid_blocks(h, kPairBlock);
-    const bool multi = h->R > 1;
-    cudaStream_t s = h->stream;
-#define MDG_PAIR(M)                                                                         \
-    do {                                                                                    \
-        if (multi) {                                                                        \
-            if (energy) lj_pair_kernel<M, true, true><<<blocks, kPairBlock, 0, s>>>(a, p, sf); \
-            else lj_pair_kernel<M, false, true><<<blocks, kPairBlock, 0, s>>>(a, p, sf);       \
-        } else {                                                                            \
-            if (energy) lj_pair_kernel<M, true><<<blocks, kPairBlock, 0, s>>>(a, p, sf);    \
-            else lj_pair_kernel<M, false><<<blocks, kPairBlock, 0, s>>>(a, p, sf);          \
-        }                                                                                   \
-    } while (0)
-    switch (mode) {
-        case FM_STORE: MDG_PAIR(FM_STORE); break;
-        case FM_FUSED_FULL: MDG_PAIR(FM_FUSED_FULL); break;
-        default: MDG_PAIR(FM_FUSED_HALF); break;
-    }
-#undef MDG_PAIR
-    return cudaGetLastError();
+    const int P = mixed_split(h->n / 2, h->ps_cap);
+    if (h->R > 1)
+        return P == 8 ? launch_pair_lj<true, 8>(h, mode, energy, sf)
+             : P == 4 ? launch_pair_lj<true, 4>(h, mode, energy, sf)
+                      : launch_pair_lj<true, 1>(h, mode, energy, sf);
+    return P == 8 ? launch_pair_lj<false, 8>(h, mode, energy, sf)
+         : P == 4 ? launch_pair_lj<false, 4>(h, mode, energy, sf)
+                  : launch_pair_lj<false, 1>(h, mode, energy, sf);
 }
 
 }  // namespace mdg

@@ -30,9 +30,10 @@ inline PairArgs make_pair_args(const md_system *h) {
     return p;
 }
 
-// Blocks of `block` threads that cover every slot a binning can make.
-inline int pair_grid_blocks(const md_system *h, int block) {
-    return (int)((pair_slots_max(h->n, h->g.ncells) + block - 1) / block);
+// Blocks of `block` threads that cover every slot a binning can make, P lanes
+// per slot.
+inline int pair_grid_blocks(const md_system *h, int block, int P = 1) {
+    return (int)((pair_slots_max(h->n, h->g.ncells) * P + block - 1) / block);
 }
 
 // Lennard-Jones pair term in float32 for the pair vector e = x_j - x_i:
@@ -99,11 +100,50 @@ __device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) {
 }
 __device__ __forceinline__ float2 dup2(float v) { return make_float2(v, v); }
 
+// Sums of a slot's P lanes, then stores, energies and epilogues of its atoms (every
+// lane of the warp calls it): t is the state of the lane's component of the first
+// atom (with eight lanes: of atom part / 4), t1 that of the second with four.
+template <int MODE, bool ENERGY, bool SPECIES, int P>
+__device__ __forceinline__ void split_slot_out(const ForceArgs &a, int i0, bool two, bool on,
+                                               int part, float2 fx, float2 fy, float2 fz,
+                                               float2 en, unsigned np0, unsigned np1,
+                                               const SplitState &t, const SplitState &t1,
+                                               int store_f) {
+    fx = make_float2(split_sum<P>(fx.x), split_sum<P>(fx.y));
+    fy = make_float2(split_sum<P>(fy.x), split_sum<P>(fy.y));
+    fz = make_float2(split_sum<P>(fz.x), split_sum<P>(fz.y));
+    if (ENERGY) {
+        en = make_float2(split_sum<P>(en.x), split_sum<P>(en.y));
+        if (on) count_pairs(a.ds, np0 + (two ? np1 : 0u));
+        if (on && part == 0) a.e_atom[i0] = 0.5 * (double)en.x;
+        if (on && two && part == 1) a.e_atom[i0 + 1] = 0.5 * (double)en.y;
+    }
+    const int c = part & 3;
+    const float F0 = c == 0 ? fx.x : (c == 1 ? fy.x : fz.x);
+    const float F1 = c == 0 ? fx.y : (c == 1 ? fy.y : fz.y);
+    const float *words = reinterpret_cast<const float *>(a.xq);
+    if (P >= 8) {
+        const bool second = (part >> 2) & 1;
+        const bool fin = on && part < 8 && (two || !second);
+        const int i = i0 + (second && two ? 1 : 0);
+        split_epilogue<MODE, SPECIES>(a, i, c, fin, (double)(second ? F1 : F0),
+                                      words[4 * (size_t)i + 3], t, store_f);
+    } else {
+        split_epilogue<MODE, SPECIES>(a, i0, c, on, (double)F0, words[4 * (size_t)i0 + 3], t, store_f);
+        const int i1 = i0 + (two ? 1 : 0);
+        split_epilogue<MODE, SPECIES>(a, i1, c, on && two, (double)F1, words[4 * (size_t)i1 + 3], t1,
+                                      store_f);
+    }
+}
+
 // MULTI (a batch of boxes, the block's boxes not all in shared memory): the
 // stencil shifts come from the slot's box's row of the global R x 27 table.
-template <int MODE, bool ENERGY, bool MULTI = false>
+// P > 1: the P lanes of the slot (this one is `part`; on: the slot exists) each
+// walk every P-th quad of its list; lane 0 adds the slot's own pair.
+template <int MODE, bool ENERGY, bool MULTI = false, int P = 1>
 __device__ __forceinline__ void lj_pair_slot(const ForceArgs &a, const PairArgs &p,
-                                             const ShiftTab *sh, int s, int store_f) {
+                                             const ShiftTab *sh, int s, int store_f, int part = 0,
+                                             bool on = true) {
     const uint32_t sa = p.slot_atom[s];
     const int i0 = (int)(sa & ~kSingle);
     const float4 *shr = MULTI ? a.shifts32 + kStencil * (int)a.rep[i0] : nullptr;
@@ -118,7 +158,7 @@ __device__ __forceinline__ void lj_pair_slot(const ForceArgs &a, const PairArgs 
         // the slot's own pair, once: f_i0 -= fs e, f_i1 += fs e
         const float ex = q1.x - q0.x, ey = q1.y - q0.y, ez = q1.z - q0.z;
         const float r2 = ex * ex + ey * ey + ez * ez;
-        if (r2 < rc2) {
+        if ((P == 1 || part == 0) && r2 < rc2) {
             float gx = 0.f, gy = 0.f, gz = 0.f, e = 0.f;
             unsigned k = 0;
             lj_term<ENERGY>(a.fc, ex, ey, ez, r2, gx, gy, gz, e, k);
@@ -165,6 +205,17 @@ __device__ __forceinline__ void lj_pair_slot(const ForceArgs &a, const PairArgs 
             np1 += in1 ? 1u : 0u;
         }
     };
+    if constexpr (P > 1) {
+        // four lanes finish an atom: with eight lanes both atoms at once
+        const int c = part & 3, k = P >= 8 ? (part >> 2) & 1 : 0;
+        const bool fin = on && part < 8;
+        SplitState t = load_split_state<MODE>(a, i0 + (two ? k : 0), c, fin);
+        SplitState t1 = P < 8 ? load_split_state<MODE>(a, i0 + (two ? 1 : 0), c, fin) : t;
+        split_quads<P>(lq, on ? nq : 0, part, pair);
+        split_slot_out<MODE, ENERGY, false, P>(a, i0, two, on, part, fx, fy, fz, en, np0, np1, t, t1,
+                                               store_f);
+        return;
+    }
     uint4 nxt = nq > 0 ? __ldcs(lq) : make_uint4(0u, 0u, 0u, 0u);
     for (int q = 0; q < nq; ++q) {
         const uint4 e4 = nxt;

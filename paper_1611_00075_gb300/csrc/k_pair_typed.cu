@@ -57,16 +57,20 @@ __device__ __forceinline__ void typed_atom_out(const ForceArgs &a, int i, double
     if (MODE != FM_STORE) vv_epilogue<MODE, true>(a, i, Fx, Fy, Fz, qw);
 }
 
-template <int MODE, bool ENERGY, int NT>
-__global__ void __launch_bounds__(kTypedPairBlock, 8)
+// P > 1: thread t serves slot t / P (as lj_pair_kernel).
+template <int MODE, bool ENERGY, int NT, int P>
+__global__ void __launch_bounds__(kTypedPairBlock, P > 1 ? 1 : 8)
 lj_typed_pair_kernel(ForceArgs a, PairArgs p, TypeTab tt, int store_f) {
     __shared__ ShiftTab sh;
     load_shifts_f32(a.g, &sh);
     __syncthreads();
     if (a.ds->status != 0) return;
     step_bookkeeping<MODE>(a);
-    const int s = blockIdx.x * blockDim.x + threadIdx.x;
-    if (s >= p.slot_start[p.ncells]) return;
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    const int nslots = p.slot_start[p.ncells];
+    if ((P > 1 ? (t & ~31) / P : t) >= nslots) return;  // P > 1: whole warps
+    const bool on = t / P < nslots;
+    const int s = on ? t / P : nslots - 1, part = t % P;
     const uint32_t sa = p.slot_atom[s];
     const int i0 = (int)(sa & ~kSingle);
     const bool two = !(sa & kSingle);
@@ -94,7 +98,7 @@ lj_typed_pair_kernel(ForceArgs a, PairArgs p, TypeTab tt, int store_f) {
         // the slot's own pair once: f_0 -= fs e, f_1 += fs e with e = x_1 - x_0
         const float ex = q1.x - q0.x, ey = q1.y - q0.y, ez = q1.z - q0.z;
         const float r2 = ex * ex + ey * ey + ez * ez;
-        if (r2 < rc2) {
+        if (part == 0 && r2 < rc2) {
             const float r2i = rcp_fast(r2);
             float s6 = row_at<NT>(s2a, t1) * r2i;
             s6 = s6 * s6 * s6;
@@ -143,6 +147,14 @@ lj_typed_pair_kernel(ForceArgs a, PairArgs p, TypeTab tt, int store_f) {
             np1 += in1 ? 1u : 0u;
         }
     };
+    if constexpr (P > 1) {
+        const int c = part & 3, k = (part >> 2) & 1;
+        const SplitState st = load_split_state<MODE>(a, i0 + (two ? k : 0), c, on && part < 8);
+        split_quads<P>(lq, on ? nq : 0, part, pair);
+        split_slot_out<MODE, ENERGY, true, P>(a, i0, two, on, part, fx, fy, fz, en, np0, np1, st, st,
+                                              store_f);
+        return;
+    }
     uint4 nxt = nq > 0 ? __ldcs(lq) : make_uint4(0u, 0u, 0u, 0u);
     for (int q = 0; q < nq; ++q) {
         const uint4 e4 = nxt;
@@ -160,36 +172,45 @@ lj_typed_pair_kernel(ForceArgs a, PairArgs p, TypeTab tt, int store_f) {
                                      store_f);
 }
 
-template <int NT>
+template <int NT, int P>
 cudaError_t launch_nt(md_system *h, int mode, bool energy, bool store_f) {
     const ForceArgs a = make_force_args(h);
     const PairArgs p = make_pair_args(h);
     const TypeTab &tt = h->types;
-    const int blocks = pair_grid_blocks(h, kTypedPairBlock);
+    const int blocks = pair_grid_blocks(h, kTypedPairBlock, P);
     const int sf = store_f ? 1 : 0;
     cudaStream_t s = h->stream;
-#define MDG_TP(M)                                                                         \
-    do {                                                                                  \
-        if (energy) lj_typed_pair_kernel<M, true, NT><<<blocks, kTypedPairBlock, 0, s>>>(a, p, tt, sf); \
-        else lj_typed_pair_kernel<M, false, NT><<<blocks, kTypedPairBlock, 0, s>>>(a, p, tt, sf);      \
-    } while (0)
     switch (mode) {
-        case FM_STORE: MDG_TP(FM_STORE); break;
-        case FM_FUSED_FULL: MDG_TP(FM_FUSED_FULL); break;
-        default: MDG_TP(FM_FUSED_HALF); break;
+        case FM_STORE:
+            if (energy)
+                lj_typed_pair_kernel<FM_STORE, true, NT, P><<<blocks, kTypedPairBlock, 0, s>>>(a, p, tt, sf);
+            else
+                lj_typed_pair_kernel<FM_STORE, false, NT, P><<<blocks, kTypedPairBlock, 0, s>>>(a, p, tt, sf);
+            break;
+        case FM_FUSED_FULL:
+            lj_typed_pair_kernel<FM_FUSED_FULL, false, NT, P><<<blocks, kTypedPairBlock, 0, s>>>(a, p, tt, sf);
+            break;
+        default:
+            lj_typed_pair_kernel<FM_FUSED_HALF, false, NT, P><<<blocks, kTypedPairBlock, 0, s>>>(a, p, tt, sf);
+            break;
     }
-#undef MDG_TP
     return cudaGetLastError();
+}
+
+template <int NT>
+cudaError_t launch_any(md_system *h, int mode, bool energy, bool store_f) {
+    return mixed_split(h->n / 2, h->ps_cap) > 1 ? launch_nt<NT, 8>(h, mode, energy, store_f)
+                                                : launch_nt<NT, 1>(h, mode, energy, store_f);
 }
 
 }  // namespace
 
 cudaError_t launch_pair_typed_forces(md_system *h, int mode, bool energy, bool store_f) {
     switch (h->fc.ntypes) {
-        case 1: return launch_nt<1>(h, mode, energy, store_f);
-        case 2: return launch_nt<2>(h, mode, energy, store_f);
-        case 3: return launch_nt<3>(h, mode, energy, store_f);
-        default: return launch_nt<4>(h, mode, energy, store_f);
+        case 1: return launch_any<1>(h, mode, energy, store_f);
+        case 2: return launch_any<2>(h, mode, energy, store_f);
+        case 3: return launch_any<3>(h, mode, energy, store_f);
+        default: return launch_any<4>(h, mode, energy, store_f);
     }
 }
 

@@ -1,0 +1,83 @@
+"""The mixed passes on both sides of their lanes-per-item limits (eight lanes up
+to 16,384 atoms or slots, four up to 65,536, then one) and where the list
+capacity alone forbids a split, against the oracle with the mixed path's bar
+(2e-4 relative, 1e-5 of the rms; atoms with a pair within rounding of the cutoff
+left out); forces stored by a step (the split epilogue) against a fresh
+evaluation at the same positions, which runs the same kernel without it."""
+import numpy as np
+import pytest
+import torch
+
+from paper_1611_00075_gb300 import inputs, md
+from test_gpu_paired import near_cutoff
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def orc():
+    import oracle
+    oracle.lib()
+    return oracle
+
+
+def jitter(s, amp, seed):
+    return np.mod(s.pos + amp * inputs.gaussian(seed, s.pos.size).reshape(-1, 3), s.box)
+
+
+def check(f, f0, bad):
+    fn = np.linalg.norm(f0, axis=1)
+    rms = np.sqrt(np.mean(fn * fn))
+    ok = np.linalg.norm(f - f0, axis=1) <= 2e-4 * fn + 1e-5 * max(1.0, rms)
+    assert np.all(ok | bad), int((~(ok | bad)).sum())
+
+
+@pytest.mark.parametrize("variant,nc", [("full", 16), ("full", 17), ("full", 25), ("full", 26),
+                                        ("paired", 20), ("paired", 21), ("paired", 32),
+                                        ("paired", 33)])
+def test_lj_sizes(orc, variant, nc):
+    s = inputs.lj_fcc(nc=nc, T=0.5)
+    pos = jitter(s, 0.05, 400 + nc)
+    off, ids = orc.neighbors_cells(pos, s.box, 2.8)
+    _, f0 = orc.lj_list(pos, s.box, off, ids)
+    bad = near_cutoff(pos, s.box, off, ids, 2.5, 1e-5)
+    fv = md.MD_FORCE_PAIRED if variant == "paired" else md.MD_FORCE_FULL
+    with md.System(pos, s.vel, s.box, precision="mixed", force_variant=fv) as a:
+        check(a.state()[2].cpu().numpy(), f0, bad)
+        a.step(3)
+        x, v, f = a.state()
+        U = sum(a.energy())
+        md.md_set_state(a.h, x, v)
+        md.md_forces(a.h)
+        g = a.state()[2]
+        # the list is new, so the order of the sums may differ: float32 rounding
+        rms = float(torch.sqrt((g * g).mean()))
+        assert float((f - g).abs().max()) < 2e-4 * max(rms, float(g.abs().max()))
+        assert abs(sum(a.energy()) - U) < 1e-6 * abs(U)
+
+
+@pytest.mark.parametrize("variant", ["full", "paired"])
+def test_two_species(orc, variant):
+    s = inputs.lj_alloy(nc=7)
+    p = s.params
+    pos = jitter(s, 0.03, 441)
+    off, ids = orc.neighbors_cells(pos, s.box, p["rc"] + p["skin"])
+    f0 = orc.lj_typed_list(pos, s.box, off, ids, p["types"], p["t_eps"], p["t_sigma"])[1]
+    bad = near_cutoff(pos, s.box, off, ids, p["rc"], 1e-5)
+    fv = md.MD_FORCE_PAIRED if variant == "paired" else md.MD_FORCE_FULL
+    with md.System(pos, s.vel, s.box, precision="mixed", force_variant=fv, rc=p["rc"],
+                   skin=p["skin"], dt=p["dt"],
+                   species=(p["types"], p["t_eps"], p["t_sigma"], p["t_mass"])) as a:
+        check(a.state()[2].cpu().numpy(), f0, bad)
+
+
+@pytest.mark.parametrize("cap", [252, 256, 260, 508, 512, 516])
+def test_capacity_limits_the_split(orc, cap):
+    """Lists of up to cap entries: four lanes carry 256, eight 512."""
+    s = inputs.lj_fcc(nc=6, T=0.5)
+    pos = jitter(s, 0.05, 451)
+    off, ids = orc.neighbors_cells(pos, s.box, 2.8)
+    _, f0 = orc.lj_list(pos, s.box, off, ids)
+    bad = near_cutoff(pos, s.box, off, ids, 2.5, 1e-5)
+    with md.System(pos, s.vel, s.box, precision="mixed", max_neighbors=cap) as a:
+        check(a.state()[2].cpu().numpy(), f0, bad)
