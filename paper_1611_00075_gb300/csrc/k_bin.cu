@@ -99,9 +99,10 @@ __global__ void bin_count_kernel(int n, const Grid *__restrict__ grids,
                                  int32_t *__restrict__ count, int32_t *__restrict__ new_cell,
                                  int32_t *__restrict__ slot, double4 *__restrict__ tabs,
                                  double4 *__restrict__ tv, bool slots, DevStatus *ds,
-                                 bool gated) {
+                                 bool gated, bool count_run) {
     if (chain_off(ds, gated)) return;
     if (blockIdx.x == 0 && threadIdx.x == 0) {
+        if (count_run) ds->cond_runs += 1;
         ds->max_cell = 0;
         reset_list_counts(ds, slots);
     }
@@ -514,7 +515,7 @@ cudaError_t launch_scan_i32(const int32_t *in, int32_t *out, int n, int32_t *bsu
     return launch_scan<int32_t>(in, out, n, bsum, ds, gated, s);
 }
 
-cudaError_t launch_bin(md_system *h, bool gated) {
+cudaError_t launch_bin(md_system *h, bool gated, bool count_run) {
     const int n = (int)h->n, nc = h->g.ncells;
     cudaStream_t s = h->stream;
     const int cur = h->cur;
@@ -523,7 +524,7 @@ cudaError_t launch_bin(md_system *h, bool gated) {
     bin_count_kernel<<<gs_blocks(n), kBlock, 0, s>>>(n, h->grids, h->rep, h->xr64[cur], h->cell,
                                                      h->xabs, h->v, h->orig, h->cell_count,
                                                      h->new_cell, h->slot, h->tmp_abs, h->tmp_v,
-                                                     paired, h->ds, gated);
+                                                     paired, h->ds, gated, count_run);
     int32_t *slot_start = paired ? h->ps_start : nullptr;
     const int nb = std::max((nc + kScanTile - 1) / kScanTile, 1);
     const bool prefixed = nb > kScanDirect;

@@ -349,11 +349,13 @@ md_status enqueue_sched_prep(md_system *h, bool gated, bool always = false) {
 }
 
 // Rebuild chain enqueued before a force evaluation.  gated: runs only if the
-// device flag asks for it.
-md_status enqueue_rebuild(md_system *h, bool gated) {
+// device flag asks for it.  count_run: its launches count when it runs (the
+// device notes it), not here.
+md_status enqueue_rebuild(md_system *h, bool gated, bool count_run = false) {
+    const long long l0 = h->launches;
     // the list build closes the rebuild unless other passes follow it
     const bool last = !h->ov_on && h->p.force_variant != MD_FORCE_CLUSTER && !uses_partition(h);
-    MD_CK(launch_bin(h, gated));
+    MD_CK(launch_bin(h, gated, count_run));
     if (h->p.force_variant == MD_FORCE_PAIRED) MD_CK(launch_pair_build(h, true, gated, last));
     else MD_CK(launch_build_list(h, true, gated, nullptr, last));
     h->launches += bin_launches(h) + 1 + (gated ? 0 : 1);  // binning, list (and its reset)
@@ -370,6 +372,10 @@ md_status enqueue_rebuild(md_system *h, bool gated) {
         if (st != MD_OK) return st;
         MD_CK(launch_finish_rebuild(h, gated));
         h->launches += 1;
+    }
+    if (count_run) {
+        h->body_launches = h->launches - l0;
+        h->launches = l0;
     }
     MD_CK(mark(h, K_REBUILD));
     return MD_OK;
@@ -530,102 +536,66 @@ md_status forces_now(md_system *h, bool energy) {
 
 __global__ void begin_steps_kernel(DevStatus *ds, int base) { ds->steps_done = base; }
 
-// ---- CUDA graphs of one full step ---------------------------------------------
+// ---- CUDA graphs of full steps -------------------------------------------------
 //
 // The launches of a step that is neither the first nor the last of an md_step
-// call -- the rebuild chain and the fused force + kick + drift -- are the
-// same every step except for the double-buffer parity, so they are captured
-// once per parity and replayed.  The rebuild chain sits in the body of a
-// conditional (IF) node whose condition a one-thread kernel sets from the
-// device's rebuild flag, so a step without a rebuild launches two kernels
-// instead of the whole gated chain.  Kernels that decide on the device
-// (status word, step counter) keep working under replay.  Any change of
-// buffers or launch choice drops the graphs; capture needs a non-default
-// stream.  With per-launch timing on, the rebuild chain still runs from its
-// graph (a conditional body may hold no event records) and the force launch
-// and the timing events are issued around it.
-
-__global__ void rebuild_cond_kernel(cudaGraphConditionalHandle c, DevStatus *ds) {
-    const unsigned run = (ds->status == 0 && ds->rebuild != 0) ? 1u : 0u;
-    if (run) ds->cond_runs += 1;
-    cudaGraphSetConditional(c, run);
-}
+// call -- the gated rebuild chain and the fused force + kick + drift -- are the
+// same every step except for the double-buffer parity, so runs of kRunSteps
+// steps are captured and replayed, and the call's last step from a graph of its
+// own.  Kernels that decide on the device (status word, rebuild flag, step
+// counter) keep working under replay.  Any change of buffers or launch choice
+// drops the graphs; capture needs a non-default stream.
+//
+// The chain is inline: an idle kernel of it costs about 0.5 us inside a graph of
+// several steps (1.5 us with a full grid), against 2 us as a launch of its own
+// and about 10 us for a conditional node around the chain, whether it runs or
+// not.  A step without a rebuild, conditional node against this: 17.0 -> 9.2 us
+// at 864 atoms, 19.5 -> 11.4 at 4,000 (both with the split force pass), 56.5 ->
+// 51.4 at 256,000, 153.0 -> 148.5 at 1,048,576 (two atoms per thread), 409.9 ->
+// 405.9 at 2,916,000.
+constexpr int kRunSteps[3] = {8, 2, 1};
 
 void drop_graphs(md_system *h) {
     for (int b = 0; b < 2; ++b) {
-        if (h->gexec[b]) {
-            cudaGraphExecDestroy(h->gexec[b]);
-            h->gexec[b] = nullptr;
-        }
-        if (h->gexec_rb[b]) {
-            cudaGraphExecDestroy(h->gexec_rb[b]);
-            h->gexec_rb[b] = nullptr;
+        for (auto &g : h->gexec_run)
+            if (g[b]) {
+                cudaGraphExecDestroy(g[b]);
+                g[b] = nullptr;
+            }
+        if (h->gexec_last[b]) {
+            cudaGraphExecDestroy(h->gexec_last[b]);
+            h->gexec_last[b] = nullptr;
         }
     }
 }
 
-// Captures, for the current parity, [condition kernel] -> [IF: rebuild chain]
-// and, with with_forces, -> [fused force + kick + drift].  On any failure the
-// handle falls back to plain launches (graphs_ok = false).
-md_status capture_step_graph(md_system *h, bool with_forces, cudaGraphExec_t *out,
-                             long long *uncond_launches) {
+bool graphs_usable(const md_system *h) { return h->graphs_ok && h->stream != nullptr; }
+
+// Captures `steps` consecutive steps from the current parity: full steps, or
+// (last) the last step of a call.
+md_status capture_run_graph(md_system *h, int steps, bool last, cudaGraphExec_t *out,
+                            long long *launches) {
     const long long l0 = h->launches;
     const bool timing = h->timing;
+    const int cur = h->cur;
     h->timing = false;  // no event records inside a graph
     md_status st = MD_OK;
     cudaGraph_t graph = nullptr;
-    cudaGraphConditionalHandle cond = 0;
-    cudaGraphNode_t knode = nullptr, inode = nullptr;
-    cudaGraphNodeParams cp = {};
-    // one stream capture into graph g after the nodes dep[0..ndep)
-    auto capture = [&](cudaGraph_t g, const cudaGraphNode_t *dep, size_t ndep,
-                       const auto &body) -> cudaError_t {
-        cudaError_t r = cudaStreamBeginCaptureToGraph(h->stream, g, dep, nullptr, ndep,
-                                                      cudaStreamCaptureModeThreadLocal);
-        if (r != cudaSuccess) return r;
-        const md_status sb = body();
-        cudaGraph_t gg = g;
-        r = cudaStreamEndCapture(h->stream, &gg);
-        if (sb != MD_OK) {
-            st = sb;
-            return cudaErrorUnknown;
+    cudaError_t e = cudaStreamBeginCapture(h->stream, cudaStreamCaptureModeThreadLocal);
+    if (e == cudaSuccess) {
+        for (int k = 0; k < steps && st == MD_OK; ++k) {
+            st = enqueue_rebuild(h, true, true);
+            if (st == MD_OK)
+                st = enqueue_forces(h, last ? FM_FUSED_HALF : FM_FUSED_FULL, false, last);
+            h->cur ^= 1;
         }
-        return r;
-    };
-    cudaError_t e = cudaGraphCreate(&graph, 0);
-    if (e == cudaSuccess)
-        e = cudaGraphConditionalHandleCreate(&cond, graph, 0, cudaGraphCondAssignDefault);
-    if (e == cudaSuccess)
-        e = capture(graph, nullptr, 0, [&]() -> md_status {
-            rebuild_cond_kernel<<<1, 1, 0, h->stream>>>(cond, h->ds);
-            h->launches += 1;
-            return cudaGetLastError() == cudaSuccess ? MD_OK : MD_ERR_CUDA;
-        });
-    if (e == cudaSuccess) {
-        size_t nn = 1;
-        e = cudaGraphGetNodes(graph, &knode, &nn);
-        if (e == cudaSuccess && nn != 1) e = cudaErrorUnknown;
+        e = cudaStreamEndCapture(h->stream, &graph);
     }
-    if (e == cudaSuccess) {
-        cp.type = cudaGraphNodeTypeConditional;
-        cp.conditional.handle = cond;
-        cp.conditional.type = cudaGraphCondTypeIf;
-        cp.conditional.size = 1;
-        e = cudaGraphAddNode(&inode, graph, &knode, nullptr, 1, &cp);
-    }
-    const long long lb = h->launches;
-    if (e == cudaSuccess)
-        e = capture(cp.conditional.phGraph_out[0], nullptr, 0,
-                    [&]() -> md_status { return enqueue_rebuild(h, true); });
-    h->body_launches = h->launches - lb;
-    h->launches = lb;  // the body's launches are counted when it runs
-    if (e == cudaSuccess && with_forces)
-        e = capture(graph, &inode, 1,
-                    [&]() -> md_status { return enqueue_forces(h, FM_FUSED_FULL, false, false); });
-    if (e == cudaSuccess) e = cudaGraphInstantiate(out, graph, 0);
+    if (e == cudaSuccess && st == MD_OK) e = cudaGraphInstantiate(out, graph, 0);
     if (graph) cudaGraphDestroy(graph);
-    *uncond_launches = h->launches - l0;
+    *launches = h->launches - l0;
     h->launches = l0;
+    h->cur = cur;
     h->timing = timing;
     if (st != MD_OK) return st;
     if (e != cudaSuccess) {
@@ -636,39 +606,44 @@ md_status capture_step_graph(md_system *h, bool with_forces, cudaGraphExec_t *ou
     return MD_OK;
 }
 
-bool graphs_usable(const md_system *h) { return h->graphs_ok && h->stream != nullptr; }
-
-// The gated rebuild chain of one step: from the parity's conditional graph
-// when graphs work, else as plain gated launches.
-md_status enqueue_rebuild_step(md_system *h) {
+// The last step of an md_step call with its forces stored, from a graph; false
+// in *done when it has to be launched kernel by kernel.
+md_status enqueue_last_step(md_system *h, bool *done) {
+    *done = false;
+    if (!graphs_usable(h) || h->timing) return MD_OK;
     const int par = h->cur;
-    if (graphs_usable(h)) {
-        long long nl = 0;
-        if (!h->gexec_rb[par]) {
-            md_status st = capture_step_graph(h, false, &h->gexec_rb[par], &nl);
-            if (st != MD_OK) return st;
-        }
-        if (h->gexec_rb[par]) {
-            MD_CK(cudaGraphLaunch(h->gexec_rb[par], h->stream));
-            h->launches += 1;
-            MD_CK(mark(h, K_REBUILD));
-            return MD_OK;
-        }
+    if (!h->gexec_last[par]) {
+        md_status st = capture_run_graph(h, 1, true, &h->gexec_last[par], &h->last_launches[par]);
+        if (st != MD_OK || !h->gexec_last[par]) return st;
     }
-    return enqueue_rebuild(h, true);
+    MD_CK(cudaGraphLaunch(h->gexec_last[par], h->stream));
+    h->launches += h->last_launches[par];
+    *done = true;
+    return MD_OK;
 }
 
-// One step between the first and the last of an md_step call (parity h->cur).
-md_status enqueue_full_step(md_system *h) {
+// The gated rebuild chain of one step, launched kernel by kernel (per-launch
+// timing, the default stream).  On a stream that would replay graphs its
+// launches count when it runs, as they do there.
+md_status enqueue_rebuild_step(md_system *h) { return enqueue_rebuild(h, true, graphs_usable(h)); }
+
+// Steps between the first and the last of an md_step call (parity h->cur), `left`
+// of them still to go; *took receives how many were enqueued.
+md_status enqueue_full_steps(md_system *h, int64_t left, int *took) {
     const int par = h->cur;
+    *took = 1;
     if (graphs_usable(h) && !h->timing) {
-        if (!h->gexec[par]) {
-            md_status st = capture_step_graph(h, true, &h->gexec[par], &h->graph_launches[par]);
+        int k = 0;
+        while (kRunSteps[k] > left) ++k;
+        if (!h->gexec_run[k][par]) {
+            md_status st = capture_run_graph(h, kRunSteps[k], false, &h->gexec_run[k][par],
+                                             &h->run_launches[k][par]);
             if (st != MD_OK) return st;
         }
-        if (h->gexec[par]) {
-            MD_CK(cudaGraphLaunch(h->gexec[par], h->stream));
-            h->launches += h->graph_launches[par];
+        if (h->gexec_run[k][par]) {
+            MD_CK(cudaGraphLaunch(h->gexec_run[k][par], h->stream));
+            h->launches += h->run_launches[k][par];
+            *took = kRunSteps[k];
             return MD_OK;
         }
     }
@@ -1087,10 +1062,16 @@ md_status md_step(md_system *h, int64_t nsteps) {
             h->cur = c0 ^ (int)((s - 1) & 1);
             if (h->timing) ev_at[s] = h->ev_used;
             if (s < nsteps) {
-                st = enqueue_full_step(h);
+                int took = 1;
+                st = enqueue_full_steps(h, nsteps - s, &took);
                 if (st != MD_OK) return st;
+                s += took - 1;
                 continue;
             }
+            bool done = false;
+            st = enqueue_last_step(h, &done);
+            if (st != MD_OK) return st;
+            if (done) continue;
             st = enqueue_rebuild_step(h);
             if (st != MD_OK) return st;
             st = enqueue_forces(h, FM_FUSED_HALF, false, true);

@@ -82,7 +82,7 @@ struct DevStatus {
     unsigned long long pairs_cut;     // pairs inside r_c of the last energy evaluation
     int tile_counter;                 // dynamic scheduler: next unclaimed tile
     unsigned int done_ctas;           // dynamic scheduler: CTAs finished this launch
-    long long cond_runs;              // rebuild chains run by a graph's IF node
+    long long cond_runs;              // rebuild chains run that the host did not count
     unsigned long long cluster_pairs; // (i-cluster, j-cluster) entries of the last cluster list
     unsigned long long pair_entries;  // entries of the last two-atom slot list
     int pair_max;                     // its longest row
@@ -353,11 +353,13 @@ struct md_system {
     mdg::DevStatus *ds_host = nullptr;  // pinned mirror
     double *red_host = nullptr;         // pinned
 
-    // captured full steps (one per double-buffer parity)
-    cudaGraphExec_t gexec[2] = {nullptr, nullptr};     // one full step, per parity
-    cudaGraphExec_t gexec_rb[2] = {nullptr, nullptr};  // the rebuild chain alone, per parity
-    long long graph_launches[2] = {0, 0};  // unconditional launches of gexec
-    long long body_launches = 0;           // launches of the conditional rebuild chain
+    // captured steps: runs of full steps (kRunSteps) and the last step of a
+    // call, per double-buffer parity, with their unconditional launches
+    cudaGraphExec_t gexec_run[3][2] = {};
+    cudaGraphExec_t gexec_last[2] = {nullptr, nullptr};
+    long long run_launches[3][2] = {};
+    long long last_launches[2] = {0, 0};
+    long long body_launches = 0;           // launches of a rebuild chain that runs
     bool graphs_ok = true;
 
     // per-launch timing (md_set_timing)
@@ -381,8 +383,9 @@ namespace mdg {
 // ---- binning (k_bin.cu) --------------------------------------------------
 // Gated chain: count per cell (with the absolute positions and gather
 // records), scan, scatter, order and gather every cell; under the two-atom
-// layout also the slot tables.  bin_launches kernels.
-cudaError_t launch_bin(md_system *h, bool gated);
+// layout also the slot tables.  bin_launches kernels.  count_run: a chain that
+// runs adds itself to DevStatus::cond_runs.
+cudaError_t launch_bin(md_system *h, bool gated, bool count_run = false);
 int bin_launches(const md_system *h);
 // Exclusive scan of int32 counts into int32 starts (starts[n] = total).
 cudaError_t launch_scan_i32(const int32_t *in, int32_t *out, int n, int32_t *bsum,
