@@ -11,6 +11,8 @@
 // float32 pair arithmetic carries its own pair's parameters.  Sums: float32
 // over the whole list, as for the one-species slot kernel; the
 // velocity-Verlet epilogue uses each atom's species mass.
+#include <cstring>
+
 #include "k_pair.cuh"
 
 namespace mdg {
@@ -18,6 +20,26 @@ namespace mdg {
 namespace {
 
 constexpr int kTypedPairBlock = 128;
+
+// 1 below the cutoff (r2 < rc2), else 0, on the multiply-add pipe: the saturated
+// (rc2 - r2) 2^k, with 2^k = big at least 1 / ulp(rc2), in one multiply-add whose
+// rounding keeps the sign (rb = rc2 2^k; both exact).  NaN gives 0.  A compare
+// and a select per lane run on the half-rate ALU pipe, which the species selects
+// already load: 1.15 M alloy atoms, 50 steps, 11.10 -> 10.60 ms.  (The one-species
+// and Sutton-Chen slot kernels have no ALU selects to relieve and lose by the
+// two registers: liquid 7.03 -> 7.14 ms, Sutton-Chen 33.2 -> 33.5.)
+__device__ __forceinline__ float inside(float r2, float big, float rb) {
+    float w;
+    asm("fma.rn.sat.f32 %0, %1, %2, %3;" : "=f"(w) : "f"(r2), "f"(-big), "f"(rb));
+    return w;
+}
+// biased exponent of rc2 for which 2^k of inside() is a normal number with room
+__host__ __device__ __forceinline__ bool inside_fits(unsigned exponent) {
+    return exponent >= 40 && exponent <= 200;
+}
+__device__ __forceinline__ float inside_scale(float rc2) {
+    return __uint_as_float((284u - (__float_as_uint(rc2) >> 23)) << 23);
+}
 
 // element t of a row of NT values held in registers
 template <int NT>
@@ -57,8 +79,9 @@ __device__ __forceinline__ void typed_atom_out(const ForceArgs &a, int i, double
     if (MODE != FM_STORE) vv_epilogue<MODE, true>(a, i, Fx, Fy, Fz, qw);
 }
 
-// P > 1: thread t serves slot t / P (as lj_pair_kernel).
-template <int MODE, bool ENERGY, int NT, int P>
+// P > 1: thread t serves slot t / P (as lj_pair_kernel).  SAT: the cutoff by
+// inside(); false in units whose rc2 leaves it no room.
+template <int MODE, bool ENERGY, int NT, int P, bool SAT>
 __global__ void __launch_bounds__(kTypedPairBlock, P > 1 ? 1 : 8)
 lj_typed_pair_kernel(ForceArgs a, PairArgs p, TypeTab tt, int store_f) {
     __shared__ ShiftTab sh;
@@ -92,6 +115,7 @@ lj_typed_pair_kernel(ForceArgs a, PairArgs p, TypeTab tt, int store_f) {
         row_of<NT>(tt.sh, t1, shb);
     }
     const float rc2 = a.fc.rc2f;
+    const float big = SAT ? inside_scale(rc2) : 0.f, rb = rc2 * big;
     float2 fx = dup2(0.f), fy = dup2(0.f), fz = dup2(0.f), en = dup2(0.f);
     unsigned np0 = 0, np1 = 0;
     {
@@ -130,9 +154,15 @@ lj_typed_pair_kernel(ForceArgs a, PairArgs p, TypeTab tt, int store_f) {
         const float2 s6 = mul2(mul2(s2, s2), s2);
         const float2 e48 = make_float2(row_at<NT>(e48a, tj), row_at<NT>(e48b, tj));
         float2 nfs = mul2(mul2(mul2(e48, fma2(s6, dup2(-1.0f), dup2(0.5f))), s6), r2i);
-        const bool in0 = r2.x < rc2, in1 = r2.y < rc2;
-        nfs.x = in0 ? nfs.x : 0.f;
-        nfs.y = in1 ? nfs.y : 0.f;
+        float2 in;
+        if (SAT) {
+            in = make_float2(inside(r2.x, big, rb), inside(r2.y, big, rb));
+            nfs = mul2(nfs, in);
+        } else {
+            in = make_float2(r2.x < rc2 ? 1.f : 0.f, r2.y < rc2 ? 1.f : 0.f);
+            nfs.x = r2.x < rc2 ? nfs.x : 0.f;
+            nfs.y = r2.y < rc2 ? nfs.y : 0.f;
+        }
         fx = fma2(nfs, dx, fx);
         fy = fma2(nfs, dy, fy);
         fz = fma2(nfs, dz, fz);
@@ -140,11 +170,9 @@ lj_typed_pair_kernel(ForceArgs a, PairArgs p, TypeTab tt, int store_f) {
             float2 u = add2(mul2(mul2(make_float2(row_at<NT>(e4a, tj), row_at<NT>(e4b, tj)),
                                       add2(s6, dup2(-1.0f))), s6),
                             make_float2(-row_at<NT>(sha, tj), -row_at<NT>(shb, tj)));
-            u.x = in0 ? u.x : 0.f;
-            u.y = in1 ? u.y : 0.f;
-            en = add2(en, u);
-            np0 += in0 ? 1u : 0u;
-            np1 += in1 ? 1u : 0u;
+            en = fma2(u, in, en);
+            np0 += in.x > 0.f ? 1u : 0u;
+            np1 += in.y > 0.f ? 1u : 0u;
         }
     };
     if constexpr (P > 1) {
@@ -172,7 +200,7 @@ lj_typed_pair_kernel(ForceArgs a, PairArgs p, TypeTab tt, int store_f) {
                                      store_f);
 }
 
-template <int NT, int P>
+template <int NT, int P, bool SAT = true>
 cudaError_t launch_nt(md_system *h, int mode, bool energy, bool store_f) {
     const ForceArgs a = make_force_args(h);
     const PairArgs p = make_pair_args(h);
@@ -183,15 +211,15 @@ cudaError_t launch_nt(md_system *h, int mode, bool energy, bool store_f) {
     switch (mode) {
         case FM_STORE:
             if (energy)
-                lj_typed_pair_kernel<FM_STORE, true, NT, P><<<blocks, kTypedPairBlock, 0, s>>>(a, p, tt, sf);
+                lj_typed_pair_kernel<FM_STORE, true, NT, P, SAT><<<blocks, kTypedPairBlock, 0, s>>>(a, p, tt, sf);
             else
-                lj_typed_pair_kernel<FM_STORE, false, NT, P><<<blocks, kTypedPairBlock, 0, s>>>(a, p, tt, sf);
+                lj_typed_pair_kernel<FM_STORE, false, NT, P, SAT><<<blocks, kTypedPairBlock, 0, s>>>(a, p, tt, sf);
             break;
         case FM_FUSED_FULL:
-            lj_typed_pair_kernel<FM_FUSED_FULL, false, NT, P><<<blocks, kTypedPairBlock, 0, s>>>(a, p, tt, sf);
+            lj_typed_pair_kernel<FM_FUSED_FULL, false, NT, P, SAT><<<blocks, kTypedPairBlock, 0, s>>>(a, p, tt, sf);
             break;
         default:
-            lj_typed_pair_kernel<FM_FUSED_HALF, false, NT, P><<<blocks, kTypedPairBlock, 0, s>>>(a, p, tt, sf);
+            lj_typed_pair_kernel<FM_FUSED_HALF, false, NT, P, SAT><<<blocks, kTypedPairBlock, 0, s>>>(a, p, tt, sf);
             break;
     }
     return cudaGetLastError();
@@ -199,6 +227,9 @@ cudaError_t launch_nt(md_system *h, int mode, bool energy, bool store_f) {
 
 template <int NT>
 cudaError_t launch_any(md_system *h, int mode, bool energy, bool store_f) {
+    unsigned bits;
+    std::memcpy(&bits, &h->fc.rc2f, sizeof bits);
+    if (!inside_fits(bits >> 23)) return launch_nt<NT, 1, false>(h, mode, energy, store_f);
     return mixed_split(h->n / 2, h->ps_cap) > 1 ? launch_nt<NT, 8>(h, mode, energy, store_f)
                                                 : launch_nt<NT, 1>(h, mode, energy, store_f);
 }

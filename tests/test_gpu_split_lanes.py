@@ -81,3 +81,26 @@ def test_capacity_limits_the_split(orc, cap):
     bad = near_cutoff(pos, s.box, off, ids, 2.5, 1e-5)
     with md.System(pos, s.vel, s.box, precision="mixed", max_neighbors=cap) as a:
         check(a.state()[2].cpu().numpy(), f0, bad)
+
+
+@pytest.mark.parametrize("unit", [1.0, 1e-12, 1e-14, 1e13])
+def test_two_species_cutoff_in_other_units(orc, unit):
+    """The cutoff by a saturated multiply-add (r_c^2 well inside float32's
+    range) and by comparison (1e-14 and 1e13: too close to its ends), two atoms
+    per thread: the same forces in every unit of length."""
+    s = inputs.lj_alloy(nc=6)
+    p = s.params
+    pos = jitter(s, 0.03, 461)
+    off, ids = orc.neighbors_cells(pos, s.box, p["rc"] + p["skin"])
+    f0 = orc.lj_typed_list(pos, s.box, off, ids, p["types"], p["t_eps"], p["t_sigma"])[1]
+    bad = near_cutoff(pos, s.box, off, ids, p["rc"], 1e-5)
+    with md.System(pos * unit, np.zeros_like(pos), s.box * unit, precision="mixed",
+                   force_variant=md.MD_FORCE_PAIRED, rc=p["rc"] * unit, skin=p["skin"] * unit,
+                   dt=p["dt"], species=(p["types"], p["t_eps"], p["t_sigma"] * unit,
+                                        p["t_mass"])) as a:
+        f = a.state()[2].cpu().numpy() * unit
+        pe = a.energy()[1]
+    check(f, f0, bad)
+    if unit == 1.0:
+        pe1 = orc.lj_typed_list(pos, s.box, off, ids, p["types"], p["t_eps"], p["t_sigma"])[0]
+        assert abs(pe - pe1) < 2e-5 * abs(pe1)
