@@ -207,14 +207,17 @@ struct GatherArgs {
     int32_t *orig, *cell;
     uint16_t *rep;
     const int32_t *type_orig;
+    CandGroup *cand;  // null: not the two-atom layout
 };
 
 __device__ __forceinline__ int record_orig(const double4 &a) {
     return (int)(unsigned)(__double_as_longlong(a.w) & 0xffffffffll);
 }
 
-// the atom of record s (position record a) becomes sorted atom k
-__device__ __forceinline__ void gather_atom(const GatherArgs &o, int k, int s, const double4 &a) {
+// the atom of record s (position record a) becomes sorted atom k of the cell whose
+// range starts at b
+__device__ __forceinline__ void gather_atom(const GatherArgs &o, int b, int k, int s,
+                                            const double4 &a) {
     const double4 u = o.tv[s];
     const int id = record_orig(a);
     const int c = (int)(__double_as_longlong(a.w) >> 32);
@@ -230,6 +233,14 @@ __device__ __forceinline__ void gather_atom(const GatherArgs &o, int k, int s, c
     const float4 q = make_float4((float)rx, (float)ry, (float)rz, __uint_as_float(w));
     o.xq[k] = q;
     o.xq_build[k] = q;
+    if (o.cand) {
+        float *g4 =
+            reinterpret_cast<float *>(o.cand + cell_group0(c, b) + ((k - b) >> 2)) + ((k - b) & 3);
+        g4[0] = q.x;
+        g4[4] = q.y;
+        g4[8] = q.z;
+        g4[12] = q.x * q.x + q.y * q.y + q.z * q.z;
+    }
     o.xabs[k] = make_double4(a.x, a.y, a.z, 0.0);
     const size_t n = (size_t)o.n;
     o.v[k] = u.x;
@@ -254,7 +265,7 @@ __device__ __forceinline__ void gather_by_id(const GatherArgs &o, int b, int m, 
         const int id = lane < m ? record_orig(a) : 0x7fffffff;
         int rank = 0;
         for (int q = 0; q < m; ++q) rank += (__shfl_sync(0xffffffffu, id, q) < id) ? 1 : 0;
-        if (lane < m) gather_atom(o, b + rank, s, a);
+        if (lane < m) gather_atom(o, b, b + rank, s, a);
         return;
     }
     for (int l = lane; l < m; l += 32) {
@@ -265,7 +276,17 @@ __device__ __forceinline__ void gather_by_id(const GatherArgs &o, int b, int m, 
 #pragma unroll 4
         for (int q = 0; q < m; ++q)
             rank += (int)(unsigned)(__double_as_longlong(o.tabs[src[b + q]].w) & 0xffffffffll) < id ? 1 : 0;
-        gather_atom(o, b + rank, s, a);
+        gather_atom(o, b, b + rank, s, a);
+    }
+}
+
+// the empty places of a cell's last candidate group
+__device__ __forceinline__ void pad_group(const GatherArgs &o, int c, int b, int m, int lane) {
+    if (lane < ((-m) & 3)) {
+        const int k = m + lane;
+        float *g4 = reinterpret_cast<float *>(o.cand + cell_group0(c, b) + (k >> 2)) + (k & 3);
+        g4[0] = g4[4] = g4[8] = 0.f;
+        g4[12] = __int_as_float(0x7f800000);
     }
 }
 
@@ -346,6 +367,7 @@ cell_pair_order_kernel(int ncells, const int32_t *__restrict__ start,
         const int b = start[c], m = start[c + 1] - b;
         if (m == 0) continue;
         write_slots(b, m, lane, slot_start[c], slot_atom);
+        pad_group(out, c, b, m, lane);
         if (m == 1 || m > 32) {
             gather_by_id(out, b, m, lane, src);
             continue;
@@ -392,7 +414,7 @@ cell_pair_order_kernel(int ncells, const int32_t *__restrict__ start,
             left &= ~((1u << first) | (1u << mate));
         }
         if ((left >> lane) & 1u) dst = next;
-        if (on) gather_atom(out, b + dst, sv, out.tabs[sv]);
+        if (on) gather_atom(out, b, b + dst, sv, out.tabs[sv]);
     }
 }
 
@@ -425,6 +447,7 @@ cell_pair_order2_kernel(int ncells, const int32_t *__restrict__ start,
         const int b = start[c], m = start[c + 1] - b;
         if (m == 0) continue;
         write_slots(b, m, lane, slot_start[c], slot_atom);
+        pad_group(out, c, b, m, lane);
         if (m == 1 || m > kWideCell) {
             gather_by_id(out, b, m, lane, src);
             continue;
@@ -489,11 +512,11 @@ cell_pair_order2_kernel(int ncells, const int32_t *__restrict__ start,
         if ((left >> (lane + 32)) & 1ull) dst1 = next;
         if (lane < m) {
             const int sv = __float_as_int(a0.w);
-            gather_atom(out, b + dst0, sv, out.tabs[sv]);
+            gather_atom(out, b, b + dst0, sv, out.tabs[sv]);
         }
         if (lane + 32 < m) {
             const int sv = __float_as_int(a1.w);
-            gather_atom(out, b + dst1, sv, out.tabs[sv]);
+            gather_atom(out, b, b + dst1, sv, out.tabs[sv]);
         }
         __syncwarp();  // the shared rows are rewritten by the warp's next cell
     }
@@ -549,6 +572,7 @@ cudaError_t launch_bin(md_system *h, bool gated, bool count_run) {
     o.cell = h->cell;
     o.rep = h->rep;
     o.type_orig = h->type_orig;
+    o.cand = paired ? h->cand : nullptr;
     const int warps = kOrderBlock / 32;
     const int blocks = std::max(std::min((nc + warps - 1) / warps, kGridCap * 2), 1);
     // one atom per lane while the average cell fits a warp, two per lane above

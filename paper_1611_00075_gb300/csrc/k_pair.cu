@@ -29,6 +29,7 @@
 // float64 sums) and converted once: without the float64 accumulators the
 // kernel fits 9 CTAs of 128 threads per SM.
 #include <algorithm>
+#include <type_traits>
 
 #include "k_pair.cuh"
 
@@ -43,114 +44,170 @@ __device__ __forceinline__ bool chain_off(const DevStatus *ds, bool gated) {
     return ds->status != 0 || (gated && ds->rebuild == 0);
 }
 
-__device__ __forceinline__ int row_off(int k) { return k + (k >> 2) * 124; }
-
-// One stencil cell of a slot's union-list scan (HOME: the slot's own cell,
-// the only one holding i0 and i1); returns the running entry count.
-template <bool WRITE, bool HOME>
-__device__ __forceinline__ int scan_cell(int cnt, int b, int e, const float4 *__restrict__ xq,
-                                         float sx, float sy, float sz, float ux, float uy,
-                                         float uz, float lim, int i0, int i1, uint32_t *row,
-                                         int cap, uint32_t sbits) {
-#pragma unroll 4
-    for (int j = b; j < e; ++j) {
-        const float4 qj = xq[j];
-        const float ex = qj.x - sx, ey = qj.y - sy, ez = qj.z - sz;
-        const float r2 = ex * ex + ey * ey + ez * ez;
-        const float p = ex * ux + ey * uy + ez * uz;
-        bool acc = fmaf(-2.0f, fabsf(p), r2) < lim;
-        if (HOME) acc = acc & (j != i0) & (j != i1);
-        // past the capacity the row's last entry is overwritten: the
-        // overflow status discards the list
-        if (WRITE && acc) row[row_off(min(cnt, cap - 1))] = sbits | (uint32_t)j;
-        cnt += acc ? 1 : 0;
-    }
-    return cnt;
-}
-
-// The union list of each slot: the 27 cells around the slot's cell, in
-// stencil order.  A candidate j is tested against both atoms at once from
-// the slot's midpoint m = (x0 + x1) / 2 and half separation u = (x1 - x0) / 2:
-// with e = x_j - m, the nearer atom's squared distance is
-// |e|^2 + |u|^2 - 2 |e.u|, so the test is |e|^2 - 2 |e.u| < hi - |u|^2 (one
-// difference vector and two dot products instead of two distances).  In
-// float32 the terms stay below about 16 sigma^2, so the rounding error of
-// this form is about 1e-5 sigma^2 at most, against the 2^-14 r_list^2
-// (5e-4 sigma^2) margin of hi: the list stays a superset of both atoms'
-// r_list spheres.
-// Only the home cell holds i0 and i1, so only its scan excludes them.
+// The union list of each slot: the 27 cells around the slot's cell, in stencil
+// order, their atoms four at a time (CandGroup).  A candidate j is tested
+// against both atoms at once from the slot's midpoint m = (x0 + x1) / 2 and half
+// separation u = (x1 - x0) / 2: the nearer atom's squared distance is
+// |x_j - m|^2 + |u|^2 - 2 |(x_j - m).u|, so with the record's |x_j|^2 the test
+//     |x_j|^2 - 2 m.x_j + (|m|^2 + |u|^2 - hi) < |2 u.x_j - 2 u.m|
+// is an addition and six multiply-adds -- packed, for two candidates at a time --
+// and one comparison.  m is taken in the candidate's cell frame, so every term
+// stays below about 24 r_list^2 (cells of up to 4/3 r_list), and the float32
+// rounding below about 1e-5 r_list^2, against the margin of 6e-5 r_list^2 in hi =
+// r_list^2 (1 + 2^-14): the list stays a superset of both atoms' r_list spheres.
 //
-// Measured on GB300 (porous LJ, 9.8 M atoms, 300 steps from the generated
-// state, one build of the union lists): 3.68 ms against 4.19 ms for two
-// direct distances per candidate.  Seven CTAs per SM (71 registers) against
-// 3.93 ms at eight and 4.16 ms at nine; the candidate loop unrolled by 4
-// against 4.13 ms by 2 and 4.30 ms by 8 (at eight CTAs).  Packed f32x2
-// distances for the two atoms were slower (4.98 against 4.45 ms).
+// Accepted entries go to a queue of the thread in shared memory (a store and an
+// addition, both predicated) and from there to the list in whole quads: writing
+// them one by one took eight instructions per candidate, accepted or not, and a
+// scattered 4-byte store.  Bound by the latency of the candidate loads (L1 wavefronts
+// 72 %, issue 46 %); eight blocks per SM with 40 queue rows measured best.
+// Binning and list, two distance products per candidate against this form: 4.73 ->
+// 3.80 ms at 9.8 M porous atoms, 0.565 -> 0.461 at 1 M (liquid), 1.19 -> 0.94 for
+// 2.4 M atoms in 64 boxes (binning included, itself shorter than before).  Six and
+// seven blocks with the next group prefetched: 4.14 and 4.26 ms; nine blocks: 3.86.
 // MULTI (a batch of boxes): each slot takes the geometry of its atoms' box
 // (cells numbered box after box from the box's cell0).
+constexpr int kListRows = 40;                 // queue entries per thread
+constexpr int kListChunk = 7;                 // candidate groups between queue checks
+constexpr int kListHigh = kListRows - 4 * kListChunk;  // a fuller queue is emptied first
+
 template <bool WRITE, bool MULTI = false>
-__global__ void __launch_bounds__(kPairBlock, 7)
+__global__ void __launch_bounds__(kPairBlock, 8)
 pair_list_kernel(int n, Grid g, const Grid *__restrict__ grids, const uint16_t *__restrict__ rep,
-                 float hi, const float4 *__restrict__ xq,
+                 float hi, const float4 *__restrict__ xq, const CandGroup *__restrict__ cand,
                  const int32_t *__restrict__ cell, const int32_t *__restrict__ start,
                  const int32_t *__restrict__ slot_start, const uint32_t *__restrict__ slot_atom,
                  uint32_t *__restrict__ list, int32_t *__restrict__ count, int cap, DevStatus *ds,
                  bool gated, bool close) {
+    __shared__ uint32_t s_queue[WRITE ? kListRows : 1][kPairBlock];
     if (chain_off(ds, gated)) return;
     const int nslots = slot_start[g.ncells];
     if (blockIdx.x == 0 && threadIdx.x == 0) ds->pair_slots = nslots;
     unsigned long long tot = 0;
     int overflow = 0, maxc = 0;
     const uint32_t pad = (kHomeStencil << kIndexBits) | (uint32_t)n;
+    uint32_t *const q0p = &s_queue[0][threadIdx.x];
+    const int capq = cap >> 2;
     // grid-stride over whole warps, so every lane reaches the reductions below
     const int stride = gridDim.x * blockDim.x;
     const int send = ((nslots + 31) & ~31);
     for (int s = blockIdx.x * blockDim.x + threadIdx.x; s < send; s += stride) {
-        if (s < nslots) {
-            const uint32_t sa = slot_atom[s];
-            const int i0 = (int)(sa & ~kSingle);
-            const int i1 = (sa & kSingle) ? i0 : i0 + 1;
+        const bool on = s < nslots;
+        const uint32_t sa = slot_atom[on ? s : nslots - 1];
+        const int i0 = (int)(sa & ~kSingle);
+        const int i1 = (sa & kSingle) ? i0 : i0 + 1;
+        float mx, my, mz, ux, uy, uz, lim;  // u doubled
+        {
             const float4 q0 = xq[i0], q1 = xq[i1];
-            const float ux = 0.5f * (q1.x - q0.x), uy = 0.5f * (q1.y - q0.y),
-                        uz = 0.5f * (q1.z - q0.z);
-            const float mx = q0.x + ux, my = q0.y + uy, mz = q0.z + uz;
-            const float lim = hi - (ux * ux + uy * uy + uz * uz);
-            int nx = g.nx, ny = g.ny, nz = g.nz, c0 = 0;
-            float wx = g.wf[0], wy = g.wf[1], wz = g.wf[2];
-            if (MULTI) {
-                const Grid &gb = grids[rep[i0]];
-                nx = gb.nx; ny = gb.ny; nz = gb.nz; c0 = gb.cell0;
-                wx = gb.wf[0]; wy = gb.wf[1]; wz = gb.wf[2];
+            ux = q1.x - q0.x;
+            uy = q1.y - q0.y;
+            uz = q1.z - q0.z;
+            mx = q0.x + 0.5f * ux;
+            my = q0.y + 0.5f * uy;
+            mz = q0.z + 0.5f * uz;
+            lim = 0.25f * (ux * ux + uy * uy + uz * uz) - hi;
+        }
+        int nx = g.nx, ny = g.ny, nz = g.nz, c0 = 0;
+        float wx = g.wf[0], wy = g.wf[1], wz = g.wf[2];
+        if (MULTI) {
+            const Grid &gb = grids[rep[i0]];
+            nx = gb.nx; ny = gb.ny; nz = gb.nz; c0 = gb.cell0;
+            wx = gb.wf[0]; wy = gb.wf[1]; wz = gb.wf[2];
+        }
+        const int c = cell[i0] - c0;
+        const int cx = c % nx, cy = (c / nx) % ny, cz = c / (nx * ny);
+        uint4 *const row = reinterpret_cast<uint4 *>(list + list_group(s, cap)) + (s & 31);
+        const uint32_t own0 = (kHomeStencil << kIndexBits) | (uint32_t)i0,
+                       own1 = (kHomeStencil << kIndexBits) | (uint32_t)i1;
+        uint32_t *qp = q0p;  // the queue's end
+        int nq = 0;          // quads written
+        int cnt = 0;         // entries (not WRITE)
+        // whole quads of the queue to the list, the rest to its front
+        auto empty = [&]() {
+            const uint32_t *r = q0p;
+            for (; qp - r >= 4 * kPairBlock; r += 4 * kPairBlock) {
+                if (on && nq < capq)
+                    row[(size_t)nq * 32] =
+                        make_uint4(r[0], r[kPairBlock], r[2 * kPairBlock], r[3 * kPairBlock]);
+                ++nq;
             }
-            const int c = cell[i0] - c0;
-            const int cx = c % nx, cy = (c / nx) % ny, cz = c / (nx * ny);
-            uint32_t *row = list + list_group(s, cap) + ((s & 31) << 2);
-            int cnt = 0;
-            for (int dz = -1; dz <= 1; ++dz) {
-                const int zz = (cz + dz + nz) % nz;
-                for (int dy = -1; dy <= 1; ++dy) {
-                    const int yy = (cy + dy + ny) % ny;
-                    for (int dx = -1; dx <= 1; ++dx) {
-                        const int xx = (cx + dx + nx) % nx;
-                        const int cn = c0 + (zz * ny + yy) * nx + xx;
-                        const uint32_t st = (uint32_t)((dz + 1) * 9 + (dy + 1) * 3 + (dx + 1));
-                        // the midpoint moved against the cell shift
-                        const float sx = mx - (float)dx * wx, sy = my - (float)dy * wy,
-                                    sz = mz - (float)dz * wz;
-                        const int b = start[cn], e = start[cn + 1];
-                        const uint32_t sbits = st << kIndexBits;
-                        if (st == kHomeStencil)
-                            cnt = scan_cell<WRITE, true>(cnt, b, e, xq, sx, sy, sz, ux, uy, uz,
-                                                         lim, i0, i1, row, cap, sbits);
-                        else
-                            cnt = scan_cell<WRITE, false>(cnt, b, e, xq, sx, sy, sz, ux, uy, uz,
-                                                          lim, i0, i1, row, cap, sbits);
-                    }
+            const int left = (int)(qp - r) / kPairBlock;
+            if (left > 0) q0p[0] = r[0];
+            if (left > 1) q0p[kPairBlock] = r[kPairBlock];
+            if (left > 2) q0p[2 * kPairBlock] = r[2 * kPairBlock];
+            qp = q0p + left * kPairBlock;
+        };
+        for (int dz = -1; dz <= 1; ++dz) {
+            const int zz = cz + dz < 0 ? nz - 1 : (cz + dz == nz ? 0 : cz + dz);
+            for (int dy = -1; dy <= 1; ++dy) {
+                const int yy = cy + dy < 0 ? ny - 1 : (cy + dy == ny ? 0 : cy + dy);
+                for (int dx = -1; dx <= 1; ++dx) {
+                    const int xx = cx + dx < 0 ? nx - 1 : (cx + dx == nx ? 0 : cx + dx);
+                    const int cn = c0 + (zz * ny + yy) * nx + xx;
+                    const uint32_t st = (uint32_t)((dz + 1) * 9 + (dy + 1) * 3 + (dx + 1));
+                    // the midpoint moved against the cell shift
+                    const float sx = mx - (float)dx * wx, sy = my - (float)dy * wy,
+                                sz = mz - (float)dz * wz;
+                    const float2 mx2 = dup2(-2.f * sx), my2 = dup2(-2.f * sy), mz2 = dup2(-2.f * sz);
+                    const float2 k1 = dup2(sx * sx + sy * sy + sz * sz + lim);
+                    const float2 k2 = dup2(-(ux * sx + uy * sy + uz * sz));
+                    const float2 ux2 = dup2(ux), uy2 = dup2(uy), uz2 = dup2(uz);
+                    const int b = start[cn], e = start[cn + 1];
+                    const CandGroup *gp = cand + cell_group0(cn, b);
+                    const int ng = (e - b + 3) >> 2;
+                    uint32_t ent = (st << kIndexBits) | (uint32_t)b;
+                    // HOME: the slot's own cell, the only one that holds i0 and i1
+                    auto scan = [&](auto home) {
+                        constexpr bool HOME = decltype(home)::value;
+                        for (int g0 = 0; g0 < ng; g0 += kListChunk) {
+                            const int ge = min(ng, g0 + kListChunk);
+                            for (int gi = g0; gi < ge; ++gi, ent += 4) {
+                                const float4 X = __ldg(&gp[gi].x), Y = __ldg(&gp[gi].y),
+                                             Z = __ldg(&gp[gi].z), W = __ldg(&gp[gi].w);
+                                const float2 xa = make_float2(X.x, X.y), xb = make_float2(X.z, X.w);
+                                const float2 ya = make_float2(Y.x, Y.y), yb = make_float2(Y.z, Y.w);
+                                const float2 za = make_float2(Z.x, Z.y), zb = make_float2(Z.z, Z.w);
+                                const float2 wa = make_float2(W.x, W.y), wb = make_float2(W.z, W.w);
+                                const float2 ra = fma2(za, mz2, fma2(ya, my2, fma2(xa, mx2, add2(wa, k1))));
+                                const float2 rb = fma2(zb, mz2, fma2(yb, my2, fma2(xb, mx2, add2(wb, k1))));
+                                const float2 pa = fma2(za, uz2, fma2(ya, uy2, fma2(xa, ux2, k2)));
+                                const float2 pb = fma2(zb, uz2, fma2(yb, uy2, fma2(xb, ux2, k2)));
+                                auto take = [&](float r, float p, uint32_t en) {
+                                    bool acc = r < fabsf(p);
+                                    if (HOME) acc = acc & (en != own0) & (en != own1);
+                                    if (WRITE) {
+                                        if (acc) {
+                                            *qp = en;
+                                            qp += kPairBlock;
+                                        }
+                                    } else {
+                                        cnt += acc ? 1 : 0;
+                                    }
+                                };
+                                take(ra.x, pa.x, ent);
+                                take(ra.y, pa.y, ent + 1);
+                                take(rb.x, pb.x, ent + 2);
+                                take(rb.y, pb.y, ent + 3);
+                            }
+                            if (WRITE && __any_sync(__activemask(), qp - q0p > kListHigh * kPairBlock))
+                                empty();
+                        }
+                    };
+                    if (st == kHomeStencil) scan(std::true_type{});
+                    else scan(std::false_type{});
                 }
             }
-            if (WRITE && cnt <= cap)
-                for (int k = cnt; k & 3; ++k) row[row_off(k)] = pad;
-            if (WRITE) count[s] = cnt;
+        }
+        if (WRITE) {
+            empty();
+            const int left = (int)(qp - q0p) / kPairBlock;
+            cnt = 4 * nq + left;
+            if (on && left > 0 && nq < capq)
+                row[(size_t)nq * 32] = make_uint4(q0p[0], left > 1 ? q0p[kPairBlock] : pad,
+                                                  left > 2 ? q0p[2 * kPairBlock] : pad, pad);
+            if (on) count[s] = cnt;
+        }
+        if (on) {
             maxc = max(maxc, cnt);
             tot += (unsigned long long)cnt;
             overflow |= (cnt > cap);
@@ -263,7 +320,7 @@ cudaError_t launch_pair_build(md_system *h, bool write, bool gated, bool close) 
     const int blocks = (int)std::min<int64_t>((smax + kPairBlock - 1) / kPairBlock, 152 * 16);
 #define MDG_PAIR_LIST(W, M)                                                                  \
     pair_list_kernel<W, M><<<blocks, kPairBlock, 0, s>>>(                                    \
-        n, h->g, h->grids, h->rep, h->list_hi, h->xq[h->cur], h->cell, h->cell_start,        \
+        n, h->g, h->grids, h->rep, h->list_hi, h->xq[h->cur], h->cand, h->cell, h->cell_start,       \
         h->ps_start, h->ps_atom, h->ps_list, h->ps_count, h->ps_cap, h->ds, gated, close)
     if (h->R > 1) {
         if (write) MDG_PAIR_LIST(true, true);

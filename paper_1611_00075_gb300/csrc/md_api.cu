@@ -90,7 +90,7 @@ void free_all(md_system *h) {
     for (int b = 0; b < 2; ++b) { F(h->xr64[b]); F(h->xq[b]); }
     F(h->xq_build); F(h->xabs); F(h->v); F(h->f); F(h->e_atom); F(h->orig); F(h->cell);
     F(h->cell_start); F(h->cell_count); F(h->new_cell); F(h->slot); F(h->src);
-    F(h->scan_bsum); F(h->cell_bsum); F(h->tmp_abs); F(h->tmp_v); F(h->nlist); F(h->ncount);
+    F(h->scan_bsum); F(h->cell_bsum); F(h->cand); F(h->tmp_abs); F(h->tmp_v); F(h->nlist); F(h->ncount);
     F(h->rho); F(h->dF32); F(h->dF64); F(h->xqf); F(h->partials); F(h->red_out); F(h->ds);
     F(h->exp_tmp); F(h->type_orig);
     F(h->cl_icnt); F(h->cl_jcnt); F(h->cl_ioff); F(h->cl_joff); F(h->cl_bsum); F(h->cl_icl);
@@ -145,7 +145,8 @@ cudaError_t alloc_pair(md_system *h, int cap) {
     const int64_t smax = pair_slots_max(h->n, h->g.ncells);
     cudaError_t e = cudaSuccess;
     auto A = [&](cudaError_t r) { if (e == cudaSuccess) e = r; };
-    if (!h->ps_count) {  // the last of the three
+    if (!h->ps_count) {  // the last of the four
+        A(h->cand ? cudaSuccess : dalloc(&h->cand, (size_t)cand_groups(h->n, h->g.ncells)));
         A(h->ps_start ? cudaSuccess : dalloc(&h->ps_start, C + 1));
         A(h->ps_atom ? cudaSuccess : dalloc(&h->ps_atom, (size_t)smax));
         A(dalloc(&h->ps_count, (size_t)smax));

@@ -170,6 +170,19 @@ __device__ __forceinline__ bool below_cell_width(double v, const Grid &g) {
     return (__double2hiint(v) & 0x7fffffff) < g.wsmall_hi;
 }
 
+// The cells' atoms once more for the union-list build, four at a time: group g holds
+// (x, y, z, |x|^2) of four atoms of one cell as four float4 (x of the four, y of
+// the four, ...), cell-relative float32.  Cell c's groups start at cell_group0(),
+// which leaves room for its last, partly empty group without a scan; empty places
+// hold x = 0 and an infinite |x|^2, which no distance test accepts.
+struct CandGroup {
+    float4 x, y, z, w;
+};
+__host__ __device__ __forceinline__ int64_t cell_group0(int cell, int start) {
+    return (int64_t)(start >> 2) + cell;
+}
+inline int64_t cand_groups(int64_t n, int ncells) { return n / 4 + ncells + 1; }
+
 // Per-launch scalars of the force kernels.
 struct ForceConsts {
     float rc2f, eps4f, eps48f, sig2f, shiftf;  // LJ in fp32
@@ -270,6 +283,7 @@ struct md_system {
     int32_t *cell_count = nullptr;  // ncells
     int32_t *new_cell = nullptr, *slot = nullptr, *src = nullptr;
     int32_t *scan_bsum = nullptr;
+    mdg::CandGroup *cand = nullptr;  // candidate groups (CandGroup; two-atom layout)
     long long *cell_bsum = nullptr;  // tile sums of the cell scan (slots << 32 | atoms)
     double4 *tmp_abs = nullptr;  // gather records: (x, y, z, new cell | original id)
     double4 *tmp_v = nullptr;    //                 (vx, vy, vz, replica)
