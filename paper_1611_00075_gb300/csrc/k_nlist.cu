@@ -238,6 +238,80 @@ build_list_kernel(int n, const Grid *__restrict__ grids, const uint16_t *__restr
     list_build_done(ds, close);
 }
 
+// The same lists for small systems, a warp per atom: one thread's scan is a chain
+// of some 600 candidates (42 us however few atoms there are); here the lanes take
+// a cell's candidates at once and a ballot gives each accepted one its place in
+// the row, in the same order.
+template <bool WRITE, bool HALF>
+__global__ void __launch_bounds__(kListBlock)
+warp_list_kernel(int n, const Grid *__restrict__ grids, const uint16_t *__restrict__ rep, float lo,
+                 float hi, double rl2, const float4 *__restrict__ xq,
+                 const double4 *__restrict__ xabs, const int32_t *__restrict__ cell,
+                 const int32_t *__restrict__ start, uint32_t *__restrict__ nlist,
+                 int32_t *__restrict__ ncount, int cap, DevStatus *ds, bool gated, bool close) {
+    if (chain_off(ds, gated)) return;
+    const int lane = threadIdx.x & 31;
+    const int nw = gridDim.x * (kListBlock / 32);
+    unsigned long long tot = 0;
+    int overflow = 0, maxc = 0;
+    for (int i = blockIdx.x * (kListBlock / 32) + (threadIdx.x >> 5); i < n; i += nw) {
+        const Grid &g = grids[rep ? rep[i] : 0];
+        const float4 qi = xq[i];
+        const int myo = __float_as_int(qi.w);
+        const int c = cell[i] - g.cell0;
+        const int cx = c % g.nx, cy = (c / g.nx) % g.ny, cz = c / (g.nx * g.ny);
+        // lane s holds the range of stencil cell s
+        int b = 0, e = 0, dx, dy, dz;
+        if (lane < kStencil) {
+            const int cn = stencil_cell(g, cx, cy, cz, lane, dx, dy, dz);
+            b = start[cn];
+            e = start[cn + 1];
+        }
+        uint32_t *row = nlist + list_group(i, cap) + ((i & 31) << 2);
+        const float wx = g.wf[0], wy = g.wf[1], wz = g.wf[2];
+        int cnt = 0;
+#pragma unroll 3
+        for (int s = 0; s < kStencil; ++s) {
+            const int sb = __shfl_sync(0xffffffffu, b, s), se = __shfl_sync(0xffffffffu, e, s);
+            const float hx = qi.x - (float)(s % 3 - 1) * wx, hy = qi.y - (float)((s / 3) % 3 - 1) * wy,
+                        hz = qi.z - (float)(s / 9 - 1) * wz;
+            for (int j0 = sb; j0 < se; j0 += 32) {
+                const int j = j0 + lane;
+                bool acc = false;
+                if (j < se && j != (s == 13 ? i : -1)) {
+                    const float4 qj = xq[j];
+                    const float ex = qj.x - hx, ey = qj.y - hy, ez = qj.z - hz;
+                    const float r2f = ex * ex + ey * ey + ez * ez;
+                    acc = !(r2f >= hi) && (!HALF || __float_as_int(qj.w) > myo);
+                    if (acc && !(r2f < lo)) {
+                        double shx, shy, shz;
+                        stencil_shift64(g, cx, cy, cz, s, shx, shy, shz);
+                        acc = exact_within_band(xabs, i, j, shx, shy, shz, rl2);
+                    }
+                }
+                const unsigned m = __ballot_sync(0xffffffffu, acc);
+                if (WRITE && acc) {
+                    const int k = cnt + __popc(m & ((1u << lane) - 1u));
+                    if (k < cap) row[row_off(k)] = ((uint32_t)s << kIndexBits) | (uint32_t)j;
+                }
+                cnt += __popc(m);
+            }
+        }
+        if (WRITE && cnt <= cap && lane < ((-cnt) & 3))
+            row[row_off(cnt + lane)] = (kPadStencil << kIndexBits) | (uint32_t)i;
+        if (lane == 0) ncount[i] = cnt;
+        maxc = max(maxc, cnt);
+        tot += (unsigned long long)cnt;
+        overflow |= (cnt > cap);
+    }
+    if (lane == 0) {
+        if (tot) atomicAdd(&ds->list_entries, tot);
+        if (maxc) atomicMax(&ds->max_count, maxc);
+        if (WRITE && overflow) atomicCAS(&ds->status, 0, (int)MD_ERR_LIST_OVERFLOW);
+    }
+    list_build_done(ds, close);
+}
+
 // a list build without binning counts anew
 __global__ void reset_counts_kernel(DevStatus *ds, bool slots) {
     if (ds->status == 0) reset_list_counts(ds, slots);
@@ -316,6 +390,18 @@ cudaError_t launch_build_list(md_system *h, bool write, bool gated, const float4
     if (!gated) {
         const cudaError_t e = launch_reset_counts(h, false);
         if (e != cudaSuccess) return e;
+    }
+    if (h->n <= kWarpListItems) {
+        const int nb = nblocks(n, kListBlock / 32);
+#define MDG_WARP(WR, HF)                                                                        \
+    warp_list_kernel<WR, HF><<<nb, kListBlock, 0, s>>>(n, h->grids, h->rep, h->list_lo, h->list_hi, \
+                                                       h->rl2, xq, h->xabs, h->cell,            \
+                                                       h->cell_start, h->nlist, h->ncount,      \
+                                                       h->cap, h->ds, gated, close)
+        if (write) { if (half) MDG_WARP(true, true); else MDG_WARP(true, false); }
+        else { if (half) MDG_WARP(false, true); else MDG_WARP(false, false); }
+#undef MDG_WARP
+        return cudaGetLastError();
     }
 #define MDG_LIST(WR, HF)                                                                    \
     build_list_kernel<WR, HF><<<gs_blocks(n) * (kBlock / kListBlock), kListBlock, 0, s>>>(                                \

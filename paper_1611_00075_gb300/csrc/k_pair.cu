@@ -223,6 +223,85 @@ pair_list_kernel(int n, Grid g, const Grid *__restrict__ grids, const uint16_t *
     list_build_done(ds, close);
 }
 
+// The same lists for small systems, a warp per slot (as warp_list_kernel): the
+// lanes take a cell's candidates at once.  The test is the midpoint form
+// |e|^2 - 2 |e.u| < hi - |u|^2 with e = x_j - m and u the half separation.
+template <bool WRITE>
+__global__ void __launch_bounds__(kPairBlock)
+warp_pair_list_kernel(int n, Grid g1, const Grid *__restrict__ grids,
+                      const uint16_t *__restrict__ rep, float hi, const float4 *__restrict__ xq,
+                      const int32_t *__restrict__ cell, const int32_t *__restrict__ start,
+                      const int32_t *__restrict__ slot_start,
+                      const uint32_t *__restrict__ slot_atom, uint32_t *__restrict__ list,
+                      int32_t *__restrict__ count, int cap, DevStatus *ds, bool gated, bool close) {
+    if (chain_off(ds, gated)) return;
+    const int nslots = slot_start[g1.ncells];
+    if (blockIdx.x == 0 && threadIdx.x == 0) ds->pair_slots = nslots;
+    const int lane = threadIdx.x & 31;
+    const int nw = gridDim.x * (kPairBlock / 32);
+    unsigned long long tot = 0;
+    int overflow = 0, maxc = 0;
+    for (int s = blockIdx.x * (kPairBlock / 32) + (threadIdx.x >> 5); s < nslots; s += nw) {
+        const uint32_t sa = slot_atom[s];
+        const int i0 = (int)(sa & ~kSingle);
+        const int i1 = (sa & kSingle) ? i0 : i0 + 1;
+        const Grid &g = grids[rep ? rep[i0] : 0];
+        const float4 q0 = xq[i0], q1 = xq[i1];
+        const float ux = 0.5f * (q1.x - q0.x), uy = 0.5f * (q1.y - q0.y), uz = 0.5f * (q1.z - q0.z);
+        const float mx = q0.x + ux, my = q0.y + uy, mz = q0.z + uz;
+        const float lim = hi - (ux * ux + uy * uy + uz * uz);
+        const int c = cell[i0] - g.cell0;
+        int b = 0, e = 0, dx, dy, dz;
+        if (lane < kStencil) {
+            const int cn = stencil_cell(g, c % g.nx, (c / g.nx) % g.ny, c / (g.nx * g.ny), lane, dx,
+                                        dy, dz);
+            b = start[cn];
+            e = start[cn + 1];
+        }
+        uint32_t *row = list + list_group(s, cap) + ((s & 31) << 2);
+        const float wx = g.wf[0], wy = g.wf[1], wz = g.wf[2];
+        int cnt = 0;
+#pragma unroll 3
+        for (int st = 0; st < kStencil; ++st) {
+            const int sb = __shfl_sync(0xffffffffu, b, st), se = __shfl_sync(0xffffffffu, e, st);
+            const float sx = mx - (float)(st % 3 - 1) * wx, sy = my - (float)((st / 3) % 3 - 1) * wy,
+                        sz = mz - (float)(st / 9 - 1) * wz;
+            for (int j0 = sb; j0 < se; j0 += 32) {
+                const int j = j0 + lane;
+                bool acc = false;
+                if (j < se) {
+                    const float4 qj = xq[j];
+                    const float ex = qj.x - sx, ey = qj.y - sy, ez = qj.z - sz;
+                    const float r2 = ex * ex + ey * ey + ez * ez;
+                    const float p = ex * ux + ey * uy + ez * uz;
+                    acc = fmaf(-2.0f, fabsf(p), r2) < lim;
+                    if (st == (int)kHomeStencil) acc = acc && j != i0 && j != i1;
+                }
+                const unsigned m = __ballot_sync(0xffffffffu, acc);
+                if (WRITE && acc) {
+                    const int k = cnt + __popc(m & ((1u << lane) - 1u));
+                    if (k < cap) row[k + (k >> 2) * 124] = ((uint32_t)st << kIndexBits) | (uint32_t)j;
+                }
+                cnt += __popc(m);
+            }
+        }
+        if (WRITE && cnt <= cap && lane < ((-cnt) & 3)) {
+            const int k = cnt + lane;
+            row[k + (k >> 2) * 124] = (kHomeStencil << kIndexBits) | (uint32_t)n;
+        }
+        if (lane == 0 && WRITE) count[s] = cnt;
+        maxc = max(maxc, cnt);
+        tot += (unsigned long long)cnt;
+        overflow |= (cnt > cap);
+    }
+    if (lane == 0) {
+        if (tot) atomicAdd(&ds->pair_entries, tot);
+        if (maxc) atomicMax(&ds->pair_max, maxc);
+        if (WRITE && overflow) atomicCAS(&ds->status, 0, (int)MD_ERR_LIST_OVERFLOW);
+    }
+    list_build_done(ds, close);
+}
+
 // the dummy neighbour of the padding entries, past the last atom of both
 // position buffers and of the many-body passes' (x, F') records
 __global__ void pair_dummy_kernel(float4 *xq0, float4 *xq1, float4 *xqf, int n) {
@@ -317,6 +396,15 @@ cudaError_t launch_pair_build(md_system *h, bool write, bool gated, bool close) 
         if (e != cudaSuccess) return e;
     }
     const int64_t smax = pair_slots_max(h->n, nc);
+    if (h->n / 2 <= kWarpListItems) {
+        const int nb = (int)((smax + kPairBlock / 32 - 1) / (kPairBlock / 32));
+        auto k = write ? warp_pair_list_kernel<true> : warp_pair_list_kernel<false>;
+        k<<<std::min(nb, 152 * 128), kPairBlock, 0, s>>>(n, h->g, h->grids, h->rep, h->list_hi,
+                                                         h->xq[h->cur], h->cell, h->cell_start,
+                                                         h->ps_start, h->ps_atom, h->ps_list,
+                                                         h->ps_count, h->ps_cap, h->ds, gated, close);
+        return cudaGetLastError();
+    }
     const int blocks = (int)std::min<int64_t>((smax + kPairBlock - 1) / kPairBlock, 152 * 16);
 #define MDG_PAIR_LIST(W, M)                                                                  \
     pair_list_kernel<W, M><<<blocks, kPairBlock, 0, s>>>(                                    \

@@ -147,6 +147,25 @@ struct Grid {
     const double *ctab; // cell centres (c + 0.5) w: nx for x, then ny for y, then nz for z
 };
 
+// Stencil cell s (0..26) of box-local cell (cx, cy, cz): its global id and
+// coordinates (dx, dy, dz).
+__device__ __forceinline__ int stencil_cell(const Grid &g, int cx, int cy, int cz, int s, int &dx,
+                                            int &dy, int &dz) {
+    dx = s % 3 - 1;
+    dy = (s / 3) % 3 - 1;
+    dz = s / 9 - 1;
+    const int xx = cx + dx < 0 ? g.nx - 1 : (cx + dx == g.nx ? 0 : cx + dx);
+    const int yy = cy + dy < 0 ? g.ny - 1 : (cy + dy == g.ny ? 0 : cy + dy);
+    const int zz = cz + dz < 0 ? g.nz - 1 : (cz + dz == g.nz ? 0 : cz + dz);
+    return g.cell0 + (zz * g.ny + yy) * g.nx + xx;
+}
+
+// Items (atoms or slots) up to which a warp builds each list.  One build with its
+// host side, a thread per item against a warp per item, us: per-atom lists 88 / 61
+// at 864 atoms, 110 / 64 at 4,000, 138 / 134 at 32,000, 152 / 193 at 55,296; slots
+// of two atoms 94 / 61 at 864 atoms, 110 / 96 at 32,000, 109 / 114 at 55,296.
+constexpr int64_t kWarpListItems = 24576;
+
 // Periodic wrap into [0, L): x - L*floor(x/L), then one correction each
 // way -- the rounded quotient can leave x a period off (a tiny negative x,
 // or x just below a multiple of L), and x + L can round up to L itself.
