@@ -196,6 +196,14 @@ inline int mixed_split(int64_t items, int cap) {
     if (items <= 65536 && cap <= 4 * 4 * kChunkQ) return 4;
     return 1;
 }
+// Eight lanes or one, for the passes with more work per entry; each says its limit.
+// Two-species LJ, one step with eight lanes against one, us: per-atom lists 12.7 /
+// 21.5 at 2,048 atoms, 22.1 / 24.1 at 32,000; slots of two 14.5 / 29 at 10,976
+// atoms, 30.8 / 33.5 at 70,304, 47.6 / 38.5 at 131,072.
+constexpr int64_t kTypedSplit = 32768;
+inline int split8(int64_t items, int cap, int64_t limit) {
+    return items <= limit && cap <= 8 * 4 * kChunkQ ? 8 : 1;
+}
 
 // Adds v over the converged lanes of the warp to the in-cutoff pair counter
 // (correct for any subset of lanes: each group's leader adds its own sum).

@@ -70,42 +70,57 @@ __device__ __forceinline__ double eam_F(const EamTab &t, double rho) {
     return -t.A * sqrt(rho) + t.B * rho * rho;
 }
 
+// Up to this size eight lanes share an atom (or slot).  One step (both passes,
+// per-atom lists), eight lanes against one, us: 16 / 25 at 1,024 atoms, 21 / 27 at
+// 8,192, 30 / 30 at 16,000, 44 / 28 at 35,152.
+constexpr int64_t kEamSplit = 12288;
+
 // Both mixed passes: 256-thread blocks at up to 64 registers.
-template <int NPSI>
-__global__ void __launch_bounds__(kBlock, 4) eam_density_mixed(ForceArgs a, EamTab t) {
+template <int NPSI, int P>
+__global__ void __launch_bounds__(kBlock, P > 1 ? 1 : 4) eam_density_mixed(ForceArgs a, EamTab t) {
     __shared__ ShiftTab sh;
     load_shifts_f32(a.g, &sh);
     __syncthreads();
     if (a.ds->status != 0) return;
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= a.n) return;
+    const int tid = blockIdx.x * blockDim.x + threadIdx.x;
+    const bool on = tid / P < a.n;
+    if (P == 1 && !on) return;
+    const int i = on ? tid / P : a.n - 1, part = tid % P;
     const float4 qi = a.xq[i];
     const int nq = (min(a.ncount[i], a.cap) + 3) >> 2;
     const uint4 *lq = reinterpret_cast<const uint4 *>(a.nlist + list_group(i, a.cap)) + (i & 31);
     const float rc2 = a.fc.rc2f;
     double R = 0.0;
-    uint4 nxt = nq > 0 ? __ldcs(lq) : make_uint4(0u, 0u, 0u, 0u);
-    for (int q0 = 0; q0 < nq; q0 += kChunkQ) {
-        const int q1 = min(q0 + kChunkQ, nq);
-        float r = 0.f;
-        auto pair = [&](uint32_t ent) {
-            const float4 qj = __ldg(a.xq + (ent & kIndexMask));
-            const uint32_t st = ent >> kIndexBits;
-            const float ex = (qj.x - qi.x) + sh.x[st];
-            const float ey = (qj.y - qi.y) + sh.y[st];
-            const float ez = (qj.z - qi.z) + sh.z[st];
-            const float r2 = ex * ex + ey * ey + ez * ez;
-            if (r2 < rc2) r += pieces_f32<NPSI>(t.qr, t.qa, t.npsi, r2 * rsqrt_fast(r2), nullptr);
-        };
-        for (int q = q0; q < q1; ++q) {
-            const uint4 e4 = nxt;
-            if (q + 1 < nq) nxt = __ldcs(lq + (size_t)(q + 1) * 32);
-            pair(e4.x);
-            pair(e4.y);
-            pair(e4.z);
-            pair(e4.w);
+    float r = 0.f;
+    auto pair = [&](uint32_t ent) {
+        const float4 qj = __ldg(a.xq + (ent & kIndexMask));
+        const uint32_t st = ent >> kIndexBits;
+        const float ex = (qj.x - qi.x) + sh.x[st];
+        const float ey = (qj.y - qi.y) + sh.y[st];
+        const float ez = (qj.z - qi.z) + sh.z[st];
+        const float r2 = ex * ex + ey * ey + ez * ez;
+        if (r2 < rc2) r += pieces_f32<NPSI>(t.qr, t.qa, t.npsi, r2 * rsqrt_fast(r2), nullptr);
+    };
+    if (P > 1) {
+        split_quads<P>(lq, on ? nq : 0, part, pair);
+        R = split_sum<P>((double)r);
+        if (!on || part != 0) return;
+    } else {
+        // list quads stream through once (evict-first), one quad loaded ahead
+        uint4 nxt = nq > 0 ? __ldcs(lq) : make_uint4(0u, 0u, 0u, 0u);
+        for (int q0 = 0; q0 < nq; q0 += kChunkQ) {
+            const int q1 = min(q0 + kChunkQ, nq);
+            r = 0.f;
+            for (int q = q0; q < q1; ++q) {
+                const uint4 e4 = nxt;
+                if (q + 1 < nq) nxt = __ldcs(lq + (size_t)(q + 1) * 32);
+                pair(e4.x);
+                pair(e4.y);
+                pair(e4.z);
+                pair(e4.w);
+            }
+            R += (double)r;
         }
-        R += (double)r;
     }
     a.rho[i] = R;
     const float dF = (float)eam_dF(t, R);
@@ -145,15 +160,17 @@ __global__ void __launch_bounds__(kBlock) eam_density_fp64(ForceArgs a, EamTab t
     a.dF32[i] = (float)d;
 }
 
-template <int MODE, bool ENERGY, int NPHI, int NPSI>
-__global__ void __launch_bounds__(kBlock, 4) eam_force_mixed(ForceArgs a, EamTab t, int store_f) {
+template <int MODE, bool ENERGY, int NPHI, int NPSI, int P>
+__global__ void __launch_bounds__(kBlock, P > 1 ? 1 : 4) eam_force_mixed(ForceArgs a, EamTab t, int store_f) {
     __shared__ ShiftTab sh;
     load_shifts_f32(a.g, &sh);
     __syncthreads();
     if (a.ds->status != 0) return;
     step_bookkeeping<MODE>(a);
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= a.n) return;
+    const int tid = blockIdx.x * blockDim.x + threadIdx.x;
+    const bool on = tid / P < a.n;
+    if (P == 1 && !on) return;
+    const int i = on ? tid / P : a.n - 1, part = tid % P;
     const float4 qi = a.xqf[i];  // position, F'(rho_i)
     const float dFi = qi.w;
     const int nq = (min(a.ncount[i], a.cap) + 3) >> 2;
@@ -161,34 +178,51 @@ __global__ void __launch_bounds__(kBlock, 4) eam_force_mixed(ForceArgs a, EamTab
     const float rc2 = a.fc.rc2f;
     double Fx = 0.0, Fy = 0.0, Fz = 0.0, E = 0.0;
     unsigned npair = 0;
+    float fx = 0.f, fy = 0.f, fz = 0.f, e = 0.f;
+    auto pair = [&](uint32_t ent) {
+        const float4 qj = __ldg(a.xqf + (ent & kIndexMask));  // position, F'(rho_j)
+        const uint32_t st = ent >> kIndexBits;
+        const float ex = (qj.x - qi.x) + sh.x[st];
+        const float ey = (qj.y - qi.y) + sh.y[st];
+        const float ez = (qj.z - qi.z) + sh.z[st];
+        const float r2 = ex * ex + ey * ey + ez * ez;
+        if (r2 < rc2) {
+            const float rinv = rsqrt_fast(r2);
+            const float r = r2 * rinv;
+            float dPhi, dpsi;
+            const float Phi = pieces_f32<NPHI>(t.pr, t.pa, t.nphi, r, &dPhi);
+            pieces_f32<NPSI>(t.qr, t.qa, t.npsi, r, &dpsi);
+            // f_i += g (r_j - r_i) / r with g = Phi' + (F'_i + F'_j) psi'
+            const float fs = (dPhi + (dFi + qj.w) * dpsi) * rinv;
+            fx = fmaf(fs, ex, fx);
+            fy = fmaf(fs, ey, fy);
+            fz = fmaf(fs, ez, fz);
+            if (ENERGY) {
+                e += Phi;
+                ++npair;
+            }
+        }
+    };
+    if constexpr (P > 1) {
+        const int c = part & 3;
+        const SplitState st = load_split_state<MODE>(a, i, c, on && part < 4);
+        split_quads<P>(lq, on ? nq : 0, part, pair);
+        Fx = split_sum<P>((double)fx);
+        Fy = split_sum<P>((double)fy);
+        Fz = split_sum<P>((double)fz);
+        if (ENERGY) {
+            E = split_sum<P>((double)e);
+            if (on) count_pairs(a.ds, npair);
+            if (on && part == 0) a.e_atom[i] = 0.5 * E + eam_F(t, a.rho[i]);
+        }
+        split_epilogue<MODE>(a, i, c, on && part < 4, c == 0 ? Fx : (c == 1 ? Fy : Fz),
+                             reinterpret_cast<const float *>(a.xq)[4 * (size_t)i + 3], st, store_f);
+        return;
+    }
     uint4 nxt = nq > 0 ? __ldcs(lq) : make_uint4(0u, 0u, 0u, 0u);
     for (int q0 = 0; q0 < nq; q0 += kChunkQ) {
         const int q1 = min(q0 + kChunkQ, nq);
-        float fx = 0.f, fy = 0.f, fz = 0.f, e = 0.f;
-        auto pair = [&](uint32_t ent) {
-            const float4 qj = __ldg(a.xqf + (ent & kIndexMask));  // position, F'(rho_j)
-            const uint32_t st = ent >> kIndexBits;
-            const float ex = (qj.x - qi.x) + sh.x[st];
-            const float ey = (qj.y - qi.y) + sh.y[st];
-            const float ez = (qj.z - qi.z) + sh.z[st];
-            const float r2 = ex * ex + ey * ey + ez * ez;
-            if (r2 < rc2) {
-                const float rinv = rsqrt_fast(r2);
-                const float r = r2 * rinv;
-                float dPhi, dpsi;
-                const float Phi = pieces_f32<NPHI>(t.pr, t.pa, t.nphi, r, &dPhi);
-                pieces_f32<NPSI>(t.qr, t.qa, t.npsi, r, &dpsi);
-                // f_i += g (r_j - r_i) / r with g = Phi' + (F'_i + F'_j) psi'
-                const float fs = (dPhi + (dFi + qj.w) * dpsi) * rinv;
-                fx = fmaf(fs, ex, fx);
-                fy = fmaf(fs, ey, fy);
-                fz = fmaf(fs, ez, fz);
-                if (ENERGY) {
-                    e += Phi;
-                    ++npair;
-                }
-            }
-        };
+        fx = fy = fz = e = 0.f;
         for (int q = q0; q < q1; ++q) {
             const uint4 e4 = nxt;
             if (q + 1 < nq) nxt = __ldcs(lq + (size_t)(q + 1) * 32);
@@ -308,15 +342,18 @@ __device__ __forceinline__ float2 pieces_pair(const float *knot, const float *c,
     return v;
 }
 
-template <int NPSI>
-__global__ void __launch_bounds__(kEamPairBlock, 8) eam_density_pair(ForceArgs a, PairArgs p,
+template <int NPSI, int P>
+__global__ void __launch_bounds__(kEamPairBlock, P > 1 ? 1 : 8) eam_density_pair(ForceArgs a, PairArgs p,
                                                                      EamTab t) {
     __shared__ ShiftTab sh;
     load_shifts_f32(a.g, &sh);
     __syncthreads();
     if (a.ds->status != 0) return;
-    const int s = blockIdx.x * blockDim.x + threadIdx.x;
-    if (s >= p.slot_start[p.ncells]) return;
+    const int tid = blockIdx.x * blockDim.x + threadIdx.x;
+    const int nslots = p.slot_start[p.ncells];
+    if ((P > 1 ? (tid & ~31) / P : tid) >= nslots) return;  // P > 1: whole warps
+    const bool on = tid / P < nslots;
+    const int s = on ? tid / P : nslots - 1, part = tid % P;
     const uint32_t sa = p.slot_atom[s];
     const int i0 = (int)(sa & ~kSingle);
     const bool two = !(sa & kSingle);
@@ -328,7 +365,7 @@ __global__ void __launch_bounds__(kEamPairBlock, 8) eam_density_pair(ForceArgs a
         // the slot's own pair adds to both densities
         const float ex = q1.x - q0.x, ey = q1.y - q0.y, ez = q1.z - q0.z;
         const float r2 = ex * ex + ey * ey + ez * ez;
-        if (r2 < rc2) r = dup2(pieces_f32<NPSI>(t.qr, t.qa, t.npsi, r2 * rsqrt_fast(r2), nullptr));
+        if (part == 0 && r2 < rc2) r = dup2(pieces_f32<NPSI>(t.qr, t.qa, t.npsi, r2 * rsqrt_fast(r2), nullptr));
     }
     const float2 nqx = make_float2(-q0.x, -q1.x), nqy = make_float2(-q0.y, -q1.y),
                  nqz = make_float2(-q0.z, -q1.z);
@@ -344,8 +381,15 @@ __global__ void __launch_bounds__(kEamPairBlock, 8) eam_density_pair(ForceArgs a
         r = add2(r, pieces_pair<NPSI, false>(t.qr, t.qa, t.npsi, rr, nullptr));
     };
     double R0 = 0.0, R1 = 0.0;
+    if (P > 1) {
+        split_quads<P>(lq, on ? nq : 0, part, pair);
+        R0 = split_sum<P>((double)r.x);
+        R1 = split_sum<P>((double)r.y);
+        if (!on || part != 0) return;
+        r = dup2(0.f);
+    }
     uint4 nxt = nq > 0 ? __ldcs(lq) : make_uint4(0u, 0u, 0u, 0u);
-    for (int c0 = 0; c0 < nq; c0 += kChunkQ) {
+    for (int c0 = 0; P == 1 && c0 < nq; c0 += kChunkQ) {
         const int c1 = min(c0 + kChunkQ, nq);
         for (int q = c0; q < c1; ++q) {
             const uint4 e4 = nxt;
@@ -393,16 +437,19 @@ __device__ __forceinline__ void eam_pair_atom_out(const ForceArgs &a, const EamT
         vv_epilogue<MODE>(a, i, Fx, Fy, Fz, reinterpret_cast<const float *>(a.xq)[4 * (size_t)i + 3]);
 }
 
-template <int MODE, bool ENERGY, int NPHI, int NPSI>
-__global__ void __launch_bounds__(kEamPairBlock, 8) eam_force_pair(ForceArgs a, PairArgs p,
+template <int MODE, bool ENERGY, int NPHI, int NPSI, int P>
+__global__ void __launch_bounds__(kEamPairBlock, P > 1 ? 1 : 8) eam_force_pair(ForceArgs a, PairArgs p,
                                                                    EamTab t, int store_f) {
     __shared__ ShiftTab sh;
     load_shifts_f32(a.g, &sh);
     __syncthreads();
     if (a.ds->status != 0) return;
     step_bookkeeping<MODE>(a);
-    const int s = blockIdx.x * blockDim.x + threadIdx.x;
-    if (s >= p.slot_start[p.ncells]) return;
+    const int tid = blockIdx.x * blockDim.x + threadIdx.x;
+    const int nslots = p.slot_start[p.ncells];
+    if ((P > 1 ? (tid & ~31) / P : tid) >= nslots) return;  // P > 1: whole warps
+    const bool on = tid / P < nslots;
+    const int s = on ? tid / P : nslots - 1, part = tid % P;
     const uint32_t sa = p.slot_atom[s];
     const int i0 = (int)(sa & ~kSingle);
     const bool two = !(sa & kSingle);
@@ -416,7 +463,7 @@ __global__ void __launch_bounds__(kEamPairBlock, 8) eam_force_pair(ForceArgs a, 
         // the slot's own pair once: e = x_1 - x_0, f_0 += g e / r, f_1 -= g e / r
         const float ex = q1.x - q0.x, ey = q1.y - q0.y, ez = q1.z - q0.z;
         const float r2 = ex * ex + ey * ey + ez * ez;
-        if (r2 < rc2) {
+        if (part == 0 && r2 < rc2) {
             const float rinv = rsqrt_fast(r2);
             const float rr = r2 * rinv;
             float dPhi, dpsi;
@@ -458,6 +505,23 @@ __global__ void __launch_bounds__(kEamPairBlock, 8) eam_force_pair(ForceArgs a, 
             np1 += r2.y < rc2 ? 1u : 0u;
         }
     };
+    if constexpr (P > 1) {
+        SplitState st, st1;
+        load_slot_state<MODE, P>(a, i0, two, on, part, st, st1);
+        split_quads<P>(lq, on ? nq : 0, part, pair);
+        const double F0[3] = {split_sum<P>((double)fx.x), split_sum<P>((double)fy.x),
+                              split_sum<P>((double)fz.x)};
+        const double F1[3] = {split_sum<P>((double)fx.y), split_sum<P>((double)fy.y),
+                              split_sum<P>((double)fz.y)};
+        if (ENERGY) {
+            const double E0 = split_sum<P>((double)en.x), E1 = split_sum<P>((double)en.y);
+            if (on) count_pairs(a.ds, np0 + (two ? np1 : 0u));
+            if (on && part == 0) a.e_atom[i0] = 0.5 * E0 + eam_F(t, a.rho[i0]);
+            if (on && two && part == 1) a.e_atom[i0 + 1] = 0.5 * E1 + eam_F(t, a.rho[i0 + 1]);
+        }
+        split_slot_finish<MODE, false, P>(a, i0, two, on, part, F0, F1, st, st1, store_f);
+        return;
+    }
     double F0x = 0.0, F0y = 0.0, F0z = 0.0, F1x = 0.0, F1y = 0.0, F1z = 0.0, E0 = 0.0, E1 = 0.0;
     auto flush = [&]() {
         F0x += (double)fx.x; F0y += (double)fy.x; F0z += (double)fz.x;
@@ -495,14 +559,19 @@ cudaError_t launch_eam_density(md_system *h) {
     const EamTab &t = h->eam;
     if (h->p.force_variant == MD_FORCE_PAIRED) {
         const PairArgs p = make_pair_args(h);
-        const int pb = pair_grid_blocks(h, kEamPairBlock);
-        if (t.npsi == 1) eam_density_pair<1><<<pb, kEamPairBlock, 0, h->stream>>>(a, p, t);
-        else eam_density_pair<0><<<pb, kEamPairBlock, 0, h->stream>>>(a, p, t);
+        const int P = split8(h->n / 2, h->ps_cap, kEamSplit);
+        const bool one = t.npsi == 1;
+        auto k = P > 1 ? (one ? eam_density_pair<1, 8> : eam_density_pair<0, 8>)
+                       : (one ? eam_density_pair<1, 1> : eam_density_pair<0, 1>);
+        k<<<pair_grid_blocks(h, kEamPairBlock, P), kEamPairBlock, 0, h->stream>>>(a, p, t);
         return cudaGetLastError();
     }
     if (h->p.precision == MD_MIXED) {
-        if (t.npsi == 1) eam_density_mixed<1><<<nb, kBlock, 0, h->stream>>>(a, t);
-        else eam_density_mixed<0><<<nb, kBlock, 0, h->stream>>>(a, t);
+        const int P = split8(h->n, h->cap, kEamSplit);
+        const bool one = t.npsi == 1;
+        auto k = P > 1 ? (one ? eam_density_mixed<1, 8> : eam_density_mixed<0, 8>)
+                       : (one ? eam_density_mixed<1, 1> : eam_density_mixed<0, 1>);
+        k<<<nblocks(h->n * P), kBlock, 0, h->stream>>>(a, t);
     } else {
         eam_density_fp64<<<nb, kBlock, 0, h->stream>>>(a, t);
     }
@@ -517,12 +586,14 @@ cudaError_t launch_eam_force(md_system *h, int mode, bool energy, bool store_f) 
     cudaStream_t s = h->stream;
     if (h->p.force_variant == MD_FORCE_PAIRED) {
         const PairArgs p = make_pair_args(h);
-        const int pb = pair_grid_blocks(h, kEamPairBlock);
+        const int P = split8(h->n / 2, h->ps_cap, kEamSplit);
+        const int pb = pair_grid_blocks(h, kEamPairBlock, P);
         const bool fe = (t.nphi == 7 && t.npsi == 1);
 #define MDG_EAMP(M, E)                                                                  \
     do {                                                                                \
-        if (fe) eam_force_pair<M, E, 7, 1><<<pb, kEamPairBlock, 0, s>>>(a, p, t, sf);   \
-        else eam_force_pair<M, E, 0, 0><<<pb, kEamPairBlock, 0, s>>>(a, p, t, sf);      \
+        auto k = P > 1 ? (fe ? eam_force_pair<M, E, 7, 1, 8> : eam_force_pair<M, E, 0, 0, 8>)  \
+                       : (fe ? eam_force_pair<M, E, 7, 1, 1> : eam_force_pair<M, E, 0, 0, 1>); \
+        k<<<pb, kEamPairBlock, 0, s>>>(a, p, t, sf);                                    \
     } while (0)
         switch (mode) {
             case FM_STORE: if (energy) MDG_EAMP(FM_STORE, true); else MDG_EAMP(FM_STORE, false); break;
@@ -533,12 +604,14 @@ cudaError_t launch_eam_force(md_system *h, int mode, bool energy, bool store_f) 
         return cudaGetLastError();
     }
     if (h->p.precision == MD_MIXED) {
+        const int P = split8(h->n, h->cap, kEamSplit);
         // the knot counts of the Fe-like table get compile-time loops
         const bool fe = (t.nphi == 7 && t.npsi == 1);
 #define MDG_EAM(M, E)                                                                   \
     do {                                                                                \
-        if (fe) eam_force_mixed<M, E, 7, 1><<<nb, kBlock, 0, s>>>(a, t, sf);            \
-        else eam_force_mixed<M, E, 0, 0><<<nb, kBlock, 0, s>>>(a, t, sf);               \
+        auto k = P > 1 ? (fe ? eam_force_mixed<M, E, 7, 1, 8> : eam_force_mixed<M, E, 0, 0, 8>)  \
+                       : (fe ? eam_force_mixed<M, E, 7, 1, 1> : eam_force_mixed<M, E, 0, 0, 1>); \
+        k<<<nblocks(h->n * P), kBlock, 0, s>>>(a, t, sf);                               \
     } while (0)
         switch (mode) {
             case FM_STORE: if (energy) MDG_EAM(FM_STORE, true); else MDG_EAM(FM_STORE, false); break;

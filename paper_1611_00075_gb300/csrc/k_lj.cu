@@ -695,7 +695,7 @@ cudaError_t launch_lj_typed_fp64(md_system *h, const ForceArgs &a, int mode, boo
 template <int NT>
 cudaError_t launch_lj_typed_nt(md_system *h, const ForceArgs &a, int mode, bool energy, int sf) {
     if (h->p.precision == MD_MIXED)
-        return mixed_split(h->n, h->cap) > 1 ? launch_lj_typed_mixed<NT, 8>(h, a, mode, energy, sf)
+        return split8(h->n, h->cap, kTypedSplit) > 1 ? launch_lj_typed_mixed<NT, 8>(h, a, mode, energy, sf)
                                              : launch_lj_typed_mixed<NT, 1>(h, a, mode, energy, sf);
     switch (f64_split(h->n)) {
         case 1: return launch_lj_typed_fp64<NT, 1>(h, a, mode, energy, sf);

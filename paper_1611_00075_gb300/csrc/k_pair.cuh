@@ -74,6 +74,39 @@ __device__ __forceinline__ void pair_atom_out(const ForceArgs &a, int i, double 
     if (MODE != FM_STORE) vv_epilogue<MODE>(a, i, Fx, Fy, Fz, qw);
 }
 
+// State of the components that the lane finishes: with eight lanes component
+// part % 4 of atom part / 4, with four that of both atoms.
+template <int MODE, int P>
+__device__ __forceinline__ void load_slot_state(const ForceArgs &a, int i0, bool two, bool on,
+                                                int part, SplitState &t, SplitState &t1) {
+    const int c = part & 3, k = P >= 8 ? (part >> 2) & 1 : 0;
+    t = load_split_state<MODE>(a, i0 + (two ? k : 0), c, on && part < 8);
+    t1 = P < 8 ? load_split_state<MODE>(a, i0 + (two ? 1 : 0), c, on) : t;
+}
+
+// Stores and epilogues of a slot's atoms from their forces, which every one of its
+// P lanes holds (every lane of the warp calls it).
+template <int MODE, bool SPECIES, int P>
+__device__ __forceinline__ void split_slot_finish(const ForceArgs &a, int i0, bool two, bool on,
+                                                  int part, const double *F0, const double *F1,
+                                                  const SplitState &t, const SplitState &t1,
+                                                  int store_f) {
+    const int c = part & 3;
+    const double G0 = c == 0 ? F0[0] : (c == 1 ? F0[1] : F0[2]);
+    const double G1 = c == 0 ? F1[0] : (c == 1 ? F1[1] : F1[2]);
+    const float *words = reinterpret_cast<const float *>(a.xq);
+    const int i1 = i0 + (two ? 1 : 0);
+    if (P >= 8) {
+        const bool second = (part >> 2) & 1;
+        const int i = second ? i1 : i0;
+        split_epilogue<MODE, SPECIES>(a, i, c, on && part < 8 && (two || !second), second ? G1 : G0,
+                                      words[4 * (size_t)i + 3], t, store_f);
+    } else {
+        split_epilogue<MODE, SPECIES>(a, i0, c, on, G0, words[4 * (size_t)i0 + 3], t, store_f);
+        split_epilogue<MODE, SPECIES>(a, i1, c, on && two, G1, words[4 * (size_t)i1 + 3], t1, store_f);
+    }
+}
+
 // Sums of a slot's P lanes, then stores, energies and epilogues of its atoms (every
 // lane of the warp calls it): t is the state of the lane's component of the first
 // atom (with eight lanes: of atom part / 4), t1 that of the second with four.
@@ -92,22 +125,9 @@ __device__ __forceinline__ void split_slot_out(const ForceArgs &a, int i0, bool 
         if (on && part == 0) a.e_atom[i0] = 0.5 * (double)en.x;
         if (on && two && part == 1) a.e_atom[i0 + 1] = 0.5 * (double)en.y;
     }
-    const int c = part & 3;
-    const float F0 = c == 0 ? fx.x : (c == 1 ? fy.x : fz.x);
-    const float F1 = c == 0 ? fx.y : (c == 1 ? fy.y : fz.y);
-    const float *words = reinterpret_cast<const float *>(a.xq);
-    if (P >= 8) {
-        const bool second = (part >> 2) & 1;
-        const bool fin = on && part < 8 && (two || !second);
-        const int i = i0 + (second && two ? 1 : 0);
-        split_epilogue<MODE, SPECIES>(a, i, c, fin, (double)(second ? F1 : F0),
-                                      words[4 * (size_t)i + 3], t, store_f);
-    } else {
-        split_epilogue<MODE, SPECIES>(a, i0, c, on, (double)F0, words[4 * (size_t)i0 + 3], t, store_f);
-        const int i1 = i0 + (two ? 1 : 0);
-        split_epilogue<MODE, SPECIES>(a, i1, c, on && two, (double)F1, words[4 * (size_t)i1 + 3], t1,
-                                      store_f);
-    }
+    const double F0[3] = {(double)fx.x, (double)fy.x, (double)fz.x};
+    const double F1[3] = {(double)fx.y, (double)fy.y, (double)fz.y};
+    split_slot_finish<MODE, SPECIES, P>(a, i0, two, on, part, F0, F1, t, t1, store_f);
 }
 
 // MULTI (a batch of boxes, the block's boxes not all in shared memory): the
@@ -180,11 +200,8 @@ __device__ __forceinline__ void lj_pair_slot(const ForceArgs &a, const PairArgs 
         }
     };
     if constexpr (P > 1) {
-        // four lanes finish an atom: with eight lanes both atoms at once
-        const int c = part & 3, k = P >= 8 ? (part >> 2) & 1 : 0;
-        const bool fin = on && part < 8;
-        SplitState t = load_split_state<MODE>(a, i0 + (two ? k : 0), c, fin);
-        SplitState t1 = P < 8 ? load_split_state<MODE>(a, i0 + (two ? 1 : 0), c, fin) : t;
+        SplitState t, t1;
+        load_slot_state<MODE, P>(a, i0, two, on, part, t, t1);
         split_quads<P>(lq, on ? nq : 0, part, pair);
         split_slot_out<MODE, ENERGY, false, P>(a, i0, two, on, part, fx, fy, fz, en, np0, np1, t, t1,
                                                store_f);

@@ -176,10 +176,10 @@ lj_typed_pair_kernel(ForceArgs a, PairArgs p, TypeTab tt, int store_f) {
         }
     };
     if constexpr (P > 1) {
-        const int c = part & 3, k = (part >> 2) & 1;
-        const SplitState st = load_split_state<MODE>(a, i0 + (two ? k : 0), c, on && part < 8);
+        SplitState st, st1;
+        load_slot_state<MODE, P>(a, i0, two, on, part, st, st1);
         split_quads<P>(lq, on ? nq : 0, part, pair);
-        split_slot_out<MODE, ENERGY, true, P>(a, i0, two, on, part, fx, fy, fz, en, np0, np1, st, st,
+        split_slot_out<MODE, ENERGY, true, P>(a, i0, two, on, part, fx, fy, fz, en, np0, np1, st, st1,
                                               store_f);
         return;
     }
@@ -230,7 +230,7 @@ cudaError_t launch_any(md_system *h, int mode, bool energy, bool store_f) {
     unsigned bits;
     std::memcpy(&bits, &h->fc.rc2f, sizeof bits);
     if (!inside_fits(bits >> 23)) return launch_nt<NT, 1, false>(h, mode, energy, store_f);
-    return mixed_split(h->n / 2, h->ps_cap) > 1 ? launch_nt<NT, 8>(h, mode, energy, store_f)
+    return split8(h->n / 2, h->ps_cap, kTypedSplit) > 1 ? launch_nt<NT, 8>(h, mode, energy, store_f)
                                                 : launch_nt<NT, 1>(h, mode, energy, store_f);
 }
 

@@ -58,6 +58,12 @@ __device__ __forceinline__ double rpowd(double x, int k) {
     return r;
 }
 
+// Up to these sizes eight lanes share an atom or a slot.  One step (both passes),
+// eight lanes against one, us: per-atom lists 16.5 / 39 at 1,372 atoms, 24.5 / 44
+// at 6,912, 36 / 45 at 16,384, 56 / 46 at 32,000; slots of two 19.7 / 61, 23.7 /
+// 82, 31 / 69, 48 / 72 and, at 55,296 atoms, 106 / 110.
+constexpr int64_t kScSplitAtoms = 20480, kScSplitSlots = 24576;
+
 // (a/r)^K from s = (a/r)^2 and ar = a/r (ar only used for odd K).
 template <int K>
 __device__ __forceinline__ float ar_pow(float s, float ar) {
@@ -75,49 +81,58 @@ __device__ __forceinline__ double sc_embed_deriv_f64(double rho, double ec) {
 
 // Both mixed passes run 256-thread blocks at up to 64 registers (4 per SM),
 // measured 2 % faster than at 48.
-template <int ME>
-__global__ void __launch_bounds__(kBlock, 4) sc_density_mixed(ForceArgs a) {
+template <int ME, int P>
+__global__ void __launch_bounds__(kBlock, P > 1 ? 1 : 4) sc_density_mixed(ForceArgs a) {
     __shared__ ShiftTab sh;
     load_shifts_f32(a.g, &sh);
     __syncthreads();
     if (a.ds->status != 0) return;
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= a.n) return;
+    const int tid = blockIdx.x * blockDim.x + threadIdx.x;
+    const bool on = tid / P < a.n;
+    if (P == 1 && !on) return;
+    const int i = on ? tid / P : a.n - 1, part = tid % P;
     const float4 qi = a.xq[i];
     const int nq = (min(a.ncount[i], a.cap) + 3) >> 2;
     const uint4 *lq = reinterpret_cast<const uint4 *>(a.nlist + list_group(i, a.cap)) + (i & 31);
     const float rc2 = a.fc.rc2f, af = a.fc.sc_af, a2 = af * af;
     const int m = a.fc.sc_m;
     double R = 0.0;
-    // list quads stream through once (evict-first), one quad loaded ahead
-    uint4 nxt = nq > 0 ? __ldcs(lq) : make_uint4(0u, 0u, 0u, 0u);
-    for (int q0 = 0; q0 < nq; q0 += kChunkQ) {
-        const int q1 = min(q0 + kChunkQ, nq);
-        float r = 0.f;
-        auto pair = [&](uint32_t ent) {
-            const float4 qj = __ldg(a.xq + (ent & kIndexMask));
-            const uint32_t st = ent >> kIndexBits;
-            const float ex = (qj.x - qi.x) + sh.x[st];
-            const float ey = (qj.y - qi.y) + sh.y[st];
-            const float ez = (qj.z - qi.z) + sh.z[st];
-            const float r2 = ex * ex + ey * ey + ez * ez;
-            if (r2 < rc2) {
-                const float s = a2 * rcp_fast(r2);
-                float psi;
-                if (ME > 0) psi = ar_pow<ME>(s, (ME & 1) ? af * rsqrt_fast(r2) : 0.f);
-                else psi = (m & 1) ? rpow(s, m / 2) * af * rsqrt_fast(r2) : rpow(s, m / 2);
-                r += psi;
-            }
-        };
-        for (int q = q0; q < q1; ++q) {
-            const uint4 e4 = nxt;
-            if (q + 1 < nq) nxt = __ldcs(lq + (size_t)(q + 1) * 32);
-            pair(e4.x);
-            pair(e4.y);
-            pair(e4.z);
-            pair(e4.w);
+    float r = 0.f;
+    auto pair = [&](uint32_t ent) {
+        const float4 qj = __ldg(a.xq + (ent & kIndexMask));
+        const uint32_t st = ent >> kIndexBits;
+        const float ex = (qj.x - qi.x) + sh.x[st];
+        const float ey = (qj.y - qi.y) + sh.y[st];
+        const float ez = (qj.z - qi.z) + sh.z[st];
+        const float r2 = ex * ex + ey * ey + ez * ez;
+        if (r2 < rc2) {
+            const float s = a2 * rcp_fast(r2);
+            float psi;
+            if (ME > 0) psi = ar_pow<ME>(s, (ME & 1) ? af * rsqrt_fast(r2) : 0.f);
+            else psi = (m & 1) ? rpow(s, m / 2) * af * rsqrt_fast(r2) : rpow(s, m / 2);
+            r += psi;
         }
-        R += (double)r;
+    };
+    if (P > 1) {
+        split_quads<P>(lq, on ? nq : 0, part, pair);
+        R = split_sum<P>((double)r);
+        if (!on || part != 0) return;
+    } else {
+        // list quads stream through once (evict-first), one quad loaded ahead
+        uint4 nxt = nq > 0 ? __ldcs(lq) : make_uint4(0u, 0u, 0u, 0u);
+        for (int q0 = 0; q0 < nq; q0 += kChunkQ) {
+            const int q1 = min(q0 + kChunkQ, nq);
+            r = 0.f;
+            for (int q = q0; q < q1; ++q) {
+                const uint4 e4 = nxt;
+                if (q + 1 < nq) nxt = __ldcs(lq + (size_t)(q + 1) * 32);
+                pair(e4.x);
+                pair(e4.y);
+                pair(e4.z);
+                pair(e4.w);
+            }
+            R += (double)r;
+        }
     }
     a.rho[i] = R;
     const float dF = sc_embed_deriv_f32(R, a.fc.sc_ecf);
@@ -172,15 +187,17 @@ __global__ void __launch_bounds__(kF64Block) sc_density_fp64(ForceArgs a) {
     a.dF32[i] = (float)d;
 }
 
-template <int MODE, bool ENERGY, int NE, int ME>
-__global__ void __launch_bounds__(kBlock, 4) sc_force_mixed(ForceArgs a, int store_f) {
+template <int MODE, bool ENERGY, int NE, int ME, int P>
+__global__ void __launch_bounds__(kBlock, P > 1 ? 1 : 4) sc_force_mixed(ForceArgs a, int store_f) {
     __shared__ ShiftTab sh;
     load_shifts_f32(a.g, &sh);
     __syncthreads();
     if (a.ds->status != 0) return;
     step_bookkeeping<MODE>(a);
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= a.n) return;
+    const int tid = blockIdx.x * blockDim.x + threadIdx.x;
+    const bool on = tid / P < a.n;
+    if (P == 1 && !on) return;
+    const int i = on ? tid / P : a.n - 1, part = tid % P;
     const float4 qi = a.xqf[i];  // position, F'(rho_i)
     const float dFi = qi.w;
     const int nq = (min(a.ncount[i], a.cap) + 3) >> 2;
@@ -191,42 +208,59 @@ __global__ void __launch_bounds__(kBlock, 4) sc_force_mixed(ForceArgs a, int sto
     const float nf = (float)(NE > 0 ? NE : nexp), mf = (float)(ME > 0 ? ME : mexp);
     double Fx = 0.0, Fy = 0.0, Fz = 0.0, E = 0.0;
     unsigned npair = 0;
+    float fx = 0.f, fy = 0.f, fz = 0.f, e = 0.f;
+    auto pair = [&](uint32_t ent) {
+        const float4 qj = __ldg(a.xqf + (ent & kIndexMask));  // position, F'(rho_j)
+        const uint32_t st = ent >> kIndexBits;
+        const float ex = (qj.x - qi.x) + sh.x[st];
+        const float ey = (qj.y - qi.y) + sh.y[st];
+        const float ez = (qj.z - qi.z) + sh.z[st];
+        const float r2 = ex * ex + ey * ey + ez * ez;
+        if (r2 < rc2) {
+            // with an odd exponent a/r comes from one reciprocal square
+            // root, and (a/r)^2 and 1/r^2 from it without a reciprocal
+            const bool odd = (NE > 0) ? ((NE | ME) & 1) : ((nexp | mexp) & 1);
+            const float ar = odd ? af * rsqrt_fast(r2) : 0.f;
+            const float r2i = odd ? ar * ar * inv_a2 : rcp_fast(r2);
+            const float s = odd ? ar * ar : a2 * r2i;
+            float Phi, psi;
+            if (NE > 0) {
+                Phi = epsf * ar_pow<NE>(s, ar);
+                psi = ar_pow<ME>(s, ar);
+            } else {
+                Phi = epsf * ((nexp & 1) ? rpow(s, nexp / 2) * ar : rpow(s, nexp / 2));
+                psi = (mexp & 1) ? rpow(s, mexp / 2) * ar : rpow(s, mexp / 2);
+            }
+            const float fs = (nf * Phi + mf * (dFi + qj.w) * psi) * r2i;
+            fx -= fs * ex;
+            fy -= fs * ey;
+            fz -= fs * ez;
+            if (ENERGY) {
+                e += Phi;
+                ++npair;
+            }
+        }
+    };
+    if constexpr (P > 1) {
+        const int c = part & 3;
+        const SplitState st = load_split_state<MODE>(a, i, c, on && part < 4);
+        split_quads<P>(lq, on ? nq : 0, part, pair);
+        Fx = split_sum<P>((double)fx);
+        Fy = split_sum<P>((double)fy);
+        Fz = split_sum<P>((double)fz);
+        if (ENERGY) {
+            E = split_sum<P>((double)e);
+            if (on) count_pairs(a.ds, npair);
+            if (on && part == 0) a.e_atom[i] = 0.5 * E - a.fc.sc_ec * sqrt(a.rho[i]);
+        }
+        split_epilogue<MODE>(a, i, c, on && part < 4, c == 0 ? Fx : (c == 1 ? Fy : Fz),
+                             reinterpret_cast<const float *>(a.xq)[4 * (size_t)i + 3], st, store_f);
+        return;
+    }
     uint4 nxt = nq > 0 ? __ldcs(lq) : make_uint4(0u, 0u, 0u, 0u);
     for (int q0 = 0; q0 < nq; q0 += kChunkQ) {
         const int q1 = min(q0 + kChunkQ, nq);
-        float fx = 0.f, fy = 0.f, fz = 0.f, e = 0.f;
-        auto pair = [&](uint32_t ent) {
-            const float4 qj = __ldg(a.xqf + (ent & kIndexMask));  // position, F'(rho_j)
-            const uint32_t st = ent >> kIndexBits;
-            const float ex = (qj.x - qi.x) + sh.x[st];
-            const float ey = (qj.y - qi.y) + sh.y[st];
-            const float ez = (qj.z - qi.z) + sh.z[st];
-            const float r2 = ex * ex + ey * ey + ez * ez;
-            if (r2 < rc2) {
-                // with an odd exponent a/r comes from one reciprocal square
-                // root, and (a/r)^2 and 1/r^2 from it without a reciprocal
-                const bool odd = (NE > 0) ? ((NE | ME) & 1) : ((nexp | mexp) & 1);
-                const float ar = odd ? af * rsqrt_fast(r2) : 0.f;
-                const float r2i = odd ? ar * ar * inv_a2 : rcp_fast(r2);
-                const float s = odd ? ar * ar : a2 * r2i;
-                float Phi, psi;
-                if (NE > 0) {
-                    Phi = epsf * ar_pow<NE>(s, ar);
-                    psi = ar_pow<ME>(s, ar);
-                } else {
-                    Phi = epsf * ((nexp & 1) ? rpow(s, nexp / 2) * ar : rpow(s, nexp / 2));
-                    psi = (mexp & 1) ? rpow(s, mexp / 2) * ar : rpow(s, mexp / 2);
-                }
-                const float fs = (nf * Phi + mf * (dFi + qj.w) * psi) * r2i;
-                fx -= fs * ex;
-                fy -= fs * ey;
-                fz -= fs * ez;
-                if (ENERGY) {
-                    e += Phi;
-                    ++npair;
-                }
-            }
-        };
+        fx = fy = fz = e = 0.f;
         for (int q = q0; q < q1; ++q) {
             const uint4 e4 = nxt;
             if (q + 1 < nq) nxt = __ldcs(lq + (size_t)(q + 1) * 32);
@@ -374,14 +408,17 @@ __device__ __forceinline__ float2 ar_pow_rt(float2 s, float2 ar, int k) {
     return r;
 }
 
-template <int ME>
-__global__ void __launch_bounds__(kScPairBlock, 8) sc_density_pair(ForceArgs a, PairArgs p) {
+template <int ME, int P>
+__global__ void __launch_bounds__(kScPairBlock, P > 1 ? 1 : 8) sc_density_pair(ForceArgs a, PairArgs p) {
     __shared__ ShiftTab sh;
     load_shifts_f32(a.g, &sh);
     __syncthreads();
     if (a.ds->status != 0) return;
-    const int s = blockIdx.x * blockDim.x + threadIdx.x;
-    if (s >= p.slot_start[p.ncells]) return;
+    const int tid = blockIdx.x * blockDim.x + threadIdx.x;
+    const int nslots = p.slot_start[p.ncells];
+    if ((P > 1 ? (tid & ~31) / P : tid) >= nslots) return;  // P > 1: whole warps
+    const bool on = tid / P < nslots;
+    const int s = on ? tid / P : nslots - 1, part = tid % P;
     const uint32_t sa = p.slot_atom[s];
     const int i0 = (int)(sa & ~kSingle);
     const bool two = !(sa & kSingle);
@@ -394,7 +431,7 @@ __global__ void __launch_bounds__(kScPairBlock, 8) sc_density_pair(ForceArgs a, 
         // the slot's own pair adds to both densities
         const float ex = q1.x - q0.x, ey = q1.y - q0.y, ez = q1.z - q0.z;
         const float r2 = ex * ex + ey * ey + ez * ez;
-        if (r2 < rc2) {
+        if (part == 0 && r2 < rc2) {
             const float sp = a2 * rcp_fast(r2);
             const float psi = ME > 0 ? ar_pow<ME>(sp, (ME & 1) ? af * rsqrt_fast(r2) : 0.f)
                                      : ((m & 1) ? rpow(sp, m / 2) * af * rsqrt_fast(r2)
@@ -425,8 +462,15 @@ __global__ void __launch_bounds__(kScPairBlock, 8) sc_density_pair(ForceArgs a, 
         r = add2(r, psi);
     };
     double R0 = 0.0, R1 = 0.0;
+    if (P > 1) {
+        split_quads<P>(lq, on ? nq : 0, part, pair);
+        R0 = split_sum<P>((double)r.x);
+        R1 = split_sum<P>((double)r.y);
+        if (!on || part != 0) return;
+        r = dup2(0.f);
+    }
     uint4 nxt = nq > 0 ? __ldcs(lq) : make_uint4(0u, 0u, 0u, 0u);
-    for (int c0 = 0; c0 < nq; c0 += kChunkQ) {
+    for (int c0 = 0; P == 1 && c0 < nq; c0 += kChunkQ) {
         const int c1 = min(c0 + kChunkQ, nq);
         for (int q = c0; q < c1; ++q) {
             const uint4 e4 = nxt;
@@ -473,16 +517,19 @@ __device__ __forceinline__ void sc_pair_atom_out(const ForceArgs &a, int i, doub
         vv_epilogue<MODE>(a, i, Fx, Fy, Fz, reinterpret_cast<const float *>(a.xq)[4 * (size_t)i + 3]);
 }
 
-template <int MODE, bool ENERGY, int NE, int ME>
-__global__ void __launch_bounds__(kScPairBlock, 7) sc_force_pair(ForceArgs a, PairArgs p,
+template <int MODE, bool ENERGY, int NE, int ME, int P>
+__global__ void __launch_bounds__(kScPairBlock, P > 1 ? 1 : 7) sc_force_pair(ForceArgs a, PairArgs p,
                                                                  int store_f) {
     __shared__ ShiftTab sh;
     load_shifts_f32(a.g, &sh);
     __syncthreads();
     if (a.ds->status != 0) return;
     step_bookkeeping<MODE>(a);
-    const int s = blockIdx.x * blockDim.x + threadIdx.x;
-    if (s >= p.slot_start[p.ncells]) return;
+    const int tid = blockIdx.x * blockDim.x + threadIdx.x;
+    const int nslots = p.slot_start[p.ncells];
+    if ((P > 1 ? (tid & ~31) / P : tid) >= nslots) return;  // P > 1: whole warps
+    const bool on = tid / P < nslots;
+    const int s = on ? tid / P : nslots - 1, part = tid % P;
     const uint32_t sa = p.slot_atom[s];
     const int i0 = (int)(sa & ~kSingle);
     const bool two = !(sa & kSingle);
@@ -500,7 +547,7 @@ __global__ void __launch_bounds__(kScPairBlock, 7) sc_force_pair(ForceArgs a, Pa
         // the slot's own pair once: e = x_1 - x_0, f_0 -= fs e, f_1 += fs e
         const float ex = q1.x - q0.x, ey = q1.y - q0.y, ez = q1.z - q0.z;
         const float r2 = ex * ex + ey * ey + ez * ez;
-        if (r2 < rc2) {
+        if (part == 0 && r2 < rc2) {
             const float r2i = rcp_fast(r2);
             const float sp = a2 * r2i;
             const float ar = odd ? af * rsqrt_fast(r2) : 0.f;
@@ -569,6 +616,23 @@ __global__ void __launch_bounds__(kScPairBlock, 7) sc_force_pair(ForceArgs a, Pa
             np1 += in1 ? 1u : 0u;
         }
     };
+    if constexpr (P > 1) {
+        SplitState st, st1;
+        load_slot_state<MODE, P>(a, i0, two, on, part, st, st1);
+        split_quads<P>(lq, on ? nq : 0, part, pair);
+        const double F0[3] = {split_sum<P>((double)fx.x), split_sum<P>((double)fy.x),
+                              split_sum<P>((double)fz.x)};
+        const double F1[3] = {split_sum<P>((double)fx.y), split_sum<P>((double)fy.y),
+                              split_sum<P>((double)fz.y)};
+        if (ENERGY) {
+            const double E0 = split_sum<P>((double)en.x), E1 = split_sum<P>((double)en.y);
+            if (on) count_pairs(a.ds, np0 + (two ? np1 : 0u));
+            if (on && part == 0) a.e_atom[i0] = 0.5 * E0 - a.fc.sc_ec * sqrt(a.rho[i0]);
+            if (on && two && part == 1) a.e_atom[i0 + 1] = 0.5 * E1 - a.fc.sc_ec * sqrt(a.rho[i0 + 1]);
+        }
+        split_slot_finish<MODE, false, P>(a, i0, two, on, part, F0, F1, st, st1, store_f);
+        return;
+    }
     double F0x = 0.0, F0y = 0.0, F0z = 0.0, F1x = 0.0, F1y = 0.0, F1z = 0.0, E0 = 0.0, E1 = 0.0;
     auto flush = [&]() {
         F0x += (double)fx.x; F0y += (double)fy.x; F0z += (double)fz.x;
@@ -605,13 +669,19 @@ cudaError_t launch_sc_density(md_system *h) {
     const int nb = nblocks(a.n);
     if (h->p.force_variant == MD_FORCE_PAIRED) {
         const PairArgs p = make_pair_args(h);
-        if (a.fc.sc_m == 6) sc_density_pair<6><<<pair_grid_blocks(h, kScPairBlock), kScPairBlock, 0, h->stream>>>(a, p);
-        else sc_density_pair<0><<<pair_grid_blocks(h, kScPairBlock), kScPairBlock, 0, h->stream>>>(a, p);
+        const int P = split8(h->n / 2, h->ps_cap, kScSplitSlots);
+        const bool six = a.fc.sc_m == 6;
+        auto k = P > 1 ? (six ? sc_density_pair<6, 8> : sc_density_pair<0, 8>)
+                       : (six ? sc_density_pair<6, 1> : sc_density_pair<0, 1>);
+        k<<<pair_grid_blocks(h, kScPairBlock, P), kScPairBlock, 0, h->stream>>>(a, p);
         return cudaGetLastError();
     }
     if (h->p.precision == MD_MIXED) {
-        if (a.fc.sc_m == 6) sc_density_mixed<6><<<nb, kBlock, 0, h->stream>>>(a);
-        else sc_density_mixed<0><<<nb, kBlock, 0, h->stream>>>(a);
+        const int P = split8(h->n, h->cap, kScSplitAtoms);
+        const bool six = a.fc.sc_m == 6;
+        auto k = P > 1 ? (six ? sc_density_mixed<6, 8> : sc_density_mixed<0, 8>)
+                       : (six ? sc_density_mixed<6, 1> : sc_density_mixed<0, 1>);
+        k<<<nblocks(h->n * P), kBlock, 0, h->stream>>>(a);
     } else {
         return launch_sc_fp64_any(a, true, FM_STORE, false, 0, h->stream);
     }
@@ -625,12 +695,14 @@ cudaError_t launch_sc_force(md_system *h, int mode, bool energy, bool store_f) {
     cudaStream_t s = h->stream;
     if (h->p.force_variant == MD_FORCE_PAIRED) {
         const PairArgs p = make_pair_args(h);
-        const int pb = pair_grid_blocks(h, kScPairBlock);
+        const int P = split8(h->n / 2, h->ps_cap, kScSplitSlots);
+        const int pb = pair_grid_blocks(h, kScPairBlock, P);
         const bool cu = (a.fc.sc_n == 9 && a.fc.sc_m == 6);
 #define MDG_SCP(M, E)                                                                   \
     do {                                                                                \
-        if (cu) sc_force_pair<M, E, 9, 6><<<pb, kScPairBlock, 0, s>>>(a, p, sf);        \
-        else sc_force_pair<M, E, 0, 0><<<pb, kScPairBlock, 0, s>>>(a, p, sf);           \
+        auto k = P > 1 ? (cu ? sc_force_pair<M, E, 9, 6, 8> : sc_force_pair<M, E, 0, 0, 8>)  \
+                       : (cu ? sc_force_pair<M, E, 9, 6, 1> : sc_force_pair<M, E, 0, 0, 1>); \
+        k<<<pb, kScPairBlock, 0, s>>>(a, p, sf);                                        \
     } while (0)
         switch (mode) {
             case FM_STORE: if (energy) MDG_SCP(FM_STORE, true); else MDG_SCP(FM_STORE, false); break;
@@ -641,11 +713,13 @@ cudaError_t launch_sc_force(md_system *h, int mode, bool energy, bool store_f) {
         return cudaGetLastError();
     }
     if (h->p.precision == MD_MIXED) {
+        const int P = split8(h->n, h->cap, kScSplitAtoms);
         const bool cu = (a.fc.sc_n == 9 && a.fc.sc_m == 6);
 #define MDG_SC(M, E)                                                                    \
     do {                                                                                \
-        if (cu) sc_force_mixed<M, E, 9, 6><<<nb, kBlock, 0, s>>>(a, sf);                \
-        else sc_force_mixed<M, E, 0, 0><<<nb, kBlock, 0, s>>>(a, sf);                   \
+        auto k = P > 1 ? (cu ? sc_force_mixed<M, E, 9, 6, 8> : sc_force_mixed<M, E, 0, 0, 8>)  \
+                       : (cu ? sc_force_mixed<M, E, 9, 6, 1> : sc_force_mixed<M, E, 0, 0, 1>); \
+        k<<<nblocks(h->n * P), kBlock, 0, s>>>(a, sf);                                  \
     } while (0)
         switch (mode) {
             case FM_STORE: if (energy) MDG_SC(FM_STORE, true); else MDG_SC(FM_STORE, false); break;

@@ -104,3 +104,38 @@ def test_two_species_cutoff_in_other_units(orc, unit):
     if unit == 1.0:
         pe1 = orc.lj_typed_list(pos, s.box, off, ids, p["types"], p["t_eps"], p["t_sigma"])[0]
         assert abs(pe - pe1) < 2e-5 * abs(pe1)
+
+
+@pytest.mark.parametrize("variant,nc", [("full", 7), ("full", 17), ("full", 18), ("paired", 7),
+                                        ("paired", 23), ("paired", 24)])
+def test_sutton_chen_sizes(orc, variant, nc):
+    """Eight lanes up to 20,480 atoms or 24,576 slots, one above."""
+    s = inputs.sc_fcc(nc=nc)
+    p = s.params
+    pos = jitter(s, 0.02, 470 + nc)
+    kw = dict(eps=p["eps"], sigma=p["sigma"], c=p["c"], n_exp=p["n_exp"], m_exp=p["m_exp"],
+              rc=p["rc"], skin=p["skin"], dt=p["dt"])
+    U, f0 = orc.forces_once(orc.make_params(potential=orc.POT_SC, **kw), pos, s.box)
+    off, ids = orc.neighbors_cells(pos, s.box, p["rc"] + p["skin"])
+    bad = near_cutoff(pos, s.box, off, ids, p["rc"], 1e-5)
+    fv = md.MD_FORCE_PAIRED if variant == "paired" else md.MD_FORCE_FULL
+    with md.System(pos, s.vel, s.box, potential="sc", precision="mixed", force_variant=fv, **kw) as a:
+        check(a.state()[2].cpu().numpy(), f0, bad)
+        ke, pe = a.energy()
+        assert abs(pe - U) < 2e-6 * abs(U) + 1e-3 * bad.sum()
+
+
+@pytest.mark.parametrize("variant,nc", [("full", 8), ("full", 18), ("full", 19), ("paired", 8),
+                                        ("paired", 24)])
+def test_embedded_atom_sizes(orc, variant, nc):
+    """Eight lanes up to 12,288 atoms or slots, one above."""
+    s = inputs.eam_bcc(nc=nc)
+    p = s.params
+    keys = ("phi_r", "phi_a", "psi_r", "psi_a", "F_sqrt", "F_quad")
+    pos = jitter(s, 0.04, 480 + nc)
+    off, ids = orc.neighbors_cells(pos, s.box, p["rc"] + p["skin"])
+    f0 = orc.eam_list(pos, s.box, off, ids, orc.make_eam(*[p[k] for k in keys]), p["rc"])[1]
+    fv = md.MD_FORCE_PAIRED if variant == "paired" else md.MD_FORCE_FULL
+    with md.System(pos, s.vel, s.box, precision="mixed", force_variant=fv, rc=p["rc"],
+                   skin=p["skin"], dt=p["dt"], eam={k: p[k] for k in keys}) as a:
+        check(a.state()[2].cpu().numpy(), f0, np.zeros(len(pos), bool))
