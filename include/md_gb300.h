@@ -234,10 +234,9 @@ md_status md_forces(md_system *h);
 /* Advances nsteps >= 0 velocity-Verlet steps (Sec. 3.3).  Lists are rebuilt
  * on the device when the half-skin rule (or rebuild_every) asks for it; a
  * neighbour-capacity overflow is repaired on the host (capacity grown,
- * list rebuilt) and the remaining steps continue.  On a non-default stream
- * the steps replay CUDA graphs captured on first use (several steps each, the
- * rebuild chain inside, gated by the device's rebuild flag); on the
- * default stream every kernel is launched on its own.  Synchronizes the
+ * list rebuilt) and the remaining steps continue.  The steps replay CUDA
+ * graphs captured on first use (several steps each, the rebuild chain inside,
+ * gated by the device's rebuild flag).  Synchronizes the
  * stream once at the end to read the device status word. */
 md_status md_step(md_system *h, int64_t nsteps);
 

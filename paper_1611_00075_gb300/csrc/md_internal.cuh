@@ -394,6 +394,7 @@ struct md_system {
     long long last_launches[2] = {0, 0};
     long long body_launches = 0;           // launches of a rebuild chain that runs
     bool graphs_ok = true;
+    cudaStream_t cap_stream = nullptr;     // captures the default stream's steps; never runs
 
     // per-launch timing (md_set_timing)
     bool timing = false;
