@@ -702,6 +702,20 @@ static md_status eam_table(const md_params *p, const md_eam *e, EamTab *t, std::
         t->qr[k] = (float)t->qrd[k];
         t->qa[k] = (float)t->qad[k];
     }
+    int ex = 0;
+    double top = 0.0;
+    for (int k = 0; k < kEamMaxKnots; ++k) top = std::max(top, std::max(t->prd[k], t->qrd[k]));
+    const double frac = std::frexp(top, &ex);  // top = frac 2^ex, frac in [1/2, 1)
+    if (frac == 0.5) --ex;                     // a power of two itself
+    t->s = std::ldexp(1.0f, -ex);
+    for (int k = 0; k < kEamMaxKnots; ++k) {
+        t->ps[k] = std::ldexp(t->pr[k], -ex);
+        t->p2[k] = std::ldexp(t->pa[k], 2 * ex);
+        t->p3[k] = std::ldexp(t->pa[k], 3 * ex);
+        t->qs[k] = std::ldexp(t->qr[k], -ex);
+        t->q2[k] = std::ldexp(t->qa[k], 2 * ex);
+        t->q3[k] = std::ldexp(t->qa[k], 3 * ex);
+    }
     t->A = e->F_sqrt;
     t->B = e->F_quad;
     return MD_OK;

@@ -248,6 +248,11 @@ struct EamTab {
     float pr[kEamMaxKnots], pa[kEamMaxKnots], qr[kEamMaxKnots], qa[kEamMaxKnots];
     double prd[kEamMaxKnots], pad[kEamMaxKnots], qrd[kEamMaxKnots], qad[kEamMaxKnots];
     double A, B;
+    // the float32 tables with lengths in units of 2^m >= every knot (s = 2^-m, all
+    // scalings exact): knots s r_k <= 1, coefficients a_k / s^2 and a_k / s^3
+    float s;
+    float ps[kEamMaxKnots], p2[kEamMaxKnots], p3[kEamMaxKnots];
+    float qs[kEamMaxKnots], q2[kEamMaxKnots], q3[kEamMaxKnots];
 };
 
 enum ForceMode {
