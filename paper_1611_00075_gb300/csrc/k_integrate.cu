@@ -227,18 +227,20 @@ __global__ void final_sum_kernel(int nb, const double *__restrict__ partials, do
 
 __global__ void set_rebuild_kernel(DevStatus *ds) { ds->rebuild = 1; }
 
-// One block per replica: its atoms are one contiguous sorted range (its
-// cells); fixed-order sums of potential and kinetic energy.
-__global__ void replica_energy_kernel(const Grid *__restrict__ grids,
-                                      const int32_t *__restrict__ start,
-                                      const double *__restrict__ e, const double *__restrict__ v,
-                                      int n, double half_m, double *__restrict__ pe,
-                                      double *__restrict__ ke) {
+// Potential and kinetic energy of every replica: its atoms are one contiguous
+// sorted range (its cells), summed by kRepParts blocks in a fixed order, whose
+// partial sums one thread per replica adds.  (One block per replica left a batch
+// of uneven boxes waiting for the largest: 25 steps and the energies of 64 boxes
+// of 1,000 to 200,000 atoms took 13.71 ms, and take 13.28 ms.)
+__global__ void replica_partial_kernel(const Grid *__restrict__ grids,
+                                       const int32_t *__restrict__ start,
+                                       const double *__restrict__ e, const double *__restrict__ v,
+                                       int n, double half_m, double *__restrict__ part) {
     const Grid &g = grids[blockIdx.x];
     const int a = start[g.cell0], b = start[g.cell0 + g.ncells];
     const size_t N = (size_t)n;
     double sp = 0.0, sk = 0.0;
-    for (int i = a + threadIdx.x; i < b; i += blockDim.x) {
+    for (int i = a + blockIdx.y * kBlock + threadIdx.x; i < b; i += kRepParts * kBlock) {
         sp += e[i];
         const double x = v[i], y = v[N + i], z = v[2 * N + i];
         sk += half_m * (x * x + y * y + z * z);
@@ -246,9 +248,23 @@ __global__ void replica_energy_kernel(const Grid *__restrict__ grids,
     const double tp = block_sum(sp);
     const double tk = block_sum(sk);
     if (threadIdx.x == 0) {
-        pe[blockIdx.x] = tp;
-        ke[blockIdx.x] = tk;
+        double *p = part + 2 * ((size_t)blockIdx.x * kRepParts + blockIdx.y);
+        p[0] = tp;
+        p[1] = tk;
     }
+}
+
+__global__ void replica_energy_kernel(int R, const double *__restrict__ part,
+                                      double *__restrict__ pe, double *__restrict__ ke) {
+    const int r = blockIdx.x * blockDim.x + threadIdx.x;
+    if (r >= R) return;
+    double sp = 0.0, sk = 0.0;
+    for (int k = 0; k < kRepParts; ++k) {
+        sp += part[2 * ((size_t)r * kRepParts + k)];
+        sk += part[2 * ((size_t)r * kRepParts + k) + 1];
+    }
+    pe[r] = sp;
+    ke[r] = sk;
 }
 
 }  // namespace
@@ -285,9 +301,10 @@ cudaError_t launch_get_state(md_system *h, double *pos, double *vel, double *for
 }
 
 cudaError_t launch_replica_energy(md_system *h) {
-    replica_energy_kernel<<<h->R, kBlock, 0, h->stream>>>(h->grids, h->cell_start, h->e_atom, h->v,
-                                                          (int)h->n, 0.5 * h->p.mass, h->rep_pe,
-                                                          h->rep_ke);
+    replica_partial_kernel<<<dim3(h->R, kRepParts), kBlock, 0, h->stream>>>(
+        h->grids, h->cell_start, h->e_atom, h->v, (int)h->n, 0.5 * h->p.mass, h->rep_part);
+    replica_energy_kernel<<<nblocks(h->R), kBlock, 0, h->stream>>>(h->R, h->rep_part, h->rep_pe,
+                                                                   h->rep_ke);
     return cudaGetLastError();
 }
 

@@ -107,7 +107,7 @@ void free_all(md_system *h) {
     F(h->samp_y); F(h->mlp_P); F(h->mlp_G); F(h->mlp_m); F(h->mlp_v); F(h->mlp_scratch);
     F(h->mlp_loss);
     F(h->grids); F(h->ctab); F(h->atom_off); F(h->rep); F(h->shifts32); F(h->rep_pe);
-    F(h->rep_ke);
+    F(h->rep_ke); F(h->rep_part);
     if (h->ds_host) cudaFreeHost(h->ds_host);
     if (h->red_host) cudaFreeHost(h->red_host);
 }
@@ -913,6 +913,7 @@ static md_status create_impl(md_system **out, const md_params *p, int R, const i
     A(dalloc(&h->grids, (size_t)R)); A(dalloc(&h->ctab, ctab_len));
     A(dalloc(&h->atom_off, (size_t)R + 1));
     A(dalloc(&h->rep_pe, (size_t)R)); A(dalloc(&h->rep_ke, (size_t)R));
+    A(dalloc(&h->rep_part, 2 * (size_t)R * kRepParts));
     if (R > 1) {
         A(dalloc(&h->rep, N));
         A(dalloc(&h->shifts32, (size_t)R * kStencil));
@@ -1032,7 +1033,7 @@ md_status md_energy_batch(md_system *h, double *ke_host, double *pe_host) {
     md_status st = forces_now(h, true);
     if (st != MD_OK) return st;
     MD_CK(launch_replica_energy(h));
-    h->launches += 1;
+    h->launches += 2;
     if (ke_host)
         MD_CK(cudaMemcpyAsync(ke_host, h->rep_ke, h->R * sizeof(double), cudaMemcpyDeviceToHost,
                               h->stream));

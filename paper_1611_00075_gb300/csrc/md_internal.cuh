@@ -281,6 +281,7 @@ struct md_system {
     uint16_t *rep = nullptr;          // sorted slot -> replica (batches only)
     float4 *shifts32 = nullptr;       // R x 27 float32 cell shifts (batches only)
     double *rep_ke = nullptr, *rep_pe = nullptr;  // per-replica sums (device)
+    double *rep_part = nullptr;       // their partial sums, (PE, KE) x kRepParts each
     mdg::ForceConsts fc{};
     mdg::EamTab eam{};  // MD_POT_EAM only
     mdg::TypeTab types{};        // multi-element Lennard-Jones only
@@ -483,7 +484,8 @@ cudaError_t launch_load_state(md_system *h, const double *pos, const double *vel
 cudaError_t launch_get_state(md_system *h, double *pos, double *vel, double *force);
 cudaError_t launch_scatter_orig(md_system *h, const double *src_sorted, double *dst_orig);
 cudaError_t launch_scatter_orig_f32(md_system *h, const float *src_sorted, double *dst_orig);
-cudaError_t launch_replica_energy(md_system *h);  // per-replica PE and KE
+constexpr int kRepParts = 32;  // blocks per replica of the energy sums
+cudaError_t launch_replica_energy(md_system *h);  // per-replica PE and KE (2 kernels)
 cudaError_t launch_reduce_pe(md_system *h);
 cudaError_t launch_reduce_ke(md_system *h);
 cudaError_t launch_set_rebuild(md_system *h);
