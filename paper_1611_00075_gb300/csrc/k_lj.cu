@@ -125,20 +125,6 @@ __device__ __forceinline__ void lj_mixed_atom(const ForceArgs &a, const ShiftTab
     if (MODE != FM_STORE) vv_epilogue<MODE>(a, i, Fx, Fy, Fz, qi.w);
 }
 
-// Stores and the velocity-Verlet epilogue of one atom of the float64 path.
-template <int MODE, bool ENERGY, bool SPECIES>
-__device__ __forceinline__ void f64_atom_out(const ForceArgs &a, int i, double fx, double fy,
-                                             double fz, double e, float qw, int store_f) {
-    const size_t n = (size_t)a.n;
-    if (MODE == FM_STORE || store_f) {
-        a.f[i] = fx;
-        a.f[n + i] = fy;
-        a.f[2 * n + i] = fz;
-    }
-    if (ENERGY) a.e_atom[i] = e;
-    if (MODE != FM_STORE) vv_epilogue<MODE, SPECIES>(a, i, fx, fy, fz, qw);
-}
-
 // The whole per-atom job of the plain float64 path for sorted atom i, shared by
 // P lanes (lane `part`); on: the atom exists (all lanes of a warp call this).
 // The force scalar 48 eps r^-2 s6 (s6 - 1/2) with u = (sigma/r)^2 is
@@ -149,10 +135,10 @@ __device__ __forceinline__ void lj_fp64_atom(const ForceArgs &a, const ShiftTab 
     double fx = 0.0, fy = 0.0, fz = 0.0, e = 0.0;
     unsigned npair = 0;
     float qw = 0.f;
+    load_home64<P>(a, i, part, h);
     if (on) {
         const float4 qi = a.xq[i];
         qw = qi.w;
-        load_home64(a, i, h);
         const double sig2 = a.fc.sig2, e48 = a.fc.eps48;
         const bool seeded = a.fc.f64_seeded;
         f64_pairs<P>(a, sh, h, i, part, qi, [&](int, double ex, double ey, double ez, double r2) {
@@ -169,14 +155,12 @@ __device__ __forceinline__ void lj_fp64_atom(const ForceArgs &a, const ShiftTab 
             }
         });
     }
-    if (P > 1) {
-        fx = lanes_sum<P>(fx);
-        fy = lanes_sum<P>(fy);
-        fz = lanes_sum<P>(fz);
-        if (ENERGY) e = lanes_sum<P>(e);
+    if (ENERGY) {
+        e = lanes_sum<P>(e);
+        if (on) count_pairs(a.ds, npair);
+        if (on && part == 0) a.e_atom[i] = 0.5 * e;
     }
-    if (ENERGY && on) count_pairs(a.ds, npair);
-    if (on && part == 0) f64_atom_out<MODE, ENERGY, false>(a, i, fx, fy, fz, 0.5 * e, qw, store_f);
+    f64_finish<MODE, false, P>(a, i, part, on, fx, fy, fz, qw, store_f);
 }
 
 // One thread per sorted atom; the hardware block scheduler spreads the work.
@@ -590,10 +574,10 @@ __device__ __forceinline__ void lj_typed_fp64_atom(const ForceArgs &a, const Typ
     double fx = 0.0, fy = 0.0, fz = 0.0, e = 0.0;
     unsigned npair = 0;
     float qw = 0.f;
+    load_home64<P>(a, i, part, h);
     if (on) {
         const float4 qi = a.xq[i];
         qw = qi.w;
-        load_home64(a, i, h);
         const int ti = species_of(__float_as_uint(qi.w));
         double e48[NT], e4[NT], s2[NT], shd[NT];
         load_row<NT>(tt.e48d, ti, e48);
@@ -616,14 +600,12 @@ __device__ __forceinline__ void lj_typed_fp64_atom(const ForceArgs &a, const Typ
             }
         });
     }
-    if (P > 1) {
-        fx = lanes_sum<P>(fx);
-        fy = lanes_sum<P>(fy);
-        fz = lanes_sum<P>(fz);
-        if (ENERGY) e = lanes_sum<P>(e);
+    if (ENERGY) {
+        e = lanes_sum<P>(e);
+        if (on) count_pairs(a.ds, npair);
+        if (on && part == 0) a.e_atom[i] = 0.5 * e;
     }
-    if (ENERGY && on) count_pairs(a.ds, npair);
-    if (on && part == 0) f64_atom_out<MODE, ENERGY, true>(a, i, fx, fy, fz, 0.5 * e, qw, store_f);
+    f64_finish<MODE, true, P>(a, i, part, on, fx, fy, fz, qw, store_f);
 }
 
 template <int MODE, bool ENERGY, int NT, int P>
@@ -700,6 +682,7 @@ cudaError_t launch_lj_typed_nt(md_system *h, const ForceArgs &a, int mode, bool 
     switch (f64_split(h->n)) {
         case 1: return launch_lj_typed_fp64<NT, 1>(h, a, mode, energy, sf);
         case 4: return launch_lj_typed_fp64<NT, 4>(h, a, mode, energy, sf);
+        case 8: return launch_lj_typed_fp64<NT, 8>(h, a, mode, energy, sf);
         default: return launch_lj_typed_fp64<NT, 16>(h, a, mode, energy, sf);
     }
 }
@@ -775,6 +758,7 @@ cudaError_t launch_lj(md_system *h, int mode, bool energy, bool store_f) {
         switch (f64_split(h->n)) {
             case 1: return launch_lj_fp64<1>(a, mode, energy, sf, s);
             case 4: return launch_lj_fp64<4>(a, mode, energy, sf, s);
+            case 8: return launch_lj_fp64<8>(a, mode, energy, sf, s);
             default: return launch_lj_fp64<16>(a, mode, energy, sf, s);
         }
     }

@@ -164,8 +164,8 @@ __global__ void __launch_bounds__(kF64Block) sc_density_fp64(ForceArgs a) {
     const bool on = t < (long long)a.n * P;
     const int i = on ? (int)(t / P) : 0, part = (int)(t % P);
     double R = 0.0;
+    load_home64<P>(a, i, part, &home);
     if (on) {
-        load_home64(a, i, &home);
         const double A = a.fc.sc_a, A2 = A * A;
         const int m = a.fc.sc_m;
         const bool seeded = a.fc.f64_seeded;
@@ -303,10 +303,10 @@ __global__ void __launch_bounds__(kF64Block) sc_force_fp64(ForceArgs a, int stor
     double fx = 0.0, fy = 0.0, fz = 0.0, e = 0.0;
     unsigned npair = 0;
     float qw = 0.f;
+    load_home64<P>(a, i, part, &home);
     if (on) {
         const float4 qi = a.xq[i];
         qw = qi.w;
-        load_home64(a, i, &home);
         const double dFi = a.dF64[i];
         const double A = a.fc.sc_a, A2 = A * A, eps = a.fc.sc_eps;
         const int nexp = a.fc.sc_n, mexp = a.fc.sc_m;
@@ -336,22 +336,12 @@ __global__ void __launch_bounds__(kF64Block) sc_force_fp64(ForceArgs a, int stor
                          }
                      });
     }
-    if (P > 1) {
-        fx = lanes_sum<P>(fx);
-        fy = lanes_sum<P>(fy);
-        fz = lanes_sum<P>(fz);
-        if (ENERGY) e = lanes_sum<P>(e);
+    if (ENERGY) {
+        e = lanes_sum<P>(e);
+        if (on) count_pairs(a.ds, npair);
+        if (on && part == 0) a.e_atom[i] = 0.5 * e - a.fc.sc_ec * sqrt(a.rho[i]);
     }
-    if (ENERGY && on) count_pairs(a.ds, npair);
-    if (!on || part != 0) return;
-    const size_t n = (size_t)a.n;
-    if (MODE == FM_STORE || store_f) {
-        a.f[i] = fx;
-        a.f[n + i] = fy;
-        a.f[2 * n + i] = fz;
-    }
-    if (ENERGY) a.e_atom[i] = 0.5 * e - a.fc.sc_ec * sqrt(a.rho[i]);
-    if (MODE != FM_STORE) vv_epilogue<MODE>(a, i, fx, fy, fz, qw);
+    f64_finish<MODE, false, P>(a, i, part, on, fx, fy, fz, qw, store_f);
 }
 
 template <int NE, int ME, int P>
@@ -385,6 +375,7 @@ cudaError_t launch_sc_fp64_any(const ForceArgs &a, bool density, int mode, bool 
     switch (f64_split(a.n)) {
         case 1: return MDG_SC64(1);
         case 4: return MDG_SC64(4);
+        case 8: return MDG_SC64(8);
         default: return MDG_SC64(16);
     }
 #undef MDG_SC64

@@ -1,5 +1,6 @@
 """The float64 passes on both sides of their lanes-per-atom limits (16 up to
-4,096 atoms, 4 up to 32,768, then one), with lists whose last quad is ragged,
+3,072 atoms, 8 up to 8,192, 4 up to 32,768, then one), with lists whose last
+quad is ragged,
 and in units whose squared lengths float32 cannot hold.
 
 Tolerance: a force is a sum of about 60 (Sutton-Chen: 150) terms of at most
@@ -33,7 +34,7 @@ def jitter(s, amp, seed):
     return np.mod(s.pos + amp * inputs.gaussian(seed, s.pos.size).reshape(-1, 3), s.box)
 
 
-@pytest.mark.parametrize("nc", [6, 10, 11, 20, 21])  # 864, 4000 | 5324, 32000 | 37044 atoms
+@pytest.mark.parametrize("nc", [6, 10, 11, 20, 21])  # 864 | 4000, 5324 | 32000 | 37044 atoms
 def test_lj(orc, nc):
     s = inputs.lj_fcc(nc=nc, T=0.5)
     pos = jitter(s, 0.06, 300 + nc)
