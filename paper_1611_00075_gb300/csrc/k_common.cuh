@@ -69,7 +69,7 @@ struct ForceArgs {
     float4 *__restrict__ xqf;     // many-body, mixed: (x, y, z, F'(rho)) per atom
     double *__restrict__ dF64;    // many-body: F'(rho_i) in float64
     const uint16_t *__restrict__ rep;     // batches: replica of each sorted atom
-    const float4 *__restrict__ shifts32;  // batches: R x 27 float32 cell shifts
+    const float4 *__restrict__ widths32;  // batches: float32 cell widths of each box
     DevStatus *ds;
     Grid g;
     ForceConsts fc;
@@ -79,6 +79,42 @@ struct ForceArgs {
 // memory, one array per component: the lanes of a warp read up to 27
 // distinct words of one array, which sit in 27 distinct banks, so each read
 // is a single wavefront (a float4 table costs several).
+// The stencil coordinates (-1, 0 or 1 per axis) of a list entry, whose top five
+// bits hold 9 (z + 1) + 3 (y + 1) + (x + 1).  One funnel shift makes the float
+// 2^23 + that number, and six additions and multiply-adds split it (every
+// quotient is rounded to an integer by adding and subtracting 1.5 x 2^23; all of
+// it is exact).  A pair kernel that reads the cell shift from a table in shared
+// memory spends three of its 16 L1 wavefronts per entry on it, and L1 wavefronts
+// are what these kernels are short of; the multiply-add that applies the shift
+// (exactly: +-w or 0) replaces the addition of the table's value.
+// Against the table, whole runs: 331 k atoms (per-atom lists) 5.28 -> 4.84 ms,
+// liquid of 1 M 6.59 -> 6.13, 64 boxes 13.28 -> 12.32, Sutton-Chen 32.8 -> 31.1,
+// EAM 14.28 -> 13.55, alloy 10.43 -> 10.06, porous 9.8 M 66.2 -> 64.0; same bits.
+// (The same split in shifts and masks was slower than the table: they run on the
+// half-rate pipe of the comparisons.)
+__device__ __forceinline__ float3 stencil_of(uint32_t ent) {
+    const float kRound = 12582912.f;
+    const float c = __uint_as_float(__funnelshift_l(ent, 0x02580000u, 5)) - 8388621.f;
+    const float z = fmaf(c, 1.f / 9.f, kRound) - kRound;
+    const float r = fmaf(z, -9.f, c);
+    const float y = fmaf(r, 1.f / 3.f, kRound) - kRound;
+    return make_float3(fmaf(y, -3.f, r), y, z);
+}
+static_assert(kIndexBits == 27, "stencil_of's shift");
+
+// |e|^2 in the rounding that every pass over the same pairs uses (the compiler
+// orders ex ex + ey ey + ez ez by what the operands come from): one pair must not
+// be inside r_c for one pass and outside for another.
+__device__ __forceinline__ float dist2(float ex, float ey, float ez) {
+    return fmaf(ez, ez, fmaf(ex, ex, ey * ey));
+}
+
+// The cell widths of replica r of a batch.
+__device__ __forceinline__ float3 replica_width(const ForceArgs &a, int r) {
+    const float4 w = a.widths32[r];
+    return make_float3(w.x, w.y, w.z);
+}
+
 struct ShiftTab {
     float x[32], y[32], z[32];
 };

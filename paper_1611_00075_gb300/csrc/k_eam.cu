@@ -91,9 +91,6 @@ constexpr int64_t kEamSplit = 12288;
 // Both mixed passes: 256-thread blocks at up to 64 registers.
 template <int NPSI, int P>
 __global__ void __launch_bounds__(kBlock, P > 1 ? 1 : 4) eam_density_mixed(ForceArgs a, EamTab t) {
-    __shared__ ShiftTab sh;
-    load_shifts_f32(a.g, &sh);
-    __syncthreads();
     if (a.ds->status != 0) return;
     const int tid = blockIdx.x * blockDim.x + threadIdx.x;
     const bool on = tid / P < a.n;
@@ -107,11 +104,11 @@ __global__ void __launch_bounds__(kBlock, P > 1 ? 1 : 4) eam_density_mixed(Force
     float r = 0.f;
     auto pair = [&](uint32_t ent) {
         const float4 qj = __ldg(a.xq + (ent & kIndexMask));
-        const uint32_t st = ent >> kIndexBits;
-        const float ex = (qj.x - qi.x) + sh.x[st];
-        const float ey = (qj.y - qi.y) + sh.y[st];
-        const float ez = (qj.z - qi.z) + sh.z[st];
-        const float r2 = ex * ex + ey * ey + ez * ez;
+        const float3 st = stencil_of(ent);
+        const float ex = fmaf(st.x, a.g.wf[0], qj.x - qi.x);
+        const float ey = fmaf(st.y, a.g.wf[1], qj.y - qi.y);
+        const float ez = fmaf(st.z, a.g.wf[2], qj.z - qi.z);
+        const float r2 = dist2(ex, ey, ez);
         if (r2 < rc2) r += pieces_f32<NPSI>(t.qs, t.q2, t.q3, t.npsi, t.s * r2, rsqrt_fast(r2), nullptr);
     };
     if (P > 1) {
@@ -175,9 +172,6 @@ __global__ void __launch_bounds__(kBlock) eam_density_fp64(ForceArgs a, EamTab t
 
 template <int MODE, bool ENERGY, int NPHI, int NPSI, int P>
 __global__ void __launch_bounds__(kBlock, P > 1 ? 1 : 4) eam_force_mixed(ForceArgs a, EamTab t, int store_f) {
-    __shared__ ShiftTab sh;
-    load_shifts_f32(a.g, &sh);
-    __syncthreads();
     if (a.ds->status != 0) return;
     step_bookkeeping<MODE>(a);
     const int tid = blockIdx.x * blockDim.x + threadIdx.x;
@@ -194,11 +188,11 @@ __global__ void __launch_bounds__(kBlock, P > 1 ? 1 : 4) eam_force_mixed(ForceAr
     float fx = 0.f, fy = 0.f, fz = 0.f, e = 0.f;
     auto pair = [&](uint32_t ent) {
         const float4 qj = __ldg(a.xqf + (ent & kIndexMask));  // position, F'(rho_j)
-        const uint32_t st = ent >> kIndexBits;
-        const float ex = (qj.x - qi.x) + sh.x[st];
-        const float ey = (qj.y - qi.y) + sh.y[st];
-        const float ez = (qj.z - qi.z) + sh.z[st];
-        const float r2 = ex * ex + ey * ey + ez * ez;
+        const float3 st = stencil_of(ent);
+        const float ex = fmaf(st.x, a.g.wf[0], qj.x - qi.x);
+        const float ey = fmaf(st.y, a.g.wf[1], qj.y - qi.y);
+        const float ez = fmaf(st.z, a.g.wf[2], qj.z - qi.z);
+        const float r2 = dist2(ex, ey, ez);
         if (r2 < rc2) {
             const float rinv = rsqrt_fast(r2);
             float dPhi, dpsi;
@@ -353,9 +347,6 @@ __device__ __forceinline__ float2 pieces_pair(const float *ks, const float *c2, 
 template <int NPSI, int P>
 __global__ void __launch_bounds__(kEamPairBlock, P > 1 ? 1 : 8) eam_density_pair(ForceArgs a, PairArgs p,
                                                                      EamTab t) {
-    __shared__ ShiftTab sh;
-    load_shifts_f32(a.g, &sh);
-    __syncthreads();
     if (a.ds->status != 0) return;
     const int tid = blockIdx.x * blockDim.x + threadIdx.x;
     const int nslots = p.slot_start[p.ncells];
@@ -381,8 +372,8 @@ __global__ void __launch_bounds__(kEamPairBlock, P > 1 ? 1 : 8) eam_density_pair
     const uint4 *lq = reinterpret_cast<const uint4 *>(p.list + list_group(s, p.cap)) + (s & 31);
     auto pair = [&](uint32_t ent) {
         const float4 qj = __ldg(a.xq + (ent & kIndexMask));
-        const uint32_t st = ent >> kIndexBits;
-        const float tx = qj.x + sh.x[st], ty = qj.y + sh.y[st], tz = qj.z + sh.z[st];
+        const float3 st = stencil_of(ent);
+        const float tx = fmaf(st.x, a.g.wf[0], qj.x), ty = fmaf(st.y, a.g.wf[1], qj.y), tz = fmaf(st.z, a.g.wf[2], qj.z);
         const float2 dx = add2(dup2(tx), nqx), dy = add2(dup2(ty), nqy), dz = add2(dup2(tz), nqz);
         const float2 r2 = fma2(dz, dz, fma2(dy, dy, mul2(dx, dx)));
         const float2 rinv = make_float2(rsqrt_fast(r2.x), rsqrt_fast(r2.y));
@@ -448,9 +439,6 @@ __device__ __forceinline__ void eam_pair_atom_out(const ForceArgs &a, const EamT
 template <int MODE, bool ENERGY, int NPHI, int NPSI, int P>
 __global__ void __launch_bounds__(kEamPairBlock, P > 1 ? 1 : 8) eam_force_pair(ForceArgs a, PairArgs p,
                                                                    EamTab t, int store_f) {
-    __shared__ ShiftTab sh;
-    load_shifts_f32(a.g, &sh);
-    __syncthreads();
     if (a.ds->status != 0) return;
     step_bookkeeping<MODE>(a);
     const int tid = blockIdx.x * blockDim.x + threadIdx.x;
@@ -493,8 +481,8 @@ __global__ void __launch_bounds__(kEamPairBlock, P > 1 ? 1 : 8) eam_force_pair(F
     // f_i += g (x_j - x_i) / r with g = Phi' + (F'_i + F'_j) psi'
     auto pair = [&](uint32_t ent) {
         const float4 qj = __ldg(a.xqf + (ent & kIndexMask));  // position, F'(rho_j)
-        const uint32_t st = ent >> kIndexBits;
-        const float tx = qj.x + sh.x[st], ty = qj.y + sh.y[st], tz = qj.z + sh.z[st];
+        const float3 st = stencil_of(ent);
+        const float tx = fmaf(st.x, a.g.wf[0], qj.x), ty = fmaf(st.y, a.g.wf[1], qj.y), tz = fmaf(st.z, a.g.wf[2], qj.z);
         const float2 dx = add2(dup2(tx), nqx), dy = add2(dup2(ty), nqy), dz = add2(dup2(tz), nqz);
         const float2 r2 = fma2(dz, dz, fma2(dy, dy, mul2(dx, dx)));
         const float2 rinv = make_float2(rsqrt_fast(r2.x), rsqrt_fast(r2.y));

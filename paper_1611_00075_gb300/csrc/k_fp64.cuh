@@ -177,8 +177,7 @@ __device__ __forceinline__ void f64_finish(const ForceArgs &a, int i, int part, 
 // of the lanes' largest shares.  Measured (LJ, force launch, us) with
 // 1 / 4 / 8 / 16 lanes: 864 atoms 85 / 30 / 21 / 16, 2,048 atoms
 // 90 / 31 / 21 / 20, 2,916 atoms 90 / 31 / 27 / 25, 4,000 atoms
-// 90 / 31 / 27 / 31, 6,912 atoms
-// 90 / 39 / 34 / 43, 10,976 atoms 92 / 49 / 51 / 63, 32,000 atoms
+// 90 / 31 / 27 / 31, 6,912 atoms 90 / 39 / 34 / 43, 10,976 atoms 92 / 49 / 51 / 63, 32,000 atoms
 // 108 / 103 / 125 / 156, 87,808 atoms 222 / 257 / 309 / 402 (one lane per atom
 // and the plain loop: 150 us up to 32,000 atoms, 437 us at 87,808; without the
 // early load of the next position and the epilogue by components 33 at 4,000

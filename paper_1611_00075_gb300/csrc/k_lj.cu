@@ -13,7 +13,7 @@
 // Precision:
 //   MIXED  the pair vector, r^2, 1/r^2, (s/r)^6 and the force scalar are
 //          float32, computed from cell-relative float32 coordinates plus the
-//          float32 cell shift of the entry's stencil cell; each chunk of
+//          float32 cell shift of the entry's stencil cell (stencil_of); each chunk of
 //          64 entries is summed in float32 and the chunk sums are added in
 //          float64 (the GPU form of the paper's blocked pair loop).  Entries
 //          arrive four at a time (one 16-byte load), so four gathers are in
@@ -35,14 +35,16 @@ namespace mdg {
 
 // The whole per-atom job of the mixed path for sorted atom i: pair loop over
 // its list, stores, and the velocity-Verlet epilogue.  MULTI (systems of
-// several boxes) reads the cell shifts of the atom's own box from a global
-// R x 27 table instead of the block's shared table.  P > 1: the P lanes of the
-// atom (this one is `part`; on: the atom exists) each walk every P-th quad and
-// add their sums.
-template <int MODE, bool ENERGY, bool MULTI = false, int P = 1>
-__device__ __forceinline__ void lj_mixed_atom(const ForceArgs &a, const ShiftTab *sh, int i,
-                                              int store_f, int part = 0, bool on = true) {
-    const float4 *shr = MULTI ? a.shifts32 + 27 * (int)a.rep[i] : nullptr;
+// several boxes) takes the cell widths of the atom's own box.  P > 1: the P
+// lanes of the atom (this one is `part`; on: the atom exists) each walk every P-th
+// quad and add their sums.  TABLE: the cell shifts come from sh (the same bits as
+// computed ones).
+template <int MODE, bool ENERGY, bool MULTI = false, int P = 1, bool TABLE = false>
+__device__ __forceinline__ void lj_mixed_atom(const ForceArgs &a, int i, int store_f,
+                                              int part = 0, bool on = true,
+                                              const ShiftTab *sh = nullptr) {
+    const float3 w = MULTI ? replica_width(a, (int)a.rep[i])
+                           : make_float3(a.g.wf[0], a.g.wf[1], a.g.wf[2]);
     const float4 qi = a.xq[i];
     const int nq = (min(a.ncount[i], a.cap) + 3) >> 2;
     const uint4 *lq = reinterpret_cast<const uint4 *>(a.nlist + list_group(i, a.cap)) + (i & 31);
@@ -52,12 +54,19 @@ __device__ __forceinline__ void lj_mixed_atom(const ForceArgs &a, const ShiftTab
     float fx = 0.f, fy = 0.f, fz = 0.f, e = 0.f;
     auto pair = [&](uint32_t ent) {
         const float4 qj = __ldg(a.xq + (ent & kIndexMask));
-        const uint32_t st = ent >> kIndexBits;
-        const float4 sf = MULTI ? __ldg(shr + st) : make_float4(sh->x[st], sh->y[st], sh->z[st], 0.f);
-        const float ex = (qj.x - qi.x) + sf.x;
-        const float ey = (qj.y - qi.y) + sf.y;
-        const float ez = (qj.z - qi.z) + sf.z;
-        const float r2 = ex * ex + ey * ey + ez * ez;
+        float ex, ey, ez;
+        if (TABLE) {
+            const uint32_t st = ent >> kIndexBits;
+            ex = (qj.x - qi.x) + sh->x[st];
+            ey = (qj.y - qi.y) + sh->y[st];
+            ez = (qj.z - qi.z) + sh->z[st];
+        } else {
+            const float3 st = stencil_of(ent);
+            ex = fmaf(st.x, w.x, qj.x - qi.x);
+            ey = fmaf(st.y, w.y, qj.y - qi.y);
+            ez = fmaf(st.z, w.z, qj.z - qi.z);
+        }
+        const float r2 = dist2(ex, ey, ez);
         if (r2 < rc2) {
             const float r2i = rcp_fast(r2);
             float s6 = sig2 * r2i;
@@ -164,10 +173,6 @@ __device__ __forceinline__ void lj_fp64_atom(const ForceArgs &a, const ShiftTab 
 }
 
 // One thread per sorted atom; the hardware block scheduler spreads the work.
-// MULTI: a block's atoms are consecutive, so they belong to one or two boxes
-// (more only when a box holds fewer atoms than a block); the shift tables of
-// those boxes go to shared memory like a single box's, and a block that
-// spans more boxes reads the global R x 27 table.
 // Block shape of the grid kernel, measured on GB300: 128 threads for one
 // box and 256 for batches, each at up to 56 registers (4-9 % faster than
 // 256 threads at 48 registers).
@@ -179,46 +184,15 @@ constexpr int grid_block() { return MULTI ? 256 : 128; }
 template <int MODE, bool ENERGY, bool MULTI = false, int P = 1>
 __global__ void __launch_bounds__(P > 1 ? 128 : grid_block<MULTI>(), P > 1 ? 1 : (MULTI ? 4 : 5))
 lj_mixed_kernel(ForceArgs a, int store_f) {
-    __shared__ ShiftTab sh[MULTI ? 2 : 1];
-    __shared__ int s_r0, s_span;
-    if (!MULTI) {
-        load_shifts_f32(a.g, &sh[0]);
-    } else {
-        const int i0 = blockIdx.x * (blockDim.x / P);
-        const int r0 = a.rep[i0], r1 = a.rep[min(a.n, i0 + (int)blockDim.x / P) - 1];
-        if (threadIdx.x < 2 * kStencil) {
-            const int t = threadIdx.x / kStencil, st = threadIdx.x % kStencil;
-            if (t <= r1 - r0) {
-                const float4 v = a.shifts32[kStencil * (r0 + t) + st];
-                sh[t].x[st] = v.x;
-                sh[t].y[st] = v.y;
-                sh[t].z[st] = v.z;
-            }
-        }
-        if (threadIdx.x == 0) {
-            s_r0 = r0;
-            s_span = r1 - r0;
-        }
-    }
-    __syncthreads();
     if (a.ds->status != 0) return;
     step_bookkeeping<MODE>(a);
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
     if constexpr (P > 1) {
-        const int t = blockIdx.x * blockDim.x + threadIdx.x;
         const bool on = t / P < a.n;
-        const int i = on ? t / P : a.n - 1;
-        if (MULTI && s_span <= 1)
-            lj_mixed_atom<MODE, ENERGY, false, P>(a, &sh[(int)a.rep[i] - s_r0], i, store_f, t % P, on);
-        else
-            lj_mixed_atom<MODE, ENERGY, MULTI, P>(a, &sh[0], i, store_f, t % P, on);
-        return;
+        lj_mixed_atom<MODE, ENERGY, MULTI, P>(a, on ? t / P : a.n - 1, store_f, t % P, on);
+    } else if (t < a.n) {
+        lj_mixed_atom<MODE, ENERGY, MULTI>(a, t, store_f);
     }
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= a.n) return;
-    if (MULTI && s_span <= 1)
-        lj_mixed_atom<MODE, ENERGY, false>(a, &sh[(int)a.rep[i] - s_r0], i, store_f);
-    else
-        lj_mixed_atom<MODE, ENERGY, MULTI>(a, &sh[0], i, store_f);
 }
 
 // Persistent variant: gridDim.x CTAs stay resident; each warp processes tiles
@@ -258,8 +232,7 @@ __device__ __forceinline__ void prefetch_l2(const void *p) {
 // porous system.
 constexpr int kPersistBlock = kPersistThreads;
 static_assert(kPersistBlock == kF64Block, "the float64 job's shared columns");
-// The slot job holds twice the accumulators: its persistent kernel gets up to
-// 64 registers (8 CTAs per SM) instead of spilling at 56.
+// The slot job fits 56 registers too.
 constexpr int kPersistPairedCtas = 9;
 
 template <int MODE, bool ENERGY, bool DYNAMIC, bool TIMING, bool MULTI = false, bool F64 = false,
@@ -269,11 +242,16 @@ lj_mixed_persist(ForceArgs a, int store_f, SchedArgs sa, PairArgs pa) {
 
     static_assert(!(F64 && MULTI), "batches run the mixed path");
     static_assert(!(PAIRED && (F64 || MULTI || ENERGY)), "slots: one box, mixed path, forces");
-    __shared__ ShiftTab sh;
+    // Per-atom tiles of one box read the cell shifts from a table here: computed
+    // ones made the tiles' timings, which train the cost model, noisier (held-out
+    // spread of 64 parts 0.0215-0.0225 against 0.0224-0.0269) and the launch no
+    // shorter.
+    constexpr bool kTable = F64 || !(MULTI || PAIRED);
+    __shared__ typename std::conditional<kTable, ShiftTab, int>::type sh;
     __shared__ typename std::conditional<F64, Home64, int>::type home;
     __shared__ int s_first[kSchedRounds], s_pre[kSchedRounds + 1], s_next;  // this CTA's ranges
     __shared__ int s_stop;
-    if (!MULTI) load_shifts_f32(a.g, &sh);
+    if constexpr (kTable) load_shifts_f32(a.g, &sh);
     // one read of the status word for the whole CTA: every thread must take the
     // same branch, since the CTA meets barriers below
     if (threadIdx.x == 0) s_stop = a.ds->status;
@@ -390,8 +368,9 @@ lj_mixed_persist(ForceArgs a, int store_f, SchedArgs sa, PairArgs pa) {
         if constexpr (F64) {
             lj_fp64_atom<MODE, ENERGY, 1>(a, &sh, &home, active ? i : 0, 0, active, store_f);
         } else if (active) {
-            if (PAIRED) lj_pair_slot<MODE, false>(a, pa, &sh, i, store_f);
-            else lj_mixed_atom<MODE, ENERGY, MULTI>(a, &sh, i, store_f);
+            if constexpr (PAIRED) lj_pair_slot<MODE, false>(a, pa, i, store_f);
+            else if constexpr (MULTI) lj_mixed_atom<MODE, ENERGY, true>(a, i, store_f);
+            else lj_mixed_atom<MODE, ENERGY, false, 1, true>(a, i, store_f, 0, true, &sh);
         }
         if (TIMING) {
             __syncwarp();
@@ -481,8 +460,7 @@ __device__ __forceinline__ void load_row(const T *tab, int ti, T *row) {
 
 template <int MODE, bool ENERGY, int NT, int P>
 __device__ __forceinline__ void lj_typed_mixed_atom(const ForceArgs &a, const TypeTab &tt,
-                                                    const ShiftTab *sh, int i, int store_f,
-                                                    int part, bool on) {
+                                                    int i, int store_f, int part, bool on) {
     const float4 qi = a.xq[i];
     const int ti = species_of(__float_as_uint(qi.w));
     float e48[NT], e4[NT], s2[NT], shf[NT];
@@ -498,11 +476,11 @@ __device__ __forceinline__ void lj_typed_mixed_atom(const ForceArgs &a, const Ty
     float fx = 0.f, fy = 0.f, fz = 0.f, e = 0.f;
     auto pair = [&](uint32_t ent) {
         const float4 qj = __ldg(a.xq + (ent & kIndexMask));
-        const uint32_t st = ent >> kIndexBits;
-        const float ex = (qj.x - qi.x) + sh->x[st];
-        const float ey = (qj.y - qi.y) + sh->y[st];
-        const float ez = (qj.z - qi.z) + sh->z[st];
-        const float r2 = ex * ex + ey * ey + ez * ez;
+        const float3 st = stencil_of(ent);
+        const float ex = fmaf(st.x, a.g.wf[0], qj.x - qi.x);
+        const float ey = fmaf(st.y, a.g.wf[1], qj.y - qi.y);
+        const float ez = fmaf(st.z, a.g.wf[2], qj.z - qi.z);
+        const float r2 = dist2(ex, ey, ez);
         if (r2 < rc2) {
             const int tj = species_of(__float_as_uint(qj.w));
             const float r2i = rcp_fast(r2);
@@ -625,15 +603,12 @@ __global__ void __launch_bounds__(kF64Block) lj_typed_fp64_kernel(ForceArgs a, T
 
 template <int MODE, bool ENERGY, int NT, int P>
 __global__ void __launch_bounds__(128) lj_typed_kernel(ForceArgs a, TypeTab tt, int store_f) {
-    __shared__ ShiftTab sh;
-    load_shifts_f32(a.g, &sh);
-    __syncthreads();
     if (a.ds->status != 0) return;
     step_bookkeeping<MODE>(a);
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     const bool on = t / P < a.n;
     if (P == 1 && !on) return;
-    lj_typed_mixed_atom<MODE, ENERGY, NT, P>(a, tt, &sh, on ? t / P : a.n - 1, store_f, t % P, on);
+    lj_typed_mixed_atom<MODE, ENERGY, NT, P>(a, tt, on ? t / P : a.n - 1, store_f, t % P, on);
 }
 
 template <int NT, int P>
@@ -718,7 +693,7 @@ ForceArgs make_force_args(md_system *h) {
     a.xqf = h->xqf;
     a.dF64 = h->dF64;
     a.rep = h->rep;
-    a.shifts32 = h->shifts32;
+    a.widths32 = h->widths32;
     a.ds = h->ds;
     a.g = h->g;
     a.fc = h->fc;

@@ -27,7 +27,7 @@
 // force is summed in float32 over the whole list (about 55 entries per atom
 // at rho* = 0.8442, so one chunk of the per-atom kernel's float32-then-
 // float64 sums) and converted once: without the float64 accumulators the
-// kernel fits 9 CTAs of 128 threads per SM.
+// kernel fits 8 CTAs of 128 threads per SM.
 #include <algorithm>
 #include <type_traits>
 
@@ -311,71 +311,32 @@ __global__ void pair_dummy_kernel(float4 *xq0, float4 *xq1, float4 *xqf, int n) 
     if (xqf) xqf[n] = far;
 }
 
-// Measured on GB300 (porous LJ, 9.8 M atoms, one force launch): this form
-// (packed pairs, float32 sums, 56 registers, 9 CTAs per SM) 1.232 ms against
-// 1.304 ms for the per-atom kernel from the generated state, 1.342 against
-// 1.440 ms on the equilibrated one; the same arithmetic unpacked 1.387 ms
-// (issue-bound: the second atom's pair terms cost as many instructions as
-// the first's); with float64 chunk accumulators at 72 registers (7 CTAs)
-// 1.498 ms unpacked and 1.551 ms packed (latency-bound).  At 1 M atoms the
-// two layouts tie (porous) or the per-atom kernel leads by 2 % (liquid).
-//
-// MULTI (a batch of boxes): a block's slots are consecutive, so their atoms
-// belong to one or two boxes (more only when a box holds fewer slots than a
-// block); the shift tables of those boxes go to shared memory like a single
-// box's, and a block that spans more boxes reads the global R x 27 table.
+// Measured on GB300 (porous LJ, 9.8 M atoms, one force launch), with the cell
+// shifts still read from a table: packed pairs and float32 sums at 56 registers
+// 1.232 ms against 1.304 ms for the per-atom kernel from the generated state; the
+// same arithmetic unpacked 1.387 ms (issue-bound: the second atom's pair terms
+// cost as many instructions as the first's); with float64 chunk accumulators at
+// 72 registers (7 CTAs) 1.498 ms unpacked and 1.551 ms packed (latency-bound).
+// With the shifts computed (stencil_of), 9 / 8 / 7 CTAs per SM, whole runs: liquid
+// of 1 M atoms 6.49 / 6.17 / 6.30 ms, 64 boxes 13.93 / 12.40 / 13.28 (at 9 the
+// compiler spreads each quad's loads out to fit 56 registers).  The persistent
+// kernel, whose next tile is prefetched, keeps 9 (porous 9.8 M 64.6 / 65.0 / 66.6).
+// MULTI: a batch of boxes.
 //
 // P > 1: thread t serves slot t / P.
 template <int MODE, bool ENERGY, bool MULTI = false, int P = 1>
-__global__ void __launch_bounds__(kPairBlock, P > 1 ? 1 : 9)
+__global__ void __launch_bounds__(kPairBlock, P > 1 ? 1 : 8)
 lj_pair_kernel(ForceArgs a, PairArgs p, int store_f) {
-    __shared__ ShiftTab sh[MULTI ? 2 : 1];
-    __shared__ int s_r0, s_span;
-    const int nslots = p.slot_start[p.ncells];
-    if (!MULTI) {
-        load_shifts_f32(a.g, &sh[0]);
-    } else {
-        const int sb = blockIdx.x * (blockDim.x / P);
-        const int se = min(nslots, sb + (int)blockDim.x / P) - 1;
-        const int r0 = sb <= se ? (int)a.rep[p.slot_atom[sb] & ~kSingle] : 0;
-        const int r1 = sb <= se ? (int)a.rep[p.slot_atom[se] & ~kSingle] : 0;
-        if (threadIdx.x < 2 * kStencil) {
-            const int t = threadIdx.x / kStencil, st = threadIdx.x % kStencil;
-            if (t <= r1 - r0) {
-                const float4 v = a.shifts32[kStencil * (r0 + t) + st];
-                sh[t].x[st] = v.x;
-                sh[t].y[st] = v.y;
-                sh[t].z[st] = v.z;
-            }
-        }
-        if (threadIdx.x == 0) {
-            s_r0 = r0;
-            s_span = r1 - r0;
-        }
-    }
-    __syncthreads();
     if (a.ds->status != 0) return;
     step_bookkeeping<MODE>(a);
+    const int nslots = p.slot_start[p.ncells];
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
     if constexpr (P > 1) {
-        const int t = blockIdx.x * blockDim.x + threadIdx.x;
         if ((t & ~31) / P >= nslots) return;  // whole warps: the lanes add their sums
         const bool on = t / P < nslots;
-        const int s = on ? t / P : nslots - 1;
-        if (MULTI && s_span <= 1) {
-            const int r = (int)a.rep[p.slot_atom[s] & ~kSingle];
-            lj_pair_slot<MODE, ENERGY, false, P>(a, p, &sh[r - s_r0], s, store_f, t % P, on);
-        } else {
-            lj_pair_slot<MODE, ENERGY, MULTI, P>(a, p, &sh[0], s, store_f, t % P, on);
-        }
-        return;
-    }
-    const int s = blockIdx.x * blockDim.x + threadIdx.x;
-    if (s >= nslots) return;
-    if (MULTI && s_span <= 1) {
-        const int r = (int)a.rep[p.slot_atom[s] & ~kSingle];
-        lj_pair_slot<MODE, ENERGY, false>(a, p, &sh[r - s_r0], s, store_f);
-    } else {
-        lj_pair_slot<MODE, ENERGY, MULTI>(a, p, &sh[0], s, store_f);
+        lj_pair_slot<MODE, ENERGY, MULTI, P>(a, p, on ? t / P : nslots - 1, store_f, t % P, on);
+    } else if (t < nslots) {
+        lj_pair_slot<MODE, ENERGY, MULTI>(a, p, t, store_f);
     }
 }
 

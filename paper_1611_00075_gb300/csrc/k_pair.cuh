@@ -131,16 +131,16 @@ __device__ __forceinline__ void split_slot_out(const ForceArgs &a, int i0, bool 
 }
 
 // MULTI (a batch of boxes, the block's boxes not all in shared memory): the
-// stencil shifts come from the slot's box's row of the global R x 27 table.
+// cell widths are those of the slot's box.
 // P > 1: the P lanes of the slot (this one is `part`; on: the slot exists) each
 // walk every P-th quad of its list; lane 0 adds the slot's own pair.
 template <int MODE, bool ENERGY, bool MULTI = false, int P = 1>
-__device__ __forceinline__ void lj_pair_slot(const ForceArgs &a, const PairArgs &p,
-                                             const ShiftTab *sh, int s, int store_f, int part = 0,
-                                             bool on = true) {
+__device__ __forceinline__ void lj_pair_slot(const ForceArgs &a, const PairArgs &p, int s,
+                                             int store_f, int part = 0, bool on = true) {
     const uint32_t sa = p.slot_atom[s];
     const int i0 = (int)(sa & ~kSingle);
-    const float4 *shr = MULTI ? a.shifts32 + kStencil * (int)a.rep[i0] : nullptr;
+    const float3 w = MULTI ? replica_width(a, (int)a.rep[i0])
+                           : make_float3(a.g.wf[0], a.g.wf[1], a.g.wf[2]);
     const bool two = !(sa & kSingle);
     const float4 q0 = a.xq[i0];
     // a one-atom slot puts its second atom at the dummy's distance
@@ -174,9 +174,8 @@ __device__ __forceinline__ void lj_pair_slot(const ForceArgs &a, const PairArgs 
     // packed instructions; -fs = r2i s6 (e48 / 2 - e48 s6) is added with one fma
     auto pair = [&](uint32_t ent) {
         const float4 qj = __ldg(a.xq + (ent & kIndexMask));
-        const uint32_t st = ent >> kIndexBits;
-        const float4 sf = MULTI ? __ldg(shr + st) : make_float4(sh->x[st], sh->y[st], sh->z[st], 0.f);
-        const float tx = qj.x + sf.x, ty = qj.y + sf.y, tz = qj.z + sf.z;
+        const float3 st = stencil_of(ent);
+        const float tx = fmaf(st.x, w.x, qj.x), ty = fmaf(st.y, w.y, qj.y), tz = fmaf(st.z, w.z, qj.z);
         const float2 dx = add2(dup2(tx), nqx), dy = add2(dup2(ty), nqy), dz = add2(dup2(tz), nqz);
         const float2 r2 = fma2(dz, dz, fma2(dy, dy, mul2(dx, dx)));
         const float2 r2i = make_float2(rcp_fast(r2.x), rcp_fast(r2.y));

@@ -83,9 +83,6 @@ __device__ __forceinline__ double sc_embed_deriv_f64(double rho, double ec) {
 // measured 2 % faster than at 48.
 template <int ME, int P>
 __global__ void __launch_bounds__(kBlock, P > 1 ? 1 : 4) sc_density_mixed(ForceArgs a) {
-    __shared__ ShiftTab sh;
-    load_shifts_f32(a.g, &sh);
-    __syncthreads();
     if (a.ds->status != 0) return;
     const int tid = blockIdx.x * blockDim.x + threadIdx.x;
     const bool on = tid / P < a.n;
@@ -100,11 +97,11 @@ __global__ void __launch_bounds__(kBlock, P > 1 ? 1 : 4) sc_density_mixed(ForceA
     float r = 0.f;
     auto pair = [&](uint32_t ent) {
         const float4 qj = __ldg(a.xq + (ent & kIndexMask));
-        const uint32_t st = ent >> kIndexBits;
-        const float ex = (qj.x - qi.x) + sh.x[st];
-        const float ey = (qj.y - qi.y) + sh.y[st];
-        const float ez = (qj.z - qi.z) + sh.z[st];
-        const float r2 = ex * ex + ey * ey + ez * ez;
+        const float3 st = stencil_of(ent);
+        const float ex = fmaf(st.x, a.g.wf[0], qj.x - qi.x);
+        const float ey = fmaf(st.y, a.g.wf[1], qj.y - qi.y);
+        const float ez = fmaf(st.z, a.g.wf[2], qj.z - qi.z);
+        const float r2 = dist2(ex, ey, ez);
         if (r2 < rc2) {
             const float s = a2 * rcp_fast(r2);
             float psi;
@@ -189,9 +186,6 @@ __global__ void __launch_bounds__(kF64Block) sc_density_fp64(ForceArgs a) {
 
 template <int MODE, bool ENERGY, int NE, int ME, int P>
 __global__ void __launch_bounds__(kBlock, P > 1 ? 1 : 4) sc_force_mixed(ForceArgs a, int store_f) {
-    __shared__ ShiftTab sh;
-    load_shifts_f32(a.g, &sh);
-    __syncthreads();
     if (a.ds->status != 0) return;
     step_bookkeeping<MODE>(a);
     const int tid = blockIdx.x * blockDim.x + threadIdx.x;
@@ -211,11 +205,11 @@ __global__ void __launch_bounds__(kBlock, P > 1 ? 1 : 4) sc_force_mixed(ForceArg
     float fx = 0.f, fy = 0.f, fz = 0.f, e = 0.f;
     auto pair = [&](uint32_t ent) {
         const float4 qj = __ldg(a.xqf + (ent & kIndexMask));  // position, F'(rho_j)
-        const uint32_t st = ent >> kIndexBits;
-        const float ex = (qj.x - qi.x) + sh.x[st];
-        const float ey = (qj.y - qi.y) + sh.y[st];
-        const float ez = (qj.z - qi.z) + sh.z[st];
-        const float r2 = ex * ex + ey * ey + ez * ez;
+        const float3 st = stencil_of(ent);
+        const float ex = fmaf(st.x, a.g.wf[0], qj.x - qi.x);
+        const float ey = fmaf(st.y, a.g.wf[1], qj.y - qi.y);
+        const float ez = fmaf(st.z, a.g.wf[2], qj.z - qi.z);
+        const float r2 = dist2(ex, ey, ez);
         if (r2 < rc2) {
             // with an odd exponent a/r comes from one reciprocal square
             // root, and (a/r)^2 and 1/r^2 from it without a reciprocal
@@ -401,9 +395,6 @@ __device__ __forceinline__ float2 ar_pow_rt(float2 s, float2 ar, int k) {
 
 template <int ME, int P>
 __global__ void __launch_bounds__(kScPairBlock, P > 1 ? 1 : 8) sc_density_pair(ForceArgs a, PairArgs p) {
-    __shared__ ShiftTab sh;
-    load_shifts_f32(a.g, &sh);
-    __syncthreads();
     if (a.ds->status != 0) return;
     const int tid = blockIdx.x * blockDim.x + threadIdx.x;
     const int nslots = p.slot_start[p.ncells];
@@ -436,8 +427,8 @@ __global__ void __launch_bounds__(kScPairBlock, P > 1 ? 1 : 8) sc_density_pair(F
     const uint4 *lq = reinterpret_cast<const uint4 *>(p.list + list_group(s, p.cap)) + (s & 31);
     auto pair = [&](uint32_t ent) {
         const float4 qj = __ldg(a.xq + (ent & kIndexMask));
-        const uint32_t st = ent >> kIndexBits;
-        const float tx = qj.x + sh.x[st], ty = qj.y + sh.y[st], tz = qj.z + sh.z[st];
+        const float3 st = stencil_of(ent);
+        const float tx = fmaf(st.x, a.g.wf[0], qj.x), ty = fmaf(st.y, a.g.wf[1], qj.y), tz = fmaf(st.z, a.g.wf[2], qj.z);
         const float2 dx = add2(dup2(tx), nqx), dy = add2(dup2(ty), nqy), dz = add2(dup2(tz), nqz);
         const float2 r2 = fma2(dz, dz, fma2(dy, dy, mul2(dx, dx)));
         const float2 sp = mul2(dup2(a2), make_float2(rcp_fast(r2.x), rcp_fast(r2.y)));
@@ -511,9 +502,6 @@ __device__ __forceinline__ void sc_pair_atom_out(const ForceArgs &a, int i, doub
 template <int MODE, bool ENERGY, int NE, int ME, int P>
 __global__ void __launch_bounds__(kScPairBlock, P > 1 ? 1 : 7) sc_force_pair(ForceArgs a, PairArgs p,
                                                                  int store_f) {
-    __shared__ ShiftTab sh;
-    load_shifts_f32(a.g, &sh);
-    __syncthreads();
     if (a.ds->status != 0) return;
     step_bookkeeping<MODE>(a);
     const int tid = blockIdx.x * blockDim.x + threadIdx.x;
@@ -567,8 +555,8 @@ __global__ void __launch_bounds__(kScPairBlock, P > 1 ? 1 : 7) sc_force_pair(For
     // d = x_j - x_i per atom; f_i -= fs d with fs = (n Phi + m (F'_i + F'_j) psi) / r^2
     auto pair = [&](uint32_t ent) {
         const float4 qj = __ldg(a.xqf + (ent & kIndexMask));  // position, F'(rho_j)
-        const uint32_t st = ent >> kIndexBits;
-        const float tx = qj.x + sh.x[st], ty = qj.y + sh.y[st], tz = qj.z + sh.z[st];
+        const float3 st = stencil_of(ent);
+        const float tx = fmaf(st.x, a.g.wf[0], qj.x), ty = fmaf(st.y, a.g.wf[1], qj.y), tz = fmaf(st.z, a.g.wf[2], qj.z);
         const float2 dx = add2(dup2(tx), nqx), dy = add2(dup2(ty), nqy), dz = add2(dup2(tz), nqz);
         const float2 r2 = fma2(dz, dz, fma2(dy, dy, mul2(dx, dx)));
         // with an odd exponent a/r comes from one reciprocal square root,

@@ -106,7 +106,7 @@ void free_all(md_system *h) {
     F(h->cell_cycles); F(h->cta_cycles); F(h->samp_flag); F(h->samp_bsum); F(h->samp_X);
     F(h->samp_y); F(h->mlp_P); F(h->mlp_G); F(h->mlp_m); F(h->mlp_v); F(h->mlp_scratch);
     F(h->mlp_loss);
-    F(h->grids); F(h->ctab); F(h->atom_off); F(h->rep); F(h->shifts32); F(h->rep_pe);
+    F(h->grids); F(h->ctab); F(h->atom_off); F(h->rep); F(h->widths32); F(h->rep_pe);
     F(h->rep_ke); F(h->rep_part);
     if (h->ds_host) cudaFreeHost(h->ds_host);
     if (h->red_host) cudaFreeHost(h->red_host);
@@ -916,7 +916,7 @@ static md_status create_impl(md_system **out, const md_params *p, int R, const i
     A(dalloc(&h->rep_part, 2 * (size_t)R * kRepParts));
     if (R > 1) {
         A(dalloc(&h->rep, N));
-        A(dalloc(&h->shifts32, (size_t)R * kStencil));
+        A(dalloc(&h->widths32, (size_t)R));
     }
     if (p->potential == MD_POT_SC || p->potential == MD_POT_EAM) {
         A(dalloc(&h->rho, N)); A(dalloc(&h->dF32, N)); A(dalloc(&h->dF64, N));
@@ -947,17 +947,11 @@ static md_status create_impl(md_system **out, const md_params *p, int R, const i
         if (st == MD_OK && r != cudaSuccess)
             st = fail(h, MD_ERR_CUDA, std::string(what) + ": " + cudaGetErrorString(r));
     };
-    std::vector<float4> sh;
+    std::vector<float4> widths;
     if (R > 1) {
-        for (int r = 0; r < R; ++r)
-            for (int s = 0; s < kStencil; ++s) {
-                const Grid &g = h->grids_h[r];
-                const int dx = s % 3 - 1, dy = (s / 3) % 3 - 1, dz = s / 9 - 1;
-                sh.push_back(make_float4((float)(dx * g.w[0]), (float)(dy * g.w[1]),
-                                         (float)(dz * g.w[2]), 0.f));
-            }
-        step(cudaMemcpyAsync(h->shifts32, sh.data(), sh.size() * sizeof(float4),
-                             cudaMemcpyHostToDevice, h->stream), "copy shifts");
+        for (const Grid &g : h->grids_h) widths.push_back(make_float4(g.wf[0], g.wf[1], g.wf[2], 0.f));
+        step(cudaMemcpyAsync(h->widths32, widths.data(), widths.size() * sizeof(float4),
+                             cudaMemcpyHostToDevice, h->stream), "copy cell widths");
     }
     // cell centres (c + 0.5) w of every box, and each box's pointer into them
     std::vector<double> ctab;

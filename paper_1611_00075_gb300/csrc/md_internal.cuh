@@ -279,7 +279,7 @@ struct md_system {
     double *ctab = nullptr;           // cell-centre tables of all boxes (Grid::ctab)
     int64_t *atom_off = nullptr;      // device copy of atom_off_h
     uint16_t *rep = nullptr;          // sorted slot -> replica (batches only)
-    float4 *shifts32 = nullptr;       // R x 27 float32 cell shifts (batches only)
+    float4 *widths32 = nullptr;       // float32 cell widths of each box (batches only)
     double *rep_ke = nullptr, *rep_pe = nullptr;  // per-replica sums (device)
     double *rep_part = nullptr;       // their partial sums, (PE, KE) x kRepParts each
     mdg::ForceConsts fc{};

@@ -1,7 +1,6 @@
 """The float64 passes on both sides of their lanes-per-atom limits (16 up to
 3,072 atoms, 8 up to 8,192, 4 up to 32,768, then one), with lists whose last
-quad is ragged,
-and in units whose squared lengths float32 cannot hold.
+quad is ragged, and in units whose squared lengths float32 cannot hold.
 
 Tolerance: a force is a sum of about 60 (Sutton-Chen: 150) terms of at most
 some 30 times the rms force, each right to a few units of 2^-53, so it is
