@@ -296,8 +296,9 @@ md_status md_get_atom_energy(md_system *h, double *e_dev);
  * Sutton-Chen and the embedded-atom potential, and batches, under
  * MD_SCHED_GRID); the persistent schedulers drive the one-box, one-species
  * full-list Lennard-Jones pass of either precision and its two-atom pass,
- * and every other combination runs one thread per atom (per slot, per
- * i-cluster). */
+ * and every other combination -- and a system whose items all fit the
+ * resident CTAs -- runs one thread per atom (per slot, per i-cluster; small
+ * systems several lanes). */
 md_status md_set_variant(md_system *h, int32_t force_variant, int32_t scheduler);
 
 /* Colour of every cell of an ncell_host[0] x [1] x [2] grid (each >= 3) as
