@@ -94,6 +94,7 @@ struct DevStatus {
 // its own when a list is built without binning): the slot lists' counts or the
 // per-atom rows'.
 __device__ __forceinline__ void reset_list_counts(DevStatus *ds, bool slots) {
+    ds->list_done = 0;  // a build that overflowed stops its later blocks uncounted
     if (slots) {
         ds->pair_max = 0;
         ds->pair_entries = 0;
