@@ -243,9 +243,10 @@ lj_mixed_persist(ForceArgs a, int store_f, SchedArgs sa, PairArgs pa) {
     static_assert(!(F64 && MULTI), "batches run the mixed path");
     static_assert(!(PAIRED && (F64 || MULTI || ENERGY)), "slots: one box, mixed path, forces");
     // Per-atom tiles of one box read the cell shifts from a table here: computed
-    // ones made the tiles' timings, which train the cost model, noisier (held-out
-    // spread of 64 parts 0.0215-0.0225 against 0.0224-0.0269) and the launch no
-    // shorter.
+    // ones made the launch 6-8 % shorter (2.1 M porous atoms: 319 -> 293 us) but the
+    // tiles' timings, which train the cost model, noisier: the model's held-out
+    // spread over 64 parts went from 0.0215-0.0225 to 0.0224-0.0269, no longer
+    // surely below the pair count's.
     constexpr bool kTable = F64 || !(MULTI || PAIRED);
     __shared__ typename std::conditional<kTable, ShiftTab, int>::type sh;
     __shared__ typename std::conditional<F64, Home64, int>::type home;
