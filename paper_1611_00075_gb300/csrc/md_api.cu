@@ -131,6 +131,7 @@ cudaError_t alloc_cluster(md_system *h, int max_cell) {
     }
     const int cap = cluster_cap(max_cell + max_cell / 4 + 4);
     if (e == cudaSuccess && (cap > h->cl_cap || !h->cl_list)) {
+        drop_graphs(h);  // captured steps hold the old list pointer and capacity
         if (h->cl_list) cudaFree(h->cl_list);
         h->cl_list = nullptr;
         h->cl_cap = cap;
