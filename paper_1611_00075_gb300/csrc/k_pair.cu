@@ -155,11 +155,14 @@ pair_list_kernel(int n, Grid g, const Grid *__restrict__ grids, const uint16_t *
                     const int b = start[cn], e = start[cn + 1];
                     const CandGroup *gp = cand + cell_group0(cn, b);
                     const int ng = (e - b + 3) >> 2;
+                    // every lane makes the warp's largest number of rounds, so that
+                    // all of them vote together on emptying the queues
+                    const int ngw = (int)__reduce_max_sync(0xffffffffu, (unsigned)ng);
                     uint32_t ent = (st << kIndexBits) | (uint32_t)b;
                     // HOME: the slot's own cell, the only one that holds i0 and i1
                     auto scan = [&](auto home) {
                         constexpr bool HOME = decltype(home)::value;
-                        for (int g0 = 0; g0 < ng; g0 += kListChunk) {
+                        for (int g0 = 0; g0 < ngw; g0 += kListChunk) {
                             const int ge = min(ng, g0 + kListChunk);
                             for (int gi = g0; gi < ge; ++gi, ent += 4) {
                                 const float4 X = __ldg(&gp[gi].x), Y = __ldg(&gp[gi].y),
@@ -189,7 +192,7 @@ pair_list_kernel(int n, Grid g, const Grid *__restrict__ grids, const uint16_t *
                                 take(rb.x, pb.x, ent + 2);
                                 take(rb.y, pb.y, ent + 3);
                             }
-                            if (WRITE && __any_sync(__activemask(), qp - q0p > kListHigh * kPairBlock))
+                            if (WRITE && __any_sync(0xffffffffu, qp - q0p > kListHigh * kPairBlock))
                                 empty();
                         }
                     };
