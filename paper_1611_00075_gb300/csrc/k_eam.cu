@@ -77,7 +77,7 @@ __device__ __forceinline__ double eam_dF(const EamTab &t, double rho) {
     // float32 rate (986 k atoms, 50 steps: 14.83 -> 14.66 ms).
     const double d = 2.0 * t.B * rho;
     if (!(rho > 0.0)) return d;
-    return fma(-0.5 * t.A, rsqrt_f64(rho, rho > 1e-30 && rho < 1e30), d);
+    return fma(-0.5 * t.A, rsqrt_f64(rho, rho < 1e30 ? kSeedHi : kNoSeed), d);
 }
 __device__ __forceinline__ double eam_F(const EamTab &t, double rho) {
     return -t.A * sqrt(rho) + t.B * rho * rho;

@@ -46,16 +46,19 @@ __device__ __forceinline__ double f64_bits(float f) {
 }
 
 // 1/x (Newton's iteration with its second-order term) and 1/sqrt(x) (the
-// binomial series of the residual), from a float32 seed; x positive.  seeded =
-// false (r_c^2 far outside float32's comfortable range): the library's forms.
-__device__ __forceinline__ double rcp_f64(double x, bool seeded) {
-    if (!seeded) return 1.0 / x;
+// binomial series of the residual), from a float32 seed; x not negative.  An x
+// whose high word lies below seed_hi takes the library's forms: x = 0 (two atoms
+// at one place: infinity) and anything below float32's normal range, which
+// f32_bits cannot hold, or (kNoSeed) every x, where r_c^2 itself is far outside
+// float32's comfortable range.
+__device__ __forceinline__ double rcp_f64(double x, int seed_hi) {
+    if (__double2hiint(x) < seed_hi) return 1.0 / x;
     const double y = f64_bits(rcp_fast(f32_bits(x)));
     const double e = fma(-x, y, 1.0);
     return fma(y, fma(e, e, e), y);
 }
-__device__ __forceinline__ double rsqrt_f64(double x, bool seeded) {
-    if (!seeded) return 1.0 / sqrt(x);
+__device__ __forceinline__ double rsqrt_f64(double x, int seed_hi) {
+    if (__double2hiint(x) < seed_hi) return 1.0 / sqrt(x);
     const double y = f64_bits(rsqrt_fast(f32_bits(x)));
     const double e = fma(-(x * y), y, 1.0);
     return fma(y * e, fma(e, 0.375, 0.5), y);

@@ -149,9 +149,9 @@ __device__ __forceinline__ void lj_fp64_atom(const ForceArgs &a, const ShiftTab 
         const float4 qi = a.xq[i];
         qw = qi.w;
         const double sig2 = a.fc.sig2, e48 = a.fc.eps48;
-        const bool seeded = a.fc.f64_seeded;
+        const int seed_hi = a.fc.f64_seed_hi;
         f64_pairs<P>(a, sh, h, i, part, qi, [&](int, double ex, double ey, double ez, double r2) {
-            const double r2i = rcp_f64(r2, seeded);
+            const double r2i = rcp_f64(r2, seed_hi);
             double s6 = sig2 * r2i;
             s6 = s6 * s6 * s6;
             const double fs = (e48 * r2i) * fma(s6, s6, -0.5 * s6);
@@ -563,10 +563,10 @@ __device__ __forceinline__ void lj_typed_fp64_atom(const ForceArgs &a, const Typ
         load_row<NT>(tt.e4d, ti, e4);
         load_row<NT>(tt.s2d, ti, s2);
         load_row<NT>(tt.shd, ti, shd);
-        const bool seeded = a.fc.f64_seeded;
+        const int seed_hi = a.fc.f64_seed_hi;
         f64_pairs<P>(a, sh, h, i, part, qi, [&](int j, double ex, double ey, double ez, double r2) {
             const int tj = species_of(__float_as_uint(__ldg(&a.xq[j].w)));
-            const double r2i = rcp_f64(r2, seeded);
+            const double r2i = rcp_f64(r2, seed_hi);
             double s6 = pick_row<NT>(s2, tj) * r2i;
             s6 = s6 * s6 * s6;
             const double fs = (pick_row<NT>(e48, tj) * r2i) * fma(s6, s6, -0.5 * s6);

@@ -165,14 +165,14 @@ __global__ void __launch_bounds__(kF64Block) sc_density_fp64(ForceArgs a) {
     if (on) {
         const double A = a.fc.sc_a, A2 = A * A;
         const int m = a.fc.sc_m;
-        const bool seeded = a.fc.f64_seeded;
+        const int seed_hi = a.fc.f64_seed_hi;
         f64_pairs<P>(a, &sh, &home, i, part, a.xq[i],
                      [&](int, double, double, double, double r2) {
                          if (ME > 0 ? (ME & 1) : (m & 1)) {
-                             const double ar = A * rsqrt_f64(r2, seeded);
+                             const double ar = A * rsqrt_f64(r2, seed_hi);
                              R += ar_pow_f64<ME>(ar * ar, ar, m);
                          } else {
-                             R += ar_pow_f64<ME>(A2 * rcp_f64(r2, seeded), 0.0, m);
+                             R += ar_pow_f64<ME>(A2 * rcp_f64(r2, seed_hi), 0.0, m);
                          }
                      });
     }
@@ -306,16 +306,16 @@ __global__ void __launch_bounds__(kF64Block) sc_force_fp64(ForceArgs a, int stor
         const int nexp = a.fc.sc_n, mexp = a.fc.sc_m;
         const double nd = (double)(NE > 0 ? NE : nexp), mD = (double)(ME > 0 ? ME : mexp);
         const bool odd = NE > 0 ? ((NE | ME) & 1) : ((nexp | mexp) & 1);
-        const bool seeded = a.fc.f64_seeded;
+        const int seed_hi = a.fc.f64_seed_hi;
         f64_pairs<P>(a, &sh, &home, i, part, qi,
                      [&](int j, double ex, double ey, double ez, double r2) {
                          double ar = 0.0, r2i;
                          if (odd) {
-                             const double y = rsqrt_f64(r2, seeded);
+                             const double y = rsqrt_f64(r2, seed_hi);
                              ar = A * y;
                              r2i = y * y;
                          } else {
-                             r2i = rcp_f64(r2, seeded);
+                             r2i = rcp_f64(r2, seed_hi);
                          }
                          const double s = A2 * r2i;
                          const double Phi = eps * ar_pow_f64<NE>(s, ar, nexp);

@@ -891,10 +891,11 @@ static md_status create_impl(md_system **out, const md_params *p, int R, const i
     // float32 decides distances to a band of 2^-14 while squared lengths stay
     // far from its limits; in units beyond that the float64 path decides all
     // of them in float64 (NaN bounds fail every comparison)
-    fc.f64_seeded = rc2 > 1e-24 && h->rl2 < 1e24;
-    fc.scr_lo = fc.f64_seeded ? (float)(rc2 * (1.0 - 1.0 / 16384.0)) : NAN;
-    fc.scr_hi = fc.f64_seeded ? (float)(rc2 * (1.0 + 1.0 / 16384.0)) : NAN;
-    if (p->precision == MD_FP64 && !fc.f64_seeded) h->list_lo = h->list_hi = NAN;
+    const bool seeded = rc2 > 1e-24 && h->rl2 < 1e24;
+    fc.f64_seed_hi = seeded ? kSeedHi : kNoSeed;
+    fc.scr_lo = seeded ? (float)(rc2 * (1.0 - 1.0 / 16384.0)) : NAN;
+    fc.scr_hi = seeded ? (float)(rc2 * (1.0 + 1.0 / 16384.0)) : NAN;
+    if (p->precision == MD_FP64 && !seeded) h->list_lo = h->list_hi = NAN;
 
     const size_t N = (size_t)n, C = (size_t)cells_total;
     const size_t scan_len = std::max(N, C + 1) / (kBlock * 8) + 4;

@@ -203,6 +203,10 @@ __host__ __device__ __forceinline__ int64_t cell_group0(int cell, int start) {
 }
 inline int64_t cand_groups(int64_t n, int ncells) { return n / 4 + ncells + 1; }
 
+// High words of float64: float32's smallest normal number (2^-126), and one above
+// every number's (no float32 seeds).
+constexpr int kSeedHi = 0x38100000, kNoSeed = 0x7fffffff;
+
 // Per-launch scalars of the force kernels.
 struct ForceConsts {
     float rc2f, eps4f, eps48f, sig2f, shiftf;  // LJ in fp32
@@ -215,9 +219,10 @@ struct ForceConsts {
     double dt, inv_m;
     float half_skin2f;
     // float64 passes: the float32 screen around r_c^2 (NaN: undecided, every
-    // entry goes to the float64 test) and whether float32 seeds serve
+    // entry goes to the float64 test) and the high word of the smallest squared
+    // distance whose reciprocal starts from a float32 seed
     float scr_lo, scr_hi;
-    bool f64_seeded;
+    int f64_seed_hi;
     // multi-element Lennard-Jones: species count (0 = one species) and the
     // inverse mass of each species; an atom's species sits in bits 27-28 of
     // its float32 position's w word, above the original id
