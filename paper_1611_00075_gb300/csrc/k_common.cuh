@@ -37,6 +37,55 @@ __device__ __forceinline__ T split_sum(T x) {
     return x;
 }
 
+// A normal float32 as float64 by integer operations (the conversion instruction runs
+// on the float64 pipe).
+__device__ __forceinline__ bool normal_f32(float f) {
+    return (__float_as_uint(f) & 0x7fffffffu) - 0x00800000u < 0x7f000000u;
+}
+__device__ __forceinline__ double widen_f32(float f) {
+    const unsigned b = __float_as_uint(f);
+    return __hiloint2double(
+        (int)((((b & 0x7fffffffu) >> 3) + 0x38000000u) | (b & 0x80000000u)), (int)(b << 29));
+}
+
+// s + e = a + b exactly (Knuth's two-sum), s the rounded sum.
+__device__ __forceinline__ void two_sum(float a, float b, float &s, float &e) {
+    s = __fadd_rn(a, b);
+    const float t = __fsub_rn(s, a);
+    e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, t)), __fsub_rn(b, t));
+}
+
+// The sums over an item's P lanes (4 or 8, aligned) of the float32 values x, y, z
+// and e: the lane with part & 3 = 0, 1, 2, 3 returns that of x, y, z, e (every lane
+// of the warp calls it).  The lanes' values are added as pairs of floats, 48 bits,
+// and once in float64: what is rounded off is below 2^-45 of the largest partial
+// sum, while each value carries float32's own rounding.  Each exchange halves what
+// a lane still holds.  (Float64 additions wait for a pipe of 1/64 of the float32
+// rate: one step of 16,384 atoms 17.5 us with them, 15.9 with plain float32 sums,
+// 16.2 in this form; 864 atoms 9.6, 9.4 and 9.4.)
+template <int P>
+__device__ __forceinline__ double split_component(float x, float y, float z, float e, int part) {
+    static_assert(P == 4 || P == 8, "one lane per component");
+    constexpr unsigned full = 0xffffffffu;
+    const bool hi = part & 2, lo = part & 1;
+    float s0, r0, s1, r1, s, r;
+    two_sum(hi ? z : x, __shfl_xor_sync(full, hi ? x : z, 2), s0, r0);
+    two_sum(hi ? e : y, __shfl_xor_sync(full, hi ? y : e, 2), s1, r1);
+    const float ss = __shfl_xor_sync(full, lo ? s0 : s1, 1);
+    const float rr = __shfl_xor_sync(full, lo ? r0 : r1, 1);
+    two_sum(lo ? s1 : s0, ss, s, r);
+    r += (lo ? r1 : r0) + rr;
+    if (P == 8) {
+        const float s8 = __shfl_xor_sync(full, s, 4), r8 = __shfl_xor_sync(full, r, 4);
+        float t;
+        two_sum(s, s8, s, t);
+        r += r8 + t;
+    }
+    // zero, infinity and NaN have no rest (nor has a denormal sum)
+    if (!normal_f32(s)) return (double)s;
+    return widen_f32(s) + (normal_f32(r) ? widen_f32(r) : 0.0);
+}
+
 // pair(entry) for every entry of the quads part, part + P, ... of an item's list
 // (lq: its first quad; quads lie 32 apart), one quad loaded ahead.
 template <int P, class Pair>
@@ -221,7 +270,9 @@ __device__ __forceinline__ void split_epilogue(const ForceArgs &a, int i, int c,
 // Lanes per work item (atom or two-atom slot) of the mixed passes: one item's
 // list is a serial chain of gathers, so a system that leaves most of the GPU
 // idle is split.  The lanes' float32 sums cover at most cap / P entries, kept
-// within the 64 of the one-lane kernels' chunks.  Force launch (LJ, timed by
+// within the 64 of the one-lane kernels' chunks; per-atom rows add them as
+// pairs of floats (split_component), where one lane adds its chunks in float64;
+// slots add in float32, as one lane does.  Force launch (LJ, timed by
 // events, which add about 4 us), one lane / four / eight: per-atom lists 14.0 /
 // 9.8 / 7.9 us at 864 atoms, 14.2 / 9.8 / 8.1 at 4,000, 16.0 / 13.8 / 24 at
 // 32,000, 22.5 / 33 / 51 at 87,808 (float64 instructions of the epilogue); slots

@@ -15,7 +15,8 @@
 //          float32, computed from cell-relative float32 coordinates plus the
 //          float32 cell shift of the entry's stencil cell (stencil_of); each chunk of
 //          64 entries is summed in float32 and the chunk sums are added in
-//          float64 (the GPU form of the paper's blocked pair loop).  Entries
+//          float64 (the GPU form of the paper's blocked pair loop; where lanes
+//          share an atom, their sums of at most 64 entries as pairs of floats).  Entries
 //          arrive four at a time (one 16-byte load), so four gathers are in
 //          flight before the arithmetic that needs them.
 //   FP64   everything in float64 (the plain path).
@@ -82,20 +83,16 @@ __device__ __forceinline__ void lj_mixed_atom(const ForceArgs &a, int i, int sto
         }
     };
     if constexpr (P > 1) {
-        // the float32 sums cover a P-th of the list
+        // the float32 sums cover a P-th of the list, at most a chunk's 64 entries
         const int c = part & 3;
         const SplitState t = load_split_state<MODE>(a, i, c, on && part < 4);
         split_quads<P>(lq, on ? nq : 0, part, pair);
-        fx = split_sum<P>(fx);
-        fy = split_sum<P>(fy);
-        fz = split_sum<P>(fz);
+        const double F = split_component<P>(fx, fy, fz, e, part);
         if (ENERGY) {
-            e = split_sum<P>(e);
             if (on) count_pairs(a.ds, npair);
-            if (on && part == 0) a.e_atom[i] = 0.5 * (double)e;
+            if (on && part == 3) a.e_atom[i] = 0.5 * F;
         }
-        split_epilogue<MODE>(a, i, c, on && part < 4, (double)(c == 0 ? fx : (c == 1 ? fy : fz)),
-                             qi.w, t, store_f);
+        split_epilogue<MODE>(a, i, c, on && part < 4, F, qi.w, t, store_f);
         return;
     } else {
         // list quads stream through once (evict-first), one quad loaded ahead;
@@ -501,16 +498,12 @@ __device__ __forceinline__ void lj_typed_mixed_atom(const ForceArgs &a, const Ty
         const int c = part & 3;
         const SplitState t = load_split_state<MODE>(a, i, c, on && part < 4);
         split_quads<P>(lq, on ? nq : 0, part, pair);
-        fx = split_sum<P>(fx);
-        fy = split_sum<P>(fy);
-        fz = split_sum<P>(fz);
+        const double F = split_component<P>(fx, fy, fz, e, part);
         if (ENERGY) {
-            e = split_sum<P>(e);
             if (on) count_pairs(a.ds, npair);
-            if (on && part == 0) a.e_atom[i] = 0.5 * (double)e;
+            if (on && part == 3) a.e_atom[i] = 0.5 * F;
         }
-        split_epilogue<MODE, true>(a, i, c, on && part < 4,
-                                   (double)(c == 0 ? fx : (c == 1 ? fy : fz)), qi.w, t, store_f);
+        split_epilogue<MODE, true>(a, i, c, on && part < 4, F, qi.w, t, store_f);
         return;
     }
     uint4 nxt = nq > 0 ? __ldcs(lq) : make_uint4(0u, 0u, 0u, 0u);
