@@ -272,15 +272,20 @@ __device__ __forceinline__ void split_epilogue(const ForceArgs &a, int i, int c,
 // idle is split.  The lanes' float32 sums cover at most cap / P entries, kept
 // within the 64 of the one-lane kernels' chunks; per-atom rows add them as
 // pairs of floats (split_component), where one lane adds its chunks in float64;
-// slots add in float32, as one lane does.  Force launch (LJ, timed by
-// events, which add about 4 us), one lane / four / eight: per-atom lists 14.0 /
-// 9.8 / 7.9 us at 864 atoms, 14.2 / 9.8 / 8.1 at 4,000, 16.0 / 13.8 / 24 at
-// 32,000, 22.5 / 33 / 51 at 87,808 (float64 instructions of the epilogue); slots
-// of two atoms 22.0 / - / 8.7 at 864, 24.1 / - / 8.6 at 4,000, 23.8 / 16.7 at
-// 32,000, 26.1 / 25.7 at 87,808 atoms.
-inline int mixed_split(int64_t items, int cap) {
-    if (items <= 16384 && cap <= 8 * 4 * kChunkQ) return 8;
-    if (items <= 65536 && cap <= 4 * 4 * kChunkQ) return 4;
+// slots add in float32, as one lane does.
+// One step (LJ, replayed, disordered fcc), us.  Four lanes end where one lane takes
+// the same time: per-atom rows, four / one, 17.6 / 19.6 at 42,592 atoms, 19.7 / 20.1
+// at 46,552, 20.1 / 19.7 at 48,668, 21.2 / 20.2 at 55,296; slots of two, by atoms,
+// 26.6 / 30.5 at 87,808, 32.6 / 32.6 at 119,164, 34.6 / 34.4 at 131,072.  Eight lanes
+// against four: rows 9.9 / 11.4 at 864 atoms, 11.7 / 11.9 at 5,324, 13.0 / 12.5 at
+// 8,788, 16.0 / 14.8 at 16,384; slots 11.7 / 13.0 at 864, 13.7 / 14.0 at 13,500,
+// 19.9 / 17.6 at 32,000.  They go past the crossing (6,000 atoms, 7,000 slots) because
+// lanes set the order of an item's sums: a batch moves its boxes bit for bit as they
+// move alone only while the batch and each box have the same lanes.
+constexpr int64_t kEightLanes = 16384, kFourLanesAtoms = 47104, kFourLanesSlots = 61440;
+inline int mixed_split(int64_t items, int cap, int64_t four) {
+    if (items <= kEightLanes && cap <= 8 * 4 * kChunkQ) return 8;
+    if (items <= four && cap <= 4 * 4 * kChunkQ) return 4;
     return 1;
 }
 // Eight lanes or one, for the passes with more work per entry; each says its limit.

@@ -715,7 +715,7 @@ cudaError_t launch_lj(md_system *h, int mode, bool energy, bool store_f) {
     cudaStream_t s = h->stream;
     if (h->fc.ntypes > 0) return launch_lj_typed(h, a, mode, energy, sf);
     if (h->p.precision == MD_MIXED) {
-        const int P = mixed_split(h->n, h->cap);
+        const int P = mixed_split(h->n, h->cap, kFourLanesAtoms);
         if (h->R > 1)
             return P == 8 ? launch_lj_mixed<true, 8>(a, mode, energy, sf, s)
                  : P == 4 ? launch_lj_mixed<true, 4>(a, mode, energy, sf, s)

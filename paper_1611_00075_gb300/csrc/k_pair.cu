@@ -410,7 +410,7 @@ static cudaError_t launch_pair_lj(md_system *h, int mode, bool energy, int sf) {
 cudaError_t launch_pair_forces(md_system *h, int mode, bool energy, bool store_f) {
     if (h->fc.ntypes > 0) return launch_pair_typed_forces(h, mode, energy, store_f);
     const int sf = store_f ? 1 : 0;
-    const int P = mixed_split(h->n / 2, h->ps_cap);
+    const int P = mixed_split(h->n / 2, h->ps_cap, kFourLanesSlots);
     if (h->R > 1)
         return P == 8 ? launch_pair_lj<true, 8>(h, mode, energy, sf)
              : P == 4 ? launch_pair_lj<true, 4>(h, mode, energy, sf)
