@@ -1438,6 +1438,18 @@ md_status md_get_cell_costs(md_system *h, float *cycles_dev, int64_t *predicted_
     return MD_OK;
 }
 
+// The forces as the system's own launch gives them, after timed passes of the
+// persistent kernel: where lanes share an item, that kernel (one lane per item)
+// sums in another order, and the next step would start from its bits.
+static md_status restore_forces(md_system *h) {
+    if (persistent_path(h)) return MD_OK;
+    const bool timing = h->timing;
+    h->timing = false;  // no interval of its own
+    const md_status st = enqueue_forces(h, FM_STORE, false, true);
+    h->timing = timing;
+    return st;
+}
+
 // Per-CTA cycles of one timed force pass, reduced on the host to max / mean.
 md_status cta_imbalance(md_system *h, float *out) {
     std::vector<float> c((size_t)h->sched_ctas);
@@ -1483,6 +1495,8 @@ md_status md_cost_model(md_system *h, int32_t op, float *loss_out) {
             MD_CK(cudaMemsetAsync(h->cta_cycles, 0, (size_t)h->sched_ctas * sizeof(float),
                                   h->stream));
             for (int r = 0; r < kPasses; ++r) MD_CK(launch_lj_persist(h, FM_STORE, true, true, true));
+            st = restore_forces(h);
+            if (st != MD_OK) return st;
             MD_CK(launch_cell_features(h, false, false));
             int32_t *cnt_dev = h->samp_flag + 2 * ((size_t)h->g.ncells + 1);
             MD_CK(launch_make_samples(h, kPasses, cnt_dev));
@@ -1539,6 +1553,8 @@ md_status md_cost_model(md_system *h, int32_t op, float *loss_out) {
                                         h->p.scheduler != MD_SCHED_PAIRCOUNT &&
                                             h->p.scheduler != MD_SCHED_MLP,
                                         true));
+            st = restore_forces(h);
+            if (st != MD_OK) return st;
             st = read_status(h);
             if (st != MD_OK) return st;
             h->forces_valid = true;
