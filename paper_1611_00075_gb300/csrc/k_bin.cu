@@ -89,7 +89,8 @@ __device__ __forceinline__ double pack2(int hi, int lo) {
 // Cell of every atom, its slot in the cell (atomic count) and its gather
 // records: (x, y, z, new cell | original id) and (v, replica).  The counts are
 // zero on entry (the scan clears them behind itself).  Resets what the later
-// passes of the rebuild count.
+// passes of the rebuild count (not the list's counts when no list build follows:
+// the last list's stay).
 __global__ void bin_count_kernel(int n, const Grid *__restrict__ grids,
                                  const uint16_t *__restrict__ rep,
                                  const double4 *__restrict__ xr,
@@ -98,13 +99,13 @@ __global__ void bin_count_kernel(int n, const Grid *__restrict__ grids,
                                  const double *__restrict__ v, const int32_t *__restrict__ orig,
                                  int32_t *__restrict__ count, int32_t *__restrict__ new_cell,
                                  int32_t *__restrict__ slot, double4 *__restrict__ tabs,
-                                 double4 *__restrict__ tv, bool slots, DevStatus *ds,
-                                 bool gated, bool count_run) {
+                                 double4 *__restrict__ tv, bool slots, bool list_follows,
+                                 DevStatus *ds, bool gated, bool count_run) {
     if (chain_off(ds, gated)) return;
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         if (count_run) ds->cond_runs += 1;
         ds->max_cell = 0;
-        reset_list_counts(ds, slots);
+        if (list_follows) reset_list_counts(ds, slots);
     }
     const bool fresh = ds->abs_fresh != 0;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
@@ -538,7 +539,7 @@ cudaError_t launch_scan_i32(const int32_t *in, int32_t *out, int n, int32_t *bsu
     return launch_scan<int32_t>(in, out, n, bsum, ds, gated, s);
 }
 
-cudaError_t launch_bin(md_system *h, bool gated, bool count_run) {
+cudaError_t launch_bin(md_system *h, bool gated, bool count_run, bool list_follows) {
     const int n = (int)h->n, nc = h->g.ncells;
     cudaStream_t s = h->stream;
     const int cur = h->cur;
@@ -547,7 +548,8 @@ cudaError_t launch_bin(md_system *h, bool gated, bool count_run) {
     bin_count_kernel<<<gs_blocks(n), kBlock, 0, s>>>(n, h->grids, h->rep, h->xr64[cur], h->cell,
                                                      h->xabs, h->v, h->orig, h->cell_count,
                                                      h->new_cell, h->slot, h->tmp_abs, h->tmp_v,
-                                                     paired, h->ds, gated, count_run);
+                                                     paired, list_follows, h->ds, gated,
+                                                     count_run);
     int32_t *slot_start = paired ? h->ps_start : nullptr;
     const int nb = std::max((nc + kScanTile - 1) / kScanTile, 1);
     const bool prefixed = nb > kScanDirect;

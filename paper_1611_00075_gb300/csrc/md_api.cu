@@ -1042,7 +1042,7 @@ md_status md_energy_batch(md_system *h, double *ke_host, double *pe_host) {
 
 md_status md_bin_cells(md_system *h) {
     if (!h) return fail(nullptr, MD_ERR_INVALID, "md_bin_cells: null handle");
-    MD_CK(launch_bin(h, false));
+    MD_CK(launch_bin(h, false, false, false));
     MD_CK(launch_set_rebuild(h));  // list entries now refer to the old order
     h->list_valid = false;
     h->forces_valid = false;

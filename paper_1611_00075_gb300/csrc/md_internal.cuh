@@ -430,8 +430,9 @@ namespace mdg {
 // Gated chain: count per cell (with the absolute positions and gather
 // records), scan, scatter, order and gather every cell; under the two-atom
 // layout also the slot tables.  bin_launches kernels.  count_run: a chain that
-// runs adds itself to DevStatus::cond_runs.
-cudaError_t launch_bin(md_system *h, bool gated, bool count_run = false);
+// runs adds itself to DevStatus::cond_runs.  list_follows: a list build comes next
+// and counts from zero.
+cudaError_t launch_bin(md_system *h, bool gated, bool count_run = false, bool list_follows = true);
 int bin_launches(const md_system *h);
 // Exclusive scan of int32 counts into int32 starts (starts[n] = total).
 cudaError_t launch_scan_i32(const int32_t *in, int32_t *out, int n, int32_t *bsum,
