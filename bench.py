@@ -43,7 +43,8 @@ POROUS_DESC = ("porous Lennard-Jones solid: 160^3 fcc cells = 16,384,000 sites a
 # kernel sources still hash to the captured version.
 FORCE_SOURCES = ("paper_1611_00075_gb300/csrc/k_lj.cu", "paper_1611_00075_gb300/csrc/k_common.cuh",
                  "paper_1611_00075_gb300/csrc/md_internal.cuh",
-                 "paper_1611_00075_gb300/csrc/k_pair.cuh")
+                 "paper_1611_00075_gb300/csrc/k_pair.cuh",
+                 "paper_1611_00075_gb300/csrc/k_packed.cuh")
 PROFILED_TRAFFIC = {
     # kernel: (sources sha1[:16], DRAM bytes per atom, capture)
     "lj_mixed_persist_paired": ("766f90ca9261abed", 365.8,

@@ -322,7 +322,8 @@ md_status md_cost_model(md_system *h, int32_t op, float *loss_out);
  * each rebuild chain, force evaluation and integrator launch it enqueues
  * (on the handle's stream) and md_stats reports the summed milliseconds and
  * counts per kind, plus the number of kernels launched (those of a rebuild
- * chain only when it ran).  Resets the sums and the launch count.
+ * chain only when it ran; on the default stream those of every step's chain,
+ * whose kernels return at once when no rebuild is due).  Resets the sums and the launch count.
  * Synchronizes. */
 md_status md_set_timing(md_system *h, int32_t on);
 

@@ -18,12 +18,12 @@
 //
 // Launches: five (counting, two of the scan, scatter, order and gather); the
 // slot tables of the two-atom layout come out of the scan (slots per cell, beside
-// the atoms) and of the last pass.  Most steps need no rebuild, and on the
-// default stream they still launch the gated chain, 2 us per idle kernel: with
-// seven launches fewer per step (14 fewer under the two-atom layout) 864 atoms on
-// the default stream run 50 steps in 2.11 instead of 2.60 ms, and the rebuilds
-// of 9.8 M porous atoms, which now read the records once, bring 40 steps from
-// 69.7 to 68.6 ms.
+// the atoms) and of the last pass.  Every step holds the gated chain, and an idle
+// kernel of it costs 0.5 us in a replayed step (2 us where the steps are launched
+// one by one), so the chain is kept short: with the list build six launches, where
+// passes of their own (zeroing, sorting, gathering, slot tables, closing) made
+// eleven, eighteen under the two-atom layout.  The records are read once: 40 steps
+// of 9.8 M porous atoms went from 69.7 to 68.6 ms.
 //
 // A system of several boxes (replicas) numbers its cells consecutively, box
 // after box, so each box's atoms stay one contiguous range of the sorted

@@ -11,11 +11,10 @@ namespace mdg {
 constexpr int kChunkQ = 16;
 
 // 1/x and 1/sqrt(x) in one special-function instruction, within 1 ulp and
-// 2^-22.9 relative.  The .ftz forms: __fdividef and rsqrtf compiled without
-// -ftz also scale denormal and huge arguments (predicated multiplies per call),
-// which no squared distance the cutoff accepts needs.  The pair kernels return
-// the same bits as with those forms on every system measured, and whole runs got
-// shorter: alloy 12.00 -> 11.43 ms, Sutton-Chen 34.8 -> 33.4, batch 15.42 -> 15.07,
+// 2^-22.9 relative.  The .ftz forms: __fdividef and rsqrtf without -ftz also hold
+// for denormal and huge arguments, which no squared distance the cutoff accepts
+// needs, and take longer: the pair kernels return the same bits as with those
+// forms on every system measured, and whole runs got shorter: alloy 12.00 -> 11.43 ms, Sutton-Chen 34.8 -> 33.4, batch 15.42 -> 15.07,
 // porous 9.8 M 71.3 -> 69.7, EAM 15.30 -> 15.11 (the cases' own step counts).
 __device__ __forceinline__ float rcp_fast(float x) {
     float r;
@@ -124,10 +123,6 @@ struct ForceArgs {
     ForceConsts fc;
 };
 
-// Float32 cell shifts (dx, dy, dz) * w of the 27 stencil cells, in shared
-// memory, one array per component: the lanes of a warp read up to 27
-// distinct words of one array, which sit in 27 distinct banks, so each read
-// is a single wavefront (a float4 table costs several).
 // The stencil coordinates (-1, 0 or 1 per axis) of a list entry, whose top five
 // bits hold 9 (z + 1) + 3 (y + 1) + (x + 1).  One funnel shift makes the float
 // 2^23 + that number, and six additions and multiply-adds split it (every
@@ -151,9 +146,9 @@ __device__ __forceinline__ float3 stencil_of(uint32_t ent) {
 }
 static_assert(kIndexBits == 27, "stencil_of's shift");
 
-// |e|^2 in the rounding that every pass over the same pairs uses (the compiler
-// orders ex ex + ey ey + ez ez by what the operands come from): one pair must not
-// be inside r_c for one pass and outside for another.
+// |e|^2 in the rounding that every pass over the same pairs uses (left to the
+// contraction rules, ex ex + ey ey + ez ez gave other bits in other kernels): one
+// pair must not be inside r_c for one pass and outside for another.
 __device__ __forceinline__ float dist2(float ex, float ey, float ez) {
     return fmaf(ez, ez, fmaf(ex, ex, ey * ey));
 }
@@ -164,6 +159,10 @@ __device__ __forceinline__ float3 replica_width(const ForceArgs &a, int r) {
     return make_float3(w.x, w.y, w.z);
 }
 
+// Float32 cell shifts (dx, dy, dz) * w of the 27 stencil cells, in shared
+// memory, one array per component: the lanes of a warp read up to 27
+// distinct words of one array, which sit in 27 distinct banks, so each read
+// is a single wavefront (a float4 table costs several).
 struct ShiftTab {
     float x[32], y[32], z[32];
 };

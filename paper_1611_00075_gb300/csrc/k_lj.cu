@@ -176,7 +176,6 @@ __device__ __forceinline__ void lj_fp64_atom(const ForceArgs &a, const ShiftTab 
 template <bool MULTI>
 constexpr int grid_block() { return MULTI ? 256 : 128; }
 
-//
 // P > 1: thread t serves atom t / P (blocks of 128).
 template <int MODE, bool ENERGY, bool MULTI = false, int P = 1>
 __global__ void __launch_bounds__(P > 1 ? 128 : grid_block<MULTI>(), P > 1 ? 1 : (MULTI ? 4 : 5))

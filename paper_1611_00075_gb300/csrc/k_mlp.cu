@@ -81,7 +81,9 @@ struct GradSmem {
 // sample: FP32-bound.  One block holds 66 KB of shared memory, three run per SM, and
 // the grid is at most one wave, so the second stage adds 456 partials at most
 // (one block per 64 samples before: 8,457 partials of 41 MB, added by one
-// serial thread per parameter in 0.92 ms at 541,199 samples).
+// serial thread per parameter in 0.92 ms at 541,199 samples).  The float32 sums grow
+// with the groups a warp takes: at 541,199 and 4,000,037 samples (10 and 69 groups)
+// the largest error is 2.6e-8 and 8.7e-8 of the gradient's largest entry.
 __global__ void __launch_bounds__(32 * kGradWarps, 3)
 mlp_grad_partial_kernel(const float *__restrict__ X, const float *__restrict__ Y, long long ns,
                         const float *__restrict__ P, float *__restrict__ partial,

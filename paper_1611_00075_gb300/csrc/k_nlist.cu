@@ -43,9 +43,8 @@ __device__ __forceinline__ bool exact_within(const double4 &ai, const double4 &a
     return r2 < rl2;
 }
 
-// The same test for the rare candidates of the float32 band, kept out of line
-// so that the compiler cannot turn it into predicated code that every
-// candidate of the hot loop would issue.
+// The same test for the rare candidates of the float32 band, kept out of line:
+// the hot loop issues none of it for the other candidates.
 __device__ __noinline__ bool exact_within_band(const double4 *__restrict__ xabs, int i, int j,
                                                double shx, double shy, double shz, double rl2) {
     return exact_within(xabs[i], xabs[j], shx, shy, shz, rl2);

@@ -321,9 +321,9 @@ __global__ void pair_dummy_kernel(float4 *xq0, float4 *xq1, float4 *xqf, int n) 
 // cost as many instructions as the first's); with float64 chunk accumulators at
 // 72 registers (7 CTAs) 1.498 ms unpacked and 1.551 ms packed (latency-bound).
 // With the shifts computed (stencil_of), 9 / 8 / 7 CTAs per SM, whole runs: liquid
-// of 1 M atoms 6.49 / 6.17 / 6.30 ms, 64 boxes 13.93 / 12.40 / 13.28 (at 9 the
-// compiler spreads each quad's loads out to fit 56 registers).  The persistent
-// kernel, whose next tile is prefetched, keeps 9 (porous 9.8 M 64.6 / 65.0 / 66.6).
+// of 1 M atoms 6.49 / 6.17 / 6.30 ms, 64 boxes 13.93 / 12.40 / 13.28
+// (9 CTAs leave 56 registers a thread, 8 leave 64).  The persistent kernel, whose
+// next tile is prefetched, keeps 9 (porous 9.8 M 64.6 / 65.0 / 66.6).
 // MULTI: a batch of boxes.
 //
 // P > 1: thread t serves slot t / P.

@@ -130,8 +130,7 @@ __device__ __forceinline__ void split_slot_out(const ForceArgs &a, int i0, bool 
     split_slot_finish<MODE, SPECIES, P>(a, i0, two, on, part, F0, F1, t, t1, store_f);
 }
 
-// MULTI (a batch of boxes, the block's boxes not all in shared memory): the
-// cell widths are those of the slot's box.
+// MULTI (a batch of boxes): the cell widths are those of the slot's box.
 // P > 1: the P lanes of the slot (this one is `part`; on: the slot exists) each
 // walk every P-th quad of its list; lane 0 adds the slot's own pair.
 template <int MODE, bool ENERGY, bool MULTI = false, int P = 1>

@@ -645,7 +645,6 @@ __global__ void __launch_bounds__(kScPairBlock, P > 1 ? 1 : 7) sc_force_pair(For
 
 cudaError_t launch_sc_density(md_system *h) {
     ForceArgs a = make_force_args(h);
-    const int nb = nblocks(a.n);
     if (h->p.force_variant == MD_FORCE_PAIRED) {
         const PairArgs p = make_pair_args(h);
         const int P = split8(h->n / 2, h->ps_cap, kScSplitSlots);
@@ -669,7 +668,6 @@ cudaError_t launch_sc_density(md_system *h) {
 
 cudaError_t launch_sc_force(md_system *h, int mode, bool energy, bool store_f) {
     ForceArgs a = make_force_args(h);
-    const int nb = nblocks(a.n);
     const int sf = store_f ? 1 : 0;
     cudaStream_t s = h->stream;
     if (h->p.force_variant == MD_FORCE_PAIRED) {

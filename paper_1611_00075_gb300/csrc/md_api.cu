@@ -578,8 +578,8 @@ bool default_stream(const md_system *h) {
     return h->stream == nullptr || h->stream == cudaStreamLegacy;
 }
 
-// A side stream counts the launches of a rebuild chain when it runs, the default
-// stream all of them.
+// A side stream counts the launches of a rebuild chain when it runs (the device
+// notes it), the default stream those of every step's chain, idle ones included.
 bool counts_when_run(const md_system *h) { return h->graphs_ok && !default_stream(h); }
 
 // Captures `steps` consecutive steps from the current parity: full steps, or
@@ -1599,7 +1599,7 @@ md_status md_set_timing(md_system *h, int32_t on) {
         h->n_kind[k] = 0;
     }
     h->launches = 0;
-    // rebuild chains run by conditional graph nodes count from here on
+    // rebuild chains counted on the device when they run count from here on
     MD_CK(cudaMemsetAsync(&h->ds->cond_runs, 0, sizeof(long long), h->stream));
     return MD_OK;
 }
