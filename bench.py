@@ -47,11 +47,11 @@ FORCE_SOURCES = ("paper_1611_00075_gb300/csrc/k_lj.cu", "paper_1611_00075_gb300/
                  "paper_1611_00075_gb300/csrc/k_packed.cuh")
 PROFILED_TRAFFIC = {
     # kernel: (sources sha1[:16], DRAM bytes per atom, capture)
-    "lj_mixed_persist_paired": ("766f90ca9261abed", 365.8,
+    "lj_mixed_persist_paired": ("059709e934a8da01", 365.8,
                                 "ncu --set full, porous 80^3 cells (1,223,941 atoms) equilibrated "
                                 "as the bench's input, two atoms per thread, one FM_FUSED_FULL "
                                 "launch of the timed range"),
-    "lj_mixed_persist": ("9e866177b4ed5d5f", 485.0,
+    "lj_mixed_persist": ("059709e934a8da01", 484.9,
                          "ncu --set full, porous 80^3 cells (1,223,941 atoms) equilibrated as the "
                          "bench's input, per-atom lists, one FM_FUSED_FULL launch of the timed "
                          "range"),
