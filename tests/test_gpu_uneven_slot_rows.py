@@ -56,3 +56,20 @@ def test_batch(orc):
         f = a.state()[2].cpu().numpy()
         for r, (p, b) in enumerate(reps):
             compare(orc, f[a.offsets[r]:a.offsets[r + 1]], p, b)
+
+
+@pytest.mark.parametrize("half", [False, True])
+@pytest.mark.parametrize("nc", [9, 20, 24])  # a warp per row (1.6 and 18 thousand atoms), a thread per row
+def test_rows_around_one_atom_cells(orc, nc, half):
+    """Per-atom rows of the same systems: exact sets, empty and one-atom cells
+    among their stencils."""
+    pos, box = blobs(nc, 850 + nc)
+    assert (len(pos) <= 24576) == (nc < 24)
+    off, ids = orc.neighbors_cells(pos, box, 2.8, half=half)
+    cells = np.diff(orc.bin_cells(pos, box, 2.8)[2])
+    assert cells.min() == 0 and (cells == 1).any()
+    fv = md.MD_FORCE_HALF_ATOMIC if half else md.MD_FORCE_FULL
+    with md.System(pos, np.zeros_like(pos), box, precision="mixed", force_variant=fv) as a:
+        goff, gids = a.neighbors(half=half)
+    np.testing.assert_array_equal(goff.cpu().numpy(), off)
+    np.testing.assert_array_equal(gids.cpu().numpy(), ids)
